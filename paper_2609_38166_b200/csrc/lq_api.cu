@@ -28,8 +28,8 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const 
   constexpr bool DIAG = GATE == LQ_GATE_DIAG;
   const Tile t;
   const size_t nh = (size_t)p.batch * p.heads_v;
-  __shared__ uint32_t todo_mask;
-  __shared__ int todo_n[32];
+  __shared__ size_t todo_bh[32];
+  __shared__ int todo_n[32], todo_count, any_due;
   LQ_STAMP(1, 0);
 #ifdef LQ_TIMING
   if (threadIdx.x == 0 && blockIdx.x < 1024) {
@@ -46,37 +46,37 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const 
   if (threadIdx.x == 0) { for (int i = 0; i < 16; i++) lq_bacc[i] = 0; lq_btick = clock64(); }
   bool first_flush_ = true;
 #endif
-  // The CTA owns heads blockIdx.x + k * gridDim.x.  Warp 0 looks at 32 of them at a time (one load each, all in
-  // flight together) and publishes which ones have work and how many records each holds; then the CTA takes
-  // them one after the other, fetching the next one's data into the other staging buffer meanwhile.
-  for (size_t base = blockIdx.x; base < nh; base += 32 * (size_t)gridDim.x) {
+  // Warp 0 puts together the next 32 heads of the CTA (a flush: of those that are due, see find_due_heads; otherwise every
+  // gridDim-th head) and how many records each holds; then the CTA takes them one after the other, fetching the next
+  // one's data into the other staging buffer meanwhile.
+  int count = 32;
+  for (size_t first = blockIdx.x; count == 32; first += 32 * (size_t)gridDim.x) {
     if (t.warp == 0) {
-      const size_t cand = base + t.lane * (size_t)gridDim.x;
-      bool want = false;
-      int n_mine = 0;
-      if (cand < nh) {
-        if (MODE != 1) n_mine = p.win_pos[cand / p.heads_v] & 0xFFFF;
-        want = MODE != 0 || n_mine == p.W || (p.force && n_mine > 0);
+      size_t bh_mine = first + t.lane * (size_t)gridDim.x;
+      int n_mine = 0, c, due = 0;
+      if (MODE == 0) {
+        c = find_due_heads(p, first, gridDim.x, t.lane, bh_mine, n_mine, due);
+      } else {
+        const bool have = bh_mine < nh;
+        if (MODE == 2 && have) n_mine = p.win_pos[bh_mine / p.heads_v] & 0xFFFF;
+        c = __popc(__ballot_sync(FULL, have));
       }
-      const uint32_t m = __ballot_sync(FULL, want);
+      todo_bh[t.lane] = bh_mine;
       todo_n[t.lane] = n_mine > p.W ? p.W : n_mine;
-      if (t.lane == 0) todo_mask = m;
-      // The arrival on win_pos (arrive_and_set: the last head of a sequence to arrive stores 0) only says "this head
-      // has read the old value", which it just did; nobody inside this kernel waits for the 0.  Made here, 32 heads
-      // at once, the atomic's round trip hides behind the wait for the first staging buffer.
-      if (MODE == 0 && want) arrive_and_set(p.win_pos, static_cast<int>(cand / p.heads_v), p.heads_v, 0);
+      if (t.lane == 0) { todo_count = c; any_due = due; }
     }
     __syncthreads();
     LQ_BTICK(0);
-    uint32_t mask = todo_mask;
+    count = todo_count;
+    // one warp reports that this CTA has seen all of win_pos, once the first head's copies are on their way (the round
+    // trip hides behind them); with nothing due there is nothing to restart
+    bool report = MODE == 0 && count < 32 && any_due > 0 && t.warp == 7;
     int buf = 0;
     bool staged = false;                     // the data of the head about to be processed is already on its way
-    while (mask) {
-      const int kbit = __ffs(mask) - 1;
-      mask &= mask - 1;
-      const size_t bh = base + kbit * (size_t)gridDim.x;
+    for (int k = 0; k < count; k++) {
+      const size_t bh = todo_bh[k];
       const int b = static_cast<int>(bh / p.heads_v);
-      const int n = todo_n[kbit];
+      const int n = todo_n[k];
       const BoundarySmem sm(smem, p.W, p.r, DIAG, R16, buf);
       float M[8][8];
       if (MODE == 1) {
@@ -90,16 +90,18 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const 
           cp_async_commit();
         }
         staged = false;
-        if (mask && stage_bufs > 1) {
-          const int knext = __ffs(mask) - 1;
+        if (k + 1 < count && stage_bufs > 1) {
           const BoundarySmem nx(smem, p.W, p.r, DIAG, R16, buf ^ 1);
-          stage_issue<GATE, R16>(p, nx, t, base + knext * (size_t)gridDim.x, todo_n[knext]);
+          stage_issue<GATE, R16>(p, nx, t, todo_bh[k + 1], todo_n[k + 1]);
           cp_async_commit();
           staged = true;
+          if (report) restart_due_windows(p, t.lane);
           cp_async_wait_but_one();
         } else {
+          if (report) restart_due_windows(p, t.lane);
           cp_async_wait_all();
         }
+        report = false;
         __syncthreads();
         LQ_BTICK(1);
 #ifdef LQ_TIMING
@@ -123,7 +125,8 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const 
       if (MODE == 1 && t.tid == 0) p.win_pos[b] = 0;      // (nobody reads win_pos in this mode)
       if (staged) buf ^= 1;
     }
-    __syncthreads();                         // todo_mask / todo_n are rewritten by the next round
+    if (report) restart_due_windows(p, t.lane);
+    __syncthreads();                         // the list is rewritten by the next round
   }
 #ifdef LQ_TIMING
   LQ_STAMP(1, 4);

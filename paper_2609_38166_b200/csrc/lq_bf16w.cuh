@@ -253,11 +253,7 @@ __device__ __forceinline__ void bf16w_boundary_head(const Params &p, unsigned ch
         ws[e] = (uint32_t)to_bf16_bits(M[2 * e][bcol]) | ((uint32_t)to_bf16_bits(M[2 * e + 1][bcol]) << 16);
       *reinterpret_cast<uint4 *>(S0T + (8 * t.tx + bcol) * D + 8 * t.ty) = make_uint4(ws[0], ws[1], ws[2], ws[3]);
     }
-    __syncthreads();
-    if (t.tid == 0) {
-      if (MODE == 0) arrive_and_set(p.win_pos, b, p.heads_v, 0);
-      else p.win_pos[b] = 0;                 // nobody reads win_pos in this mode
-    }
+    if (MODE == 1 && t.tid == 0) p.win_pos[b] = 0;           // nobody reads win_pos in this mode
   }
 }
 
@@ -265,36 +261,37 @@ template <int GATE, int MODE, bool R16>
 __global__ void __launch_bounds__(256, 2) bf16w_boundary_kernel(const Params p) {
   extern __shared__ float4 lq_bf16w_smem4[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(lq_bf16w_smem4);
-  __shared__ uint32_t todo_mask;
-  __shared__ int todo_n[32];
+  __shared__ size_t todo_bh[32];
+  __shared__ int todo_n[32], todo_count, any_due;
   __shared__ float dec_s[MAX_W];
   const Tile t;
   const size_t nh = (size_t)p.batch * p.heads_v;
   grid_dependency_wait();
-  // The CTA owns heads blockIdx.x + k * gridDim.x; warp 0 looks at 32 of them at a time (one load each, all in
-  // flight together) and publishes which are due and how many records each holds.
-  for (size_t base = blockIdx.x; base < nh; base += 32 * (size_t)gridDim.x) {
+  // Warp 0 puts together the next 32 heads of the CTA: of those that are due (find_due_heads), or every gridDim-th head.
+  int count = 32;
+  for (size_t first = blockIdx.x; count == 32; first += 32 * (size_t)gridDim.x) {
     if (t.warp == 0) {
-      const size_t cand = base + t.lane * (size_t)gridDim.x;
-      bool want = false;
-      int n_mine = 0;
-      if (cand < nh) {
-        if (MODE != 1) n_mine = p.win_pos[cand / p.heads_v] & 0xFFFF;
-        want = MODE != 0 || n_mine == p.W || (p.force && n_mine > 0);
+      size_t bh_mine = first + t.lane * (size_t)gridDim.x;
+      int n_mine = 0, c, due = 0;
+      if (MODE == 0) {
+        c = find_due_heads(p, first, gridDim.x, t.lane, bh_mine, n_mine, due);
+      } else {
+        const bool have = bh_mine < nh;
+        if (MODE == 2 && have) n_mine = p.win_pos[bh_mine / p.heads_v] & 0xFFFF;
+        c = __popc(__ballot_sync(FULL, have));
       }
-      const uint32_t m = __ballot_sync(FULL, want);
+      todo_bh[t.lane] = bh_mine;
       todo_n[t.lane] = n_mine > p.W ? p.W : n_mine;
-      if (t.lane == 0) todo_mask = m;
+      if (t.lane == 0) { todo_count = c; any_due = due; }
     }
     __syncthreads();
-    uint32_t mask = todo_mask;
-    while (mask) {
-      const int kbit = __ffs(mask) - 1;
-      mask &= mask - 1;
-      bf16w_boundary_head<GATE, MODE, R16>(p, smem, dec_s, t, base + kbit * (size_t)gridDim.x, todo_n[kbit]);
+    count = todo_count;
+    if (MODE == 0 && count < 32 && any_due > 0 && t.warp == 7) restart_due_windows(p, t.lane);
+    for (int k = 0; k < count; k++) {
+      bf16w_boundary_head<GATE, MODE, R16>(p, smem, dec_s, t, todo_bh[k], todo_n[k]);
       __syncthreads();                       // this head's use of shared memory is over
     }
-    __syncthreads();                         // todo_mask / todo_n are rewritten by the next round
+    __syncthreads();                         // the list is rewritten by the next round
   }
 }
 

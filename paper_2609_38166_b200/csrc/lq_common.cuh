@@ -333,6 +333,70 @@ __device__ __forceinline__ void row_blocks(const float (&M)[8][8], const float (
   }
 }
 
+// ---- the heads that are due for a window boundary ----
+// Position of the k-th set bit of m (k < popc(m)).
+__device__ __forceinline__ int nth_set_bit(uint32_t m, unsigned k) {
+  int pos = 0;
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    const unsigned c = __popc(m & ((1u << s) - 1u));
+    if (k >= c) { k -= c; m >>= s; pos += s; }
+  }
+  return pos;
+}
+
+// The due heads, numbered sequence by sequence, belong to CTA i mod gridDim: with the windows of a serving batch in no
+// particular order, heads handed out by their own index pile up on some CTAs (256 sequences x 32 heads in random order,
+// W = 16: up to five boundaries on one CTA and none on others; a step of 100 us, 73 us with equal shares).
+// One warp finds up to 32 of a CTA's heads in one pass over win_pos: lane l looks for due head number first + l * stride.
+// Returns how many lanes found theirs (lanes 0 .. count-1); bh and n are the head and its buffered records, `total` how
+// many sequences are due in all.
+__device__ __forceinline__ int find_due_heads(const Params &p, size_t first, size_t stride, int lane, size_t &bh, int &n,
+                                              int &total) {
+  constexpr int U = 8;                       // loads in flight per lane
+  const size_t item = first + lane * stride;
+  const unsigned want = static_cast<unsigned>(item / p.heads_v);       // rank of the head's sequence among the due ones
+  unsigned base = 0;
+  bool found = false;
+  bh = 0; n = 0;
+  for (int b0 = 0; b0 < p.batch; b0 += 32 * U) {
+    int v[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) v[u] = b0 + 32 * u + lane < p.batch ? p.win_pos[b0 + 32 * u + lane] & 0xFFFF : 0;
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const uint32_t m = __ballot_sync(FULL, v[u] == p.W || (p.force && v[u] > 0));
+      if (m == 0) continue;
+      const unsigned c = __popc(m);
+      const bool mine = want - base < c;     // (unsigned: false for ranks below base)
+      const int pos = mine ? nth_set_bit(m, want - base) : 0;
+      const int nv = __shfl_sync(FULL, v[u], pos);
+      if (mine) {
+        found = true;
+        n = nv < p.W ? nv : p.W;
+        bh = (size_t)(b0 + 32 * u + pos) * p.heads_v + (item - (size_t)want * p.heads_v);
+      }
+      base += c;
+    }
+  }
+  total = base;
+  return __popc(__ballot_sync(FULL, found));
+}
+
+// A CTA that has seen all of win_pos says so on the upper bits of win_pos[0]; the last one starts the windows of the due
+// sequences afresh (nobody reads win_pos any more, and the boundaries themselves do not need it).  One warp calls this.
+__device__ __forceinline__ void restart_due_windows(const Params &p, int lane) {
+  int old = 0;
+  if (lane == 0) old = atomicAdd(p.win_pos, 0x10000);
+  old = __shfl_sync(FULL, old, 0);
+  if ((old >> 16) != static_cast<int>(gridDim.x) - 1) return;
+  for (int b = lane; b < p.batch; b += 32) {
+    const int v = __ldcg(p.win_pos + b) & 0xFFFF;
+    const bool due = v == p.W || (p.force && v > 0);
+    if (due || b == 0) p.win_pos[b] = due ? 0 : v;
+  }
+}
+
 // Last-arrival bookkeeping on win_pos[b]: bits 16.. count the heads of sequence b that are done with
 // the value in bits 0..15.  The head that arrives last (all heads_v have read the old value by then)
 // stores the new value and thereby clears the counter.  Call from one thread per head, after a

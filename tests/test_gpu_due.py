@@ -1,0 +1,42 @@
+"""GPU: which heads a window boundary takes.  The kernels find the due sequences by looking over all window positions; the
+sizes here are where that can go wrong: one sequence, more sequences than one pass of loads covers (256), more due heads
+per CTA than one list holds (32), windows in random order, all due at once, none due."""
+import numpy as np
+import pytest
+import torch
+
+from oracle.lq_oracle import State as OState
+from paper_2609_38166_b200 import lq, synth
+from tests import gpu_util as gu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("state_bf16", [0, 1])
+@pytest.mark.parametrize("batch,heads_v,heads_qk,W,order", [(1, 1, 1, 4, "last"), (5, 3, 3, 5, "all"), (300, 3, 1, 4, "random"),
+                                                            (257, 2, 2, 3, "none"), (301, 32, 16, 2, "all")])
+def test_boundaries_of_windows_in_any_order(oracle, batch, heads_v, heads_qk, W, order, state_bf16):
+    kw = dict(r=0, smooth=0, state_bf16=1) if state_bf16 else dict(r=2)
+    wl = synth.Workload("due", batch, heads_v, heads_qk, W=W, seed=800 + batch, **kw)
+    osh, lsh = gu.shapes(wl)
+    ost = OState(osh)
+    oracle.quantize_state(osh, synth.dense_states(wl, 3), ost)
+    rng = np.random.default_rng(batch)
+    ost.win_pos[:] = {"last": np.where(np.arange(batch) == batch - 1, W - 1, np.arange(batch) % W), "all": np.full(batch, W - 1),
+                      "random": rng.integers(0, W, batch), "none": np.zeros(batch)}[order]
+    ost.buf_k[...] = rng.standard_normal(ost.buf_k.shape).astype(np.float32) * 0.1
+    ost.buf_u[...] = rng.standard_normal(ost.buf_u.shape).astype(np.float32)
+    ost.buf_a[...] = rng.uniform(0.2, 1.0, ost.buf_a.shape).astype(np.float32)
+    st = gu.state_to_dev(ost, lsh)
+    o = torch.empty((batch, heads_v, 128), dtype=torch.float32, device="cuda")
+    for step in range(2):
+        tok = synth.token_inputs(wl, step)
+        want = oracle.decode_step(osh, ost, **tok)
+        td = gu.tok_dev(tok)
+        lq.decode_step(lsh, st, td["q"], td["k"], td["v"], td["beta"], td["alpha"], o)
+        assert np.array_equal(gu.host(o), want), f"o of step {step}"
+        gu.assert_state_parity(st, ost, wl.r, f"state after step {step}")
+    lq.window_flush(lsh, st, force=True)            # every window that holds records, whatever its fill
+    oracle.window_flush(osh, ost, force=True)
+    gu.assert_state_parity(st, ost, wl.r, "forced flush")
+    assert st.win_pos.tolist() == [0] * batch and lq.check_device() == 0
