@@ -11,130 +11,8 @@
 #include "lq_bf16w.cuh"
 #include "lq_boundary.cuh"
 #include "lq_decode.cuh"
-#include "lq_fused.cuh"
 
 namespace lq {
-
-// ---------------------------------------------------------------------------------------------
-// Boundary kernels: a CTA of 256 threads walks over heads (grid-stride) and takes those that need work.
-// MODE 0: flush (window representation -> dense -> new window representation)
-// MODE 1: quantize dense fp32 states         MODE 2: dequantize to dense fp32 states
-// ---------------------------------------------------------------------------------------------
-// RM: the largest r the instance handles (4, 8 or MAX_R; the fit keeps its small matrices in registers, RM wide).
-template <int GATE, int MODE, bool R16, int RM>
-__global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const int stage_bufs) {
-  extern __shared__ float4 lq_smem4[];
-  float *smem = reinterpret_cast<float *>(lq_smem4);
-  constexpr bool DIAG = GATE == LQ_GATE_DIAG;
-  const Tile t;
-  const size_t nh = (size_t)p.batch * p.heads_v;
-  __shared__ size_t todo_bh[32];
-  __shared__ int todo_n[32], todo_count, any_due;
-  LQ_STAMP(1, 0);
-#ifdef LQ_TIMING
-  if (threadIdx.x == 0 && blockIdx.x < 1024) {
-    unsigned smid_;
-    asm volatile("mov.u32 %0, %smid;" : "=r"(smid_));
-    g_timeline[p.gen & 3][1][5][blockIdx.x] = smid_;
-  }
-#endif
-  grid_dependency_wait();                    // everything the kernel before this one wrote is visible from here on
-  LQ_STAMP(1, 1);
-  // the decode kernel ahead of a flush counts the tickets of its pool of heads in the state's scratch words
-  if (MODE == 0 && p.work != nullptr && blockIdx.x == 0 && threadIdx.x == 0) p.work[0] = 0;
-#ifdef LQ_TIMING
-  if (threadIdx.x == 0) { for (int i = 0; i < 16; i++) lq_bacc[i] = 0; lq_btick = clock64(); }
-  bool first_flush_ = true;
-#endif
-  // Warp 0 puts together the next 32 heads of the CTA (a flush: of those that are due, see find_due_heads; otherwise every
-  // gridDim-th head) and how many records each holds; then the CTA takes them one after the other, fetching the next
-  // one's data into the other staging buffer meanwhile.
-  int count = 32;
-  for (size_t first = blockIdx.x; count == 32; first += 32 * (size_t)gridDim.x) {
-    if (t.warp == 0) {
-      size_t bh_mine = first + t.lane * (size_t)gridDim.x;
-      int n_mine = 0, c, due = 0;
-      if (MODE == 0) {
-        c = find_due_heads(p, first, gridDim.x, t.lane, bh_mine, n_mine, due);
-      } else {
-        const bool have = bh_mine < nh;
-        if (MODE == 2 && have) n_mine = p.win_pos[bh_mine / p.heads_v] & 0xFFFF;
-        c = __popc(__ballot_sync(FULL, have));
-      }
-      todo_bh[t.lane] = bh_mine;
-      todo_n[t.lane] = n_mine > p.W ? p.W : n_mine;
-      if (t.lane == 0) { todo_count = c; any_due = due; }
-    }
-    __syncthreads();
-    LQ_BTICK(0);
-    count = todo_count;
-    // one warp reports that this CTA has seen all of win_pos, once the first head's copies are on their way (the round
-    // trip hides behind them); with nothing due there is nothing to restart
-    bool report = MODE == 0 && count < 32 && any_due > 0 && t.warp == 7;
-    int buf = 0;
-    bool staged = false;                     // the data of the head about to be processed is already on its way
-    for (int k = 0; k < count; k++) {
-      const size_t bh = todo_bh[k];
-      const int b = static_cast<int>(bh / p.heads_v);
-      const int n = todo_n[k];
-      const BoundarySmem sm(smem, p.W, p.r, DIAG, R16, buf);
-      float M[8][8];
-      if (MODE == 1) {
-        const float *S = p.S + bh * (size_t)(D * D);
-#pragma unroll
-        for (int a = 0; a < 8; a++) load8(S + (8 * t.ty + a) * D + 8 * t.tx, M[a]);
-      } else {
-        // (the barrier that ended the previous head's work also freed both staging buffers for writing)
-        if (!staged) {
-          stage_issue<GATE, R16>(p, sm, t, bh, n);
-          cp_async_commit();
-        }
-        staged = false;
-        if (k + 1 < count && stage_bufs > 1) {
-          const BoundarySmem nx(smem, p.W, p.r, DIAG, R16, buf ^ 1);
-          stage_issue<GATE, R16>(p, nx, t, todo_bh[k + 1], todo_n[k + 1]);
-          cp_async_commit();
-          staged = true;
-          if (report) restart_due_windows(p, t.lane);
-          cp_async_wait_but_one();
-        } else {
-          if (report) restart_due_windows(p, t.lane);
-          cp_async_wait_all();
-        }
-        report = false;
-        __syncthreads();
-        LQ_BTICK(1);
-#ifdef LQ_TIMING
-        if (first_flush_) LQ_STAMP(1, 2);
-#endif
-        reconstruct_tile<GATE, R16>(p, sm, t, bh, n, M);
-      }
-      if (MODE == 2) {
-        float *S = p.S + bh * (size_t)(D * D);
-#pragma unroll
-        for (int a = 0; a < 8; a++) store8(S + (8 * t.ty + a) * D + 8 * t.tx, M[a]);
-      } else {
-        quantize_tile<RM>(p, sm, t, bh, MODE == 0 ? n : 0, M);
-      }
-      __syncthreads();                       // this head's use of shared memory is over
-      LQ_BTICK(9);
-#ifdef LQ_TIMING
-      if (first_flush_) LQ_STAMP(1, 3);
-      first_flush_ = false;
-#endif
-      if (MODE == 1 && t.tid == 0) p.win_pos[b] = 0;      // (nobody reads win_pos in this mode)
-      if (staged) buf ^= 1;
-    }
-    if (report) restart_due_windows(p, t.lane);
-    __syncthreads();                         // the list is rewritten by the next round
-  }
-#ifdef LQ_TIMING
-  LQ_STAMP(1, 4);
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < 16; i++) atomicAdd(&g_phase_cycles[32 + i], (unsigned long long)lq_bacc[i]);
-  }
-#endif
-}
 
 // ---------------------------------------------------------------------------------------------
 // Baseline: Eq. 1 on a dense state that is read and written in full every token.
@@ -453,74 +331,35 @@ static lq_status launch_bf16w_boundary(const lq_shape *s, const Params &p, cudaS
               : launch_dependent(bf16w_boundary_kernel<LQ_GATE_SCALAR, MODE, false>, grid, 256, smem, stream, p);
 }
 
+// The boundary kernels are persistent: as many CTAs as are resident at once, each striding over its heads.
+template <int GATE, int MODE, bool R16, int RM>
+static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStream_t stream) {
+  const size_t smem = BoundarySmem<RM>(s->W, s->r, GATE == LQ_GATE_DIAG, R16, MODE != 1, s->n_iter > 1).bytes;
+  auto kernel = boundary_kernel<GATE, MODE, R16, RM>;
+  if (!smem_opt_in(reinterpret_cast<const void *>(kernel), smem)) return LQ_ERR_CUDA;
+  const long resident = (long)ctas_per_sm(reinterpret_cast<const void *>(kernel), 256, smem) * sm_count();
+  if (resident < 1) return LQ_ERR_CUDA;
+  const long nh = (long)s->batch * s->heads_v;
+  return launch_dependent(kernel, static_cast<int>(nh < resident ? nh : resident), 256, smem, stream, p);
+}
+
+template <int MODE, int RM>
+static lq_status launch_boundary_gate(const lq_shape *s, const Params &p, cudaStream_t stream) {
+  if (MODE == 1) return launch_boundary_t<LQ_GATE_SCALAR, MODE, false, RM>(s, p, stream);   // (reads no records)
+  constexpr int M_ = MODE == 1 ? 0 : MODE;
+  if (s->gate == LQ_GATE_DIAG)
+    return s->rec16 ? launch_boundary_t<LQ_GATE_DIAG, M_, true, RM>(s, p, stream) : launch_boundary_t<LQ_GATE_DIAG, M_, false, RM>(s, p, stream);
+  return s->rec16 ? launch_boundary_t<LQ_GATE_SCALAR, M_, true, RM>(s, p, stream) : launch_boundary_t<LQ_GATE_SCALAR, M_, false, RM>(s, p, stream);
+}
+
+// compiled for r <= 4, r <= 8 and any r (the small matrices of the fit live in registers); dequantizing has no fit
 template <int MODE>
 static lq_status launch_boundary(const lq_shape *s, const Params &p, cudaStream_t stream) {
+  if (s->batch == 0) return LQ_OK;
   if (s->state_bf16) return launch_bf16w_boundary<MODE>(s, p, stream);
-  const bool diag = s->gate == LQ_GATE_DIAG;
-  const bool r16 = MODE != 1 && s->rec16 != 0;               // quantizing a dense state reads no records
-  const int bufs = MODE == 1 ? 1 : BoundarySmem::buffers(s->W, s->r, diag, r16);
-  const size_t smem = BoundarySmem::bytes(s->W, s->r, diag, r16, bufs);
-  const long nh = (long)s->batch * s->heads_v;
-  // persistent: the CTAs that are resident at once (two per SM), each striding over the heads
-  const int grid = static_cast<int>(nh < 2L * sm_count() ? nh : 2L * sm_count());
-  // the flush (the hot one) is compiled for r <= 4, r <= 8 and any r; the others once
-  constexpr int M_ = MODE;
-  if (MODE == 0 && s->r <= 4) {
-    if (r16) return diag ? launch_dependent(boundary_kernel<LQ_GATE_DIAG, M_, true, 4>, grid, 256, smem, stream, p, bufs)
-                         : launch_dependent(boundary_kernel<LQ_GATE_SCALAR, M_, true, 4>, grid, 256, smem, stream, p, bufs);
-    return diag ? launch_dependent(boundary_kernel<LQ_GATE_DIAG, M_, false, 4>, grid, 256, smem, stream, p, bufs)
-                : launch_dependent(boundary_kernel<LQ_GATE_SCALAR, M_, false, 4>, grid, 256, smem, stream, p, bufs);
-  }
-  if (MODE == 0 && s->r <= 8) {
-    if (r16) return diag ? launch_dependent(boundary_kernel<LQ_GATE_DIAG, M_, true, 8>, grid, 256, smem, stream, p, bufs)
-                         : launch_dependent(boundary_kernel<LQ_GATE_SCALAR, M_, true, 8>, grid, 256, smem, stream, p, bufs);
-    return diag ? launch_dependent(boundary_kernel<LQ_GATE_DIAG, M_, false, 8>, grid, 256, smem, stream, p, bufs)
-                : launch_dependent(boundary_kernel<LQ_GATE_SCALAR, M_, false, 8>, grid, 256, smem, stream, p, bufs);
-  }
-  if (r16)
-    return diag ? launch_dependent(boundary_kernel<LQ_GATE_DIAG, MODE == 1 ? 0 : MODE, true, MAX_R>, grid, 256, smem, stream, p, bufs)
-                : launch_dependent(boundary_kernel<LQ_GATE_SCALAR, MODE == 1 ? 0 : MODE, true, MAX_R>, grid, 256, smem, stream, p, bufs);
-  return diag ? launch_dependent(boundary_kernel<LQ_GATE_DIAG, MODE, false, MAX_R>, grid, 256, smem, stream, p, bufs)
-              : launch_dependent(boundary_kernel<LQ_GATE_SCALAR, MODE, false, MAX_R>, grid, 256, smem, stream, p, bufs);
-}
-
-// The step as one cooperative kernel (lq_fused.cuh): one decode CTA and one boundary CTA per SM.
-static bool fused_step_wanted(long nh) {
-  // Off unless LQ_FUSED_STEP=1 is set: on B200 the fused kernel is slower than the two kernels (a boundary CTA
-  // alone on an SM is latency-bound and takes 21 us per head where two of them sharing an SM take 12 us each,
-  // and the registers of an SM do not hold two boundary CTAs next to the decode slots).
-  (void)nh;
-  const char *e = getenv("LQ_FUSED_STEP");
-  return e && atoi(e) != 0;
-}
-
-template <int GATE, bool R16>
-static lq_status launch_fused_step_t(const lq_shape *s, const Params &p, cudaStream_t stream) {
-  const bool diag = GATE == LQ_GATE_DIAG;
-  const size_t smem = fused_smem_bytes(s->W, s->r, diag, R16);
-  auto kernel = fused_step_kernel<GATE, R16>;
-  if (smem > 227 * 1024) return LQ_ERR_UNSUPPORTED;
-  if (!smem_opt_in(reinterpret_cast<const void *>(kernel), smem)) return LQ_ERR_UNSUPPORTED;
-  if (ctas_per_sm(reinterpret_cast<const void *>(kernel), 256, smem) < 2)
-    return LQ_ERR_UNSUPPORTED;               // two CTAs per SM are the design
-  const long nh = (long)s->batch * s->heads_v;
-  const int sms = sm_count();
-  if (nh > (long)sms * FUSED_SLOTS * FUSED_NBUF || nh > (long)sms * 2048) return LQ_ERR_UNSUPPORTED;
-  int decode_ctas = sms;
-  Params pp = p;
-  void *args[] = {&pp, &decode_ctas};
-  if (cudaLaunchCooperativeKernel(reinterpret_cast<void *>(kernel), dim3(2 * sms), dim3(256), args, smem, stream) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    return LQ_ERR_CUDA;
-  }
-  return LQ_OK;
-}
-
-static lq_status launch_fused_step(const lq_shape *s, const Params &p, cudaStream_t stream) {
-  const bool diag = s->gate == LQ_GATE_DIAG;
-  if (s->rec16) return diag ? launch_fused_step_t<LQ_GATE_DIAG, true>(s, p, stream) : launch_fused_step_t<LQ_GATE_SCALAR, true>(s, p, stream);
-  return diag ? launch_fused_step_t<LQ_GATE_DIAG, false>(s, p, stream) : launch_fused_step_t<LQ_GATE_SCALAR, false>(s, p, stream);
+  if (MODE == 2 || s->r <= 4) return launch_boundary_gate<MODE, 4>(s, p, stream);
+  if (s->r <= 8) return launch_boundary_gate<MODE, MODE == 2 ? 4 : 8>(s, p, stream);
+  return launch_boundary_gate<MODE, MODE == 2 ? 4 : MAX_R>(s, p, stream);
 }
 
 }  // namespace lq
@@ -564,10 +403,6 @@ static lq_status decode_step_impl(const lq_shape *shape, const lq_state *state, 
       return LQ_ERR_CUDA;
     }
     return launch_boundary<0>(shape, p, st);
-  }
-  if (!between && fused_step_wanted(nh)) {
-    lq_status frc = launch_fused_step(shape, p, st);
-    if (frc != LQ_ERR_UNSUPPORTED) return frc;       // does not fit this device or shape: the two kernels below
   }
   const size_t smem = DecodeSlot(shape->W, shape->r, diag, r16).bytes;
   const bool longw = shape->W - 1 > REC_SEG;               // windows whose records come in more than one segment

@@ -261,17 +261,17 @@ template <int GATE, int MODE, bool R16>
 __global__ void __launch_bounds__(256, 2) bf16w_boundary_kernel(const Params p) {
   extern __shared__ float4 lq_bf16w_smem4[];
   unsigned char *smem = reinterpret_cast<unsigned char *>(lq_bf16w_smem4);
-  __shared__ size_t todo_bh[32];
+  __shared__ unsigned todo_bh[32];
   __shared__ int todo_n[32], todo_count, any_due;
   __shared__ float dec_s[MAX_W];
   const Tile t;
-  const size_t nh = (size_t)p.batch * p.heads_v;
+  const unsigned nh = static_cast<unsigned>(p.batch) * p.heads_v;
   grid_dependency_wait();
   // Warp 0 puts together the next 32 heads of the CTA: of those that are due (find_due_heads), or every gridDim-th head.
   int count = 32;
-  for (size_t first = blockIdx.x; count == 32; first += 32 * (size_t)gridDim.x) {
+  for (unsigned first = blockIdx.x; count == 32; first += 32 * gridDim.x) {
     if (t.warp == 0) {
-      size_t bh_mine = first + t.lane * (size_t)gridDim.x;
+      unsigned bh_mine = first + t.lane * gridDim.x;
       int n_mine = 0, c, due = 0;
       if (MODE == 0) {
         c = find_due_heads(p, first, gridDim.x, t.lane, bh_mine, n_mine, due);

@@ -1,258 +1,144 @@
-// Window-boundary work on one 128x128 state held as 8x8 register tiles by a CTA of 256 threads:
-// reconstruction of the dense state from the window representation (Eq. 7) and its quantization
-// (Compensator-Token fit by power iteration on all r vectors at once, Eqs. 5-6; residual smoothing, Sec. 3.4;
-// per-value-channel symmetric 8-bit codes, Appendix B.3).
+// The window boundary of a head: rebuild the dense state from the window representation (Eq. 7), refit the Compensator
+// Tokens by power iteration on all r vectors at once (Eqs. 5-6), smooth the residual (Sec. 3.4), requantize it to 8 bits
+// per value channel (Appendix B.3) and write the head back.
+//
+// Layout.  Eight warps hold the 128x128 state in registers: a warp owns 16 columns (value channels) of all 128 rows, lane
+// (ty, tx) = (lane >> 1, lane & 1) the 8x8 tile of rows 8 ty .. 8 ty + 7 and eight of the columns, kept as column pairs
+// (two FMAs per instruction).  So everything that belongs to a column - the products with the keys, the value sides, the
+// scales, the codes - stays inside a warp, and only row sums (the products with the start vectors, the smoothing scales)
+// go through shared memory and a barrier.  Two CTAs fill the register file of an SM.
 #pragma once
+#include <type_traits>
+
 #include "lq_common.cuh"
 
 namespace lq {
 
-// Shared-memory plan of the boundary kernels (in floats).  A fixed part (working vectors of the fit, the
-// compensators widened to fp32) is followed by one or two staging buffers, each holding everything that is read
-// from global memory for one head: with two, the next head of the CTA is fetched while this one is computed.
+// Shared memory of a CTA, byte offsets: working arrays at fixed places (sized for RM vectors), then the slot (head block,
+// records), which is filled by two bulk copies.  Both parts of the slot are free again when the products with the start
+// vectors have been taken, and then receive the next head.
+template <int RM>
 struct BoundarySmem {
-  // fixed part
-  float *ck;     // [r][128]  compensator keys widened to fp32
-  float *cu;     // [r][128]  compensator values widened to fp32
-  float *vec;    // [128]     row-sum results (row mean-abs)
-  float *colv;   // [128]     1 / c
-  float *part;   // [8][4][128] per-warp column partial sums of four vectors (column maxima: [8][128])
-  float *gam;    // [128]     Gamma_{1:n}
-  float *gram;   // [16][16]  Gram matrix of the vectors being orthonormalised (lower triangle), later K^T K
-  float *chol;   // [16][16]  its Cholesky factor L (strictly lower triangle), then [16] 1 / L_hh, [16] alive flags
-  // staging buffer `buf`
-  float *kd;     // [W][128]  buffered write keys, turned in place into Gamma_{j+1:n} kt_j
-  float *bu;     // [W][128]  buffered corrections u_j
-  float *ba;     // [W][128]  diagonal-gate decays of the records (diagonal gate only), else [MAX_W]
-  float *cs;     // [128]     smoothing scales c
-  float *ss;     // [128]     code steps s_j = B_j / 127
-  uint16_t *ckh; // [r][128]  compensator keys as stored (fp16 bits)
-  uint16_t *cuh; // [r][128]  compensator values as stored
-  uint8_t *zt;   // [128][128] codes Z^T, 16-byte chunk q of row v stored at chunk q ^ ((v >> 3) & 7)
-  __half *raw;   // fp16 records only: [W] rows as stored (kt | u | (alpha)), widened into kd, bu by the decay scan
-  __host__ __device__ static constexpr int fixed_floats(int r) {
-    return 2 * r * D + 35 * D + 2 * MAX_R * MAX_R + 2 * MAX_R;
+  static constexpr int bar = 0;
+  static constexpr int invc = 16;                            // [8][16]    1 / code step, per warp
+  static constexpr int ic = invc + 4 * D;                    // [128]      1 / c
+  static constexpr int gam = ic + 4 * D;                     // [128]      Gamma_{1:n}
+  static constexpr int gram = gam + 4 * D;                   // [RM][RM]   Gram matrix (lower triangle), later K^T K (a > b)
+  static constexpr int chol = gram + 4 * RM * RM;            // L [RM][RM], 1 / L_hh [RM], alive [RM] (more than four vectors)
+  static constexpr int ub = chol + (RM > 4 ? 4 * (RM * RM + 2 * RM) : 0);      // [8][RM][16] value sides as stored, per warp
+  static constexpr int T = ub + 4 * D * RM;                  // [RM][128]  S w_h, then the keys as stored
+  static constexpr int part = T + 4 * D * RM;                // [8][RM][128] per-warp row sums; later [8][128] those of |R|
+  static constexpr int head = part + 4 * D * 8 * RM;
+  int rec, dec, kd, Wv, bytes;
+  __host__ __device__ BoundarySmem(int W, int r, bool diag, bool rec16, bool slot, bool iterate) {
+    rec = head + (slot ? head_bytes(r) : 0);                 // [W] record rows
+    dec = rec + (slot ? (rec16 ? 2 : 4) * record_floats(diag) * W : 0);        // [W] scalar gate: the records' decays
+    kd = dec + (slot && !diag ? (4 * W + 15) / 16 * 16 : 0); // [W][128] fp16 records: Gamma_{j+1:n} kt_j (fp32: in place)
+    Wv = kd + (slot && rec16 ? 4 * D * W : 0);               // [r][128] several rounds: S^T q_h
+    bytes = Wv + (iterate ? 4 * D * r : 0);
   }
-  __host__ __device__ static constexpr int stage_floats(int W, int r, bool diag, bool rec16) {
-    return 2 * W * D + (diag ? W * D : MAX_W) + 2 * D + r * D + D * D / 4 + (rec16 ? W * record_floats(diag) / 2 : 0);
-  }
-  __device__ __forceinline__ BoundarySmem(float *base, int W, int r, bool diag, bool rec16, int buf) {
-    ck = base; cu = ck + r * D; vec = cu + r * D; colv = vec + D; part = colv + D; gam = part + 32 * D;
-    gram = gam + D; chol = gram + MAX_R * MAX_R;
-    kd = base + fixed_floats(r) + buf * stage_floats(W, r, diag, rec16);
-    bu = kd + W * D; ba = bu + W * D; cs = ba + (diag ? W * D : MAX_W); ss = cs + D;
-    ckh = reinterpret_cast<uint16_t *>(ss + D); cuh = ckh + r * D;
-    zt = reinterpret_cast<uint8_t *>(cuh + r * D);
-    raw = reinterpret_cast<__half *>(zt + D * D);
-  }
-  static size_t bytes(int W, int r, bool diag, bool rec16, int bufs) {
-    return sizeof(float) * (size_t)(fixed_floats(r) + bufs * stage_floats(W, r, diag, rec16));
-  }
-  // two staging buffers while two CTAs with two buffers each still fit on an SM
-  static int buffers(int W, int r, bool diag, bool rec16) { return bytes(W, r, diag, rec16, 2) <= 110 * 1024 ? 2 : 1; }
 };
 
-// Issue the asynchronous copies that bring head bh (its codes, scales, compensators and n records) into the
-// staging buffer of sm.  The caller commits the group and later waits for it.
-template <int GATE, bool R16>
-__device__ __forceinline__ void stage_issue(const Params &p, const BoundarySmem &sm, const Tile &t, size_t bh, int n) {
-  constexpr bool DIAG = GATE == LQ_GATE_DIAG;
-  constexpr int RF = record_floats(DIAG);
-  const int r = p.r;
-  const uint8_t *hb = p.head(bh);
-  for (int e = t.tid; e < D * D / 16; e += 256) {             // codes: 1024 chunks of 16 bytes
-    const int v = e >> 3, q = e & 7;
-    cp_async16(sm.zt + v * D + 16 * (q ^ ((v >> 3) & 7)), hb + HB_CODES + 16 * e);
-  }
-  if (R16) {                                                  // the n rows are one contiguous piece of fp16 values
-    const __half *rec = p.record<__half>(bh, 0, DIAG);
-    for (int e = t.tid; e < n * (RF / 8); e += 256) cp_async16(sm.raw + 8 * e, rec + 8 * e);
-  } else {
-    const float *rec = p.record<float>(bh, 0, DIAG);
-    for (int e = t.tid; e < n * (D / 4); e += 256) {
-      const int j = e / (D / 4), q4 = 4 * (e % (D / 4));
-      cp_async16(sm.kd + j * D + q4, rec + j * RF + REC_KT + q4);
-      cp_async16(sm.bu + j * D + q4, rec + j * RF + REC_U + q4);
-      if (DIAG) cp_async16(sm.ba + j * D + q4, rec + j * RF + REC_A + q4);
-    }
-  }
-  if (!DIAG && t.tid < n) cp_async4(sm.ba + t.tid, p.decays + bh * (size_t)p.W + t.tid);
-  if (t.tid < D / 4) cp_async16(sm.ss + 4 * t.tid, hb + HB_COL_SCALE + 16 * t.tid);
-  else if (t.tid < D / 2) cp_async16(sm.cs + 4 * (t.tid - D / 4), hb + HB_ROW_SMOOTH + 16 * (t.tid - D / 4));
-  for (int e = t.tid; e < r * D / 4; e += 256)                // 2 r rows of 256 bytes, contiguous in the head block
-    cp_async16(sm.ckh + 8 * e, hb + HB_COMP_K + 16 * e);      // (cuh follows ckh in the buffer as in the block)
-}
-
-// M += x y^T on the register tile, two columns per instruction (fma.rn.f32x2 is two independent round-to-nearest
-// FMAs, so the values are those of fmaf; what it halves is the issue slots of the phases that are bound by them).
-__device__ __forceinline__ void rank1_update(float (&M)[8][8], const float (&x)[8], const float (&y)[8]) {
+// M += x y^T on the tile
+__device__ __forceinline__ void rank1_pairs(float2 (&M)[8][4], const float (&x)[8], const float2 (&y)[4]) {
 #pragma unroll
   for (int a = 0; a < 8; a++) {
-    const float2 xa = make_float2(x[a], x[a]);
+    const float2 xa = pair(x[a]);
 #pragma unroll
-    for (int b = 0; b < 8; b += 2) {
-      const float2 m = __ffma2_rn(xa, make_float2(y[b], y[b + 1]), make_float2(M[a][b], M[a][b + 1]));
-      M[a][b] = m.x;
-      M[a][b + 1] = m.y;
-    }
+    for (int c = 0; c < 4; c++) M[a][c] = __ffma2_rn(xa, y[c], M[a][c]);
   }
 }
 
-// Eq. 7 for the tile of thread t: M = Gamma_{1:n}[C (Z/127) B + Kc Uc^T] + sum_j Gamma_{j+1:n} kt_j u_j^T,
-// evaluated per element as  base = c_i*(Z_ij*s_j) with s_j the stored code step; base = fma(kc_hi, uc_hj, base) for h = 0..r-1;
-// x = gamma_i*base; x = fma(kd_ji, u_jj, x) for j = 0..n-1.  No sum crosses threads.
-// Leaves the CTA's shared memory holding the records; ends after its last read of it (no trailing barrier).
-template <int GATE, bool R16>
-__device__ __forceinline__ void reconstruct_tile(const Params &p, const BoundarySmem &sm, const Tile &t, size_t bh,
-                                                 int n, float (&M)[8][8]) {
-  const int r = p.r;
-  constexpr bool DIAG = GATE == LQ_GATE_DIAG;
-  constexpr int RF = record_floats(DIAG);
-  // the staging buffer has landed and the CTA has synchronised (the caller did both)
-  // cumulative decays, newest record first (Appendix B.2): kd_j = Gamma_{j+1:n} kt_j, gam = Gamma_{1:n};
-  // the other half of the CTA widens the compensators meanwhile
-  if (t.tid < D) {
-    const int i = t.tid;
-    // record j's write key and decay for channel i (fp16 records are widened here, on the way into kd)
-    auto kt_at = [&](int jj) { return R16 ? __half2float(sm.raw[jj * RF + REC_KT + i]) : sm.kd[jj * D + i]; };
-    auto a_at = [&](int jj) {
-      return !DIAG ? sm.ba[jj] : R16 ? __half2float(sm.raw[jj * RF + REC_A + i]) : sm.ba[jj * D + i];
-    };
-    float g = 1.0f;
-    int j = n - 1;
-    for (; j >= 3; j -= 4) {                                  // four records per trip: the loads go out together
-      float kt[4], a[4];
+// Which of the lane's eight columns a column_tree leaves with it
+__device__ __forceinline__ int column_of(int lane) { return (lane & 2 ? 4 : 0) + (lane & 4 ? 2 : 0) + (lane & 8 ? 1 : 0); }
+// Combine the eight per-column values p over the 16 lanes ty (lane bits 1..4), neighbouring blocks first, by halving
+// exchanges; returns the result of column column_of(lane), the same in lanes that differ in bit 4.
+template <typename Op>
+__device__ __forceinline__ float column_tree(const float (&p)[8], int lane, Op op) {
+  const bool u0 = lane & 2, u1 = lane & 4, u2 = lane & 8;
+  float q4[4], q2[2], q1;
 #pragma unroll
-      for (int e = 0; e < 4; e++) {
-        kt[e] = kt_at(j - e);
-        a[e] = a_at(j - e);
-      }
-#pragma unroll
-      for (int e = 0; e < 4; e++) {
-        sm.kd[(j - e) * D + i] = g * kt[e];
-        g = g * a[e];
-      }
-    }
-    for (; j >= 0; j--) {
-      sm.kd[j * D + i] = g * kt_at(j);
-      g = g * a_at(j);
-    }
-    sm.gam[i] = g;
-  } else {
-    for (int e = t.tid - D; e < 2 * r * D; e += 256 - D) sm.ck[e] = f16_bits(sm.ckh[e]);   // ck and cu are adjacent
-    if (R16)                                                  // fp16 records: the u rows, widened
-      for (int e = t.tid - D; e < n * D; e += 256 - D) sm.bu[e] = __half2float(sm.raw[(e / D) * RF + REC_U + (e % D)]);
-  }
-  __syncthreads();
-  LQ_BTICK(2);
-
-  float ci[8], gi[8], sj[8];
-  load8(sm.cs + 8 * t.ty, ci);
-  load8(sm.gam + 8 * t.ty, gi);
-  load8(sm.ss + 8 * t.tx, sj);
-#pragma unroll
-  for (int b = 0; b < 8; b++) {
-    // column v = 8 tx + b of the tile: bytes 8 ty .. 8 ty + 7 of row v of Z^T (chunk ty / 2, swizzled by tx)
-    const uint2 zz = *reinterpret_cast<const uint2 *>(sm.zt + (8 * t.tx + b) * D + 16 * ((t.ty >> 1) ^ (t.tx & 7)) +
-                                                      8 * (t.ty & 1));
-    // int8 -> fp32 without the conversion unit: byte + 128 placed in the low mantissa bits of 2^23, minus 2^23 + 128
-    const uint32_t lo = zz.x ^ 0x80808080u, hi = zz.y ^ 0x80808080u;
-#pragma unroll
-    for (int a = 0; a < 8; a++) {
-      const uint32_t word = a < 4 ? lo : hi;
-      const float zf = __uint_as_float(__byte_perm(word, 0x4B000000u, 0x7540 | (a & 3))) - 8388736.0f;
-      M[a][b] = ci[a] * (zf * sj[b]);
-    }
-  }
-  for (int h = 0; h < r; h++) {
-    float kc[8], uc[8];
-    load8(sm.ck + h * D + 8 * t.ty, kc);
-    load8(sm.cu + h * D + 8 * t.tx, uc);
-    rank1_update(M, kc, uc);
+  for (int e = 0; e < 4; e++) {
+    const float keep = u0 ? p[e + 4] : p[e], send = u0 ? p[e] : p[e + 4];
+    q4[e] = op(keep, __shfl_xor_sync(FULL, send, 2));
   }
 #pragma unroll
-  for (int a = 0; a < 8; a++)
-#pragma unroll
-    for (int b = 0; b < 8; b++) M[a][b] = gi[a] * M[a][b];
-  for (int j = 0; j < n; j++) {
-    float kj[8], uj[8];
-    load8(sm.kd + j * D + 8 * t.ty, kj);
-    load8(sm.bu + j * D + 8 * t.tx, uj);
-    rank1_update(M, kj, uj);
+  for (int e = 0; e < 2; e++) {
+    const float keep = u1 ? q4[e + 2] : q4[e], send = u1 ? q4[e] : q4[e + 2];
+    q2[e] = op(keep, __shfl_xor_sync(FULL, send, 4));
   }
-  LQ_BTICK(3);
+  {
+    const float keep = u2 ? q2[1] : q2[0], send = u2 ? q2[0] : q2[1];
+    q1 = op(keep, __shfl_xor_sync(FULL, send, 8));
+  }
+  return op(q1, __shfl_xor_sync(FULL, q1, 16));
 }
-
-// ---- pieces of the Compensator-Token fit: power iteration on all r vectors at once ----
+// S^T x for the lane's eight columns: even and odd rows as two chains of the block
+__device__ __forceinline__ void column_blocks(const float2 (&M)[8][4], const float (&x)[8], float (&pc)[8]) {
+#pragma unroll
+  for (int c = 0; c < 4; c++) {
+    float2 even = __fmul2_rn(pair(x[0]), M[0][c]), odd = __fmul2_rn(pair(x[1]), M[1][c]);
+#pragma unroll
+    for (int a = 2; a < 8; a += 2) {
+      even = __ffma2_rn(pair(x[a]), M[a][c], even);
+      odd = __ffma2_rn(pair(x[a + 1]), M[a + 1][c], odd);
+    }
+    const float2 s = __fadd2_rn(even, odd);
+    pc[2 * c] = s.x; pc[2 * c + 1] = s.y;
+  }
+}
+// Row values of the two lanes tx added; the lane keeps rows 8 ty + 4 tx .. + 3 and puts them into dst[128]
+__device__ __forceinline__ void store_row_pairs(const float (&p)[8], int ty, int tx, float *dst) {
+  float q[4];
+#pragma unroll
+  for (int e = 0; e < 4; e++) {
+    const float keep = tx ? p[e + 4] : p[e], send = tx ? p[e] : p[e + 4];
+    q[e] = keep + __shfl_xor_sync(FULL, send, 1);
+  }
+  *reinterpret_cast<float4 *>(dst + 8 * ty + 4 * tx) = make_float4(q[0], q[1], q[2], q[3]);
+}
+// the sum of what the eight warps left for one row (rows of the warps `stride` floats apart)
+__device__ __forceinline__ float sum_warps(const float *c, int stride) {
+  return ((c[0] + c[stride]) + (c[2 * stride] + c[3 * stride])) + ((c[4 * stride] + c[5 * stride]) + (c[6 * stride] + c[7 * stride]));
+}
 
 // Entry j of start vector h where no buffered record supplies one: -1 where h and j share an odd number of bits
 __device__ __forceinline__ float walsh_entry(int h, int j) { return (__popc(h & j) & 1) ? -1.0f : 1.0f; }
 
-// Lower triangle of the Gram matrix of the nv vectors X[0..nv-1] (rows of 128 floats in shared memory), one dot
-// product per half-warp and trip.  Barrier before (X complete) and after (G complete) are the caller's.
-__device__ __forceinline__ void gram_lower(const float *X, int nv, float *G, const Tile &t, bool with_diagonal) {
-  const int hw = t.tid >> 4, c = t.lane & 15;
-  const int npairs = with_diagonal ? nv * (nv + 1) / 2 : nv * (nv - 1) / 2;
-  for (int base = 0; base < npairs; base += 16) {            // the same trip count for every thread of the CTA
+// Lower triangle of the Gram matrix of the r vectors X (rows of 128 floats in shared memory), one dot product per
+// half-warp and trip.
+template <int RM>
+__device__ __forceinline__ void gram_lower(const float *X, int r, float *G, bool with_diagonal) {
+  const int hw = threadIdx.x >> 4, c = threadIdx.x & 15;
+  const int npairs = with_diagonal ? r * (r + 1) / 2 : r * (r - 1) / 2;
+  for (int base = 0; base < npairs; base += 16) {            // the same trip count for every thread
     const int idx = base + hw;
     const int ii = idx < npairs ? idx : 0;
-    int a = 0;                                               // ii = a (a + 1) / 2 + b with b <= a, without a loop
+    int a = 0;                                               // ii = a (a + 1) / 2 + b with b <= a
 #pragma unroll
-    for (int e = 1; e < MAX_R; e++) a += ii >= e * (e + 1) / 2;
-    int b = ii - a * (a + 1) / 2;
+    for (int e = 1; e < RM; e++) a += ii >= e * (e + 1) / 2;
+    const int b = ii - a * (a + 1) / 2;
     if (!with_diagonal) a += 1;                              // pairs b < a only
     const float d = dot128_shared(X + a * D, X + b * D, c);
-    if (idx < npairs && c == 0) G[a * MAX_R + b] = d;
-  }
-}
-
-// Cholesky factor of the Gram matrix of up to four vectors, by one thread, in registers (all loads first):
-// L (strictly lower part), inv[h] = 1 / L_hh, alive[h], to shared memory.  Same arithmetic as the warp's version below.
-__device__ __forceinline__ void cholesky_lower_4(const float *G, int nv, float *L) {
-  float *inv = L + MAX_R * MAX_R, *alive = inv + MAX_R;
-  float g[4][4], l[4][4], iv[4];
-#pragma unroll
-  for (int h = 0; h < 4; h++)
-#pragma unroll
-    for (int j = 0; j <= h; j++) g[h][j] = h < nv ? G[h * MAX_R + j] : 0.0f;
-#pragma unroll
-  for (int h = 0; h < 4; h++) {
-#pragma unroll
-    for (int j = 0; j < h; j++) {
-      float sacc = g[h][j];
-#pragma unroll
-      for (int m = 0; m < j; m++) sacc = fmaf(-l[h][m], l[j][m], sacc);
-      l[h][j] = sacc * iv[j];
-    }
-    float d = g[h][h];
-#pragma unroll
-    for (int m = 0; m < h; m++) d = fmaf(-l[h][m], l[h][m], d);
-    const bool ok = g[h][h] >= 1e-30f && d > 1e-6f * g[h][h];
-    iv[h] = ok ? 1.0f / sqrtf(d) : 0.0f;
-    if (h < nv) {
-#pragma unroll
-      for (int j = 0; j < h; j++) L[h * MAX_R + j] = l[h][j];
-      inv[h] = iv[h];
-      alive[h] = ok ? 1.0f : 0.0f;
-    }
+    if (idx < npairs && c == 0) G[a * RM + b] = d;
   }
 }
 
 // Cholesky factor of the Gram matrix, by one warp: lane h owns row h of L.  Column by column: lane j finishes
 // L_jj from its own row, the lanes below it their entry of column j (the entries of row j they need come by
 // shuffle from lane j); the arithmetic of an entry is  s = G_hj; s = fma(-L_hm, L_jm, s) for m < j; L_hj = s / L_jj.
-// Writes L (strictly lower part), inv[h] = 1 / L_hh and alive[h] to shared memory.
+// Writes L (strictly lower part), then inv[h] = 1 / L_hh and alive[h], to shared memory.
 // A vector whose squared length is below 1e-30, or of which the vectors before it leave no more than 1e-6 of its
 // squared length, is dropped: inv = 0, which makes its orthonormalised vector and all its L entries zero.
-// RM: the largest number of vectors this instance is compiled for (nv <= RM <= MAX_R).
+// RM: the largest number of vectors this instance is compiled for (nv <= RM), the row length of G and L.
 template <int RM>
 __device__ __forceinline__ void cholesky_lower_warp(const float *G, int nv, float *L, int lane) {
-  float *inv = L + MAX_R * MAX_R, *alive = inv + MAX_R;
+  float *inv = L + RM * RM, *alive = inv + RM;
   const int h = lane;
   float g[RM], l[RM];
 #pragma unroll
   for (int j = 0; j < RM; j++) {
-    g[j] = (h < nv && j <= h) ? G[h * MAX_R + j] : 0.0f;
+    g[j] = (h < nv && j <= h) ? G[h * RM + j] : 0.0f;
     l[j] = 0.0f;
   }
   float inv_h = 0.0f;
@@ -276,51 +162,77 @@ __device__ __forceinline__ void cholesky_lower_warp(const float *G, int nv, floa
   if (h < nv) {
 #pragma unroll
     for (int j = 0; j < RM; j++)
-      if (j < h) L[h * MAX_R + j] = l[j];
+      if (j < h) L[h * RM + j] = l[j];
     inv[h] = inv_h;
     alive[h] = ok_h ? 1.0f : 0.0f;
   }
 }
 
-// Orthonormalise the nv vectors X (rows of 128 floats in shared memory) in place, in order:
-// q_h = (x_h - sum_{j<h} L_hj q_j) / L_hh, one thread per element index, its nv values in registers.
-// With FINAL the results are then rounded to fp16 (what is stored as compensator keys), written to comp_k of
-// head bh and kept in X as the stored values.  Begins and ends with a barrier.
+// Orthonormalise the r vectors X (rows of 128 floats in shared memory) in place, in order:
+// q_h = (x_h - sum_{j<h} L_hj q_j) / L_hh, one thread per element index (the upper half of the threads computes the same
+// and stores nothing).  With FINAL the results are rounded to fp16 (what is stored as compensator keys), written to keys
+// and kept in X as stored.  Up to four vectors: every thread computes the factor itself, in registers (no barriers around
+// a chain of four 1/sqrt); more: one warp does, through shared memory.
+// Returns the bit mask of the vectors that were not dropped.  Begins and ends with a barrier.
 template <bool FINAL, int RM>
-__device__ __forceinline__ void orthonormalize(const Params &p, const BoundarySmem &sm, const Tile &t, float *X,
-                                               int nv, size_t bh) {
+__device__ __forceinline__ uint32_t orthonormalize(float *X, int r, float *gram, float *chol, uint16_t *keys) {
+  const int tid = threadIdx.x, i = tid & (D - 1);
   __syncthreads();
-  gram_lower(X, nv, sm.gram, t, true);
+  gram_lower<RM>(X, r, gram, true);
   __syncthreads();
   LQ_BTICK(7);
-  if (RM <= 4) {                                             // four dependent 1/sqrt: one thread is the shortest chain
-    if (t.tid == 0) cholesky_lower_4(sm.gram, nv, sm.chol);
-  } else if (t.warp == 0) {
-    cholesky_lower_warp<RM>(sm.gram, nv, sm.chol, t.lane);
-  }
-  __syncthreads();
-  LQ_BTICK(8);
-  if (t.tid < D) {
-    const float *L = sm.chol, *inv = L + MAX_R * MAX_R, *alive = inv + MAX_R;
-    const int i = t.tid;
-    float x[RM];
+  uint32_t alive = 0;
+  float x[RM];
 #pragma unroll
-    for (int h = 0; h < RM; h++) x[h] = h < nv ? X[h * D + i] : 0.0f;
+  for (int h = 0; h < RM; h++) x[h] = h < r ? X[h * D + i] : 0.0f;
+  if constexpr (RM <= 4) {
+    float l[4][4], iv[4];
+#pragma unroll
+    for (int h = 0; h < 4; h++) {
+      float gr[4];
+#pragma unroll
+      for (int j = 0; j <= h; j++) gr[j] = h < r ? gram[h * RM + j] : 0.0f;
+#pragma unroll
+      for (int j = 0; j < h; j++) {
+        float s = gr[j];
+#pragma unroll
+        for (int m = 0; m < j; m++) s = fmaf(-l[h][m], l[j][m], s);
+        l[h][j] = s * iv[j];
+      }
+      float d = gr[h];
+#pragma unroll
+      for (int m = 0; m < h; m++) d = fmaf(-l[h][m], l[h][m], d);
+      const bool ok = gr[h] >= 1e-30f && d > 1e-6f * gr[h];
+      alive |= ok ? 1u << h : 0u;
+      iv[h] = ok ? 1.0f / sqrtf(d) : 0.0f;
+#pragma unroll
+      for (int j = 0; j < h; j++) x[h] = fmaf(-l[h][j], x[j], x[h]);
+      x[h] = x[h] * iv[h];
+    }
+    __syncthreads();                         // (two threads share an element of X)
+  } else {
+    if (tid < 32) cholesky_lower_warp<RM>(gram, r, chol, tid);
+    __syncthreads();
+    const float *iv = chol + RM * RM;
 #pragma unroll
     for (int h = 0; h < RM; h++) {
-      if (h < nv) {
+      if (h < r) {
 #pragma unroll
-        for (int j = 0; j < h; j++) x[h] = fmaf(-L[h * MAX_R + j], x[j], x[h]);
-        x[h] = x[h] * inv[h];
+        for (int j = 0; j < h; j++) x[h] = fmaf(-chol[h * RM + j], x[j], x[h]);
+        x[h] = x[h] * iv[h];
+        alive |= iv[RM + h] != 0.0f ? 1u << h : 0u;
       }
     }
+  }
+  LQ_BTICK(8);
+  if (tid < D) {
 #pragma unroll
     for (int h = 0; h < RM; h++) {
-      if (h < nv) {
+      if (h < r) {
         float out = x[h];
         if (FINAL) {
-          const uint16_t bits = alive[h] != 0.0f ? to_f16_bits_sat(out) : static_cast<uint16_t>(0);
-          p.comp_k(bh)[h * D + i] = bits;
+          const uint16_t bits = (alive >> h) & 1u ? to_f16_bits_sat(out) : static_cast<uint16_t>(0);
+          keys[h * D + i] = bits;
           out = f16_bits(bits);
         }
         X[h * D + i] = out;
@@ -328,210 +240,359 @@ __device__ __forceinline__ void orthonormalize(const Params &p, const BoundarySm
     }
   }
   __syncthreads();
+  return alive;
 }
 
-// T[h] = M w_h for the nv vectors w_h (two at a time), into Tm (rows of 128 floats).  `wsrc(h, w)` loads the eight
-// entries of w_h for this thread's columns.  No barrier inside.
-template <typename WSrc>
-__device__ __forceinline__ void rows_times_vectors(const float (&M)[8][8], const Tile &t, int nv, float *Tm, WSrc wsrc) {
-  for (int h0 = 0; h0 < nv; h0 += 2) {
-    const bool two = h0 + 1 < nv;
-    float w0[8], w1[8], pr0[8], pr1[8];
-    wsrc(h0, w0);
-    wsrc(two ? h0 + 1 : h0, w1);
-    row_blocks(M, w0, pr0);
-    row_blocks(M, w1, pr1);
-    int sel;
-    const float t0 = row_tree(pr0, t.lane, sel);
-    const float t1 = row_tree(pr1, t.lane, sel);
-    if (t.tx < 8) {
-      Tm[h0 * D + 8 * t.ty + sel] = t0;
-      if (two) Tm[(h0 + 1) * D + 8 * t.ty + sel] = t1;
+// MODE 0 flush (window representation -> dense -> new window representation), 1 quantize dense fp32 states,
+// 2 dequantize to dense fp32 states.  RM: the largest r the instance handles.
+template <int GATE, int MODE, bool R16, int RM>
+__global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
+  constexpr bool DIAG = GATE == LQ_GATE_DIAG, SLOT = MODE != 1;
+  constexpr int RF = record_floats(DIAG);
+  using rec_t = typename std::conditional<R16, __half, float>::type;
+  using Lay = BoundarySmem<RM>;
+  extern __shared__ __align__(128) unsigned char lq_bsm[];
+  __shared__ unsigned todo_bh[32];
+  __shared__ int todo_n[32], todo_count, any_due;
+  const int W = p.W, r = p.r, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 1, tx = lane & 1;
+  const int v0 = 16 * warp + 8 * tx;         // the lane's first column
+  const unsigned nh = static_cast<unsigned>(p.batch) * p.heads_v;
+  const Lay L(W, r, DIAG, R16, SLOT, p.n_iter > 1);
+  rec_t *rec = reinterpret_cast<rec_t *>(lq_bsm + L.rec);
+  float *dec = reinterpret_cast<float *>(lq_bsm + L.dec), *gam = reinterpret_cast<float *>(lq_bsm + Lay::gam);
+  const uint8_t *zt = lq_bsm + Lay::head + HB_CODES;
+  const float *ss = reinterpret_cast<const float *>(lq_bsm + Lay::head + HB_COL_SCALE);
+  const float *cs = reinterpret_cast<const float *>(lq_bsm + Lay::head + HB_ROW_SMOOTH);
+  const uint16_t *ckh = reinterpret_cast<const uint16_t *>(lq_bsm + Lay::head + HB_COMP_K), *cuh = ckh + r * D;
+  float *part = reinterpret_cast<float *>(lq_bsm + Lay::part), *T = reinterpret_cast<float *>(lq_bsm + Lay::T);
+  float *Wv = reinterpret_cast<float *>(lq_bsm + L.Wv), *gram = reinterpret_cast<float *>(lq_bsm + Lay::gram);
+  float *chol = reinterpret_cast<float *>(lq_bsm + Lay::chol), *ub = reinterpret_cast<float *>(lq_bsm + Lay::ub) + warp * 16 * RM;
+  float *ic_s = reinterpret_cast<float *>(lq_bsm + Lay::ic), *invc = reinterpret_cast<float *>(lq_bsm + Lay::invc) + 16 * warp;
+  const uint32_t bar = smem_addr(lq_bsm + Lay::bar);
+  auto kd_row = [&](int j) -> float * {      // Gamma_{j+1:n} kt_j
+    if constexpr (R16) return reinterpret_cast<float *>(lq_bsm + L.kd) + j * D;
+    else return rec + j * RF + REC_KT;
+  };
+
+  LQ_STAMP(1, 0);
+  if (SLOT && tid == 0) mbar_init(bar, 1);
+  grid_dependency_wait();                    // everything the kernel before this one wrote is visible from here on
+  LQ_STAMP(1, 1);
+#ifdef LQ_TIMING
+  if (tid == 0) { for (int i = 0; i < 16; i++) lq_bacc[i] = 0; lq_btick = clock64(); }
+#endif
+  // the decode kernel ahead of a flush counts the tickets of its pool of heads in the state's scratch words
+  if (MODE == 0 && p.work != nullptr && blockIdx.x == 0 && tid == 0) p.work[0] = 0;
+
+  uint32_t parity = 0;
+  float dec_next = 0.0f;                     // this thread's decay of the head on its way (scalar gate, tid < n)
+  auto request = [&](size_t bh, int n) {     // bring head bh and its n records into the slot
+    if (!DIAG && tid < n) dec_next = p.decays[bh * (size_t)W + tid];
+    if (tid == 0) {
+      const uint32_t rb = static_cast<uint32_t>(sizeof(rec_t)) * RF * n;
+      mbar_expect_tx(bar, head_bytes(r) + rb);
+      bulk_g2s(smem_addr(lq_bsm + Lay::head), p.head(bh), head_bytes(r), bar);
+      if (n > 0) bulk_g2s(smem_addr(lq_bsm + L.rec), p.record<rec_t>(bh, 0, DIAG), rb, bar);
     }
-  }
-}
+  };
 
-// Out[h] = M^T x_h for the nv vectors x_h in Xm (rows of 128 floats in shared memory), four to a round of barriers.
-// Column sums in the fixed order: this thread's eight rows, its neighbour in the warp (lane ^ 16), then the
-// eight warps as a balanced tree.  Begins after a barrier of the caller (Xm complete); ends with a barrier.
-__device__ __forceinline__ void columns_times_vectors(const float (&M)[8][8], const BoundarySmem &sm, const Tile &t,
-                                                      int nv, const float *Xm, float *Out) {
-  const bool up = t.lane & 16;
-  for (int h0 = 0; h0 < nv; h0 += 4) {
-    const int nh = nv - h0 < 4 ? nv - h0 : 4;
-    if (h0 > 0) __syncthreads();                              // the previous round's partial sums have been read
-    for (int hh = 0; hh < nh; hh++) {                         // first half: own rows, then the neighbour's
-      float x[8], pc[8], rr[4];
-      load8(Xm + (h0 + hh) * D + 8 * t.ty, x);
-      col_blocks(M, x, pc);
-#pragma unroll
-      for (int e = 0; e < 4; e++) {
-        const float keep = up ? pc[e + 4] : pc[e], send = up ? pc[e] : pc[e + 4];
-        rr[e] = keep + __shfl_xor_sync(FULL, send, 16);
+  // Warp 0 puts together the next 32 heads of the CTA (a flush: of those that are due, see find_due_heads; otherwise every
+  // gridDim-th head) and how many records each holds; then the CTA takes them one after the other.
+  int count = 32;
+  for (unsigned first = blockIdx.x; count == 32; first += 32 * gridDim.x) {
+    if (warp == 0) {
+      unsigned bh_mine = first + lane * gridDim.x;
+      int n_mine = 0, c, due = 0;
+      if (MODE == 0) {
+        c = find_due_heads(p, first, gridDim.x, lane, bh_mine, n_mine, due);
+      } else {
+        const bool have = bh_mine < nh;
+        if (MODE == 2 && have) n_mine = p.win_pos[bh_mine / p.heads_v] & 0xFFFF;
+        c = __popc(__ballot_sync(FULL, have));
       }
-      *reinterpret_cast<float4 *>(sm.part + (t.warp * 4 + hh) * D + 8 * t.tx + (up ? 4 : 0)) =
-          make_float4(rr[0], rr[1], rr[2], rr[3]);
+      todo_bh[lane] = bh_mine;
+      todo_n[lane] = n_mine > W ? W : n_mine;
+      if (lane == 0) { todo_count = c; any_due = due; }
     }
     __syncthreads();
-    for (int idx = t.tid; idx < nh * D; idx += 256) {         // second half: the eight warps
-      const int v = idx >> 7, col = idx & (D - 1);
-      const float *c = sm.part + v * D + col;
-      Out[(h0 + v) * D + col] =
-          ((c[0] + c[4 * D]) + (c[8 * D] + c[12 * D])) + ((c[16 * D] + c[20 * D]) + (c[24 * D] + c[28 * D]));
-    }
-  }
-  __syncthreads();
-}
+    count = todo_count;
+    if (SLOT && count > 0) request(todo_bh[0], todo_n[0]);
+    // one warp reports that this CTA has seen all of win_pos, once the first head's copies are on their way (the round
+    // trip hides behind them); with nothing due there is nothing to restart
+    if (MODE == 0 && count < 32 && any_due > 0 && warp == 7) restart_due_windows(p, lane);
+    LQ_BTICK(0);
 
-// Quantize the dense state held in M (destroyed) and write codes, scales and compensators of head bh.
-// Uses the fixed part of shared memory (ck, cu, vec, colv, part, gram, chol); begins with a barrier so that it
-// may follow any other use of it.
-// Compensator Tokens (Eqs. 5-6): power iteration on all r vectors at once.  T = M W, orthonormalise, W = M^T T,
-// orthonormalise, ... n_iter times, ending on the key side; column h of W starts from the value side u of the
-// (h+1)-th newest of the n records in sm.bu, from a Walsh vector where there is no such record.  The keys are
-// rounded to fp16; value side h is M^T k_h - sum_{a<h} u_a (k_a^T k_h) with the stored values (the least-squares
-// answer for what components 0..h-1 leave), rounded to fp16 in turn; then M -= K U^T with the stored values.
-// RM: the largest r this instance is compiled for (the small matrices of the fit live in registers, RM wide).
-template <int RM>
-__device__ __forceinline__ void quantize_tile(const Params &p, const BoundarySmem &sm, const Tile &t, size_t bh,
-                                              int n, float (&M)[8][8]) {
-  const int r = p.r;
-  __syncthreads();
-  if (r > 0) {
-    float *Tm = sm.ck, *Wm = sm.cu;                           // [r][128] each; the old compensators are done with
-    for (int it = 0; it < p.n_iter; it++) {
-      if (it == 0) {
-        rows_times_vectors(M, t, r, Tm, [&](int h, float (&w)[8]) {
-          if (h < n) {
-            load8(sm.bu + (n - 1 - h) * D + 8 * t.tx, w);
+    for (int k = 0; k < count; k++) {
+      const size_t bh = todo_bh[k];
+      const int n = todo_n[k];
+      if (SLOT) {
+        if (!DIAG && tid < n) dec[tid] = dec_next;
+        if (!mbar_wait(bar, parity) && lane == 0) atomicOr(&g_device_error, 1);
+        parity ^= 1u;
+        if (!DIAG) __syncthreads();
+        if (k == 0) LQ_STAMP(1, 2);
+        LQ_BTICK(1);
+        // cumulative decays, newest record first (Appendix B.2): kd_j = Gamma_{j+1:n} kt_j, gam = Gamma_{1:n}
+        if (tid < D) {
+          auto kt_at = [&](int j) { return static_cast<float>(rec[j * RF + REC_KT + tid]); };
+          auto a_at = [&](int j) { return DIAG ? static_cast<float>(rec[j * RF + REC_A + tid]) : dec[j]; };
+          float g = 1.0f;
+          int j = n - 1;
+          for (; j >= 3; j -= 4) {                            // four records per trip: the loads go out together
+            float kt[4], a[4];
+#pragma unroll
+            for (int e = 0; e < 4; e++) { kt[e] = kt_at(j - e); a[e] = a_at(j - e); }
+#pragma unroll
+            for (int e = 0; e < 4; e++) { kd_row(j - e)[tid] = g * kt[e]; g = g * a[e]; }
+          }
+          for (; j >= 0; j--) { const float kt = kt_at(j); kd_row(j)[tid] = g * kt; g = g * a_at(j); }
+          gam[tid] = g;
+        }
+        __syncthreads();
+        LQ_BTICK(2);
+      }
+
+      float2 M[8][4];                                         // rows 8 ty + a, columns v0 + 2 c, v0 + 2 c + 1
+      // ---- the dense state (Eq. 7) ----
+      if constexpr (SLOT) {
+        {
+          float ci[8];
+          float2 sj[4];
+          load8(cs + 8 * ty, ci);
+          load8p(ss + v0, sj);
+          uint2 zz[8];
+#pragma unroll
+          for (int b = 0; b < 8; b++) {
+            zz[b] = *reinterpret_cast<const uint2 *>(zt + (v0 + b) * D + 8 * ty);
+            zz[b].x ^= 0x80808080u; zz[b].y ^= 0x80808080u;
+          }
+          // int8 -> fp32 without the conversion unit: byte + 128 in the low mantissa bits of 2^23, minus 2^23 + 128
+#pragma unroll
+          for (int a = 0; a < 8; a++)
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+              const float2 raw = make_float2(
+                  __uint_as_float(__byte_perm(a < 4 ? zz[2 * c].x : zz[2 * c].y, 0x4B000000u, 0x7540 | (a & 3))),
+                  __uint_as_float(__byte_perm(a < 4 ? zz[2 * c + 1].x : zz[2 * c + 1].y, 0x4B000000u, 0x7540 | (a & 3))));
+              M[a][c] = __fmul2_rn(pair(ci[a]), __fmul2_rn(__fadd2_rn(raw, pair(-8388736.0f)), sj[c]));
+            }
+        }
+#pragma unroll 1
+        for (int h = 0; h < r; h++) {
+          float kc[8];
+          float2 uc[4];
+          load8(reinterpret_cast<const __half *>(ckh + h * D + 8 * ty), kc);
+          load8p(reinterpret_cast<const __half *>(cuh + h * D + v0), uc);
+          rank1_pairs(M, kc, uc);
+        }
+        {
+          float gi[8];
+          load8(gam + 8 * ty, gi);
+#pragma unroll
+          for (int a = 0; a < 8; a++)
+#pragma unroll
+            for (int c = 0; c < 4; c++) M[a][c] = __fmul2_rn(pair(gi[a]), M[a][c]);
+        }
+#pragma unroll 1
+        for (int j = 0; j < n; j++) {
+          float kj[8];
+          float2 uj[4];
+          load8(kd_row(j) + 8 * ty, kj);
+          load8p(rec + j * RF + REC_U + v0, uj);
+          rank1_pairs(M, kj, uj);
+        }
+        LQ_BTICK(3);
+      } else {
+        const float *S = p.S + bh * (size_t)(D * D) + 8 * ty * D + v0;
+#pragma unroll
+        for (int a = 0; a < 8; a++) load8p(S + a * D, M[a]);
+      }
+      if constexpr (MODE == 2) {
+        float *S = p.S + bh * (size_t)(D * D) + 8 * ty * D + v0;
+#pragma unroll
+        for (int a = 0; a < 8; a++) store8p(S + a * D, M[a]);
+      } else {
+        // T_h = S w_h; w_h is the value side of the (h+1)-th newest record, or Walsh function h
+#pragma unroll 1
+        for (int h = 0; h < r; h++) {
+          float2 w[4];
+          if (SLOT && h < n) {
+            load8p(rec + (n - 1 - h) * RF + REC_U + v0, w);
           } else {
 #pragma unroll
-            for (int b = 0; b < 8; b++) w[b] = walsh_entry(h, 8 * t.tx + b);
+            for (int c = 0; c < 4; c++) w[c] = make_float2(walsh_entry(h, v0 + 2 * c), walsh_entry(h, v0 + 2 * c + 1));
           }
-        });
-      } else {
-        rows_times_vectors(M, t, r, Tm, [&](int h, float (&w)[8]) { load8(Wm + h * D + 8 * t.tx, w); });
-      }
-      LQ_BTICK(10);
-      if (it + 1 < p.n_iter) {
-        orthonormalize<false, RM>(p, sm, t, Tm, r, bh);
-        columns_times_vectors(M, sm, t, r, Tm, Wm);
-        orthonormalize<false, RM>(p, sm, t, Wm, r, bh);
-      }
-    }
-    orthonormalize<true, RM>(p, sm, t, Tm, r, bh);                // Tm now holds the keys as stored
-    LQ_BTICK(11);
-    gram_lower(Tm, r, sm.gram, t, false);                     // k_a^T k_h, a < h, in gram[h][a]
-    columns_times_vectors(M, sm, t, r, Tm, Wm);               // M^T k_h (its barriers also publish gram)
-    LQ_BTICK(13);
-    if (t.tid < D) {
-      const float *alive = sm.chol + MAX_R * MAX_R + MAX_R;
-      const int j = t.tid;
-      float x[RM], uf[RM];                                    // this column's sums, then its stored values u_a
-      uint16_t ub[RM];
+          float pr[8];
 #pragma unroll
-      for (int h = 0; h < RM; h++) x[h] = h < r ? Wm[h * D + j] : 0.0f;
-#pragma unroll
-      for (int h = 0; h < RM; h++) {
-        if (h < r) {
-#pragma unroll
-          for (int a = 0; a < h; a++) x[h] = fmaf(-uf[a], sm.gram[h * MAX_R + a], x[h]);
-          ub[h] = alive[h] != 0.0f ? to_f16_bits_sat(x[h]) : static_cast<uint16_t>(0);
-          uf[h] = f16_bits(ub[h]);
+          for (int a = 0; a < 8; a++) pr[a] = block8(M[a], w);
+          store_row_pairs(pr, ty, tx, part + (warp * RM + h) * D);
         }
       }
-#pragma unroll
-      for (int h = 0; h < RM; h++) {
-        if (h < r) {
-          p.comp_u(bh)[h * D + j] = ub[h];
-          Wm[h * D + j] = uf[h];
-        }
-      }
-    }
-    __syncthreads();
-    LQ_BTICK(14);
-    for (int h = 0; h < r; h++) {                             // M -= k u^T with the stored values
-      float kf[8], uf[8], nk[8];
-      load8(Tm + h * D + 8 * t.ty, kf);
-      load8(Wm + h * D + 8 * t.tx, uf);
-#pragma unroll
-      for (int a = 0; a < 8; a++) nk[a] = -kf[a];
-      rank1_update(M, nk, uf);
-    }
-  }
-  LQ_BTICK(4);
+      // the slot is free when all have come here: the next head may land while this one is worked on
+      if (SLOT) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      __syncthreads();
+      if (SLOT && k + 1 < count) request(todo_bh[k + 1], todo_n[k + 1]);
+      if (MODE == 1 && k + 1 < count && tid < 8)              // (dense states: at least into the L2)
+        bulk_prefetch_l2(p.S + todo_bh[k + 1] * (size_t)(D * D) + tid * (D * D / 8), D * D / 2);
 
-  // residual smoothing: c_i = max(sqrt(mean_j |R_ij|), 1e-6)
-  float c[8];
-  __syncthreads();   // every read of sm.vec / sm.part above is done
-  if (p.smooth) {
-    float pr[8];
+      if constexpr (MODE != 2) {
+        uint32_t alive = 0;
+        if (r > 0) {
+          for (int idx = tid; idx < r * D; idx += 256) T[idx] = sum_warps(part + idx, RM * D);
+          LQ_BTICK(10);
+          // further rounds: W_h = S^T q_h, orthonormalise, T_h = S q_h
+          for (int it = 1; it < p.n_iter; it++) {
+            orthonormalize<false, RM>(T, r, gram, chol, nullptr);
+#pragma unroll 1
+            for (int h = 0; h < r; h++) {
+              float x[8], pc[8];
+              load8(T + h * D + 8 * ty, x);
+              column_blocks(M, x, pc);
+              const float s = column_tree(pc, lane, [](float a, float b) { return a + b; });
+              if (lane < 16) Wv[h * D + v0 + column_of(lane)] = s;
+            }
+            orthonormalize<false, RM>(Wv, r, gram, chol, nullptr);
+#pragma unroll 1
+            for (int h = 0; h < r; h++) {
+              float2 w[4];
+              load8p(Wv + h * D + v0, w);
+              float pr[8];
 #pragma unroll
-    for (int a = 0; a < 8; a++) {                             // even and odd columns as two chains
-      float even = fabsf(M[a][0]), odd = fabsf(M[a][1]);
+              for (int a = 0; a < 8; a++) pr[a] = block8(M[a], w);
+              store_row_pairs(pr, ty, tx, part + (warp * RM + h) * D);
+            }
+            __syncthreads();
+            for (int idx = tid; idx < r * D; idx += 256) T[idx] = sum_warps(part + idx, RM * D);
+          }
+          alive = orthonormalize<true, RM>(T, r, gram, chol, p.comp_k(bh));       // T now holds the keys as stored
+          LQ_BTICK(11);
+          gram_lower<RM>(T, r, gram, false);                  // k_a^T k_h (published by the barrier in front of the value sides)
+
+          // ---- value sides and removal of the stored tokens ----
+          float x[RM];                                        // S^T k_h for the lane's column
 #pragma unroll
-      for (int b = 2; b < 8; b += 2) { even = even + fabsf(M[a][b]); odd = odd + fabsf(M[a][b + 1]); }
-      pr[a] = even + odd;
+          for (int h = 0; h < RM; h++) {
+            x[h] = 0.0f;
+            if (h < r) {
+              float kf[8], pc[8];
+              load8(T + h * D + 8 * ty, kf);
+              column_blocks(M, kf, pc);
+              x[h] = column_tree(pc, lane, [](float a, float b) { return a + b; });
+            }
+          }
+          __syncthreads();                                    // K^T K is complete
+          LQ_BTICK(13);
+          // u_h = S^T k_h - sum_{a<h} u_a (k_a^T k_h) with the stored values: what tokens 0..h-1 leave
+          float uf[RM];
+          const int col = column_of(lane);
+          uint16_t *cu_out = p.comp_u(bh) + v0 + col;
+#pragma unroll
+          for (int h = 0; h < RM; h++) {
+            uf[h] = 0.0f;
+            if (h < r) {
+#pragma unroll
+              for (int a = 0; a < h; a++) x[h] = fmaf(-uf[a], gram[h * RM + a], x[h]);
+              const uint16_t bits = (alive >> h) & 1u ? to_f16_bits_sat(x[h]) : static_cast<uint16_t>(0);
+              uf[h] = f16_bits(bits);
+              if (lane < 16) {
+                cu_out[h * D] = bits;
+                ub[16 * h + 8 * tx + col] = uf[h];
+              }
+            }
+          }
+          __syncwarp();
+          LQ_BTICK(14);
+#pragma unroll 1
+          for (int h = 0; h < r; h++) {                       // M -= k u^T with the stored values
+            float kf[8];
+            float2 uv[4];
+            load8(T + h * D + 8 * ty, kf);
+            load8p(ub + 16 * h + 8 * tx, uv);
+#pragma unroll
+            for (int a = 0; a < 8; a++) kf[a] = -kf[a];
+            rank1_pairs(M, kf, uv);
+          }
+        }
+        LQ_BTICK(4);
+        // ---- residual smoothing: c_i = max(sqrt(mean_j |R_ij|), 1e-6) ----
+        {
+          float pr[8];
+#pragma unroll
+          for (int a = 0; a < 8; a++) {                       // even and odd columns as two chains
+            float even = fabsf(M[a][0].x), odd = fabsf(M[a][0].y);
+#pragma unroll
+            for (int c = 1; c < 4; c++) { even = even + fabsf(M[a][c].x); odd = odd + fabsf(M[a][c].y); }
+            pr[a] = even + odd;
+          }
+          store_row_pairs(pr, ty, tx, part + warp * D);
+        }
+        __syncthreads();
+        if (tid < D) {
+          const float ci = p.smooth ? fmaxf(sqrtf(sum_warps(part + tid, D) / static_cast<float>(D)), 1e-6f) : 1.0f;
+          ic_s[tid] = p.smooth ? 1.0f / ci : 1.0f;
+          p.row_smooth(bh)[tid] = ci;
+        }
+        __syncthreads();
+        LQ_BTICK(5);
+
+        // ---- code steps and codes ----
+        {
+          float ic[8];
+          load8(ic_s + 8 * ty, ic);
+#pragma unroll
+          for (int a = 0; a < 8; a++)
+#pragma unroll
+            for (int c = 0; c < 4; c++) M[a][c] = __fmul2_rn(M[a][c], pair(ic[a]));
+        }
+        float m[8];
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          m[2 * c] = fabsf(M[0][c].x); m[2 * c + 1] = fabsf(M[0][c].y);
+#pragma unroll
+          for (int a = 1; a < 8; a++) {
+            m[2 * c] = fmaxf(m[2 * c], fabsf(M[a][c].x));
+            m[2 * c + 1] = fmaxf(m[2 * c + 1], fabsf(M[a][c].y));
+          }
+        }
+        const float amax = column_tree(m, lane, [](float a, float b) { return fmaxf(a, b); });
+        if (lane < 16) {
+          const int col = column_of(lane);
+          p.col_scale(bh)[v0 + col] = amax / 127.0f;          // stored as the step of the code, B_j / 127
+          invc[8 * tx + col] = amax > 0.0f ? 127.0f / amax : 0.0f;
+        }
+        __syncwarp();
+        LQ_BTICK(6);
+        float2 inv[4];
+        load8p(invc + 8 * tx, inv);
+        int8_t *ZT = p.codes(bh) + v0 * D + 8 * ty;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          // |X * inv| <= 127 (1 + 2^-23): adding 1.5 * 2^23 leaves the nearest integer (ties to even) in the low byte
+          // (product and sum are rounded one after the other; written as a packed addition the two would get fused)
+          float2 z[8];
+#pragma unroll
+          for (int a = 0; a < 8; a++) z[a] = __ffma2_rn(__fmul2_rn(M[a][c], inv[c]), pair(1.0f), pair(12582912.0f));
+          auto bytes4 = [](float x0, float x1, float x2, float x3) {
+            return __byte_perm(__byte_perm(__float_as_uint(x0), __float_as_uint(x1), 0x0040),
+                               __byte_perm(__float_as_uint(x2), __float_as_uint(x3), 0x0040), 0x5410);
+          };
+          *reinterpret_cast<uint2 *>(ZT + (2 * c) * D) =
+              make_uint2(bytes4(z[0].x, z[1].x, z[2].x, z[3].x), bytes4(z[4].x, z[5].x, z[6].x, z[7].x));
+          *reinterpret_cast<uint2 *>(ZT + (2 * c + 1) * D) =
+              make_uint2(bytes4(z[0].y, z[1].y, z[2].y, z[3].y), bytes4(z[4].y, z[5].y, z[6].y, z[7].y));
+        }
+        if (MODE == 1 && tid == 0) p.win_pos[bh / p.heads_v] = 0;      // (nobody reads win_pos in this mode)
+      }
+      if (k == 0) LQ_STAMP(1, 3);
+      LQ_BTICK(9);
     }
-    int sel;
-    const float tot = row_tree(pr, t.lane, sel);
-    if (t.tx < 8) {                                           // one thread per row: c_i and 1 / c_i
-      const float ci = fmaxf(sqrtf(tot / static_cast<float>(D)), 1e-6f);
-      sm.vec[8 * t.ty + sel] = ci;
-      sm.colv[8 * t.ty + sel] = 1.0f / ci;
-    }
-    __syncthreads();
-    load8(sm.vec + 8 * t.ty, c);
-    if (t.tx == 0) store8(p.row_smooth(bh) + 8 * t.ty, c);
-    LQ_BTICK(5);
-    load8(sm.colv + 8 * t.ty, c);                             // from here on c holds 1 / c_i
-#pragma unroll
-    for (int a = 0; a < 8; a++) {
-#pragma unroll
-      for (int b = 0; b < 8; b++) M[a][b] = M[a][b] * c[a];
-    }
-  } else {
-#pragma unroll
-    for (int a = 0; a < 8; a++) c[a] = 1.0f;                  // X = R / 1 = R
-    if (t.tx == 0) store8(p.row_smooth(bh) + 8 * t.ty, c);
+    __syncthreads();                         // the list is rewritten by the next round
   }
-  // per-value-channel scale: column maximum of |X| (exact in any order); one thread per column finishes it
-  {
-    float m[8];
-#pragma unroll
-    for (int b = 0; b < 8; b++) {
-      float s = fabsf(M[0][b]);
-#pragma unroll
-      for (int a = 1; a < 8; a++) s = fmaxf(s, fabsf(M[a][b]));
-      m[b] = fmaxf(s, __shfl_xor_sync(FULL, s, 16));
-    }
-    if (t.lane < 16) store8(sm.part + t.warp * D + 8 * t.tx, m);
-    __syncthreads();
-    const int col = threadIdx.x;
-    if (col < D) {
-      float amax = sm.part[col];
-#pragma unroll
-      for (int wv = 1; wv < 8; wv++) amax = fmaxf(amax, sm.part[wv * D + col]);
-      p.col_scale(bh)[col] = amax / 127.0f;                   // stored as the step of the code, B_j / 127
-      sm.cs[col] = amax > 0.0f ? 127.0f / amax : 0.0f;
-    }
-    __syncthreads();
-  }
-  LQ_BTICK(6);
-  float inv[8];
-  load8(sm.cs + 8 * t.tx, inv);
-  int8_t *ZT = p.codes(bh);
-#pragma unroll
-  for (int b = 0; b < 8; b++) {
-    // |X * inv| <= 127 (1 + 2^-23), so the nearest integer (ties to even) is already inside [-127, 127]
-    int z[8];
-#pragma unroll
-    for (int a = 0; a < 8; a++) z[a] = __float_as_int(M[a][b] * inv[b] + 12582912.0f);   // + 1.5 * 2^23: the low
-    // mantissa byte of the sum is the nearest integer (ties to even) in two's complement
-    const uint32_t lo = __byte_perm(__byte_perm(z[0], z[1], 0x0040), __byte_perm(z[2], z[3], 0x0040), 0x5410);
-    const uint32_t hi = __byte_perm(__byte_perm(z[4], z[5], 0x0040), __byte_perm(z[6], z[7], 0x0040), 0x5410);
-    *reinterpret_cast<uint2 *>(ZT + (8 * t.tx + b) * D + 8 * t.ty) = make_uint2(lo, hi);
-  }
+  LQ_STAMP(1, 4);
+#ifdef LQ_TIMING
+  if (tid == 0)
+    for (int i = 0; i < 16; i++) atomicAdd(&g_phase_cycles[32 + i], (unsigned long long)lq_bacc[i]);
+#endif
 }
 
 }  // namespace lq

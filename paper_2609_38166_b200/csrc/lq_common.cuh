@@ -101,6 +101,54 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // all but the most recently committed group have landed
 __device__ __forceinline__ void cp_async_wait_but_one() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
+// ---- mbarrier / TMA bulk copy (1-D) ----
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
+__device__ __forceinline__ void mbar_init(uint32_t bar, int count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+}
+// The arrival that announces the bytes of the next copies.  Relaxed: nothing this thread wrote has to be
+// visible to anybody through this barrier (the copies' own completion is what the waiters acquire), and the
+// default release form stalls the warp for about 800 cycles here.
+__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.relaxed.cta.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+}
+// global -> shared bulk copy; addresses and size are multiples of 16 bytes
+__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+// The same with an L2 eviction priority for the lines the copy brings in.
+__device__ __forceinline__ void bulk_g2s_hint(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;\n" ::"r"(dst),
+      "l"(src), "r"(bytes), "r"(bar), "l"(policy)
+      : "memory");
+}
+// Ask the L2 for a piece of global memory (no data comes back, nothing waits for it).
+__device__ __forceinline__ void bulk_prefetch_l2(const void *src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(src), "r"(bytes) : "memory");
+}
+// Bounded wait for phase `parity`; false if the limit of LIMIT polls ran out (the caller then reports and bails out).
+template <int LIMIT = (1 << 20)>
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+  for (int spin = 0; spin < LIMIT; spin++) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+
+// Set when a bounded wait gave up (bit 0: a wait for bulk copies; bit 3: the wait of lq_selftest_bounded_wait).  Never cleared
+// by kernels: lq_clear_device_flags.
+__device__ int g_device_error = 0;
+
 // ---- sum of sixteen block results held by sixteen neighbouring lanes (tree levels 1, 2, 4, 8) ----
 __device__ __forceinline__ float tree16(float x) {
   x = x + __shfl_xor_sync(FULL, x, 1);
@@ -351,11 +399,11 @@ __device__ __forceinline__ int nth_set_bit(uint32_t m, unsigned k) {
 // One warp finds up to 32 of a CTA's heads in one pass over win_pos: lane l looks for due head number first + l * stride.
 // Returns how many lanes found theirs (lanes 0 .. count-1); bh and n are the head and its buffered records, `total` how
 // many sequences are due in all.
-__device__ __forceinline__ int find_due_heads(const Params &p, size_t first, size_t stride, int lane, size_t &bh, int &n,
+__device__ __forceinline__ int find_due_heads(const Params &p, unsigned first, unsigned stride, int lane, unsigned &bh, int &n,
                                               int &total) {
   constexpr int U = 8;                       // loads in flight per lane
-  const size_t item = first + lane * stride;
-  const unsigned want = static_cast<unsigned>(item / p.heads_v);       // rank of the head's sequence among the due ones
+  const unsigned item = first + lane * stride;
+  const unsigned want = item / static_cast<unsigned>(p.heads_v);       // rank of the head's sequence among the due ones
   unsigned base = 0;
   bool found = false;
   bh = 0; n = 0;
@@ -374,7 +422,7 @@ __device__ __forceinline__ int find_due_heads(const Params &p, size_t first, siz
       if (mine) {
         found = true;
         n = nv < p.W ? nv : p.W;
-        bh = (size_t)(b0 + 32 * u + pos) * p.heads_v + (item - (size_t)want * p.heads_v);
+        bh = static_cast<unsigned>(b0 + 32 * u + pos) * p.heads_v + (item - want * p.heads_v);
       }
       base += c;
     }
@@ -401,15 +449,9 @@ __device__ __forceinline__ void restart_due_windows(const Params &p, int lane) {
 // the value in bits 0..15.  The head that arrives last (all heads_v have read the old value by then)
 // stores the new value and thereby clears the counter.  Call from one thread per head, after a
 // __syncthreads() that follows the head's last global write.
-// FENCED: for readers inside the same kernel, who take the new value as the sign that every head's writes are
-// there (each arriving head fences before the call, the last one again before it stores).
-template <bool FENCED = false>
 __device__ __forceinline__ void arrive_and_set(int32_t *win_pos, int b, int heads_v, int new_value) {
   const int old = atomicAdd(win_pos + b, 0x10000);
-  if ((old >> 16) == heads_v - 1) {
-    if (FENCED) __threadfence();
-    win_pos[b] = new_value;
-  }
+  if ((old >> 16) == heads_v - 1) win_pos[b] = new_value;
 }
 
 }  // namespace lq

@@ -36,10 +36,6 @@
 
 namespace lq {
 
-// Set when a bounded wait gave up (bit 0: a decode warp's wait for one of its bulk copies; bits 1, 2: the fused step
-// kernel's waits; bit 3: the wait of lq_selftest_bounded_wait).  Never cleared by kernels: lq_clear_device_flags.
-__device__ int g_device_error = 0;
-
 // Rows of the record buffer that a decode slot holds at a time (a multiple of four: the walk takes the records four
 // at a time from the newest back, so a group of four never straddles two segments).
 constexpr int REC_SEG = 32;                // (16 was tried: no faster at W = 32 or 64)
@@ -81,50 +77,6 @@ __device__ __forceinline__ void fixed_point_scales(float xmax, float &scale, flo
   const int e = static_cast<int>((__float_as_uint(xmax) >> 23) & 0xFF) - 127;
   scale = __uint_as_float(static_cast<uint32_t>(29 - e + 127) << 23);
   back = __uint_as_float(static_cast<uint32_t>(e - 29 + 127) << 23);
-}
-
-// ---- mbarrier / TMA bulk copy (1-D) ----
-__device__ __forceinline__ uint32_t smem_addr(const void *p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
-__device__ __forceinline__ void mbar_init(uint32_t bar, int count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
-  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-}
-// The arrival that announces the bytes of the next copies.  Relaxed: nothing this thread wrote has to be
-// visible to anybody through this barrier (the copies' own completion is what the waiters acquire), and the
-// default release form stalls the warp for about 800 cycles here.
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.relaxed.cta.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
-}
-// global -> shared bulk copy; addresses and size are multiples of 16 bytes
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
-}
-// The same with an L2 eviction priority for the lines the copy brings in.
-__device__ __forceinline__ void bulk_g2s_hint(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar, uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;\n" ::"r"(dst),
-      "l"(src), "r"(bytes), "r"(bar), "l"(policy)
-      : "memory");
-}
-// Ask the L2 for a piece of global memory (no data comes back, nothing waits for it).
-__device__ __forceinline__ void bulk_prefetch_l2(const void *src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(src), "r"(bytes) : "memory");
-}
-// Bounded wait for phase `parity`; false if the limit of LIMIT polls ran out (the caller then reports and bails out).
-template <int LIMIT = (1 << 20)>
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  for (int spin = 0; spin < LIMIT; spin++) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
 }
 
 __device__ __forceinline__ void widen8_bf16(const uint4 w, float (&x)[8]) {
@@ -196,42 +148,14 @@ __device__ __forceinline__ void load_token(const Params &p, const HeadIdx h, int
   }
 }
 
-// Counters of the fused step kernel (lq_fused.cuh): decode slots that are through with the heads whose window
-// becomes full, and CTAs that have left; the last CTA to leave clears both.
-__device__ unsigned g_fused_boundary_heads_done = 0, g_fused_exit_ticket = 0;
-
 // The work of one pair of warps (role 0: stream warp, role 1: dot warp) on its shared-memory slot: heads
-// first, first + G, first + 2G, ...  The named barriers it uses are bar0 + 1 .. bar0 + 5.
-// FUSED (the step kernel that also takes the window boundaries): two passes over the heads, first those whose
-// window becomes full with this token, so that their boundaries can start while the rest is decoded; the
-// arrival on win_pos comes after BOTH warps' global writes of the head, because another CTA acts on it;
-// and the window positions of all of the slot's heads are read once, up front, into nbuf (a sequence whose
-// boundary is taken meanwhile goes back to position 0, which must not be mistaken for a fresh window).
-// Before the first pass: the slot's two copy barriers, and (fused) the window positions of all its heads.
-template <int GATE, bool R16, bool FUSED>
-__device__ __forceinline__ void decode_slot_init(const Params &p, unsigned char *slot, const int lane, const int role,
-                                                 const int bar0, const unsigned first, const unsigned G, uint16_t *nbuf) {
-  const DecodeSlot L(p.W, p.r, GATE == LQ_GATE_DIAG, R16);
-  const uint32_t barA = smem_addr(slot + L.mbar), barR = barA + 8;
-  if (role == 0 && lane == 0) { mbar_init(barA, 1); mbar_init(barR, 1); }
-  if (FUSED) {
-    const unsigned nh = static_cast<unsigned>(p.batch) * p.heads_v;
-    for (unsigned k = 32 * role + lane; first + k * G < nh; k += 64)
-      nbuf[k] = static_cast<uint16_t>(p.win_pos[(first + k * G) / p.heads_v] & 0xFFFF);
-  }
-  named_wait(bar0 + 1);                      // both warps: the barriers are initialised, nbuf is complete
-}
-
-// PASS: 0 in the ordinary kernel; in the fused one 0 = the heads whose window fills with this token, 1 = the
-// others (two instances of the code: only the first carries the fences that publish a head to other CTAs, and a
-// fence anywhere in the loop costs every trip).  parA, parR: the phases of the two copy barriers, carried over.
+// first, first + G, first + 2G, ...
 // LONGW: the window may hold more records than the slot stages at a time (W - 1 > REC_SEG); in the instances for
 // shorter windows everything to do with a second segment drops out at compile time.
-template <int GATE, bool R16, bool FUSED, int PASS, bool LONGW = true>
+template <int GATE, bool R16, bool LONGW>
 __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot, const int lane, const int role,
-                                            const int bar0, const unsigned first, const unsigned G,
-                                            uint16_t *nbuf, uint32_t &parA, uint32_t &parR) {
-  constexpr int pass = PASS;
+                                            const unsigned first, const unsigned G) {
+  uint32_t parA = 0, parR = 0;               // phases of the slot's two copy barriers
   constexpr bool DIAG = GATE == LQ_GATE_DIAG;
   constexpr int RF = record_floats(DIAG);
   const int W = p.W, r = p.r;
@@ -311,7 +235,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
   // A pair stops when a ticket is beyond the pool.
   const int rounds_all = static_cast<int>(nh / G);             // rounds in which every pair has a head
   const int DRAWN_ROUNDS = rounds_all >= 6 ? 2 : 1;            // (with few rounds, more of them in turn)
-  const bool draw = !FUSED && p.work != nullptr && rounds_all >= 3;
+  const bool draw = p.work != nullptr && rounds_all >= 3;
   const int S = draw ? rounds_all - DRAWN_ROUNDS : 0;
   const unsigned pool = draw ? nh - static_cast<unsigned>(S) * G : 0;
   // Per-head scalars of this CTA's heads, 32 heads at a time: lane l holds those of the CTA's (32*batch+l)-th head
@@ -320,8 +244,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
   auto load_scalars = [&](unsigned first_bh) {
     const unsigned bh = first_bh + lane * G;  // (once per 32 heads: a division is fine here)
     if (bh < (draw ? static_cast<unsigned>(S) * G : nh)) {     // (the heads taken in turn)
-      sc_n = FUSED ? nbuf[(first_bh - first) / G + lane]
-                   : p.win_pos[bh / Hv];    // bits 16.. are the arrival counter of this launch: masked at use
+      sc_n = p.win_pos[bh / Hv];             // bits 16.. are the arrival counter of this launch: masked at use
       sc_beta = p.beta[bh];
       if (!DIAG) sc_alpha = p.alpha[bh];
     }
@@ -331,8 +254,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
   // value, which this head did when its scalars were loaded.  The dot warp makes the arrival, at the end of its
   // work: it has slack, the stream warp (the longer of the two) has none to sit out the atomic's round trip.
   // A head whose window is already full (n >= W) gets no token: it is neither requested nor waited for.
-  // which heads this pass takes: all that get a token, or (fused) those at / not at their last free record
-  auto wanted = [&](int n_) { return n_ < W && (!FUSED || (n_ == W - 1) == (pass == 0)); };
+  auto wanted = [&](int n_) { return n_ < W; };
   load_scalars(first);
   TokenRaw nxt;                               // the token of the head about to start
   nxt.ba_lo = nxt.ba_hi = 1.0f;
@@ -415,9 +337,9 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         if (role == 1) {
           if (lane == 0) *qidx = ticket;
           __syncwarp();
-          named_arrive(bar0 + 1);
+          named_arrive(1);
         } else {
-          named_wait(bar0 + 1);
+          named_wait(1);
         }
       }
       continue;
@@ -514,7 +436,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
       for (int jt = n - 1; jt >= 0; jt -= 4) {       // records jt, jt-1, jt-2, jt-3
         if (LONGW && jt < base) {                    // the segment is walked: fetch the one before it
           __syncwarp();
-          if (DIAG) named_wait(bar0 + 4);            // (the stream warp has taken this segment's decays as well)
+          if (DIAG) named_wait(4);            // (the stream warp has taken this segment's decays as well)
           request_segment(bh, n, base);
           base = seg_base(base);
           wait_for(barR, parR);
@@ -589,19 +511,19 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         }
       }
       __syncwarp();
-      named_arrive(bar0 + 3);                       // the compensator projections are in pk, pq; this warp is done with the head block
+      named_arrive(3);                       // the compensator projections are in pk, pq; this warp is done with the head block
       LQ_TICK(4);
-      if (DIAG) named_wait(bar0 + 4);               // diagonal gate: the stream warp read the records' decays too
+      if (DIAG) named_wait(4);               // diagonal gate: the stream warp read the records' decays too
       {
         const int n_next = n_next_now();
         if (wanted(n_next)) request_records(bh_next, n_next);
       }
-      named_wait(bar0 + 2);                         // the stream warp has taken its sums out of y
+      named_wait(2);                         // the stream warp has taken its sums out of y
       *reinterpret_cast<float4 *>(y + 4 * lane) = make_float4(rk_rec[0], rk_rec[1], rk_rec[2], rk_rec[3]);
       *reinterpret_cast<float4 *>(y + D + 4 * lane) = make_float4(rq_rec[0], rq_rec[1], rq_rec[2], rq_rec[3]);
       if (draws && lane == 0) *qidx = ticket;
       __syncwarp();
-      named_arrive(bar0 + 1);                       // the record terms are in shared memory (and the ticket)
+      named_arrive(1);                       // the record terms are in shared memory (and the ticket)
       LQ_TICK(5);
       // append the key side of the record (and its decay)
       {
@@ -612,11 +534,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
           else if (lane == 0) p.decays[bh * (size_t)W + n] = a8[0];
         }
       }
-      if (FUSED && pass == 0) {              // a boundary CTA will read this head's record: the stream warp's u is
-        named_wait(bar0 + 5);                // out as well, and both warps' writes are ordered before the arrival
-        __threadfence();
-      }
-      if (lane == 0) arrive_and_set<FUSED && PASS == 0>(p.win_pos, b, p.heads_v, n + 1);
+      if (lane == 0) arrive_and_set(p.win_pos, b, p.heads_v, n + 1);
       LQ_TICK(7);
     } else {
       // =========================== STREAM WARP ===========================
@@ -636,7 +554,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
             for (int e = 0; e < 8; e++) gam[e] = gam[e] * aj[e];
           }
           __syncwarp();
-          named_arrive(bar0 + 4);                   // this warp is done with the segment
+          named_arrive(4);                   // this warp is done with the segment
           if (lo == 0) break;
           hi = lo;
         }
@@ -741,8 +659,8 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         const float v4[4] = {__uint_as_float(v_raw.x << 16), __uint_as_float(v_raw.x & 0xFFFF0000u),
                              __uint_as_float(v_raw.y << 16), __uint_as_float(v_raw.y & 0xFFFF0000u)};
         LQ_TICK(6);
-        named_arrive(bar0 + 2);                     // y has been read: the dot warp may put the record terms there
-        named_wait(bar0 + 3);                       // the compensator projections are complete
+        named_arrive(2);                     // y has been read: the dot warp may put the record terms there
+        named_wait(3);                       // the compensator projections are complete
         LQ_TICK(7);
 #pragma unroll 2
         for (int h = 0; h < r; h++) {
@@ -759,7 +677,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
           const int n_next = n_next_now();
           if (wanted(n_next)) request_head(bh_next, n_next);   // it before barrier 3): the next head's may land
         }
-        named_wait(bar0 + 1);                       // the record terms are complete
+        named_wait(1);                       // the record terms are complete
         {
           const float4 tk = *reinterpret_cast<const float4 *>(y + 4 * lane);
           const float4 tq = *reinterpret_cast<const float4 *>(y + D + 4 * lane);
@@ -773,17 +691,9 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         LQ_TICK(8);
         *reinterpret_cast<float4 *>(p.o + bh * D + 4 * lane) = make_float4(o[0], o[1], o[2], o[3]);
         store4(p.record<rec_t>(bh, n, DIAG) + REC_U + 4 * lane, u[0], u[1], u[2], u[3]);
-        if (FUSED && pass == 0) {
-          __threadfence();
-          named_arrive(bar0 + 5);
-        }
       }
       LQ_TICK(9);
     }
-  }
-  if (FUSED && pass == 0 && role == 1 && lane == 0) {       // every head of this slot whose window fills has arrived
-    __threadfence();
-    atomicAdd(&g_fused_boundary_heads_done, 1u);
   }
 #ifdef LQ_TIMING
   if (lane == 0)
@@ -802,11 +712,15 @@ __global__ void __launch_bounds__(64, 6) decode_kernel(const Params p) {
   if (threadIdx.x == 0 && blockIdx.x < static_cast<unsigned>(p.batch) * p.heads_v)
     bulk_prefetch_l2(p.head(blockIdx.x), head_bytes(p.r));
   const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
-  uint32_t parA = 0, parR = 0;
-  decode_slot_init<GATE, R16, false>(p, lq_slot, lane, role, 0, blockIdx.x, gridDim.x, nullptr);      // (shared memory only)
+  if (threadIdx.x == 0) {                    // the slot's two copy barriers (shared memory only)
+    const uint32_t bar = smem_addr(lq_slot + DecodeSlot(p.W, p.r, GATE == LQ_GATE_DIAG, R16).mbar);
+    mbar_init(bar, 1);
+    mbar_init(bar + 8, 1);
+  }
+  __syncthreads();
   grid_dependency_wait();                    // no data in global memory is read or written above this line
   LQ_STAMP(0, 1);
-  decode_slot<GATE, R16, false, 0, LONGW>(p, lq_slot, lane, role, 0, blockIdx.x, gridDim.x, nullptr, parA, parR);
+  decode_slot<GATE, R16, LONGW>(p, lq_slot, lane, role, blockIdx.x, gridDim.x);
   LQ_STAMP(0, 3);
 #ifdef LQ_TIMING
   if (threadIdx.x == 0 && blockIdx.x < 1024) {
