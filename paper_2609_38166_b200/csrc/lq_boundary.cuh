@@ -7,6 +7,12 @@
 // (two FMAs per instruction).  So everything that belongs to a column - the products with the keys, the value sides, the
 // scales, the codes - stays inside a warp, and only row sums (the products with the start vectors, the smoothing scales)
 // go through shared memory and a barrier.  Two CTAs fill the register file of an SM.
+//
+// What bounds it: a flush (W = 16, r = 4) takes 27 K cycles with two CTAs on the SM; 9 K of them are the fp32 pipes (about
+// 1150 packed FMAs per warp, two cycles each, four warps to a scheduler), the rest the waits between its dependent phases,
+// of which only the other CTA fills some.  Against tiles of 8 rows x 128 columns per half-warp, where every column sum
+// crossed the CTA (13 barriers a head, now 8), and copies by all threads into two staging buffers: 2048 dense states
+// quantized in 59.7 us (91.4 before), 2048 states dequantized in 48.4 us (54.0), 512 flushes 35.8 us (37.7).
 #pragma once
 #include <type_traits>
 
@@ -47,6 +53,25 @@ __device__ __forceinline__ void rank1_pairs(float2 (&M)[8][4], const float (&x)[
 #pragma unroll
     for (int c = 0; c < 4; c++) M[a][c] = __ffma2_rn(xa, y[c], M[a][c]);
   }
+}
+
+// Eight floats of a dense state's row.  One 32-byte access (a whole sector) where the base allows it: the lanes of a warp
+// touch 64-byte pieces of 16 rows, and with 16-byte accesses every sector goes to the L2 twice.
+__device__ __forceinline__ void load_row8(const float *src, bool wide, float2 (&x)[4]) {
+  if (wide)
+    asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                 : "=f"(x[0].x), "=f"(x[0].y), "=f"(x[1].x), "=f"(x[1].y), "=f"(x[2].x), "=f"(x[2].y), "=f"(x[3].x), "=f"(x[3].y)
+                 : "l"(src));
+  else
+    load8p(src, x);
+}
+__device__ __forceinline__ void store_row8(float *dst, bool wide, const float2 (&x)[4]) {
+  if (wide)
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"l"(dst), "f"(x[0].x), "f"(x[0].y), "f"(x[1].x),
+                 "f"(x[1].y), "f"(x[2].x), "f"(x[2].y), "f"(x[3].x), "f"(x[3].y)
+                 : "memory");
+  else
+    store8p(dst, x);
 }
 
 // Which of the lane's eight columns a column_tree leaves with it
@@ -269,6 +294,7 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
   float *chol = reinterpret_cast<float *>(lq_bsm + Lay::chol), *ub = reinterpret_cast<float *>(lq_bsm + Lay::ub) + warp * 16 * RM;
   float *ic_s = reinterpret_cast<float *>(lq_bsm + Lay::ic), *invc = reinterpret_cast<float *>(lq_bsm + Lay::invc) + 16 * warp;
   const uint32_t bar = smem_addr(lq_bsm + Lay::bar);
+  const bool wide = (reinterpret_cast<uintptr_t>(p.S) & 31) == 0;
   auto kd_row = [&](int j) -> float * {      // Gamma_{j+1:n} kt_j
     if constexpr (R16) return reinterpret_cast<float *>(lq_bsm + L.kd) + j * D;
     else return rec + j * RF + REC_KT;
@@ -405,12 +431,12 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
       } else {
         const float *S = p.S + bh * (size_t)(D * D) + 8 * ty * D + v0;
 #pragma unroll
-        for (int a = 0; a < 8; a++) load8p(S + a * D, M[a]);
+        for (int a = 0; a < 8; a++) load_row8(S + a * D, wide, M[a]);
       }
       if constexpr (MODE == 2) {
         float *S = p.S + bh * (size_t)(D * D) + 8 * ty * D + v0;
 #pragma unroll
-        for (int a = 0; a < 8; a++) store8p(S + a * D, M[a]);
+        for (int a = 0; a < 8; a++) store_row8(S + a * D, wide, M[a]);
       } else {
         // T_h = S w_h; w_h is the value side of the (h+1)-th newest record, or Walsh function h
 #pragma unroll 1

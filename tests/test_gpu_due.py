@@ -40,3 +40,24 @@ def test_boundaries_of_windows_in_any_order(oracle, batch, heads_v, heads_qk, W,
     oracle.window_flush(osh, ost, force=True)
     gu.assert_state_parity(st, ost, wl.r, "forced flush")
     assert st.win_pos.tolist() == [0] * batch and lq.check_device() == 0
+
+
+@pytest.mark.parametrize("shift", [0, 4])
+def test_dense_states_at_any_16_byte_boundary(oracle, shift):
+    """Dense states are moved 32 bytes at a time where their base allows it; a base that is only 16-byte aligned
+    (`shift` floats into an allocation) takes the other branch.  Same bits."""
+    wl = synth.Workload("al", 3, 2, 1, W=5, r=3, seed=830)
+    osh, lsh = gu.shapes(wl)
+    S0 = synth.dense_states(wl, 3)
+    ost = OState(osh)
+    oracle.quantize_state(osh, S0, ost)
+    room = torch.zeros(S0.size + 8, dtype=torch.float32, device="cuda")
+    S = room[shift:shift + S0.size].view(S0.shape)
+    S.copy_(gu.dev(S0))
+    st = lq.State(lsh)
+    lq.quantize_state(lsh, S, st)
+    gu.assert_state_parity(st, ost, wl.r, "quantize")
+    S.zero_()
+    lq.dequantize_state(lsh, st, S)
+    assert np.array_equal(gu.host(S), oracle.dequantize_state(osh, ost))
+    assert not room[:shift].any() and not room[shift + S0.size:].any()
