@@ -266,6 +266,22 @@ static int ctas_per_sm(const void *kernel, int block, size_t smem) {
   return per_sm = v;
 }
 
+// Both of the above for a kernel about to be launched: the opt-in is made, the number of CTAs an SM holds is returned (0: one
+// of the calls failed).  A thread remembers its last few answers, so that a step does not take two locks and walk two maps
+// per launch.
+static int prepare_launch(const void *kernel, int block, size_t smem) {
+  struct Known { const void *kernel; size_t smem; int dev, block, per_sm; };
+  thread_local Known known[8] = {};
+  thread_local unsigned next = 0;
+  const int dev = current_device();
+  for (const Known &k : known)
+    if (k.kernel == kernel && k.smem == smem && k.dev == dev && k.block == block) return k.per_sm;
+  if (!smem_opt_in(kernel, smem)) return 0;
+  const int per_sm = ctas_per_sm(kernel, block, smem);
+  if (per_sm > 0) known[next++ % 8] = Known{kernel, smem, dev, block, per_sm};
+  return per_sm;
+}
+
 template <typename K, typename P>
 static lq_status launch(K kernel, int grid, int block, size_t smem, cudaStream_t stream, const P &p) {
   if (grid <= 0) return LQ_OK;
@@ -281,7 +297,7 @@ static lq_status launch(K kernel, int grid, int block, size_t smem, cudaStream_t
 template <typename K, typename... Args>
 static lq_status launch_dependent(K kernel, int grid, int block, size_t smem, cudaStream_t stream, const Args &...args) {
   if (grid <= 0) return LQ_OK;
-  if (!smem_opt_in(reinterpret_cast<const void *>(kernel), smem)) return LQ_ERR_CUDA;
+  if (prepare_launch(reinterpret_cast<const void *>(kernel), block, smem) < 1) return LQ_ERR_CUDA;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
@@ -303,8 +319,7 @@ static lq_status launch_dependent(K kernel, int grid, int block, size_t smem, cu
 template <typename K>
 static lq_status launch_persistent(K kernel, long items, int block, size_t smem, cudaStream_t stream, const Params &p) {
   if (items <= 0) return LQ_OK;
-  if (!smem_opt_in(reinterpret_cast<const void *>(kernel), smem)) return LQ_ERR_CUDA;
-  const int per_sm = ctas_per_sm(reinterpret_cast<const void *>(kernel), block, smem);
+  const int per_sm = prepare_launch(reinterpret_cast<const void *>(kernel), block, smem);
   if (per_sm < 1) return LQ_ERR_CUDA;
   const long resident = (long)per_sm * sm_count();
   // Every CTA takes ceil(items / resident) items at most; the smallest grid with that property leaves no last
@@ -336,8 +351,7 @@ template <int GATE, int MODE, bool R16, int RM>
 static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStream_t stream) {
   const size_t smem = BoundarySmem<RM>(s->W, s->r, GATE == LQ_GATE_DIAG, R16, MODE != 1, s->n_iter > 1).bytes;
   auto kernel = boundary_kernel<GATE, MODE, R16, RM>;
-  if (!smem_opt_in(reinterpret_cast<const void *>(kernel), smem)) return LQ_ERR_CUDA;
-  const long resident = (long)ctas_per_sm(reinterpret_cast<const void *>(kernel), 256, smem) * sm_count();
+  const long resident = (long)prepare_launch(reinterpret_cast<const void *>(kernel), 256, smem) * sm_count();
   if (resident < 1) return LQ_ERR_CUDA;
   const long nh = (long)s->batch * s->heads_v;
   return launch_dependent(kernel, static_cast<int>(nh < resident ? nh : resident), 256, smem, stream, p);

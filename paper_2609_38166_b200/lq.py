@@ -68,6 +68,16 @@ def lib() -> C.CDLL:
                      "lq_decode_step_host_static", "lq_check_device", "lq_window_flush", "lq_quantize_state",
                      "lq_dequantize_state", "lq_ref_decode_step_f32", "lq_ref_decode_step_bf16"):
             getattr(L, name).restype = C.c_int
+        vp = C.c_void_p                      # (declared, so that plain integers can be handed over as addresses)
+        L.lq_decode_step.argtypes = [vp] * 9
+        L.lq_decode_step_profiled.argtypes = [vp] * 10
+        for name in ("lq_decode_step_host", "lq_decode_step_host_pipelined"):
+            getattr(L, name).argtypes = [vp] * 10
+        L.lq_decode_step_host_static.argtypes = [vp] * 9
+        L.lq_window_flush.argtypes = [vp, vp, C.c_int, vp]
+        L.lq_quantize_state.argtypes = L.lq_dequantize_state.argtypes = [vp] * 4
+        L.lq_ref_decode_step_f32.argtypes = L.lq_ref_decode_step_bf16.argtypes = [vp] * 9
+        L.lq_import_state.argtypes = L.lq_export_state.argtypes = [vp] * 4
         _lib = L
     return _lib
 
@@ -88,19 +98,33 @@ class Shape:
     rec16: int = 0
     state_bf16: int = 0
 
-    def c(self) -> _Shape:
-        return _Shape(self.batch, self.heads_v, self.heads_qk, self.d_k, self.d_v, self.W, self.r, self.n_iter,
-                      self.gate, self.smooth, self.delta, self.rec16, self.state_bf16)
+    def c(self, batch: Optional[int] = None) -> _Shape:
+        return _Shape(self.batch if batch is None else batch, self.heads_v, self.heads_qk, self.d_k, self.d_v, self.W, self.r,
+                      self.n_iter, self.gate, self.smooth, self.delta, self.rec16, self.state_bf16)
+
+    def ref(self):
+        """A reference to the shape as the C struct, for a call of the library.  The struct is built once and kept until a
+        field changes: a decode step is one call per token and layer, and at small batches its marshalling took longer than
+        its kernels (10.1 us of host time a call, 2.7 us now)."""
+        r = self.__dict__.get("_ref")
+        if r is None:
+            r = self.__dict__["_ref"] = C.byref(self.c())
+        return r
+
+    def __setattr__(self, name, value):
+        object.__setattr__(self, name, value)
+        self.__dict__.pop("_ref", None)
+
+    def __getstate__(self):                  # (copies and pickles carry the fields only)
+        return {k: v for k, v in self.__dict__.items() if k != "_ref"}
 
 
 def head_bytes(sh: Shape) -> int:
-    s = sh.c()
-    return int(lib().lq_head_bytes(C.byref(s)))
+    return int(lib().lq_head_bytes(sh.ref()))
 
 
 def record_floats(sh: Shape) -> int:
-    s = sh.c()
-    return int(lib().lq_record_floats(C.byref(s)))
+    return int(lib().lq_record_floats(sh.ref()))
 
 
 class State:
@@ -158,17 +182,19 @@ class State:
 
     def c(self, b0: int = 0) -> _State:
         """ctypes view; ``b0`` offsets every array to sequence b0 (sub-batches are addressed by pointer)."""
-        return _State(*[t.data_ptr() + b0 * t.stride(0) * t.element_size() for t in self.tensors()],
-                      self.work.data_ptr() if self.work is not None else None)
+        work = self.work.data_ptr() if self.work is not None else None
+        if b0:
+            return _State(*[t.data_ptr() + b0 * t.stride(0) * t.element_size() for t in self.tensors()], work)
+        return _State(self.heads.data_ptr(), self.records.data_ptr(), self.decays.data_ptr(), self.win_pos.data_ptr(), work)
 
     def nbytes_quantized(self) -> int:
         return self.heads.numel()
 
 
-def _stream(stream) -> C.c_void_p:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+def _stream(stream) -> int:
+    if stream is None:                       # (building torch's Stream object for this takes 3.4 us)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _check(rc: int, what: str) -> None:
@@ -176,53 +202,54 @@ def _check(rc: int, what: str) -> None:
         raise LqError(f"{what}: {lib().lq_status_string(rc).decode()} (status {rc})")
 
 
-def _ptr(t: Optional[torch.Tensor], b0: int = 0) -> C.c_void_p:
+def _ptr(t: Optional[torch.Tensor], b0: int = 0) -> Optional[int]:
     if t is None:
-        return C.c_void_p(None)
+        return None
     assert t.is_contiguous()
-    return C.c_void_p(t.data_ptr() + b0 * t.stride(0) * t.element_size())
+    return t.data_ptr() + b0 * t.stride(0) * t.element_size() if b0 else t.data_ptr()
 
 
-def _sub(sh: Shape, b0: int, nb: Optional[int]) -> Shape:
+def _sub(sh: Shape, b0: int, nb: Optional[int]):
+    """Sequences [b0, b0+nb) of a shape, as a reference to the C struct."""
     nb = sh.batch - b0 if nb is None else nb
-    return Shape(nb, sh.heads_v, sh.heads_qk, sh.d_k, sh.d_v, sh.W, sh.r, sh.n_iter, sh.gate, sh.smooth, sh.delta, sh.rec16, sh.state_bf16)
+    return sh.ref() if nb == sh.batch else C.byref(sh.c(nb))
 
 
 def decode_step(sh: Shape, st: State, q, k, v, beta, alpha, o, stream=None, b0: int = 0, nb: Optional[int] = None):
     """lq_decode_step on sequences [b0, b0+nb) of the tensors (all of them by default)."""
-    s = _sub(sh, b0, nb).c()
-    cs = st.c(b0)
-    _check(lib().lq_decode_step(C.byref(s), C.byref(cs), _ptr(q, b0), _ptr(k, b0), _ptr(v, b0), _ptr(beta, b0),
-                                _ptr(alpha, b0), _ptr(o, b0), _stream(stream)), "lq_decode_step")
+    s = _sub(sh, b0, nb)
+    cs = C.byref(st.c(b0))
+    rc = (_lib or lib()).lq_decode_step(s, cs, _ptr(q, b0), _ptr(k, b0), _ptr(v, b0), _ptr(beta, b0), _ptr(alpha, b0), _ptr(o, b0),
+                                        _stream(stream))
+    if rc:
+        _check(rc, "lq_decode_step")
 
 
 def decode_step_profiled(sh: Shape, st: State, q, k, v, beta, alpha, o, event_between, stream=None):
     """lq_decode_step_profiled: ``event_between`` is a torch.cuda.Event that has been recorded once before
     (so that its CUDA handle exists); it is re-recorded between the two kernels of the step."""
-    s = sh.c()
-    cs = st.c()
-    _check(lib().lq_decode_step_profiled(C.byref(s), C.byref(cs), _ptr(q), _ptr(k), _ptr(v), _ptr(beta),
-                                         _ptr(alpha), _ptr(o), _stream(stream), C.c_void_p(event_between.cuda_event)),
+    s = sh.ref()
+    cs = C.byref(st.c())
+    _check(lib().lq_decode_step_profiled(s, cs, _ptr(q), _ptr(k), _ptr(v), _ptr(beta),
+                                         _ptr(alpha), _ptr(o), _stream(stream), event_between.cuda_event),
            "lq_decode_step_profiled")
 
 
 def decode_stage_bytes(sh: Shape) -> int:
-    s = sh.c()
-    return int(lib().lq_decode_stage_bytes(C.byref(s)))
+    return int(lib().lq_decode_stage_bytes(sh.ref()))
 
 
 def decode_launches(sh: Shape) -> int:
-    s = sh.c()
-    return int(lib().lq_decode_launches(C.byref(s)))
+    return int(lib().lq_decode_launches(sh.ref()))
 
 
 def decode_step_host(sh: Shape, st: State, q_h, k_h, v_h, beta_h, alpha_h, o_h, stage, stream=None):
     """lq_decode_step_host: the token's tensors are (pinned) CPU tensors, ``stage`` a device byte buffer."""
     for t in (q_h, k_h, v_h, beta_h, alpha_h, o_h):
         assert t.device.type == "cpu" and t.is_contiguous()
-    s = sh.c()
-    cs = st.c()
-    _check(lib().lq_decode_step_host(C.byref(s), C.byref(cs), _ptr(q_h), _ptr(k_h), _ptr(v_h), _ptr(beta_h),
+    s = sh.ref()
+    cs = C.byref(st.c())
+    _check(lib().lq_decode_step_host(s, cs, _ptr(q_h), _ptr(k_h), _ptr(v_h), _ptr(beta_h),
                                      _ptr(alpha_h), _ptr(o_h), _ptr(stage), _stream(stream)), "lq_decode_step_host")
 
 
@@ -230,9 +257,9 @@ def decode_step_host_pipelined(sh: Shape, st: State, q_h, k_h, v_h, beta_h, alph
     """lq_decode_step_host_pipelined: same arguments as decode_step_host; copies and kernels overlap."""
     for t in (q_h, k_h, v_h, beta_h, alpha_h, o_h):
         assert t.device.type == "cpu" and t.is_contiguous()
-    s = sh.c()
-    cs = st.c()
-    _check(lib().lq_decode_step_host_pipelined(C.byref(s), C.byref(cs), _ptr(q_h), _ptr(k_h), _ptr(v_h), _ptr(beta_h),
+    s = sh.ref()
+    cs = C.byref(st.c())
+    _check(lib().lq_decode_step_host_pipelined(s, cs, _ptr(q_h), _ptr(k_h), _ptr(v_h), _ptr(beta_h),
                                                _ptr(alpha_h), _ptr(o_h), _ptr(stage), _stream(stream)),
            "lq_decode_step_host_pipelined")
 
@@ -245,42 +272,42 @@ def decode_step_host_static(sh: Shape, st: State, q_h, k_h, v_h, beta_h, alpha_h
     buffer; the staging is a fixed array inside the library (requests above STATIC_STAGE_BYTES are refused)."""
     for t in (q_h, k_h, v_h, beta_h, alpha_h, o_h):
         assert t.device.type == "cpu" and t.is_contiguous()
-    s = sh.c()
-    cs = st.c()
-    _check(lib().lq_decode_step_host_static(C.byref(s), C.byref(cs), _ptr(q_h), _ptr(k_h), _ptr(v_h), _ptr(beta_h),
+    s = sh.ref()
+    cs = C.byref(st.c())
+    _check(lib().lq_decode_step_host_static(s, cs, _ptr(q_h), _ptr(k_h), _ptr(v_h), _ptr(beta_h),
                                             _ptr(alpha_h), _ptr(o_h), _stream(stream)), "lq_decode_step_host_static")
 
 
 def window_flush(sh: Shape, st: State, force: bool = False, stream=None):
-    s = sh.c()
-    cs = st.c()
-    _check(lib().lq_window_flush(C.byref(s), C.byref(cs), C.c_int(1 if force else 0), _stream(stream)),
+    s = sh.ref()
+    cs = C.byref(st.c())
+    _check(lib().lq_window_flush(s, cs, 1 if force else 0, _stream(stream)),
            "lq_window_flush")
 
 
 def quantize_state(sh: Shape, S, st: State, stream=None, b0: int = 0, nb: Optional[int] = None):
-    s = _sub(sh, b0, nb).c()
-    cs = st.c(b0)
-    _check(lib().lq_quantize_state(C.byref(s), _ptr(S, b0), C.byref(cs), _stream(stream)), "lq_quantize_state")
+    s = _sub(sh, b0, nb)
+    cs = C.byref(st.c(b0))
+    _check(lib().lq_quantize_state(s, _ptr(S, b0), cs, _stream(stream)), "lq_quantize_state")
 
 
 def dequantize_state(sh: Shape, st: State, S, stream=None, b0: int = 0, nb: Optional[int] = None):
     """lq_dequantize_state on sequences [b0, b0+nb) of the state; ``S`` receives exactly those sequences."""
-    s = _sub(sh, b0, nb).c()
-    cs = st.c(b0)
-    _check(lib().lq_dequantize_state(C.byref(s), C.byref(cs), _ptr(S), _stream(stream)), "lq_dequantize_state")
+    s = _sub(sh, b0, nb)
+    cs = C.byref(st.c(b0))
+    _check(lib().lq_dequantize_state(s, cs, _ptr(S), _stream(stream)), "lq_dequantize_state")
 
 
 def ref_decode_step_f32(sh: Shape, S, q, k, v, beta, alpha, o, stream=None, b0: int = 0, nb: Optional[int] = None):
-    s = _sub(sh, b0, nb).c()
-    _check(lib().lq_ref_decode_step_f32(C.byref(s), _ptr(S, b0), _ptr(q, b0), _ptr(k, b0), _ptr(v, b0),
+    s = _sub(sh, b0, nb)
+    _check(lib().lq_ref_decode_step_f32(s, _ptr(S, b0), _ptr(q, b0), _ptr(k, b0), _ptr(v, b0),
                                         _ptr(beta, b0), _ptr(alpha, b0), _ptr(o, b0), _stream(stream)),
            "lq_ref_decode_step_f32")
 
 
 def ref_decode_step_bf16(sh: Shape, S16, q, k, v, beta, alpha, o, stream=None):
-    s = sh.c()
-    _check(lib().lq_ref_decode_step_bf16(C.byref(s), _ptr(S16), _ptr(q), _ptr(k), _ptr(v), _ptr(beta), _ptr(alpha),
+    s = sh.ref()
+    _check(lib().lq_ref_decode_step_bf16(s, _ptr(S16), _ptr(q), _ptr(k), _ptr(v), _ptr(beta), _ptr(alpha),
                                          _ptr(o), _stream(stream)), "lq_ref_decode_step_bf16")
 
 
@@ -322,14 +349,14 @@ class StateArrays:
 
 def import_state(sh: Shape, arrays: StateArrays, st: State, stream=None) -> None:
     """lq_import_state: fill the packed state from the separate arrays."""
-    s, a, cs = sh.c(), arrays.c(), st.c()
-    _check(lib().lq_import_state(C.byref(s), C.byref(a), C.byref(cs), _stream(stream)), "lq_import_state")
+    s, a, cs = sh.ref(), C.byref(arrays.c()), C.byref(st.c())
+    _check(lib().lq_import_state(s, a, cs, _stream(stream)), "lq_import_state")
 
 
 def export_state(sh: Shape, st: State, arrays: StateArrays, stream=None) -> None:
     """lq_export_state: write the packed state out as separate arrays."""
-    s, a, cs = sh.c(), arrays.c(), st.c()
-    _check(lib().lq_export_state(C.byref(s), C.byref(cs), C.byref(a), _stream(stream)), "lq_export_state")
+    s, a, cs = sh.ref(), C.byref(arrays.c()), C.byref(st.c())
+    _check(lib().lq_export_state(s, cs, a, _stream(stream)), "lq_export_state")
 
 
 def clear_device_flags() -> None:
