@@ -366,11 +366,12 @@ static lq_status launch_boundary_gate(const lq_shape *s, const Params &p, cudaSt
   return s->rec16 ? launch_boundary_t<LQ_GATE_SCALAR, M_, true, RM>(s, p, stream) : launch_boundary_t<LQ_GATE_SCALAR, M_, false, RM>(s, p, stream);
 }
 
-// compiled for r <= 4, r <= 8 and any r (the small matrices of the fit live in registers); dequantizing has no fit
+// compiled for r = 0, r <= 4, r <= 8 and any r (the small matrices of the fit live in registers)
 template <int MODE>
 static lq_status launch_boundary(const lq_shape *s, const Params &p, cudaStream_t stream) {
   if (s->batch == 0) return LQ_OK;
   if (s->state_bf16) return launch_bf16w_boundary<MODE>(s, p, stream);
+  if (s->r == 0) return launch_boundary_gate<MODE, 0>(s, p, stream);
   if (MODE == 2 || s->r <= 4) return launch_boundary_gate<MODE, 4>(s, p, stream);
   if (s->r <= 8) return launch_boundary_gate<MODE, MODE == 2 ? 4 : 8>(s, p, stream);
   return launch_boundary_gate<MODE, MODE == 2 ? 4 : MAX_R>(s, p, stream);

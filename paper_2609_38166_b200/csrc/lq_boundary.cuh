@@ -34,7 +34,7 @@ struct BoundarySmem {
   static constexpr int ub = chol + (RM > 4 ? 4 * (RM * RM + 2 * RM) : 0);      // [8][RM][16] value sides as stored, per warp
   static constexpr int T = ub + 4 * D * RM;                  // [RM][128]  S w_h, then the keys as stored
   static constexpr int part = T + 4 * D * RM;                // [8][RM][128] per-warp row sums; later [8][128] those of |R|
-  static constexpr int head = part + 4 * D * 8 * RM;
+  static constexpr int head = part + 4 * D * 8 * (RM > 0 ? RM : 1);
   int rec, dec, kd, Wv, bytes;
   __host__ __device__ BoundarySmem(int W, int r, bool diag, bool rec16, bool slot, bool iterate) {
     rec = head + (slot ? head_bytes(r) : 0);                 // [W] record rows
@@ -269,7 +269,8 @@ __device__ __forceinline__ uint32_t orthonormalize(float *X, int r, float *gram,
 }
 
 // MODE 0 flush (window representation -> dense -> new window representation), 1 quantize dense fp32 states,
-// 2 dequantize to dense fp32 states.  RM: the largest r the instance handles.
+// 2 dequantize to dense fp32 states.  RM: the largest r the instance handles; 0: no compensators at all (an instance of its
+// own: told apart inside the others, the two ways cost 400 bytes of spills).
 template <int GATE, int MODE, bool R16, int RM>
 __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
   constexpr bool DIAG = GATE == LQ_GATE_DIAG, SLOT = MODE != 1;
@@ -281,6 +282,7 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
   __shared__ int todo_n[32], todo_count, any_due;
   const int W = p.W, r = p.r, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 1, tx = lane & 1;
   const int v0 = 16 * warp + 8 * tx;         // the lane's first column
+  if (RM > 0 && r < 1) return;               // (not launched)
   const unsigned nh = static_cast<unsigned>(p.batch) * p.heads_v;
   const Lay L(W, r, DIAG, R16, SLOT, p.n_iter > 1);
   rec_t *rec = reinterpret_cast<rec_t *>(lq_bsm + L.rec);
@@ -419,7 +421,8 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
 #pragma unroll
             for (int c = 0; c < 4; c++) M[a][c] = __fmul2_rn(pair(gi[a]), M[a][c]);
         }
-#pragma unroll 1
+        constexpr int AHEAD = MODE == 2 ? 1 : 2;              // (dequantizing spills with two records at a time)
+#pragma unroll AHEAD
         for (int j = 0; j < n; j++) {
           float kj[8];
           float2 uj[4];
@@ -439,7 +442,7 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
         for (int a = 0; a < 8; a++) store_row8(S + a * D, wide, M[a]);
       } else {
         // T_h = S w_h; w_h is the value side of the (h+1)-th newest record, or Walsh function h
-#pragma unroll 1
+#pragma unroll 2
         for (int h = 0; h < r; h++) {
           float2 w[4];
           if (SLOT && h < n) {
@@ -463,7 +466,7 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
 
       if constexpr (MODE != 2) {
         uint32_t alive = 0;
-        if (r > 0) {
+        if constexpr (RM > 0) {
           for (int idx = tid; idx < r * D; idx += 256) T[idx] = sum_warps(part + idx, RM * D);
           LQ_BTICK(10);
           // further rounds: W_h = S^T q_h, orthonormalise, T_h = S q_h
