@@ -169,15 +169,8 @@ struct DueList {
   unsigned bh[64];
   int n[64], count;
 };
-// Where a warp stands in its heads, kept while its CTA performs boundaries.
-struct PairState {
-  PairHead cur, nx;                          // the head at hand and the next one
-  bool have_cur, have_nx, drawing, reported;
-  int t0, taken, due_next, trips;
-  uint32_t todo, parities;
-};
-constexpr int SLOTS_AT = 128, STATES_AT = 640, SLOTS_AT_LIST = STATES_AT + 8 * 80;
-static_assert(64 + sizeof(DueList) <= STATES_AT && sizeof(PairState) <= 80, "what lies in front of the slots");
+constexpr int SLOTS_AT = 128, SLOTS_AT_LIST = 640;
+static_assert(64 + sizeof(DueList) <= SLOTS_AT_LIST, "the list fits in front of the slots");
 
 // The boundary of head bh, whose block and W records are in `slot` (the newest record in the slot's digits region, its
 // decay at dec[W - 1]).  Called by the 256 threads of a CTA after a barrier; ends with one.  (A function of its own: the
@@ -221,22 +214,18 @@ __device__ __noinline__ void flush_slot(const Params &p, unsigned char *slot, un
 // boundary where they are; nothing is read again.
 // LONGW: the window may hold more records than the slot stages at a time (W - 1 > REC_SEG); in the instances for
 // shorter windows everything to do with a second segment drops out at compile time.
-// Returns true when the pair has come to a boundary (its state is then in shared memory, `first` is false for the next call),
-// false when all is done.  Nothing of this function lives across a boundary: the boundary takes all registers, and what the
-// compiler spilled around a call from inside the loop it reloaded in every trip (1 KB a thread; twice the time).
 template <int GATE, bool R16, bool LONGW, int RM>
-__device__ __forceinline__ bool decode_pair(const Params &p, unsigned char *smem, const StepPlan &plan, const bool first_call) {
+__device__ __forceinline__ void decode_pair(const Params &p, unsigned char *smem, const StepPlan &plan) {
   constexpr bool DIAG = GATE == LQ_GATE_DIAG, BOUNDARY = RM >= 0;
   static_assert(!(BOUNDARY && LONGW), "the boundary needs all records of the window in the slot");
   constexpr int RF = record_floats(DIAG);
   const int W = p.W, r = p.r;
   using rec_t = typename std::conditional<R16, __half, float>::type;   // element type of the record rows
   const DecodeSlot L(W, r, DIAG, R16);
-  int tid = threadIdx.x;
-  if (BOUNDARY) asm volatile("" : "+r"(tid));          // (so that nothing derived from it is kept across a boundary)
-  const int lane = tid & 31, role = (tid >> 5) & 1, pr = BOUNDARY ? tid >> 6 : 0;
+  const int lane = threadIdx.x & 31, role = (threadIdx.x >> 5) & 1, pr = BOUNDARY ? threadIdx.x >> 6 : 0;
   const int PAIRS = BOUNDARY ? plan.pairs : 1, B0 = BOUNDARY ? pr * (DIAG ? 4 : 3) : 0;     // B0: named barriers of the pair
-  unsigned char *slots = smem + (BOUNDARY ? SLOTS_AT_LIST : SLOTS_AT), *slot = slots + pr * L.bytes;
+  const bool lender = BOUNDARY && pr >= PAIRS;                         // a warp without a slot
+  unsigned char *slots = smem + (BOUNDARY ? SLOTS_AT_LIST : SLOTS_AT), *slot = slots + (lender ? 0 : pr) * L.bytes;
   const int c = lane & 15, half = lane >> 4, g = lane >> 2, t = lane & 3;
   const int8_t *zt = reinterpret_cast<const int8_t *>(slot + L.head + HB_CODES);
   const float *bs = reinterpret_cast<const float *>(slot + L.head + HB_COL_SCALE);
@@ -312,8 +301,8 @@ __device__ __forceinline__ bool decode_pair(const Params &p, unsigned char *smem
   // A pair stops when a ticket is beyond the pool.
   const int rounds = static_cast<int>(nh / P);                 // rounds in which every pair has a head
   const bool draw = p.work != nullptr && rounds >= 3;
-  const int S = draw ? rounds - (BOUNDARY ? (rounds >= 6 ? 3 : 2) : rounds >= 6 ? 2 : 1)
-                         : me < nh ? static_cast<int>((nh - 1 - me) / P) + 1 : 0;
+  const int S = lender ? 0 : draw ? rounds - (BOUNDARY ? (rounds >= 6 ? 3 : 2) : rounds >= 6 ? 2 : 1)
+                                  : me < nh ? static_cast<int>((nh - 1 - me) / P) + 1 : 0;
   const unsigned pool = draw ? nh - static_cast<unsigned>(S) * P : 0;
   auto is_due = [&](int n) { return BOUNDARY && (n == W - 1 || n == W); };
   auto in_turn = [&](int n) { return n < (BOUNDARY ? W - 1 : W); };    // (a full window gets no token)
@@ -349,20 +338,42 @@ __device__ __forceinline__ bool decode_pair(const Params &p, unsigned char *smem
     h.due = false;
     return true;
   };
-  const DueList &list = *reinterpret_cast<const DueList *>(smem + 64);
-  const int due = BOUNDARY ? list.count : 0;           // boundaries of this CTA
-  int due_next = 0;                                    // how many of them have been taken up
-  auto take_due = [&](PairHead &h) {                   // this pair's part in the next plan.hold of them
+  DueList &list = *reinterpret_cast<DueList *>(smem + 64);
+  auto load_list = [&](unsigned d0) {        // entries d0 .. d0 + 31 of the CTA's list of boundaries, by one warp
+    unsigned bh_due;
+    int n_due, total;
+    const int found = find_due_heads(p, is_due, blockIdx.x + d0 * G, G, lane, bh_due, n_due, total);
+    const unsigned items = static_cast<unsigned>(total) * Hv, at = (d0 + lane) & 63;
+    if (lane < found) { list.bh[at] = bh_due; list.n[at] = n_due; }
+    if (lane == 0) list.count = items > blockIdx.x ? static_cast<int>((items - 1 - blockIdx.x) / G) + 1 : 0;
+  };
+  int due = 0, due_next = 0;                 // boundaries of this CTA, and how many of them have been taken up
+  const int hold = BOUNDARY ? plan.hold : 1;
+  auto take_due = [&](PairHead &h) {         // this pair's part in the next `hold` of them
     const int m = due_next + pr;
     h = PairHead{NO_HEAD, 0u, W, 0u, true};
-    if (pr < plan.hold && m < due) {
+    if (pr < hold && m < due) {
       h.bh = list.bh[m & 63];
       h.b = h.bh / Hv;
       h.n = list.n[m & 63];
       h.ba = p.beta[h.bh];
       if (!DIAG) h.ba |= static_cast<uint32_t>(p.alpha[h.bh]) << 16;
     }
-    due_next += plan.hold;
+    due_next += hold;
+  };
+  // All warps of the CTA: the boundaries of entries m0 .. m0 + hold - 1, each in the slot of the pair that gave it its token.
+  auto perform_boundaries = [&](int m0) {
+    __syncthreads();                         // the tokens are complete in the slots, the others are free
+    const int m1 = m0 + hold < due ? m0 + hold : due;
+#pragma unroll 1
+    for (int m = m0; m < m1; m++) {
+      if constexpr (BOUNDARY) flush_slot<GATE, R16, RM>(p, slots + (m - m0) * L.bytes, slots + plan.scratch, list.bh[m & 63]);
+    }
+    // (entries are taken up to three rounds ahead: the next 32 are found when the first of these 32 are done with)
+    if (m0 > 0 && m0 % 32 == 0 && m0 + 32 < due) {
+      if (threadIdx.x < 32) load_list(static_cast<unsigned>(m0 + 32));
+      __syncthreads();
+    }
   };
   // The pair has read all it will of win_pos (report_seen): the last of the pairs to say so moves the windows on, and puts
   // the ticket counter back to zero.
@@ -381,36 +392,45 @@ __device__ __forceinline__ bool decode_pair(const Params &p, unsigned char *smem
     if (role == 0) request_head(cur.bh, cur.n & 0xFFFF);
     else request_records(cur.bh, cur.n & 0xFFFF);
   };
-  // (the two CTAs of an SM take their boundaries at different times, so that one of them keeps the memory busy)
-  const int due_at = 2 * blockIdx.x >= G && S > 3 ? S / 2 : 1;
-  int taken = 0;
+  load_window();
+  bool have_cur = take_in_turn(cur);
+  if (have_cur) start();
+  int taken = have_cur, due_at = 0;
+  if (BOUNDARY) {
+    // the list of boundaries, while the first heads are on their way (by a warp without a slot, if there is one)
+    if (threadIdx.x >= blockDim.x - 32) {
+      load_list(0);
+      __syncwarp();
+      if (list.count > 32) load_list(32);
+    }
+    __syncthreads();
+    due = list.count;
+    if (lender) {
+      for (int m0 = 0; m0 < due; m0 += hold) perform_boundaries(m0);
+      return;
+    }
+    // (the two CTAs of an SM take their boundaries at different times, so that one of them keeps the memory busy)
+    due_at = 2 * blockIdx.x >= G && S > 3 ? S / 2 : 1;
+  }
   auto take = [&](PairHead &h) {
     if (BOUNDARY && due_next < due && taken >= due_at) { take_due(h); return true; }
     if (take_in_turn(h)) { taken++; return true; }
     if (BOUNDARY && due_next < due) { take_due(h); return true; }
     return false;
   };
-  bool have_cur, have_nx, drawing = draw, reported = false;    // drawing: no ticket has been beyond the pool yet
-  int trips = 0;
-  PairState &kept = *reinterpret_cast<PairState *>(smem + STATES_AT + 80 * (tid >> 5));
-  if (first_call) {
-    load_window();
+  if (!have_cur) {
     have_cur = take(cur);
     if (have_cur && wanted(cur)) start();
-    have_nx = have_cur && take(nx);
-  } else {
-    cur = kept.cur; nx = kept.nx; have_cur = kept.have_cur; have_nx = kept.have_nx; drawing = kept.drawing; reported = kept.reported;
-    t0 = kept.t0; taken = kept.taken; due_next = kept.due_next; trips = kept.trips;
-    parA = kept.parities & 1; parR = kept.parities >> 1;
-    if (have_cur && wanted(cur)) start();
-    load_window();
-    todo = kept.todo;
   }
+  bool have_nx = have_cur && take(nx);
 #ifdef LQ_TIMING
   tick_ = clock64();
 #endif
   unsigned *qidx = reinterpret_cast<unsigned *>(pk + r);      // (a spare word of the projection area)
   unsigned ticket = 0xFFFFFFFFu;             // (dot warp, lane 0) what was drawn in this trip
+  bool drawing = draw;                       // no ticket has been beyond the pool yet
+  bool reported = false;
+  int trips = 0, done = 0;                   // done: boundaries performed
   while (have_cur || have_nx || drawing) {
     const bool turn_over = !more_in_turn() && due_next >= due;  // nothing is left to take but what is drawn
     const bool draws = drawing && turn_over;                    // a ticket is drawn in this trip
@@ -852,12 +872,9 @@ __device__ __forceinline__ bool decode_pair(const Params &p, unsigned char *smem
     nx = after; have_nx = have_after;
     trips++;
     if (was_due) {
-      if (lane == 0) {
-        kept.cur = cur; kept.nx = nx; kept.have_cur = have_cur; kept.have_nx = have_nx; kept.drawing = drawing; kept.reported = reported;
-        kept.t0 = t0; kept.taken = taken; kept.due_next = due_next; kept.trips = trips;
-        kept.todo = todo; kept.parities = parA | parR << 1;
-      }
-      return true;
+      perform_boundaries(done);
+      done += hold;
+      if (have_cur && wanted(cur)) start();
     }
   }
   if (!reported) {                           // the last trips had no head: the pair reports when both warps are here
@@ -872,48 +889,6 @@ __device__ __forceinline__ bool decode_pair(const Params &p, unsigned char *smem
   if (lane == 0)
     for (int i = 0; i < 12; i++) atomicAdd(&g_phase_cycles[16 * role + i], (unsigned long long)acc_[i]);
 #endif
-  return false;
-}
-
-// The life of a CTA that also performs the boundaries: its pairs decode until all of them have come to one, then all eight
-// warps perform it, and so on.
-template <int GATE, bool R16, int RM>
-__device__ __forceinline__ void decode_with_boundaries(const Params &p, unsigned char *smem, const StepPlan &plan) {
-  DueList &list = *reinterpret_cast<DueList *>(smem + 64);
-  auto load_list = [&](unsigned d0) {        // entries d0 .. d0 + 31 of the CTA's list of boundaries, by one warp
-    const int lane = threadIdx.x & 31;
-    unsigned bh_due;
-    int n_due, total;
-    const int found = find_due_heads(p, [&](int n) { return n == p.W - 1 || n == p.W; }, blockIdx.x + d0 * gridDim.x, gridDim.x, lane,
-                                     bh_due, n_due, total);
-    const unsigned items = static_cast<unsigned>(total) * p.heads_v, at = (d0 + lane) & 63;
-    if (lane < found) { list.bh[at] = bh_due; list.n[at] = n_due; }
-    if (lane == 0) list.count = items > blockIdx.x ? static_cast<int>((items - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
-    __syncwarp();
-  };
-  if (threadIdx.x < 32) {
-    load_list(0);
-    if (list.count > 32) load_list(32);
-  }
-  __syncthreads();
-  const bool paired = static_cast<int>(threadIdx.x >> 6) < plan.pairs;        // (the other warps only lend a hand)
-  bool more = true;
-#pragma unroll 1
-  for (int m0 = 0;; m0 += plan.hold) {
-    if (paired && more) more = decode_pair<GATE, R16, false, RM>(p, smem, plan, m0 == 0);
-    if (m0 >= list.count) break;
-    __syncthreads();                         // the tokens are complete in the slots, the other slots are free
-    const int m1 = min(m0 + plan.hold, list.count);
-#pragma unroll 1
-    for (int m = m0; m < m1; m++)
-      flush_slot<GATE, R16, RM>(p, smem + SLOTS_AT_LIST + (m - m0) * DecodeSlot(p.W, p.r, GATE == LQ_GATE_DIAG, R16).bytes,
-                                smem + SLOTS_AT_LIST + plan.scratch, list.bh[m & 63]);
-    // (entries are taken up to three rounds ahead: the next 32 are found when the first of these 32 are done with)
-    if (m0 > 0 && m0 % 32 == 0 && m0 + 32 < list.count) {
-      if (threadIdx.x < 32) load_list(static_cast<unsigned>(m0 + 32));
-      __syncthreads();
-    }
-  }
 }
 
 // Persistent kernel: CTAs of one pair of warps (RM < 0), or of eight warps that also perform the boundaries.
@@ -934,8 +909,7 @@ __global__ void __launch_bounds__(RM >= 0 ? 256 : 64, RM >= 0 ? 2 : 6) decode_ke
   __syncthreads();
   grid_dependency_wait();                    // no data in global memory is read or written above this line
   LQ_STAMP(0, 1);
-  if constexpr (RM >= 0) decode_with_boundaries<GATE, R16, RM>(p, lq_smem, plan);
-  else decode_pair<GATE, R16, LONGW, RM>(p, lq_smem, plan, true);
+  decode_pair<GATE, R16, LONGW, RM>(p, lq_smem, plan);
   LQ_STAMP(0, 3);
 #ifdef LQ_TIMING
   if (threadIdx.x == 0 && blockIdx.x < 1024) {
