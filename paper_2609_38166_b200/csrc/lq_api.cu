@@ -315,6 +315,22 @@ static lq_status launch_dependent(K kernel, int grid, int block, size_t smem, cu
   return LQ_OK;
 }
 
+// grid <= min(work items, CTAs that fit on the device at once), for kernels that stride over their work
+template <typename K>
+static lq_status launch_persistent(K kernel, long items, int block, size_t smem, cudaStream_t stream, const Params &p) {
+  if (items <= 0) return LQ_OK;
+  const int per_sm = prepare_launch(reinterpret_cast<const void *>(kernel), block, smem);
+  if (per_sm < 1) return LQ_ERR_CUDA;
+  const long resident = (long)per_sm * sm_count();
+  // Every CTA takes ceil(items / resident) items at most; the smallest grid with that property leaves no last
+  // round in which a fraction of the CTAs works while the others have left (8192 heads: 820 CTAs of 10 heads
+  // instead of 888 of which 200 take a tenth).  With scratch words in the state the items of a partial last round
+  // go to the CTAs that get there first (decode_slot), and every CTA that fits is launched.
+  const long rounds = (items + resident - 1) / resident;
+  const long grid = p.work != nullptr ? (items < resident ? items : resident) : (items + rounds - 1) / rounds;
+  return launch_dependent(kernel, static_cast<int>(grid), block, smem, stream, p);
+}
+
 // per-window BF16: persistent CTAs that stride over the heads
 template <int MODE>
 static lq_status launch_bf16w_boundary(const lq_shape *s, const Params &p, cudaStream_t stream) {
@@ -361,54 +377,6 @@ static lq_status launch_boundary(const lq_shape *s, const Params &p, cudaStream_
   return launch_boundary_gate<MODE, MODE == 2 ? 4 : MAX_R>(s, p, stream);
 }
 
-// ---- the decode kernel ----
-// One pair of warps per CTA, the boundary left to a kernel of its own.
-template <int GATE, bool R16, bool LONGW>
-static lq_status launch_decode(const lq_shape *s, const Params &p, cudaStream_t stream) {
-  const StepPlan plan = {1, 0, 0, SLOTS_AT + DecodeSlot(s->W, s->r, GATE == LQ_GATE_DIAG, R16).bytes};
-  auto kernel = decode_kernel<GATE, R16, LONGW, -1>;
-  const int per_sm = prepare_launch(reinterpret_cast<const void *>(kernel), 64, plan.bytes);
-  if (per_sm < 1) return LQ_ERR_CUDA;
-  const long nh = (long)s->batch * s->heads_v, resident = (long)per_sm * sm_count();
-  // Every CTA takes ceil(nh / resident) heads at most; the smallest grid with that property leaves no last round in which
-  // a fraction of the CTAs works while the others have left (8192 heads: 820 CTAs of 10 heads instead of 888 of which 200
-  // take a tenth).  With scratch words in the state the heads of the last rounds go to the CTAs that get there first
-  // (decode_pair), and every CTA that fits is launched.
-  const long rounds = (nh + resident - 1) / resident;
-  const long grid = p.work != nullptr ? std::min(nh, resident) : (nh + rounds - 1) / rounds;
-  return launch_dependent(kernel, static_cast<int>(grid), 64, plan.bytes, stream, p, plan);
-}
-
-// The plan of a CTA that also performs the boundaries; pairs == 0: not possible for this shape.  Two such CTAs share an SM.
-// All W records of a due head have to be in its slot, and beside `hold` slots there has to be room for the working arrays.
-static StepPlan step_plan(const lq_shape *s) {
-  const bool diag = s->gate == LQ_GATE_DIAG, r16 = s->rec16 != 0, iterate = s->n_iter > 1;
-  const int budget = 228 * 1024 / 2 - 1024 - SLOTS_AT_LIST, slot = DecodeSlot(s->W, s->r, diag, r16).bytes;
-  const int scratch = s->r == 0 ? flush_scratch_bytes<0>(s->W, s->r, r16, iterate)
-                      : s->r <= 4 ? flush_scratch_bytes<4>(s->W, s->r, r16, iterate) : flush_scratch_bytes<8>(s->W, s->r, r16, iterate);
-  StepPlan plan = {std::min(diag ? 3 : 4, budget / slot), 2, 0, 0};
-  while (plan.hold > 0 && (plan.hold > plan.pairs || plan.hold * slot + scratch > budget)) plan.hold /= 2;
-  if (s->state_bf16 || s->W - 1 > REC_SEG || s->r > 8 || plan.pairs < 2 || plan.hold < 1) return StepPlan{0, 0, 0, 0};
-  const int area = std::max(plan.pairs * slot, (plan.hold * slot + scratch + 127) / 128 * 128);
-  plan.scratch = (area - scratch) / 128 * 128;
-  plan.bytes = SLOTS_AT_LIST + area;
-  return plan;
-}
-
-template <int GATE, bool R16, int RM>
-static lq_status launch_step_t(const lq_shape *s, const Params &p, const StepPlan &plan, cudaStream_t stream) {
-  auto kernel = decode_kernel<GATE, R16, false, RM>;
-  const int per_sm = prepare_launch(reinterpret_cast<const void *>(kernel), 256, plan.bytes);
-  if (per_sm < 1) return LQ_ERR_CUDA;
-  const long nh = (long)s->batch * s->heads_v, resident = (long)per_sm * sm_count();
-  return launch_dependent(kernel, static_cast<int>(std::min(nh, resident)), 256, plan.bytes, stream, p, plan);
-}
-template <int GATE, bool R16>
-static lq_status launch_step(const lq_shape *s, const Params &p, const StepPlan &plan, cudaStream_t stream) {
-  return s->r == 0 ? launch_step_t<GATE, R16, 0>(s, p, plan, stream)
-         : s->r <= 4 ? launch_step_t<GATE, R16, 4>(s, p, plan, stream) : launch_step_t<GATE, R16, 8>(s, p, plan, stream);
-}
-
 }  // namespace lq
 
 using namespace lq;
@@ -451,19 +419,22 @@ static lq_status decode_step_impl(const lq_shape *shape, const lq_state *state, 
     }
     return launch_boundary<0>(shape, p, st);
   }
-  if (nh <= 0) return LQ_OK;
-  if (!between) {                            // decode and boundaries in one kernel, where that is possible
-    const StepPlan plan = step_plan(shape);
-    if (plan.pairs > 0 && !getenv("LQ_TWO"))
-      return diag ? r16 ? launch_step<LQ_GATE_DIAG, true>(shape, p, plan, st) : launch_step<LQ_GATE_DIAG, false>(shape, p, plan, st)
-                  : r16 ? launch_step<LQ_GATE_SCALAR, true>(shape, p, plan, st) : launch_step<LQ_GATE_SCALAR, false>(shape, p, plan, st);
-  }
-  if (shape->W - 1 > REC_SEG) {              // windows whose records come in more than one segment
-    if (r16) rc = diag ? launch_decode<LQ_GATE_DIAG, true, true>(shape, p, st) : launch_decode<LQ_GATE_SCALAR, true, true>(shape, p, st);
-    else rc = diag ? launch_decode<LQ_GATE_DIAG, false, true>(shape, p, st) : launch_decode<LQ_GATE_SCALAR, false, true>(shape, p, st);
+  const size_t smem = DecodeSlot(shape->W, shape->r, diag, r16).bytes;
+  const bool longw = shape->W - 1 > REC_SEG;               // windows whose records come in more than one segment
+  if (longw) {
+    if (r16)
+      rc = diag ? launch_persistent(decode_kernel<LQ_GATE_DIAG, true, true>, nh, 64, smem, st, p)
+                : launch_persistent(decode_kernel<LQ_GATE_SCALAR, true, true>, nh, 64, smem, st, p);
+    else
+      rc = diag ? launch_persistent(decode_kernel<LQ_GATE_DIAG, false, true>, nh, 64, smem, st, p)
+                : launch_persistent(decode_kernel<LQ_GATE_SCALAR, false, true>, nh, 64, smem, st, p);
   } else {
-    if (r16) rc = diag ? launch_decode<LQ_GATE_DIAG, true, false>(shape, p, st) : launch_decode<LQ_GATE_SCALAR, true, false>(shape, p, st);
-    else rc = diag ? launch_decode<LQ_GATE_DIAG, false, false>(shape, p, st) : launch_decode<LQ_GATE_SCALAR, false, false>(shape, p, st);
+    if (r16)
+      rc = diag ? launch_persistent(decode_kernel<LQ_GATE_DIAG, true, false>, nh, 64, smem, st, p)
+                : launch_persistent(decode_kernel<LQ_GATE_SCALAR, true, false>, nh, 64, smem, st, p);
+    else
+      rc = diag ? launch_persistent(decode_kernel<LQ_GATE_DIAG, false, false>, nh, 64, smem, st, p)
+                : launch_persistent(decode_kernel<LQ_GATE_SCALAR, false, false>, nh, 64, smem, st, p);
   }
   if (rc != LQ_OK) return rc;
   if (between && cudaEventRecord(between, st) != cudaSuccess) {
@@ -992,9 +963,7 @@ int lq_debug_phase_cycles(unsigned long long *out) {
 }
 #endif
 
-int lq_decode_launches(const lq_shape *shape) {
-  return check_shape(shape) == LQ_OK && shape->batch > 0 ? (step_plan(shape).pairs > 0 ? 1 : 2) : 0;
-}
+int lq_decode_launches(const lq_shape *shape) { return check_shape(shape) == LQ_OK && shape->batch > 0 ? 2 : 0; }
 
 const char *lq_status_string(lq_status status) {
   switch (status) {

@@ -17,13 +17,6 @@ __device__ __forceinline__ uint16_t *bf16w_state(const Params &p, size_t bh) {
   return reinterpret_cast<uint16_t *>(p.heads + bh * (size_t)BF16W_HEAD_BYTES);
 }
 
-// Last-arrival bookkeeping on win_pos[b]: bits 16.. count the heads of sequence b that are done with the value in bits
-// 0..15; the head that arrives last stores the new value and thereby clears the counter.  One thread per head.
-__device__ __forceinline__ void arrive_and_set(int32_t *win_pos, int b, int heads_v, int new_value) {
-  const int old = atomicAdd(win_pos + b, 0x10000);
-  if ((old >> 16) == heads_v - 1) win_pos[b] = new_value;
-}
-
 // eight bfloat16 values as four (even, odd) pairs
 __device__ __forceinline__ void widen8_bf16(const uint4 &w, float2 (&x)[4]) {
   const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
@@ -281,7 +274,7 @@ __global__ void __launch_bounds__(256, 2) bf16w_boundary_kernel(const Params p) 
       unsigned bh_mine = first + t.lane * gridDim.x;
       int n_mine = 0, c, due = 0;
       if (MODE == 0) {
-        c = find_due_heads(p, [&](int v) { return v == p.W || (p.force && v > 0); }, first, gridDim.x, t.lane, bh_mine, n_mine, due);
+        c = find_due_heads(p, first, gridDim.x, t.lane, bh_mine, n_mine, due);
       } else {
         const bool have = bh_mine < nh;
         if (MODE == 2 && have) n_mine = p.win_pos[bh_mine / p.heads_v] & 0xFFFF;

@@ -268,266 +268,9 @@ __device__ __forceinline__ uint32_t orthonormalize(float *X, int r, float *gram,
   return alive;
 }
 
-// Cumulative decays, newest record first (Appendix B.2): kd_j = Gamma_{j+1:n} kt_j, gam = Gamma_{1:n}; thread tid < 128 takes
-// channel tid.  row(j): record j as stored; kd_row(j): where kd_j goes (may be the record's own write key).
-template <bool DIAG, typename Row, typename KdRow>
-__device__ __forceinline__ void decay_records(int n, Row row, KdRow kd_row, const float *dec, float *gam) {
-  const int tid = threadIdx.x;
-  auto kt_at = [&](int j) { return static_cast<float>(row(j)[REC_KT + tid]); };
-  auto a_at = [&](int j) { return DIAG ? static_cast<float>(row(j)[REC_A + tid]) : dec[j]; };
-  float g = 1.0f;
-  int j = n - 1;
-  for (; j >= 3; j -= 4) {                                    // four records per trip: the loads go out together
-    float kt[4], a[4];
-#pragma unroll
-    for (int e = 0; e < 4; e++) { kt[e] = kt_at(j - e); a[e] = a_at(j - e); }
-#pragma unroll
-    for (int e = 0; e < 4; e++) { kd_row(j - e)[tid] = g * kt[e]; g = g * a[e]; }
-  }
-  for (; j >= 0; j--) { const float kt = kt_at(j); kd_row(j)[tid] = g * kt; g = g * a_at(j); }
-  gam[tid] = g;
-}
-
-// The lane's tile of the dense state (Eq. 7) from the head block in shared memory, the decayed records and Gamma_{1:n}:
-// x = gam_i (c_i (Z_ij s_j) + sum_h kc_hi uc_hj) + sum_j kd_ji u_jj, one fused multiply-add per term, oldest record first.
-// AHEAD: records in flight.
-template <int AHEAD, typename Row, typename KdRow>
-__device__ __forceinline__ void rebuild_tile(const unsigned char *head, int r, int n, Row row, KdRow kd_row, const float *gam,
-                                             float2 (&M)[8][4]) {
-  const int lane = threadIdx.x & 31, ty = lane >> 1, v0 = 16 * (threadIdx.x >> 5) + 8 * (lane & 1);
-  const uint8_t *zt = head + HB_CODES;
-  const uint16_t *ckh = reinterpret_cast<const uint16_t *>(head + HB_COMP_K), *cuh = ckh + r * D;
-  {
-    float ci[8];
-    float2 sj[4];
-    load8(reinterpret_cast<const float *>(head + HB_ROW_SMOOTH) + 8 * ty, ci);
-    load8p(reinterpret_cast<const float *>(head + HB_COL_SCALE) + v0, sj);
-    uint2 zz[8];
-#pragma unroll
-    for (int b = 0; b < 8; b++) {
-      zz[b] = *reinterpret_cast<const uint2 *>(zt + (v0 + b) * D + 8 * ty);
-      zz[b].x ^= 0x80808080u; zz[b].y ^= 0x80808080u;
-    }
-    // int8 -> fp32 without the conversion unit: byte + 128 in the low mantissa bits of 2^23, minus 2^23 + 128
-#pragma unroll
-    for (int a = 0; a < 8; a++)
-#pragma unroll
-      for (int c = 0; c < 4; c++) {
-        const float2 raw = make_float2(
-            __uint_as_float(__byte_perm(a < 4 ? zz[2 * c].x : zz[2 * c].y, 0x4B000000u, 0x7540 | (a & 3))),
-            __uint_as_float(__byte_perm(a < 4 ? zz[2 * c + 1].x : zz[2 * c + 1].y, 0x4B000000u, 0x7540 | (a & 3))));
-        M[a][c] = __fmul2_rn(pair(ci[a]), __fmul2_rn(__fadd2_rn(raw, pair(-8388736.0f)), sj[c]));
-      }
-  }
-#pragma unroll 1
-  for (int h = 0; h < r; h++) {
-    float kc[8];
-    float2 uc[4];
-    load8(reinterpret_cast<const __half *>(ckh + h * D + 8 * ty), kc);
-    load8p(reinterpret_cast<const __half *>(cuh + h * D + v0), uc);
-    rank1_pairs(M, kc, uc);
-  }
-  {
-    float gi[8];
-    load8(gam + 8 * ty, gi);
-#pragma unroll
-    for (int a = 0; a < 8; a++)
-#pragma unroll
-      for (int c = 0; c < 4; c++) M[a][c] = __fmul2_rn(pair(gi[a]), M[a][c]);
-  }
-#pragma unroll AHEAD
-  for (int j = 0; j < n; j++) {
-    float kj[8];
-    float2 uj[4];
-    load8(kd_row(j) + 8 * ty, kj);
-    load8p(row(j) + REC_U + v0, uj);
-    rank1_pairs(M, kj, uj);
-  }
-}
-
-// Per-warp row sums of S w_h into part [8][RM][128]; w_h is the value side of the (h+1)-th newest of the n records (RECORDS),
-// or Walsh function h where there is no such record.
-template <int RM, bool RECORDS, typename Row>
-__device__ __forceinline__ void start_products(const float2 (&M)[8][4], int r, int n, Row row, float *part) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ty = lane >> 1, tx = lane & 1, v0 = 16 * warp + 8 * tx;
-#pragma unroll 2
-  for (int h = 0; h < r; h++) {
-    float2 w[4];
-    if (RECORDS && h < n) {
-      load8p(row(n - 1 - h) + REC_U + v0, w);
-    } else {
-#pragma unroll
-      for (int c = 0; c < 4; c++) w[c] = make_float2(walsh_entry(h, v0 + 2 * c), walsh_entry(h, v0 + 2 * c + 1));
-    }
-    float pr[8];
-#pragma unroll
-    for (int a = 0; a < 8; a++) pr[a] = block8(M[a], w);
-    store_row_pairs(pr, ty, tx, part + (warp * RM + h) * D);
-  }
-}
-
-// The dense state in the tiles M (destroyed) to the new window representation of head bh, from the products with the start
-// vectors in `part` on (a barrier has been passed since).  work: the arrays of BoundarySmem<RM>; Wv: [r][128], used when
-// n_iter > 1.  Called by 256 threads; the last barrier it contains is the one in front of the code steps.
-template <int RM>
-__device__ __forceinline__ void requantize_tile(const Params &p, const int r, unsigned char *work, float *Wv, const size_t bh,
-                                                float2 (&M)[8][4]) {
-  using Lay = BoundarySmem<RM>;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 1, tx = lane & 1, v0 = 16 * warp + 8 * tx;
-  float *part = reinterpret_cast<float *>(work + Lay::part), *T = reinterpret_cast<float *>(work + Lay::T);
-  float *gram = reinterpret_cast<float *>(work + Lay::gram), *chol = reinterpret_cast<float *>(work + Lay::chol);
-  float *ub = reinterpret_cast<float *>(work + Lay::ub) + warp * 16 * RM;
-  float *ic_s = reinterpret_cast<float *>(work + Lay::ic), *invc = reinterpret_cast<float *>(work + Lay::invc) + 16 * warp;
-  uint32_t alive = 0;
-  if constexpr (RM > 0) {
-    for (int idx = tid; idx < r * D; idx += 256) T[idx] = sum_warps(part + idx, RM * D);
-    LQ_BTICK(10);
-    // further rounds: W_h = S^T q_h, orthonormalise, T_h = S q_h
-    for (int it = 1; it < p.n_iter; it++) {
-      orthonormalize<false, RM>(T, r, gram, chol, nullptr);
-#pragma unroll 1
-      for (int h = 0; h < r; h++) {
-        float x[8], pc[8];
-        load8(T + h * D + 8 * ty, x);
-        column_blocks(M, x, pc);
-        const float s = column_tree(pc, lane, [](float a, float b) { return a + b; });
-        if (lane < 16) Wv[h * D + v0 + column_of(lane)] = s;
-      }
-      orthonormalize<false, RM>(Wv, r, gram, chol, nullptr);
-#pragma unroll 1
-      for (int h = 0; h < r; h++) {
-        float2 w[4];
-        load8p(Wv + h * D + v0, w);
-        float pr[8];
-#pragma unroll
-        for (int a = 0; a < 8; a++) pr[a] = block8(M[a], w);
-        store_row_pairs(pr, ty, tx, part + (warp * RM + h) * D);
-      }
-      __syncthreads();
-      for (int idx = tid; idx < r * D; idx += 256) T[idx] = sum_warps(part + idx, RM * D);
-    }
-    alive = orthonormalize<true, RM>(T, r, gram, chol, p.comp_k(bh));       // T now holds the keys as stored
-    LQ_BTICK(11);
-    gram_lower<RM>(T, r, gram, false);                  // k_a^T k_h (published by the barrier in front of the value sides)
-
-    // ---- value sides and removal of the stored tokens ----
-    float x[RM];                                        // S^T k_h for the lane's column
-#pragma unroll
-    for (int h = 0; h < RM; h++) {
-      x[h] = 0.0f;
-      if (h < r) {
-        float kf[8], pc[8];
-        load8(T + h * D + 8 * ty, kf);
-        column_blocks(M, kf, pc);
-        x[h] = column_tree(pc, lane, [](float a, float b) { return a + b; });
-      }
-    }
-    __syncthreads();                                    // K^T K is complete
-    LQ_BTICK(13);
-    // u_h = S^T k_h - sum_{a<h} u_a (k_a^T k_h) with the stored values: what tokens 0..h-1 leave
-    float uf[RM];
-    const int col = column_of(lane);
-    uint16_t *cu_out = p.comp_u(bh) + v0 + col;
-#pragma unroll
-    for (int h = 0; h < RM; h++) {
-      uf[h] = 0.0f;
-      if (h < r) {
-#pragma unroll
-        for (int a = 0; a < h; a++) x[h] = fmaf(-uf[a], gram[h * RM + a], x[h]);
-        const uint16_t bits = (alive >> h) & 1u ? to_f16_bits_sat(x[h]) : static_cast<uint16_t>(0);
-        uf[h] = f16_bits(bits);
-        if (lane < 16) {
-          cu_out[h * D] = bits;
-          ub[16 * h + 8 * tx + col] = uf[h];
-        }
-      }
-    }
-    __syncwarp();
-    LQ_BTICK(14);
-#pragma unroll 1
-    for (int h = 0; h < r; h++) {                       // M -= k u^T with the stored values
-      float kf[8];
-      float2 uv[4];
-      load8(T + h * D + 8 * ty, kf);
-      load8p(ub + 16 * h + 8 * tx, uv);
-#pragma unroll
-      for (int a = 0; a < 8; a++) kf[a] = -kf[a];
-      rank1_pairs(M, kf, uv);
-    }
-  }
-  LQ_BTICK(4);
-  // ---- residual smoothing: c_i = max(sqrt(mean_j |R_ij|), 1e-6) ----
-  {
-    float pr[8];
-#pragma unroll
-    for (int a = 0; a < 8; a++) {                       // even and odd columns as two chains
-      float even = fabsf(M[a][0].x), odd = fabsf(M[a][0].y);
-#pragma unroll
-      for (int c = 1; c < 4; c++) { even = even + fabsf(M[a][c].x); odd = odd + fabsf(M[a][c].y); }
-      pr[a] = even + odd;
-    }
-    store_row_pairs(pr, ty, tx, part + warp * D);
-  }
-  __syncthreads();
-  if (tid < D) {
-    const float ci = p.smooth ? fmaxf(sqrtf(sum_warps(part + tid, D) / static_cast<float>(D)), 1e-6f) : 1.0f;
-    ic_s[tid] = p.smooth ? 1.0f / ci : 1.0f;
-    p.row_smooth(bh)[tid] = ci;
-  }
-  __syncthreads();
-  LQ_BTICK(5);
-
-  // ---- code steps and codes ----
-  {
-    float ic[8];
-    load8(ic_s + 8 * ty, ic);
-#pragma unroll
-    for (int a = 0; a < 8; a++)
-#pragma unroll
-      for (int c = 0; c < 4; c++) M[a][c] = __fmul2_rn(M[a][c], pair(ic[a]));
-  }
-  float m[8];
-#pragma unroll
-  for (int c = 0; c < 4; c++) {
-    m[2 * c] = fabsf(M[0][c].x); m[2 * c + 1] = fabsf(M[0][c].y);
-#pragma unroll
-    for (int a = 1; a < 8; a++) {
-      m[2 * c] = fmaxf(m[2 * c], fabsf(M[a][c].x));
-      m[2 * c + 1] = fmaxf(m[2 * c + 1], fabsf(M[a][c].y));
-    }
-  }
-  const float amax = column_tree(m, lane, [](float a, float b) { return fmaxf(a, b); });
-  if (lane < 16) {
-    const int col = column_of(lane);
-    p.col_scale(bh)[v0 + col] = amax / 127.0f;          // stored as the step of the code, B_j / 127
-    invc[8 * tx + col] = amax > 0.0f ? 127.0f / amax : 0.0f;
-  }
-  __syncwarp();
-  LQ_BTICK(6);
-  float2 inv[4];
-  load8p(invc + 8 * tx, inv);
-  int8_t *ZT = p.codes(bh) + v0 * D + 8 * ty;
-#pragma unroll
-  for (int c = 0; c < 4; c++) {
-    // |X * inv| <= 127 (1 + 2^-23): adding 1.5 * 2^23 leaves the nearest integer (ties to even) in the low byte
-    // (product and sum are rounded one after the other; written as a packed addition the two would get fused)
-    float2 z[8];
-#pragma unroll
-    for (int a = 0; a < 8; a++) z[a] = __ffma2_rn(__fmul2_rn(M[a][c], inv[c]), pair(1.0f), pair(12582912.0f));
-    auto bytes4 = [](float x0, float x1, float x2, float x3) {
-      return __byte_perm(__byte_perm(__float_as_uint(x0), __float_as_uint(x1), 0x0040),
-                         __byte_perm(__float_as_uint(x2), __float_as_uint(x3), 0x0040), 0x5410);
-    };
-    *reinterpret_cast<uint2 *>(ZT + (2 * c) * D) =
-        make_uint2(bytes4(z[0].x, z[1].x, z[2].x, z[3].x), bytes4(z[4].x, z[5].x, z[6].x, z[7].x));
-    *reinterpret_cast<uint2 *>(ZT + (2 * c + 1) * D) =
-        make_uint2(bytes4(z[0].y, z[1].y, z[2].y, z[3].y), bytes4(z[4].y, z[5].y, z[6].y, z[7].y));
-  }
-}
-
 // MODE 0 flush (window representation -> dense -> new window representation), 1 quantize dense fp32 states,
 // 2 dequantize to dense fp32 states.  RM: the largest r the instance handles; 0: no compensators at all (an instance of its
-// own: the others are told that r >= 1, without which the two ways through them cost 400 bytes of spills).
+// own: told apart inside the others, the two ways cost 400 bytes of spills).
 template <int GATE, int MODE, bool R16, int RM>
 __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
   constexpr bool DIAG = GATE == LQ_GATE_DIAG, SLOT = MODE != 1;
@@ -537,16 +280,23 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
   extern __shared__ __align__(128) unsigned char lq_bsm[];
   __shared__ unsigned todo_bh[32];
   __shared__ int todo_n[32], todo_count, any_due;
-  const int W = p.W, r = RM > 0 ? max(p.r, 1) : 0, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 1, tx = lane & 1;
+  const int W = p.W, r = p.r, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 1, tx = lane & 1;
   const int v0 = 16 * warp + 8 * tx;         // the lane's first column
+  if (RM > 0 && r < 1) return;               // (not launched)
   const unsigned nh = static_cast<unsigned>(p.batch) * p.heads_v;
   const Lay L(W, r, DIAG, R16, SLOT, p.n_iter > 1);
   rec_t *rec = reinterpret_cast<rec_t *>(lq_bsm + L.rec);
   float *dec = reinterpret_cast<float *>(lq_bsm + L.dec), *gam = reinterpret_cast<float *>(lq_bsm + Lay::gam);
-  float *part = reinterpret_cast<float *>(lq_bsm + Lay::part), *Wv = reinterpret_cast<float *>(lq_bsm + L.Wv);
+  const uint8_t *zt = lq_bsm + Lay::head + HB_CODES;
+  const float *ss = reinterpret_cast<const float *>(lq_bsm + Lay::head + HB_COL_SCALE);
+  const float *cs = reinterpret_cast<const float *>(lq_bsm + Lay::head + HB_ROW_SMOOTH);
+  const uint16_t *ckh = reinterpret_cast<const uint16_t *>(lq_bsm + Lay::head + HB_COMP_K), *cuh = ckh + r * D;
+  float *part = reinterpret_cast<float *>(lq_bsm + Lay::part), *T = reinterpret_cast<float *>(lq_bsm + Lay::T);
+  float *Wv = reinterpret_cast<float *>(lq_bsm + L.Wv), *gram = reinterpret_cast<float *>(lq_bsm + Lay::gram);
+  float *chol = reinterpret_cast<float *>(lq_bsm + Lay::chol), *ub = reinterpret_cast<float *>(lq_bsm + Lay::ub) + warp * 16 * RM;
+  float *ic_s = reinterpret_cast<float *>(lq_bsm + Lay::ic), *invc = reinterpret_cast<float *>(lq_bsm + Lay::invc) + 16 * warp;
   const uint32_t bar = smem_addr(lq_bsm + Lay::bar);
   const bool wide = (reinterpret_cast<uintptr_t>(p.S) & 31) == 0;
-  auto row = [&](int j) { return rec + j * RF; };
   auto kd_row = [&](int j) -> float * {      // Gamma_{j+1:n} kt_j
     if constexpr (R16) return reinterpret_cast<float *>(lq_bsm + L.kd) + j * D;
     else return rec + j * RF + REC_KT;
@@ -582,7 +332,7 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
       unsigned bh_mine = first + lane * gridDim.x;
       int n_mine = 0, c, due = 0;
       if (MODE == 0) {
-        c = find_due_heads(p, [&](int v) { return v == p.W || (p.force && v > 0); }, first, gridDim.x, lane, bh_mine, n_mine, due);
+        c = find_due_heads(p, first, gridDim.x, lane, bh_mine, n_mine, due);
       } else {
         const bool have = bh_mine < nh;
         if (MODE == 2 && have) n_mine = p.win_pos[bh_mine / p.heads_v] & 0xFFFF;
@@ -602,7 +352,7 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
 
     for (int k = 0; k < count; k++) {
       const size_t bh = todo_bh[k];
-      const int n = MODE == 0 ? max(todo_n[k], 1) : todo_n[k];      // (never 0 when due)
+      const int n = todo_n[k];
       if (SLOT) {
         if (!DIAG && tid < n) dec[tid] = dec_next;
         if (!mbar_wait(bar, parity) && lane == 0) atomicOr(&g_device_error, 1);
@@ -610,7 +360,22 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
         if (!DIAG) __syncthreads();
         if (k == 0) LQ_STAMP(1, 2);
         LQ_BTICK(1);
-        if (tid < D) decay_records<DIAG>(n, row, kd_row, dec, gam);
+        // cumulative decays, newest record first (Appendix B.2): kd_j = Gamma_{j+1:n} kt_j, gam = Gamma_{1:n}
+        if (tid < D) {
+          auto kt_at = [&](int j) { return static_cast<float>(rec[j * RF + REC_KT + tid]); };
+          auto a_at = [&](int j) { return DIAG ? static_cast<float>(rec[j * RF + REC_A + tid]) : dec[j]; };
+          float g = 1.0f;
+          int j = n - 1;
+          for (; j >= 3; j -= 4) {                            // four records per trip: the loads go out together
+            float kt[4], a[4];
+#pragma unroll
+            for (int e = 0; e < 4; e++) { kt[e] = kt_at(j - e); a[e] = a_at(j - e); }
+#pragma unroll
+            for (int e = 0; e < 4; e++) { kd_row(j - e)[tid] = g * kt[e]; g = g * a[e]; }
+          }
+          for (; j >= 0; j--) { const float kt = kt_at(j); kd_row(j)[tid] = g * kt; g = g * a_at(j); }
+          gam[tid] = g;
+        }
         __syncthreads();
         LQ_BTICK(2);
       }
@@ -618,7 +383,53 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
       float2 M[8][4];                                         // rows 8 ty + a, columns v0 + 2 c, v0 + 2 c + 1
       // ---- the dense state (Eq. 7) ----
       if constexpr (SLOT) {
-        rebuild_tile<MODE == 2 ? 1 : 2>(lq_bsm + Lay::head, r, n, row, kd_row, gam, M);
+        {
+          float ci[8];
+          float2 sj[4];
+          load8(cs + 8 * ty, ci);
+          load8p(ss + v0, sj);
+          uint2 zz[8];
+#pragma unroll
+          for (int b = 0; b < 8; b++) {
+            zz[b] = *reinterpret_cast<const uint2 *>(zt + (v0 + b) * D + 8 * ty);
+            zz[b].x ^= 0x80808080u; zz[b].y ^= 0x80808080u;
+          }
+          // int8 -> fp32 without the conversion unit: byte + 128 in the low mantissa bits of 2^23, minus 2^23 + 128
+#pragma unroll
+          for (int a = 0; a < 8; a++)
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+              const float2 raw = make_float2(
+                  __uint_as_float(__byte_perm(a < 4 ? zz[2 * c].x : zz[2 * c].y, 0x4B000000u, 0x7540 | (a & 3))),
+                  __uint_as_float(__byte_perm(a < 4 ? zz[2 * c + 1].x : zz[2 * c + 1].y, 0x4B000000u, 0x7540 | (a & 3))));
+              M[a][c] = __fmul2_rn(pair(ci[a]), __fmul2_rn(__fadd2_rn(raw, pair(-8388736.0f)), sj[c]));
+            }
+        }
+#pragma unroll 1
+        for (int h = 0; h < r; h++) {
+          float kc[8];
+          float2 uc[4];
+          load8(reinterpret_cast<const __half *>(ckh + h * D + 8 * ty), kc);
+          load8p(reinterpret_cast<const __half *>(cuh + h * D + v0), uc);
+          rank1_pairs(M, kc, uc);
+        }
+        {
+          float gi[8];
+          load8(gam + 8 * ty, gi);
+#pragma unroll
+          for (int a = 0; a < 8; a++)
+#pragma unroll
+            for (int c = 0; c < 4; c++) M[a][c] = __fmul2_rn(pair(gi[a]), M[a][c]);
+        }
+        constexpr int AHEAD = MODE == 2 ? 1 : 2;              // (dequantizing spills with two records at a time)
+#pragma unroll AHEAD
+        for (int j = 0; j < n; j++) {
+          float kj[8];
+          float2 uj[4];
+          load8(kd_row(j) + 8 * ty, kj);
+          load8p(rec + j * RF + REC_U + v0, uj);
+          rank1_pairs(M, kj, uj);
+        }
         LQ_BTICK(3);
       } else {
         const float *S = p.S + bh * (size_t)(D * D) + 8 * ty * D + v0;
@@ -630,7 +441,21 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
 #pragma unroll
         for (int a = 0; a < 8; a++) store_row8(S + a * D, wide, M[a]);
       } else {
-        start_products<RM, SLOT>(M, r, n, row, part);
+        // T_h = S w_h; w_h is the value side of the (h+1)-th newest record, or Walsh function h
+#pragma unroll 2
+        for (int h = 0; h < r; h++) {
+          float2 w[4];
+          if (SLOT && h < n) {
+            load8p(rec + (n - 1 - h) * RF + REC_U + v0, w);
+          } else {
+#pragma unroll
+            for (int c = 0; c < 4; c++) w[c] = make_float2(walsh_entry(h, v0 + 2 * c), walsh_entry(h, v0 + 2 * c + 1));
+          }
+          float pr[8];
+#pragma unroll
+          for (int a = 0; a < 8; a++) pr[a] = block8(M[a], w);
+          store_row_pairs(pr, ty, tx, part + (warp * RM + h) * D);
+        }
       }
       // the slot is free when all have come here: the next head may land while this one is worked on
       if (SLOT) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -640,7 +465,151 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
         bulk_prefetch_l2(p.S + todo_bh[k + 1] * (size_t)(D * D) + tid * (D * D / 8), D * D / 2);
 
       if constexpr (MODE != 2) {
-        requantize_tile<RM>(p, r, lq_bsm, Wv, bh, M);
+        uint32_t alive = 0;
+        if constexpr (RM > 0) {
+          for (int idx = tid; idx < r * D; idx += 256) T[idx] = sum_warps(part + idx, RM * D);
+          LQ_BTICK(10);
+          // further rounds: W_h = S^T q_h, orthonormalise, T_h = S q_h
+          for (int it = 1; it < p.n_iter; it++) {
+            orthonormalize<false, RM>(T, r, gram, chol, nullptr);
+#pragma unroll 1
+            for (int h = 0; h < r; h++) {
+              float x[8], pc[8];
+              load8(T + h * D + 8 * ty, x);
+              column_blocks(M, x, pc);
+              const float s = column_tree(pc, lane, [](float a, float b) { return a + b; });
+              if (lane < 16) Wv[h * D + v0 + column_of(lane)] = s;
+            }
+            orthonormalize<false, RM>(Wv, r, gram, chol, nullptr);
+#pragma unroll 1
+            for (int h = 0; h < r; h++) {
+              float2 w[4];
+              load8p(Wv + h * D + v0, w);
+              float pr[8];
+#pragma unroll
+              for (int a = 0; a < 8; a++) pr[a] = block8(M[a], w);
+              store_row_pairs(pr, ty, tx, part + (warp * RM + h) * D);
+            }
+            __syncthreads();
+            for (int idx = tid; idx < r * D; idx += 256) T[idx] = sum_warps(part + idx, RM * D);
+          }
+          alive = orthonormalize<true, RM>(T, r, gram, chol, p.comp_k(bh));       // T now holds the keys as stored
+          LQ_BTICK(11);
+          gram_lower<RM>(T, r, gram, false);                  // k_a^T k_h (published by the barrier in front of the value sides)
+
+          // ---- value sides and removal of the stored tokens ----
+          float x[RM];                                        // S^T k_h for the lane's column
+#pragma unroll
+          for (int h = 0; h < RM; h++) {
+            x[h] = 0.0f;
+            if (h < r) {
+              float kf[8], pc[8];
+              load8(T + h * D + 8 * ty, kf);
+              column_blocks(M, kf, pc);
+              x[h] = column_tree(pc, lane, [](float a, float b) { return a + b; });
+            }
+          }
+          __syncthreads();                                    // K^T K is complete
+          LQ_BTICK(13);
+          // u_h = S^T k_h - sum_{a<h} u_a (k_a^T k_h) with the stored values: what tokens 0..h-1 leave
+          float uf[RM];
+          const int col = column_of(lane);
+          uint16_t *cu_out = p.comp_u(bh) + v0 + col;
+#pragma unroll
+          for (int h = 0; h < RM; h++) {
+            uf[h] = 0.0f;
+            if (h < r) {
+#pragma unroll
+              for (int a = 0; a < h; a++) x[h] = fmaf(-uf[a], gram[h * RM + a], x[h]);
+              const uint16_t bits = (alive >> h) & 1u ? to_f16_bits_sat(x[h]) : static_cast<uint16_t>(0);
+              uf[h] = f16_bits(bits);
+              if (lane < 16) {
+                cu_out[h * D] = bits;
+                ub[16 * h + 8 * tx + col] = uf[h];
+              }
+            }
+          }
+          __syncwarp();
+          LQ_BTICK(14);
+#pragma unroll 1
+          for (int h = 0; h < r; h++) {                       // M -= k u^T with the stored values
+            float kf[8];
+            float2 uv[4];
+            load8(T + h * D + 8 * ty, kf);
+            load8p(ub + 16 * h + 8 * tx, uv);
+#pragma unroll
+            for (int a = 0; a < 8; a++) kf[a] = -kf[a];
+            rank1_pairs(M, kf, uv);
+          }
+        }
+        LQ_BTICK(4);
+        // ---- residual smoothing: c_i = max(sqrt(mean_j |R_ij|), 1e-6) ----
+        {
+          float pr[8];
+#pragma unroll
+          for (int a = 0; a < 8; a++) {                       // even and odd columns as two chains
+            float even = fabsf(M[a][0].x), odd = fabsf(M[a][0].y);
+#pragma unroll
+            for (int c = 1; c < 4; c++) { even = even + fabsf(M[a][c].x); odd = odd + fabsf(M[a][c].y); }
+            pr[a] = even + odd;
+          }
+          store_row_pairs(pr, ty, tx, part + warp * D);
+        }
+        __syncthreads();
+        if (tid < D) {
+          const float ci = p.smooth ? fmaxf(sqrtf(sum_warps(part + tid, D) / static_cast<float>(D)), 1e-6f) : 1.0f;
+          ic_s[tid] = p.smooth ? 1.0f / ci : 1.0f;
+          p.row_smooth(bh)[tid] = ci;
+        }
+        __syncthreads();
+        LQ_BTICK(5);
+
+        // ---- code steps and codes ----
+        {
+          float ic[8];
+          load8(ic_s + 8 * ty, ic);
+#pragma unroll
+          for (int a = 0; a < 8; a++)
+#pragma unroll
+            for (int c = 0; c < 4; c++) M[a][c] = __fmul2_rn(M[a][c], pair(ic[a]));
+        }
+        float m[8];
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          m[2 * c] = fabsf(M[0][c].x); m[2 * c + 1] = fabsf(M[0][c].y);
+#pragma unroll
+          for (int a = 1; a < 8; a++) {
+            m[2 * c] = fmaxf(m[2 * c], fabsf(M[a][c].x));
+            m[2 * c + 1] = fmaxf(m[2 * c + 1], fabsf(M[a][c].y));
+          }
+        }
+        const float amax = column_tree(m, lane, [](float a, float b) { return fmaxf(a, b); });
+        if (lane < 16) {
+          const int col = column_of(lane);
+          p.col_scale(bh)[v0 + col] = amax / 127.0f;          // stored as the step of the code, B_j / 127
+          invc[8 * tx + col] = amax > 0.0f ? 127.0f / amax : 0.0f;
+        }
+        __syncwarp();
+        LQ_BTICK(6);
+        float2 inv[4];
+        load8p(invc + 8 * tx, inv);
+        int8_t *ZT = p.codes(bh) + v0 * D + 8 * ty;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          // |X * inv| <= 127 (1 + 2^-23): adding 1.5 * 2^23 leaves the nearest integer (ties to even) in the low byte
+          // (product and sum are rounded one after the other; written as a packed addition the two would get fused)
+          float2 z[8];
+#pragma unroll
+          for (int a = 0; a < 8; a++) z[a] = __ffma2_rn(__fmul2_rn(M[a][c], inv[c]), pair(1.0f), pair(12582912.0f));
+          auto bytes4 = [](float x0, float x1, float x2, float x3) {
+            return __byte_perm(__byte_perm(__float_as_uint(x0), __float_as_uint(x1), 0x0040),
+                               __byte_perm(__float_as_uint(x2), __float_as_uint(x3), 0x0040), 0x5410);
+          };
+          *reinterpret_cast<uint2 *>(ZT + (2 * c) * D) =
+              make_uint2(bytes4(z[0].x, z[1].x, z[2].x, z[3].x), bytes4(z[4].x, z[5].x, z[6].x, z[7].x));
+          *reinterpret_cast<uint2 *>(ZT + (2 * c + 1) * D) =
+              make_uint2(bytes4(z[0].y, z[1].y, z[2].y, z[3].y), bytes4(z[4].y, z[5].y, z[6].y, z[7].y));
+        }
         if (MODE == 1 && tid == 0) p.win_pos[bh / p.heads_v] = 0;      // (nobody reads win_pos in this mode)
       }
       if (k == 0) LQ_STAMP(1, 3);

@@ -398,10 +398,9 @@ __device__ __forceinline__ int nth_set_bit(uint32_t m, unsigned k) {
 // W = 16: up to five boundaries on one CTA and none on others; a step of 100 us, 73 us with equal shares).
 // One warp finds up to 32 of a CTA's heads in one pass over win_pos: lane l looks for due head number first + l * stride.
 // Returns how many lanes found theirs (lanes 0 .. count-1); bh and n are the head and its buffered records, `total` how
-// many sequences are due in all.  is_due(n): whether a window that holds n records is.
-template <typename Due>
-__device__ __forceinline__ int find_due_heads(const Params &p, Due is_due, unsigned first, unsigned stride, int lane, unsigned &bh,
-                                              int &n, int &total) {
+// many sequences are due in all.
+__device__ __forceinline__ int find_due_heads(const Params &p, unsigned first, unsigned stride, int lane, unsigned &bh, int &n,
+                                              int &total) {
   constexpr int U = 8;                       // loads in flight per lane
   const unsigned item = first + lane * stride;
   const unsigned want = item / static_cast<unsigned>(p.heads_v);       // rank of the head's sequence among the due ones
@@ -414,7 +413,7 @@ __device__ __forceinline__ int find_due_heads(const Params &p, Due is_due, unsig
     for (int u = 0; u < U; u++) v[u] = b0 + 32 * u + lane < p.batch ? p.win_pos[b0 + 32 * u + lane] & 0xFFFF : 0;
 #pragma unroll
     for (int u = 0; u < U; u++) {
-      const uint32_t m = __ballot_sync(FULL, b0 + 32 * u + lane < p.batch && is_due(v[u]));
+      const uint32_t m = __ballot_sync(FULL, v[u] == p.W || (p.force && v[u] > 0));
       if (m == 0) continue;
       const unsigned c = __popc(m);
       const bool mine = want - base < c;     // (unsigned: false for ranks below base)
@@ -432,31 +431,27 @@ __device__ __forceinline__ int find_due_heads(const Params &p, Due is_due, unsig
   return __popc(__ballot_sync(FULL, found));
 }
 
-// Whoever has seen all it needs of win_pos (the CTAs of a boundary kernel, the pairs of warps of the decode kernel) says so on
-// the upper bits of win_pos[0].  The last one to arrive moves the windows on: nobody reads win_pos any more then, and the work
-// on the heads does not need it.  report_seen (one lane) returns the old value, its upper half the number of earlier arrivals.
-__device__ __forceinline__ int report_seen(const Params &p) { return atomicAdd(p.win_pos, 0x10000); }
-// next(n): what a window of n records becomes.  One warp.
-template <typename Next>
-__device__ __forceinline__ void move_windows(const Params &p, int lane, Next next) {
-  constexpr int U = 8;                       // loads in flight per lane
-  for (int b0 = 0; b0 < p.batch; b0 += 32 * U) {
-    int v[U];
-#pragma unroll
-    for (int u = 0; u < U; u++) v[u] = b0 + 32 * u + lane < p.batch ? __ldcg(p.win_pos + b0 + 32 * u + lane) & 0xFFFF : 0;
-#pragma unroll
-    for (int u = 0; u < U; u++) {
-      const int b = b0 + 32 * u + lane, nv = next(v[u]);
-      if (b < p.batch && (nv != v[u] || b == 0)) p.win_pos[b] = nv;
-    }
-  }
-}
-// A boundary kernel's use of the two: the windows that are due start afresh.
+// A CTA that has seen all of win_pos says so on the upper bits of win_pos[0]; the last one starts the windows of the due
+// sequences afresh (nobody reads win_pos any more, and the boundaries themselves do not need it).  One warp calls this.
 __device__ __forceinline__ void restart_due_windows(const Params &p, int lane) {
   int old = 0;
-  if (lane == 0) old = report_seen(p);
-  if ((__shfl_sync(FULL, old, 0) >> 16) != static_cast<int>(gridDim.x) - 1) return;
-  move_windows(p, lane, [&](int v) { return v == p.W || (p.force && v > 0) ? 0 : v; });
+  if (lane == 0) old = atomicAdd(p.win_pos, 0x10000);
+  old = __shfl_sync(FULL, old, 0);
+  if ((old >> 16) != static_cast<int>(gridDim.x) - 1) return;
+  for (int b = lane; b < p.batch; b += 32) {
+    const int v = __ldcg(p.win_pos + b) & 0xFFFF;
+    const bool due = v == p.W || (p.force && v > 0);
+    if (due || b == 0) p.win_pos[b] = due ? 0 : v;
+  }
+}
+
+// Last-arrival bookkeeping on win_pos[b]: bits 16.. count the heads of sequence b that are done with
+// the value in bits 0..15.  The head that arrives last (all heads_v have read the old value by then)
+// stores the new value and thereby clears the counter.  Call from one thread per head, after a
+// __syncthreads() that follows the head's last global write.
+__device__ __forceinline__ void arrive_and_set(int32_t *win_pos, int b, int heads_v, int new_value) {
+  const int old = atomicAdd(win_pos + b, 0x10000);
+  if ((old >> 16) == heads_v - 1) win_pos[b] = new_value;
 }
 
 }  // namespace lq

@@ -32,7 +32,7 @@
 #pragma once
 #include <type_traits>
 
-#include "lq_boundary.cuh"
+#include "lq_common.cuh"
 
 namespace lq {
 
@@ -43,7 +43,7 @@ constexpr int REC_SEG = 32;                // (16 was tried: no faster at W = 32
 // ---- shared-memory slot of one CTA ----
 struct DecodeSlot {
   // byte offsets inside the slot; every region starts on a 16-byte boundary
-  int head, rec, bas, digits, y, pk, pq, bytes;
+  int head, rec, bas, digits, y, pk, pq, mbar, bytes;
   __host__ __device__ DecodeSlot(int W, int r, bool diag, bool rec16 = false) {
     // a window holds at most W-1 records when a token arrives; they are staged REC_SEG rows at a time (newest
     // first), which keeps the slot small for long windows
@@ -57,6 +57,7 @@ struct DecodeSlot {
     y = o; o += 2 * 4 * D;                // [2][128]: the rounded sums of the state stream, later the record terms
     pk = o; o += (4 * (r + 2) + 15) / 16 * 16;      // compensator projections against Gamma k
     pq = o; o += (4 * (r + 2) + 15) / 16 * 16;      // ... against Gamma q; pq[r], pq[r+1] hold kt^T q of alternate heads
+    mbar = o; o += 16;
     bytes = (o + 127) / 128 * 128;
   }
 };
@@ -106,15 +107,13 @@ __device__ __forceinline__ void tree16x4(float (&x)[4]) {
 }
 
 // Named barriers of the CTA (64 threads each): one side arrives, the other waits.
-//   1: dot warp -> stream warp, "the record terms (and the ticket) are in shared memory"
-//   2: stream warp -> dot warp, "its sums are out of y"
-//   3: dot warp -> stream warp, "the compensator projections are in shared memory"
-//   4: stream warp -> dot warp, "the records' decays have been read" (diagonal gate)
+//   1: dot warp -> stream warp, "the projections are in shared memory"
+//   2: stream warp -> dot warp, "the slot may be overwritten"
 __device__ __forceinline__ void named_arrive(int id) {
   __threadfence_block();
   asm volatile("bar.arrive %0, 64;\n" ::"r"(id) : "memory");
 }
-__device__ __forceinline__ void named_sync(int id) { asm volatile("bar.sync %0, 64;\n" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void named_wait(int id) { asm volatile("bar.sync %0, 64;\n" ::"r"(id) : "memory"); }
 
 // The token's vectors as raw bf16 bits, loaded one head ahead: lane c (and its twin c+16) owns key
 // channels 8c..8c+7, lane l value channels 4l..4l+3.
@@ -124,22 +123,20 @@ struct TokenRaw {
   float ba_lo, ba_hi;   // scalar gate: decays of buffered records `lane` and `lane + 32` (stale beyond n)
 };
 
-// What a pair of warps works on: a head, its sequence, the records buffered (bits 16.. of n may hold the counter of
-// report_seen), the token's beta and scalar alpha as bf16 bits (low and high half of ba).  due: an entry of the CTA's list
-// of boundaries (bh == NO_HEAD: the pair only lends its warps).
-constexpr unsigned NO_HEAD = 0xFFFFFFFFu;
-struct PairHead {
-  unsigned bh, b;
-  int n;
-  uint32_t ba;
-  bool due;
+// A head index with its sequence and value-head parts, stepped without divisions.
+struct HeadIdx {
+  unsigned bh, b, hv;
+  __device__ __forceinline__ void step(unsigned dbh, unsigned db, unsigned dhv, unsigned heads_v) {
+    bh += dbh; b += db; hv += dhv;
+    if (hv >= heads_v) { hv -= heads_v; b += 1; }
+  }
 };
 
 template <int GATE>
-__device__ __forceinline__ void load_token(const Params &p, const PairHead &h, int group, int lane, int role, TokenRaw &tk) {
+__device__ __forceinline__ void load_token(const Params &p, const HeadIdx h, int group, int lane, int role, TokenRaw &tk) {
   const int c = lane & 15;
   const size_t bh = h.bh;
-  const size_t qk_off = ((size_t)h.b * p.heads_qk + (h.bh - h.b * p.heads_v) / group) * D;
+  const size_t qk_off = ((size_t)h.b * p.heads_qk + h.hv / group) * D;
   tk.k = *reinterpret_cast<const uint4 *>(p.k + qk_off + 8 * c);
   tk.q = *reinterpret_cast<const uint4 *>(p.q + qk_off + 8 * c);
   if (role == 0) tk.v = *reinterpret_cast<const uint2 *>(p.v + bh * D + 4 * lane);
@@ -151,81 +148,19 @@ __device__ __forceinline__ void load_token(const Params &p, const PairHead &h, i
   }
 }
 
-// The plan of a CTA: `pairs` pairs of warps with a slot each.  If it takes the window boundaries as well, the working arrays
-// of a boundary are laid over the last slots, so that the first `hold` slots (a power of two) can keep a due head each.
-struct StepPlan {
-  int pairs, hold;
-  int scratch;                               // offset of the working arrays from the first slot
-  int bytes;                                 // shared memory of the CTA, with the area in front of the slots
-};
-template <int RM>
-__host__ __device__ constexpr int flush_scratch_bytes(int W, int r, bool rec16, bool iterate) {
-  return BoundarySmem<RM>::head + (rec16 ? 4 * D * W : 0) + (iterate ? 4 * D * r : 0);
-}
-
-// In front of the slots: the copy barriers of the pairs (two of eight bytes each), then what the warps of a CTA with boundaries
-// share: entries of its list of boundaries (number m at m mod 64; 32 at a time are found) and how many there are in all.
-struct DueList {
-  unsigned bh[64];
-  int n[64], count;
-};
-constexpr int SLOTS_AT = 128, SLOTS_AT_LIST = 640;
-static_assert(64 + sizeof(DueList) <= SLOTS_AT_LIST, "the list fits in front of the slots");
-
-// The boundary of head bh, whose block and W records are in `slot` (the newest record in the slot's digits region, its
-// decay at dec[W - 1]).  Called by the 256 threads of a CTA after a barrier; ends with one.  (A function of its own: the
-// decode loop around the call keeps its registers, and the warps without a slot run the same instructions.)
-template <int GATE, bool R16, int RM>
-__device__ __noinline__ void flush_slot(const Params &p, unsigned char *slot, unsigned char *work, const size_t bh) {
-  constexpr bool DIAG = GATE == LQ_GATE_DIAG;
-  constexpr int RF = record_floats(DIAG);
-  using rec_t = typename std::conditional<R16, __half, float>::type;
-  using Lay = BoundarySmem<RM>;
-  const int W = p.W, r = RM > 0 ? max(p.r, 1) : 0, tid = threadIdx.x;
-  const DecodeSlot L(W, r, DIAG, R16);
-  rec_t *rec = reinterpret_cast<rec_t *>(slot + L.rec), *newest = reinterpret_cast<rec_t *>(slot + L.digits);
-  const float *dec = reinterpret_cast<const float *>(slot + L.bas) + MAX_W;       // (the dot warp's copy of the decays)
-  float *gam = reinterpret_cast<float *>(work + Lay::gam), *part = reinterpret_cast<float *>(work + Lay::part);
-  float *kd = reinterpret_cast<float *>(work + Lay::head), *Wv = kd + (R16 ? W * D : 0);
-  auto row = [&](int j) { return j < W - 1 ? rec + j * RF : newest; };
-  auto kd_row = [&](int j) -> float * {
-    if constexpr (R16) return kd + j * D;
-    else return row(j) + REC_KT;
-  };
-  if (tid < D) decay_records<DIAG>(W, row, kd_row, dec, gam);
-  __syncthreads();
-  float2 M[8][4];
-  rebuild_tile<2>(slot + L.head, r, W, row, kd_row, gam, M);
-  start_products<RM, true>(M, r, W, row, part);
-  // (the slots were written to by ordinary stores; bulk copies write there next)
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-  __syncthreads();
-  requantize_tile<RM>(p, r, work, Wv, bh, M);
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-  __syncthreads();
-}
-
-// The work of one pair of warps (role 0: stream warp, role 1: dot warp) on its shared-memory slot, and of the warps beyond
-// the last pair.
-// RM < 0: a CTA is one pair; a window that becomes full is left at win_pos == W for the boundary kernel behind this one.
-// RM >= 0: a CTA of eight warps is up to four pairs and performs the boundaries as well, for r <= RM: the due heads (those at
-// their last free record, and those that came in with a full window) are dealt out evenly, CTA i taking numbers i, i + G, ...
-// The first plan.hold pairs give a due head each its token, then all eight warps meet and take these heads through the
-// boundary where they are; nothing is read again.
+// The work of one pair of warps (role 0: stream warp, role 1: dot warp) on its shared-memory slot: heads
+// first, first + G, first + 2G, ...
 // LONGW: the window may hold more records than the slot stages at a time (W - 1 > REC_SEG); in the instances for
 // shorter windows everything to do with a second segment drops out at compile time.
-template <int GATE, bool R16, bool LONGW, int RM>
-__device__ __forceinline__ void decode_pair(const Params &p, unsigned char *smem, const StepPlan &plan) {
-  constexpr bool DIAG = GATE == LQ_GATE_DIAG, BOUNDARY = RM >= 0;
-  static_assert(!(BOUNDARY && LONGW), "the boundary needs all records of the window in the slot");
+template <int GATE, bool R16, bool LONGW>
+__device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot, const int lane, const int role,
+                                            const unsigned first, const unsigned G) {
+  uint32_t parA = 0, parR = 0;               // phases of the slot's two copy barriers
+  constexpr bool DIAG = GATE == LQ_GATE_DIAG;
   constexpr int RF = record_floats(DIAG);
   const int W = p.W, r = p.r;
   using rec_t = typename std::conditional<R16, __half, float>::type;   // element type of the record rows
   const DecodeSlot L(W, r, DIAG, R16);
-  const int lane = threadIdx.x & 31, role = (threadIdx.x >> 5) & 1, pr = BOUNDARY ? threadIdx.x >> 6 : 0;
-  const int PAIRS = BOUNDARY ? plan.pairs : 1, B0 = BOUNDARY ? pr * (DIAG ? 4 : 3) : 0;     // B0: named barriers of the pair
-  const bool lender = BOUNDARY && pr >= PAIRS;                         // a warp without a slot
-  unsigned char *slots = smem + (BOUNDARY ? SLOTS_AT_LIST : SLOTS_AT), *slot = slots + (lender ? 0 : pr) * L.bytes;
   const int c = lane & 15, half = lane >> 4, g = lane >> 2, t = lane & 3;
   const int8_t *zt = reinterpret_cast<const int8_t *>(slot + L.head + HB_CODES);
   const float *bs = reinterpret_cast<const float *>(slot + L.head + HB_COL_SCALE);
@@ -237,11 +172,10 @@ __device__ __forceinline__ void decode_pair(const Params &p, unsigned char *smem
   int8_t *digits = reinterpret_cast<int8_t *>(slot + L.digits);
   float *y = reinterpret_cast<float *>(slot + L.y), *pk = reinterpret_cast<float *>(slot + L.pk);
   float *pq = reinterpret_cast<float *>(slot + L.pq);
-  const uint32_t barA = smem_addr(smem) + 16 * pr, barR = barA + 8, slot_a = smem_addr(slot);   // head block, records
-  uint32_t parA = 0, parR = 0;               // phases of the slot's two copy barriers
+  const uint32_t barA = smem_addr(slot + L.mbar), barR = barA + 8, slot_a = smem_addr(slot);   // head block, records
 
   const unsigned nh = static_cast<unsigned>(p.batch) * p.heads_v, Hv = p.heads_v;
-  const unsigned G = gridDim.x, P = PAIRS * G, me = pr * G + blockIdx.x;      // pairs in all, this one's number
+  const unsigned G_b = G / Hv, G_hv = G % Hv;       // one grid stride in (sequence, head) steps
   const int group = p.heads_v / p.heads_qk;
 
 #ifdef LQ_TIMING
@@ -256,13 +190,13 @@ __device__ __forceinline__ void decode_pair(const Params &p, unsigned char *smem
   // The regions the copies overwrite were only READ through ordinary loads, whose values have been used
   // before the call; the warps write only their scratch regions.  So nothing written by the generic proxy is
   // at stake and no cross-proxy fence is needed (it costs over a thousand cycles here).
-  // With the boundary in a kernel of its own, a head at its last free record (n == W - 1) is read again right after this
-  // kernel: its lines are asked to stay in the L2 until then.  No other line is read again soon.
+  // A head at its last free record (n == W - 1) goes through the window boundary right after this kernel, which
+  // reads the same head block and records again: its lines are asked to stay in the L2 until then.
   const uint64_t keep = l2_keep_policy(), stream = l2_stream_policy();
   auto request_head = [&](unsigned bh, int n) {
     if (lane == 0) {
       mbar_expect_tx(barA, head_bytes(r));
-      if (!BOUNDARY && n == W - 1) bulk_g2s_hint(slot_a + L.head, p.head(bh), head_bytes(r), barA, keep);
+      if (n == W - 1) bulk_g2s_hint(slot_a + L.head, p.head(bh), head_bytes(r), barA, keep);
       else bulk_g2s_hint(slot_a + L.head, p.head(bh), head_bytes(r), barA, stream);
     }
   };
@@ -275,7 +209,7 @@ __device__ __forceinline__ void decode_pair(const Params &p, unsigned char *smem
       const uint32_t rb = static_cast<uint32_t>(sizeof(rec_t)) * RF * (hi - lo);
       mbar_expect_tx(barR, rb);              // with no records the phase completes at once
       if (hi > lo) {
-        if (!BOUNDARY && n == W - 1) bulk_g2s_hint(slot_a + L.rec, p.record<rec_t>(bh, lo, DIAG), rb, barR, keep);
+        if (n == W - 1) bulk_g2s_hint(slot_a + L.rec, p.record<rec_t>(bh, lo, DIAG), rb, barR, keep);
         else bulk_g2s_hint(slot_a + L.rec, p.record<rec_t>(bh, lo, DIAG), rb, barR, stream);
       }
     }
@@ -290,599 +224,475 @@ __device__ __forceinline__ void decode_pair(const Params &p, unsigned char *smem
     __syncwarp();
   };
 
-  // Which heads.  Equal shares do not take equal time: pairs that share an SM with fewer others, or sit nearer the memory
-  // they read, are through with ten heads when others have done eight, and a CTA with boundaries to perform has less time
-  // for other heads.  So every pair takes only its first S heads in turn (me, me + P, ...; due heads are left out where the
-  // boundary is performed here), and with scratch words in the state (lq_state.work) the heads that are left
-  // (S P + t, t < pool) go to whoever gets there first: from the moment on at which nothing is left to take in turn after
-  // the next head, the dot warp draws a ticket t in every trip, for the head two trips on (word 0 of the scratch words
-  // counts the tickets), hands it to the stream warp with the record terms (barrier 1), and at the end of the trip both
-  // warps ask for that head's scalars, which they look at for the first time half a trip later.
+  // Equal shares do not take equal time: pairs that share an SM with fewer others, or sit nearer the memory they
+  // read, are through with ten heads when others have done eight.  With scratch words in the state (lq_state.work)
+  // every pair therefore takes only its first S heads in turn (DRAWN_ROUNDS rounds fewer than would fall to it), and
+  // the heads that are left (S G + t, t < pool) go to whoever gets there first: from its last turn but one on, the dot
+  // warp draws a ticket t in every trip, for the head two trips on (word 0 of the scratch words counts the tickets;
+  // the boundary kernel behind this one puts it back to zero), hands it to the stream warp with the record terms
+  // (barrier 1), and at the end of the trip both warps ask for that head's scalars, which they look at for the first
+  // time half a trip later (ext_*) and move to the lane registers of the other heads' at the end of the next trip.
   // A pair stops when a ticket is beyond the pool.
-  const int rounds = static_cast<int>(nh / P);                 // rounds in which every pair has a head
-  const bool draw = p.work != nullptr && rounds >= 3;
-  const int S = lender ? 0 : draw ? rounds - (BOUNDARY ? (rounds >= 6 ? 3 : 2) : rounds >= 6 ? 2 : 1)
-                                  : me < nh ? static_cast<int>((nh - 1 - me) / P) + 1 : 0;
-  const unsigned pool = draw ? nh - static_cast<unsigned>(S) * P : 0;
-  auto is_due = [&](int n) { return BOUNDARY && (n == W - 1 || n == W); };
-  auto in_turn = [&](int n) { return n < (BOUNDARY ? W - 1 : W); };    // (a full window gets no token)
-  auto wanted = [&](const PairHead &h) { const int n = h.n & 0xFFFF; return h.due ? n < W : in_turn(n); };
-
-  // The heads taken in turn, 32 at a time: lane l holds head number t0 + l of this pair and its scalars.
-  int t0 = 0, sc_n = 0;
-  uint32_t sc_ba = 0, todo = 0;              // todo: lanes whose head has not been taken up yet
-  auto load_window = [&]() {
-    const unsigned bh = me + static_cast<unsigned>(t0 + lane) * P;
-    bool mine = t0 + lane < S;
-    if (mine) {
-      sc_n = p.win_pos[bh / Hv];             // (once per 32 heads: a division is fine here)
-      sc_ba = p.beta[bh];
-      if (!DIAG) sc_ba |= static_cast<uint32_t>(p.alpha[bh]) << 16;
-      mine = in_turn(sc_n & 0xFFFF);
+  const int rounds_all = static_cast<int>(nh / G);             // rounds in which every pair has a head
+  const int DRAWN_ROUNDS = rounds_all >= 6 ? 2 : 1;            // (with few rounds, more of them in turn)
+  const bool draw = p.work != nullptr && rounds_all >= 3;
+  const int S = draw ? rounds_all - DRAWN_ROUNDS : 0;
+  const unsigned pool = draw ? nh - static_cast<unsigned>(S) * G : 0;
+  // Per-head scalars of this CTA's heads, 32 heads at a time: lane l holds those of the CTA's (32*batch+l)-th head
+  int sc_n = 0;
+  uint32_t sc_beta = 0, sc_alpha = 0;
+  auto load_scalars = [&](unsigned first_bh) {
+    const unsigned bh = first_bh + lane * G;  // (once per 32 heads: a division is fine here)
+    if (bh < (draw ? static_cast<unsigned>(S) * G : nh)) {     // (the heads taken in turn)
+      sc_n = p.win_pos[bh / Hv];             // bits 16.. are the arrival counter of this launch: masked at use
+      sc_beta = p.beta[bh];
+      if (!DIAG) sc_alpha = p.alpha[bh];
     }
-    todo = __ballot_sync(FULL, mine);
-  };
-  auto more_in_turn = [&]() { return todo != 0 || t0 + 32 < S; };     // (a window to come may turn out empty: no harm)
-  auto take_in_turn = [&](PairHead &h) {
-    while (todo == 0) {
-      if (t0 + 32 >= S) return false;
-      t0 += 32;
-      load_window();
-    }
-    const int l = __ffs(todo) - 1;
-    todo &= todo - 1;
-    h.bh = me + static_cast<unsigned>(t0 + l) * P;
-    h.b = h.bh / Hv;
-    h.n = __shfl_sync(FULL, sc_n, l);
-    h.ba = __shfl_sync(FULL, sc_ba, l);
-    h.due = false;
-    return true;
-  };
-  DueList &list = *reinterpret_cast<DueList *>(smem + 64);
-  auto load_list = [&](unsigned d0) {        // entries d0 .. d0 + 31 of the CTA's list of boundaries, by one warp
-    unsigned bh_due;
-    int n_due, total;
-    const int found = find_due_heads(p, is_due, blockIdx.x + d0 * G, G, lane, bh_due, n_due, total);
-    const unsigned items = static_cast<unsigned>(total) * Hv, at = (d0 + lane) & 63;
-    if (lane < found) { list.bh[at] = bh_due; list.n[at] = n_due; }
-    if (lane == 0) list.count = items > blockIdx.x ? static_cast<int>((items - 1 - blockIdx.x) / G) + 1 : 0;
-  };
-  int due = 0, due_next = 0;                 // boundaries of this CTA, and how many of them have been taken up
-  const int hold = BOUNDARY ? plan.hold : 1;
-  auto take_due = [&](PairHead &h) {         // this pair's part in the next `hold` of them
-    const int m = due_next + pr;
-    h = PairHead{NO_HEAD, 0u, W, 0u, true};
-    if (pr < hold && m < due) {
-      h.bh = list.bh[m & 63];
-      h.b = h.bh / Hv;
-      h.n = list.n[m & 63];
-      h.ba = p.beta[h.bh];
-      if (!DIAG) h.ba |= static_cast<uint32_t>(p.alpha[h.bh]) << 16;
-    }
-    due_next += hold;
-  };
-  // All warps of the CTA: the boundaries of entries m0 .. m0 + hold - 1, each in the slot of the pair that gave it its token.
-  auto perform_boundaries = [&](int m0) {
-    __syncthreads();                         // the tokens are complete in the slots, the others are free
-    const int m1 = m0 + hold < due ? m0 + hold : due;
-#pragma unroll 1
-    for (int m = m0; m < m1; m++) {
-      if constexpr (BOUNDARY) flush_slot<GATE, R16, RM>(p, slots + (m - m0) * L.bytes, slots + plan.scratch, list.bh[m & 63]);
-    }
-    // (entries are taken up to three rounds ahead: the next 32 are found when the first of these 32 are done with)
-    if (m0 > 0 && m0 % 32 == 0 && m0 + 32 < due) {
-      if (threadIdx.x < 32) load_list(static_cast<unsigned>(m0 + 32));
-      __syncthreads();
-    }
-  };
-  // The pair has read all it will of win_pos (report_seen): the last of the pairs to say so moves the windows on, and puts
-  // the ticket counter back to zero.
-  auto finish_step = [&](int seen) {
-    seen = __shfl_sync(FULL, seen, 0);
-    if ((seen >> 16) != static_cast<int>(P) - 1) return;
-    move_windows(p, lane, [&](int v) { return in_turn(v) ? v + 1 : BOUNDARY && v <= W ? 0 : v; });
-    if (BOUNDARY && lane == 0 && p.work != nullptr) p.work[0] = 0;     // (else the boundary kernel does that)
   };
 
+  // Arrival on win_pos (see arrive_and_set): the counter says how many heads of the sequence have READ the old
+  // value, which this head did when its scalars were loaded.  The dot warp makes the arrival, at the end of its
+  // work: it has slack, the stream warp (the longer of the two) has none to sit out the atomic's round trip.
+  // A head whose window is already full (n >= W) gets no token: it is neither requested nor waited for.
+  auto wanted = [&](int n_) { return n_ < W; };
+  load_scalars(first);
   TokenRaw nxt;                               // the token of the head about to start
   nxt.ba_lo = nxt.ba_hi = 1.0f;
-  PairHead cur{}, nx{};                       // this head and the next one
-  auto start = [&]() {                        // the head at hand, when nothing has been asked for ahead of time
-    load_token<GATE>(p, cur, group, lane, role, nxt);
-    if (role == 0) request_head(cur.bh, cur.n & 0xFFFF);
-    else request_records(cur.bh, cur.n & 0xFFFF);
-  };
-  load_window();
-  bool have_cur = take_in_turn(cur);
-  if (have_cur) start();
-  int taken = have_cur, due_at = 0;
-  if (BOUNDARY) {
-    // the list of boundaries, while the first heads are on their way (by a warp without a slot, if there is one)
-    if (threadIdx.x >= blockDim.x - 32) {
-      load_list(0);
-      __syncwarp();
-      if (list.count > 32) load_list(32);
+  HeadIdx hd{first, first / Hv, first % Hv};  // this head and the next one
+  HeadIdx hd1 = hd;
+  hd1.step(G, G_b, G_hv, Hv);
+  {
+    const int n0 = __shfl_sync(FULL, sc_n, 0) & 0xFFFF;
+    if (first < nh && wanted(n0)) {
+      load_token<GATE>(p, hd, group, lane, role, nxt);
+      if (role == 0) request_head(first, n0);
+      else request_records(first, n0);
     }
-    __syncthreads();
-    due = list.count;
-    if (lender) {
-      for (int m0 = 0; m0 < due; m0 += hold) perform_boundaries(m0);
-      return;
-    }
-    // (the two CTAs of an SM take their boundaries at different times, so that one of them keeps the memory busy)
-    due_at = 2 * blockIdx.x >= G && S > 3 ? S / 2 : 1;
   }
-  auto take = [&](PairHead &h) {
-    if (BOUNDARY && due_next < due && taken >= due_at) { take_due(h); return true; }
-    if (take_in_turn(h)) { taken++; return true; }
-    if (BOUNDARY && due_next < due) { take_due(h); return true; }
-    return false;
-  };
-  if (!have_cur) {
-    have_cur = take(cur);
-    if (have_cur && wanted(cur)) start();
-  }
-  bool have_nx = have_cur && take(nx);
 #ifdef LQ_TIMING
   tick_ = clock64();
 #endif
   unsigned *qidx = reinterpret_cast<unsigned *>(pk + r);      // (a spare word of the projection area)
   unsigned ticket = 0xFFFFFFFFu;             // (dot warp, lane 0) what was drawn in this trip
   bool drawing = draw;                       // no ticket has been beyond the pool yet
-  bool reported = false;
-  int trips = 0, done = 0;                   // done: boundaries performed
-  while (have_cur || have_nx || drawing) {
-    const bool turn_over = !more_in_turn() && due_next >= due;  // nothing is left to take but what is drawn
-    const bool draws = drawing && turn_over;                    // a ticket is drawn in this trip
+  int ext_n = 0;                             // scalars of the head drawn a trip ago, on their way
+  uint32_t ext_beta = 0, ext_alpha = 0;
+  int idx = 0;                               // position of the head in this slot's list
+  // end of a trip
+  auto finish_trip = [&]() {
+    // the next head, if it was drawn: its scalars, asked for a trip ago, go where the others' are
+    if (draw && idx + 1 >= S && lane == ((idx + 1) & 31)) { sc_n = ext_n; sc_beta = ext_beta; sc_alpha = ext_alpha; }
+    unsigned extra = nh;                     // the head after the next one, if it is a drawn one
+    if (drawing && idx + 2 >= S) {
+      const unsigned tk = role == 1 ? __shfl_sync(FULL, ticket, 0) : *reinterpret_cast<volatile unsigned *>(qidx);
+      if (tk < pool) {
+        extra = static_cast<unsigned>(S) * G + tk;
+        ext_n = p.win_pos[extra / Hv];
+        ext_beta = p.beta[extra];
+        if (!DIAG) ext_alpha = p.alpha[extra];
+      } else {
+        drawing = false;
+      }
+    }
+    hd = hd1;
+    idx++;
+    if (!draw || idx + 1 < S) {
+      hd1.step(G, G_b, G_hv, Hv);
+    } else if (extra < nh) {
+      const unsigned b_ = extra / Hv;
+      hd1 = HeadIdx{extra, b_, extra - b_ * Hv};
+    } else {
+      hd1 = HeadIdx{nh, 0u, 0u};
+    }
+  };
+  for (; hd.bh < nh; finish_trip()) {
+    const bool draws = drawing && idx + 2 >= S;                 // a ticket is drawn in this trip
     if (draws && role == 1 && lane == 0) ticket = static_cast<unsigned>(atomicAdd(p.work, 1));
-    // Before the warps meet for a boundary nothing may be on its way into the slots.
-    const bool ask = have_nx && nx.bh != NO_HEAD && !(BOUNDARY && have_cur && cur.due);     // the next head is asked for in this trip
-    const bool last = have_cur && !have_nx && turn_over && !draws;      // nothing more of win_pos is read after this head
-    const int n = cur.n & 0xFFFF;
-    const size_t bh = cur.bh;
-    const float beta = __uint_as_float(cur.ba << 16), alpha_s = __uint_as_float(cur.ba & 0xFFFF0000u);
+    const size_t bh = hd.bh;
+    const int n = __shfl_sync(FULL, sc_n, idx & 31) & 0xFFFF;
+    const float beta = __uint_as_float(__shfl_sync(FULL, sc_beta, idx & 31) << 16);
+    const float alpha_s = __uint_as_float(__shfl_sync(FULL, sc_alpha, idx & 31) << 16);
+    // the next head's scalars: from the next batch when this head is the last of its batch
+    const unsigned bh_next = hd1.bh;
+    if ((idx & 31) == 31) load_scalars(bh_next);
+    // The next head's window position.  Of a drawn head it is still on its way (ext_n, asked for at the end of the
+    // trip before): it is looked at only where the head's data is requested, half a trip from here; until then the
+    // head counts as one that gets a token (its token is loaded, which does no harm if it gets none).
+    const bool next_drawn = draw && idx + 1 >= S;
+    const int n_next_turn = bh_next < nh ? (__shfl_sync(FULL, sc_n, (idx + 1) & 31) & 0xFFFF) : W;
+    auto n_next_now = [&]() { return next_drawn ? (bh_next < nh ? (ext_n & 0xFFFF) : W) : n_next_turn; };
+    const bool next_token = next_drawn ? bh_next < nh : wanted(n_next_turn);
+    const bool active = wanted(n);
+    const int b = static_cast<int>(hd.b);
     LQ_TICK(0);
 
-    if (!have_cur || !wanted(cur)) {
-      // (Here as in a trip with a token, barrier 2 comes before barrier 1 and each of them once: a warp that arrived twice
-      // before the other came would complete the barrier by itself.)
-      const bool full = BOUNDARY && have_cur && cur.due && cur.bh != NO_HEAD;
-      if (full || draws) {                   // the stream warp is through with the trip before
-        if (role == 0) named_arrive(B0 + 2);
-        else named_sync(B0 + 2);
-      }
-      if (full) {                            // came in with a full window: no token, but its boundary
-        if (lane == 0) {
-          asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-          if (role == 0) {
-            mbar_expect_tx(barA, head_bytes(r));
-            bulk_g2s(slot_a + L.head, p.head(bh), head_bytes(r), barA);
-          } else {
-            constexpr uint32_t row_bytes = sizeof(rec_t) * RF;
-            mbar_expect_tx(barR, W * row_bytes);
-            if (W > 1) bulk_g2s(slot_a + L.rec, p.record<rec_t>(bh, 0, DIAG), (W - 1) * row_bytes, barR);
-            bulk_g2s(slot_a + L.digits, p.record<rec_t>(bh, W - 1, DIAG), row_bytes, barR);
-          }
-        }
-        if (!DIAG && role == 1)
-          for (int j = lane; j < W; j += 32) bas[j] = p.decays[bh * (size_t)W + j];
-        wait_for(barA, parA);
-        if (DIAG || role == 1) wait_for(barR, parR);
-      }
-      // nothing was requested for this head; keep the pipeline going
-      if (ask && wanted(nx)) {
-        load_token<GATE>(p, nx, group, lane, role, nxt);
-        if (role == 0) request_head(nx.bh, nx.n & 0xFFFF);
-        else request_records(nx.bh, nx.n & 0xFFFF);
+    if (!active) {                           // nothing was requested for this head; keep the pipeline going
+      const int n_next = n_next_now();
+      if (wanted(n_next)) {
+        load_token<GATE>(p, hd1, group, lane, role, nxt);
+        if (role == 0) request_head(bh_next, n_next);
+        else request_records(bh_next, n_next);
       }
       if (draws) {                           // the ticket changes hands outside the usual place
         if (role == 1) {
           if (lane == 0) *qidx = ticket;
           __syncwarp();
-          named_arrive(B0 + 1);
+          named_arrive(1);
         } else {
-          named_sync(B0 + 1);
+          named_wait(1);
         }
       }
+      continue;
+    }
+
+    // ---- this head's token (loaded while the previous head was being worked on); once it is unpacked
+    // the registers are free for the next head's, whose load is then issued ----
+    float k8[8], q8[8], a8[8];
+    widen8_bf16(nxt.k, k8);
+    widen8_bf16(nxt.q, q8);
+    const uint2 v_raw = nxt.v;
+    if (DIAG) {
+      widen8_bf16(nxt.a, a8);
     } else {
-      // ---- this head's token (loaded while the previous head was being worked on); once it is unpacked
-      // the registers are free for the next head's, whose load is then issued ----
-      float k8[8], q8[8], a8[8];
-      widen8_bf16(nxt.k, k8);
-      widen8_bf16(nxt.q, q8);
-      const uint2 v_raw = nxt.v;
-      if (DIAG) {
-        widen8_bf16(nxt.a, a8);
-      } else {
 #pragma unroll
-        for (int e = 0; e < 8; e++) a8[e] = alpha_s;
-        bas[lane] = nxt.ba_lo;
-        bas[lane + 32] = nxt.ba_hi;
-      }
-      if (ask) load_token<GATE>(p, nx, group, lane, role, nxt);                // used one trip from now (harmless if that head gets none)
-      // scalar gate: Gamma_{1:l}, the chain of decays from the newest record back (Appendix B.2), needs nothing
-      // from the slot, so the stream warp takes it before it waits
-      float gsc = alpha_s;
-      if (!DIAG) {
-        __syncwarp();
+      for (int e = 0; e < 8; e++) a8[e] = alpha_s;
+      bas[lane] = nxt.ba_lo;
+      bas[lane + 32] = nxt.ba_hi;
+    }
+    if (next_token) load_token<GATE>(p, hd1, group, lane, role, nxt);        // used one trip from now
+    // scalar gate: Gamma_{1:l}, the chain of decays from the newest record back (Appendix B.2), needs nothing
+    // from the slot, so the stream warp takes it before it waits
+    float gsc = alpha_s;
+    if (!DIAG) {
+      __syncwarp();
 #pragma unroll 4
-        for (int j = n - 1; j >= 0; j--) gsc = gsc * bas[j];
+      for (int j = n - 1; j >= 0; j--) gsc = gsc * bas[j];
+    }
+    // kt^T q needs only the token: the dot warp takes it before the wait as well.  It goes to one of two places
+    // in turn, because the stream warp may still be reading the previous head's.
+    if (role == 1) {
+      float2 k2p[4], q2p[4];
+#pragma unroll
+      for (int cc = 0; cc < 4; cc++) {
+        k2p[cc] = __fmul2_rn(pair(beta), make_float2(k8[2 * cc], k8[2 * cc + 1]));
+        q2p[cc] = make_float2(q8[2 * cc], q8[2 * cc + 1]);
       }
-      // kt^T q needs only the token: the dot warp takes it before the wait as well.  It goes to one of two places
-      // in turn, because the stream warp may still be reading the previous head's.
-      if (role == 1) {
-        float2 k2p[4], q2p[4];
+      const float ktq_pre = tree16(block8(k2p, q2p));
+      if (lane == 0) pq[r + (idx & 1)] = ktq_pre;
+    }
+    LQ_TICK(1);
+
+    // ---- the stream warp waits for the head block; the dot warp first takes the records, which it asked for
+    // earlier and which need nothing from the head block, and waits for the block when it gets to the compensators ----
+    if (role == 0 && !DIAG) wait_for(barA, parA);  // (diagonal gate: after its own walk of the records' decays)
+    LQ_TICK(2);
+    if (idx == 0) LQ_STAMP(0, 2);
+
+    if (role == 1) {
+      // =========================== DOT WARP ===========================
+      // Projections.  A dot product of 128 terms is taken by sixteen lanes (lane c owns block c of eight
+      // terms); the two halves of the warp work on different vectors, two per half and trip, so that four
+      // shuffle trees overlap.  Both halves make the same number of trips (the shuffles name all 32 lanes);
+      // an index outside the range recomputes a valid item and is not stored.
+      // Records are walked from the newest back, with g8 = Gamma_{j+1:l} kept up on the way (Appendix B.2).
+      float2 k2[4], q2[4], a2[4], g2[4], kt2[4];
 #pragma unroll
-        for (int cc = 0; cc < 4; cc++) {
-          k2p[cc] = __fmul2_rn(pair(beta), make_float2(k8[2 * cc], k8[2 * cc + 1]));
-          q2p[cc] = make_float2(q8[2 * cc], q8[2 * cc + 1]);
-        }
-        const float ktq_pre = tree16(block8(k2p, q2p));
-        if (lane == 0) pq[r + (trips & 1)] = ktq_pre;
+      for (int cc = 0; cc < 4; cc++) {
+        k2[cc] = make_float2(k8[2 * cc], k8[2 * cc + 1]);
+        q2[cc] = make_float2(q8[2 * cc], q8[2 * cc + 1]);
+        a2[cc] = make_float2(a8[2 * cc], a8[2 * cc + 1]);
+        g2[cc] = a2[cc];
+        kt2[cc] = __fmul2_rn(pair(beta), k2[cc]);
       }
-      LQ_TICK(1);
-
-      // ---- the stream warp waits for the head block; the dot warp first takes the records, which it asked for
-      // earlier and which need nothing from the head block, and waits for the block when it gets to the compensators ----
-      if (role == 0 && !DIAG) wait_for(barA, parA);  // (diagonal gate: after its own walk of the records' decays)
-      LQ_TICK(2);
-      if (trips == 0) LQ_STAMP(0, 2);
-
-      if (role == 1) {
-        // =========================== DOT WARP ===========================
-        // Projections.  A dot product of 128 terms is taken by sixteen lanes (lane c owns block c of eight
-        // terms); the two halves of the warp work on different vectors, two per half and trip, so that four
-        // shuffle trees overlap.  Both halves make the same number of trips (the shuffles name all 32 lanes);
-        // an index outside the range recomputes a valid item and is not stored.
-        // Records are walked from the newest back, with g8 = Gamma_{j+1:l} kept up on the way (Appendix B.2).
-        float2 k2[4], q2[4], a2[4], g2[4], kt2[4];
+      wait_for(barR, parR);                  // the newest segment of the records
+      // Compensator keys against Gamma_{1:l} k and Gamma_{1:l} q (the projections go to pk[h], pq[h]).
+      auto project_compensators = [&](const float2 (&gam)[4]) {
+        float2 gk2[4], gq2[4];
 #pragma unroll
-        for (int cc = 0; cc < 4; cc++) {
-          k2[cc] = make_float2(k8[2 * cc], k8[2 * cc + 1]);
-          q2[cc] = make_float2(q8[2 * cc], q8[2 * cc + 1]);
-          a2[cc] = make_float2(a8[2 * cc], a8[2 * cc + 1]);
-          g2[cc] = a2[cc];
-          kt2[cc] = __fmul2_rn(pair(beta), k2[cc]);
-        }
-        wait_for(barR, parR);                  // the newest segment of the records
-        // Compensator keys against Gamma_{1:l} k and Gamma_{1:l} q (the projections go to pk[h], pq[h]).
-        auto project_compensators = [&](const float2 (&gam)[4]) {
-          float2 gk2[4], gq2[4];
-#pragma unroll
-          for (int cc = 0; cc < 4; cc++) { gk2[cc] = __fmul2_rn(gam[cc], k2[cc]); gq2[cc] = __fmul2_rn(gam[cc], q2[cc]); }
-          for (int hb = 0; hb < r; hb += 4) {
-            float s4[4];
-            int ho[2];
-#pragma unroll
-            for (int u = 0; u < 2; u++) {
-              ho[u] = hb + 2 * u + half;
-              const int h = ho[u] < r ? ho[u] : r - 1;
-              float x8[8];
-              widen8_f16(*reinterpret_cast<const uint4 *>(ckh + h * D + 8 * c), x8);
-              float2 x2[4];
-#pragma unroll
-              for (int cc = 0; cc < 4; cc++) x2[cc] = make_float2(x8[2 * cc], x8[2 * cc + 1]);
-              s4[2 * u] = block8(x2, gk2);
-              s4[2 * u + 1] = block8(x2, gq2);
-            }
-            tree16x4(s4);
-#pragma unroll
-            for (int u = 0; u < 2; u++)
-              if (c == 0 && ho[u] < r) { pk[ho[u]] = s4[2 * u]; pq[ho[u]] = s4[2 * u + 1]; }
-          }
-        };
-        float rk_rec[4] = {0.0f, 0.0f, 0.0f, 0.0f}, rq_rec[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        int base = seg_base(n);                        // the slot holds records base .. (row = record - base)
-        for (int jt = n - 1; jt >= 0; jt -= 4) {       // records jt, jt-1, jt-2, jt-3
-          if (LONGW && jt < base) {                    // the segment is walked: fetch the one before it
-            __syncwarp();
-            if (DIAG) named_sync(B0 + 4);            // (the stream warp has taken this segment's decays as well)
-            request_segment(bh, n, base);
-            base = seg_base(base);
-            wait_for(barR, parR);
-          }
+        for (int cc = 0; cc < 4; cc++) { gk2[cc] = __fmul2_rn(gam[cc], k2[cc]); gq2[cc] = __fmul2_rn(gam[cc], q2[cc]); }
+        for (int hb = 0; hb < r; hb += 4) {
           float s4[4];
-          int jo[2];
+          int ho[2];
 #pragma unroll
           for (int u = 0; u < 2; u++) {
-            // the decays of the two records of this pair; the half that owns the older one steps over the newer
-            const int jn = jt - 2 * u, jold = jn - 1;  // newer, older
-            float2 an[4], ao[4], gmine[4];
-            if (DIAG) {
-              load8p(rec + ((jn > 0 ? jn : 0) - base) * RF + REC_A + 8 * c, an);
-              load8p(rec + ((jold > 0 ? jold : 0) - base) * RF + REC_A + 8 * c, ao);
-            } else {
-              const float2 x = pair(bas[jn > 0 ? jn : 0]), z = pair(bas[jold > 0 ? jold : 0]);
+            ho[u] = hb + 2 * u + half;
+            const int h = ho[u] < r ? ho[u] : r - 1;
+            float x8[8];
+            widen8_f16(*reinterpret_cast<const uint4 *>(ckh + h * D + 8 * c), x8);
+            float2 x2[4];
 #pragma unroll
-              for (int cc = 0; cc < 4; cc++) { an[cc] = x; ao[cc] = z; }
-            }
-#pragma unroll
-            for (int cc = 0; cc < 4; cc++) {
-              const float2 gn = g2[cc], go = __fmul2_rn(gn, an[cc]);   // Gamma_{jn+1:l}, Gamma_{jold+1:l}
-              gmine[cc] = half ? go : gn;
-              // past both records; the chain stops at record 0, so that it ends as Gamma_{1:l} exactly
-              // (selects: a branch for the last trip of a long head was slower)
-              g2[cc] = (!DIAG || jold >= 0) ? __fmul2_rn(go, ao[cc]) : (jn >= 0 ? go : gn);
-            }
-            jo[u] = jn - half;
-            const int j = jo[u] >= 0 ? jo[u] : 0;      // (record 0 is in the slot whenever an index runs below it)
-            float2 x2[4], yk2[4], yq2[4];
-            load8p(rec + (j - base) * RF + REC_KT + 8 * c, x2);
-#pragma unroll
-            for (int cc = 0; cc < 4; cc++) { yk2[cc] = __fmul2_rn(gmine[cc], k2[cc]); yq2[cc] = __fmul2_rn(gmine[cc], q2[cc]); }
-            s4[2 * u] = block8(x2, yk2);
-            s4[2 * u + 1] = block8(x2, yq2);
+            for (int cc = 0; cc < 4; cc++) x2[cc] = make_float2(x8[2 * cc], x8[2 * cc + 1]);
+            s4[2 * u] = block8(x2, gk2);
+            s4[2 * u + 1] = block8(x2, gq2);
           }
           tree16x4(s4);
-          // The record terms sum_j u_j (kt_j^T Gamma k) and the same for q, channels 4 lane .. 4 lane + 3, as one
-          // chain from the newest record back.  Half 0 holds the projections of records jt and jt-2, half 1
-          // those of jt-1 and jt-3: swap them, then take the four records in order.
-          {
-            float oth[4];
 #pragma unroll
-            for (int e = 0; e < 4; e++) oth[e] = __shfl_xor_sync(FULL, s4[e], 16);
-#pragma unroll
-            for (int i4 = 0; i4 < 4; i4++) {
-              const int j = jt - i4;
-              if (j < 0) break;                                  // the same for every lane
-              const int u = i4 >> 1;
-              const bool mine = (i4 & 1) == half;
-              const float pkj = mine ? s4[2 * u] : oth[2 * u], pqj = mine ? s4[2 * u + 1] : oth[2 * u + 1];
-              const float4 u4 = load4(rec + (j - base) * RF + REC_U + 4 * lane);
-              rk_rec[0] = fmaf(u4.x, pkj, rk_rec[0]); rq_rec[0] = fmaf(u4.x, pqj, rq_rec[0]);
-              rk_rec[1] = fmaf(u4.y, pkj, rk_rec[1]); rq_rec[1] = fmaf(u4.y, pqj, rq_rec[1]);
-              rk_rec[2] = fmaf(u4.z, pkj, rk_rec[2]); rq_rec[2] = fmaf(u4.z, pqj, rq_rec[2]);
-              rk_rec[3] = fmaf(u4.w, pkj, rk_rec[3]); rq_rec[3] = fmaf(u4.w, pqj, rq_rec[3]);
-            }
-          }
+          for (int u = 0; u < 2; u++)
+            if (c == 0 && ho[u] < r) { pk[ho[u]] = s4[2 * u]; pq[ho[u]] = s4[2 * u + 1]; }
         }
-        LQ_TICK(3);
-        // Now the head block: the compensators are projected with Gamma_{1:l}, which for the diagonal gate is where
-        // the walk's chain of decays has arrived (g2), for the scalar gate the product taken before the wait.
-        wait_for(barA, parA);
-        if (r > 0) {
+      };
+      float rk_rec[4] = {0.0f, 0.0f, 0.0f, 0.0f}, rq_rec[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      int base = seg_base(n);                        // the slot holds records base .. (row = record - base)
+      for (int jt = n - 1; jt >= 0; jt -= 4) {       // records jt, jt-1, jt-2, jt-3
+        if (LONGW && jt < base) {                    // the segment is walked: fetch the one before it
+          __syncwarp();
+          if (DIAG) named_wait(4);            // (the stream warp has taken this segment's decays as well)
+          request_segment(bh, n, base);
+          base = seg_base(base);
+          wait_for(barR, parR);
+        }
+        float s4[4];
+        int jo[2];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          // the decays of the two records of this pair; the half that owns the older one steps over the newer
+          const int jn = jt - 2 * u, jold = jn - 1;  // newer, older
+          float2 an[4], ao[4], gmine[4];
           if (DIAG) {
-            project_compensators(g2);
+            load8p(rec + ((jn > 0 ? jn : 0) - base) * RF + REC_A + 8 * c, an);
+            load8p(rec + ((jold > 0 ? jold : 0) - base) * RF + REC_A + 8 * c, ao);
           } else {
-            float2 gam[4];
+            const float2 x = pair(bas[jn > 0 ? jn : 0]), z = pair(bas[jold > 0 ? jold : 0]);
 #pragma unroll
-            for (int cc = 0; cc < 4; cc++) gam[cc] = pair(gsc);
-            project_compensators(gam);
+            for (int cc = 0; cc < 4; cc++) { an[cc] = x; ao[cc] = z; }
           }
+#pragma unroll
+          for (int cc = 0; cc < 4; cc++) {
+            const float2 gn = g2[cc], go = __fmul2_rn(gn, an[cc]);   // Gamma_{jn+1:l}, Gamma_{jold+1:l}
+            gmine[cc] = half ? go : gn;
+            // past both records; the chain stops at record 0, so that it ends as Gamma_{1:l} exactly
+            // (selects: a branch for the last trip of a long head was slower)
+            g2[cc] = (!DIAG || jold >= 0) ? __fmul2_rn(go, ao[cc]) : (jn >= 0 ? go : gn);
+          }
+          jo[u] = jn - half;
+          const int j = jo[u] >= 0 ? jo[u] : 0;      // (record 0 is in the slot whenever an index runs below it)
+          float2 x2[4], yk2[4], yq2[4];
+          load8p(rec + (j - base) * RF + REC_KT + 8 * c, x2);
+#pragma unroll
+          for (int cc = 0; cc < 4; cc++) { yk2[cc] = __fmul2_rn(gmine[cc], k2[cc]); yq2[cc] = __fmul2_rn(gmine[cc], q2[cc]); }
+          s4[2 * u] = block8(x2, yk2);
+          s4[2 * u + 1] = block8(x2, yq2);
         }
-        __syncwarp();
-        named_arrive(B0 + 3);                       // the compensator projections are in pk, pq; this warp is done with the head block
-        LQ_TICK(4);
-        if (DIAG) named_sync(B0 + 4);               // diagonal gate: the stream warp read the records' decays too
-        if (ask && wanted(nx)) request_records(nx.bh, nx.n & 0xFFFF);
-        named_sync(B0 + 2);                    // the stream warp has taken its sums out of y
-        int seen = 0;
-        if (last && lane == 0) seen = report_seen(p);           // (this pair has read all it will of win_pos)
-        *reinterpret_cast<float4 *>(y + 4 * lane) = make_float4(rk_rec[0], rk_rec[1], rk_rec[2], rk_rec[3]);
-        *reinterpret_cast<float4 *>(y + D + 4 * lane) = make_float4(rq_rec[0], rq_rec[1], rq_rec[2], rq_rec[3]);
-        if (draws && lane == 0) *qidx = ticket;
-        __syncwarp();
-        named_arrive(B0 + 1);                       // the record terms are in shared memory (and the ticket)
-        LQ_TICK(5);
-        // append the key side of the record (and its decay)
+        tree16x4(s4);
+        // The record terms sum_j u_j (kt_j^T Gamma k) and the same for q, channels 4 lane .. 4 lane + 3, as one
+        // chain from the newest record back.  Half 0 holds the projections of records jt and jt-2, half 1
+        // those of jt-1 and jt-3: swap them, then take the four records in order.
         {
-          rec_t *row = p.record<rec_t>(bh, n, DIAG);
-          if (half == 0) {
-            store8p(row + REC_KT + 8 * c, kt2);
-            if (DIAG) store8(row + REC_A + 8 * c, a8);
-            else if (lane == 0) p.decays[bh * (size_t)W + n] = a8[0];
+          float oth[4];
+#pragma unroll
+          for (int e = 0; e < 4; e++) oth[e] = __shfl_xor_sync(FULL, s4[e], 16);
+#pragma unroll
+          for (int i4 = 0; i4 < 4; i4++) {
+            const int j = jt - i4;
+            if (j < 0) break;                                  // the same for every lane
+            const int u = i4 >> 1;
+            const bool mine = (i4 & 1) == half;
+            const float pkj = mine ? s4[2 * u] : oth[2 * u], pqj = mine ? s4[2 * u + 1] : oth[2 * u + 1];
+            const float4 u4 = load4(rec + (j - base) * RF + REC_U + 4 * lane);
+            rk_rec[0] = fmaf(u4.x, pkj, rk_rec[0]); rq_rec[0] = fmaf(u4.x, pqj, rq_rec[0]);
+            rk_rec[1] = fmaf(u4.y, pkj, rk_rec[1]); rq_rec[1] = fmaf(u4.y, pqj, rq_rec[1]);
+            rk_rec[2] = fmaf(u4.z, pkj, rk_rec[2]); rq_rec[2] = fmaf(u4.z, pqj, rq_rec[2]);
+            rk_rec[3] = fmaf(u4.w, pkj, rk_rec[3]); rq_rec[3] = fmaf(u4.w, pqj, rq_rec[3]);
           }
         }
-        if (BOUNDARY && cur.due) {             // the boundary reads the newest record here (the digits are done with)
-          rec_t *row = reinterpret_cast<rec_t *>(digits);
-          if (half == 0) store8p(row + REC_KT + 8 * c, kt2);
-          if (!DIAG && lane == 0) bas[n] = a8[0];
-        }
-        if (last) finish_step(seen);
-        LQ_TICK(7);
-      } else {
-        // =========================== STREAM WARP ===========================
-        // Gamma_{1:l}: the chain of decays from the newest record back (Appendix B.2)
-        float gam[8];
-#pragma unroll
-        for (int e = 0; e < 8; e++) gam[e] = a8[e];
+      }
+      LQ_TICK(3);
+      // Now the head block: the compensators are projected with Gamma_{1:l}, which for the diagonal gate is where
+      // the walk's chain of decays has arrived (g2), for the scalar gate the product taken before the wait.
+      wait_for(barA, parA);
+      if (r > 0) {
         if (DIAG) {
-          for (int hi = n;;) {                        // segment after segment, in step with the dot warp
-            const int lo = seg_base(hi);
-            wait_for(barR, parR);
-#pragma unroll 2
-            for (int j = hi - 1; j >= lo; j--) {
-              float aj[8];
-              load8(rec + (j - lo) * RF + REC_A + 8 * c, aj);
-#pragma unroll
-              for (int e = 0; e < 8; e++) gam[e] = gam[e] * aj[e];
-            }
-            __syncwarp();
-            named_arrive(B0 + 4);                   // this warp is done with the segment
-            if (lo == 0) break;
-            hi = lo;
-          }
-          wait_for(barA, parA);
+          project_compensators(g2);
         } else {
+          float2 gam[4];
 #pragma unroll
-          for (int e = 0; e < 8; e++) gam[e] = gsc;
+          for (int cc = 0; cc < 4; cc++) gam[cc] = pair(gsc);
+          project_compensators(gam);
         }
-        LQ_TICK(3);
-        // C Gamma k (lanes 0..15) and C Gamma q (lanes 16..31) on their fixed-point grids, as digit planes
-        float back_own;
-        {
-          float c8[8], x8[8];
-          load8(cs + 8 * c, c8);
-          float m = 0.0f;
-#pragma unroll
-          for (int e = 0; e < 8; e++) {
-            x8[e] = c8[e] * (gam[e] * (half ? q8[e] : k8[e]));
-            m = fmaxf(m, fabsf(x8[e]));
-          }
-#pragma unroll
-          for (int s = 1; s <= 8; s <<= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, s));
-          float scale;
-          fixed_point_scales(m, scale, back_own);
-          // X = d0 + 256 d1 + 65536 d2 + 2^24 d3 with digits in [-128, 127]: the digit is the low byte read as
-          // signed, and taking it off is (X + 128) >> 8.  The bytes of the four stages of an element are the
-          // four digits; prmt gathers the same digit of four elements into one word.
-          uint32_t st[8][4];
-#pragma unroll
-          for (int e = 0; e < 8; e++) {
-            int X = __float2int_rn(x8[e] * scale);
-#pragma unroll
-            for (int d = 0; d < 4; d++) { st[e][d] = static_cast<uint32_t>(X); X = (X + 128) >> 8; }
-          }
-#pragma unroll
-          for (int d = 0; d < 4; d++) {
-            const uint32_t lo = __byte_perm(__byte_perm(st[0][d], st[1][d], 0x0040), __byte_perm(st[2][d], st[3][d], 0x0040), 0x5410);
-            const uint32_t hi = __byte_perm(__byte_perm(st[4][d], st[5][d], 0x0040), __byte_perm(st[6][d], st[7][d], 0x0040), 0x5410);
-            *reinterpret_cast<uint2 *>(digits + (4 * half + d) * D + 8 * c) = make_uint2(lo, hi);
-          }
-        }
-        const float back_other = __shfl_xor_sync(FULL, back_own, 16);
-        const float back_k = half ? back_other : back_own, back_q = half ? back_own : back_other;
-        __syncwarp();                          // the digit planes are visible to the warp
-        LQ_TICK(4);
-
-        // The state stream on the tensor cores: eight 16-row tiles of Z^T, K = 128 as four k-blocks.  A
-        // thread's 16 bytes of a row hold key channels 64p+16t..64p+16t+15 and serve two k-blocks; the digit
-        // planes are read with the same permutation of the key index.  The two 64-channel halves of a tile
-        // accumulate separately (exact integers: any split gives the same sum), which halves the dependent
-        // chain of MMAs.  Digit pairs are recombined in int32 (|sum| < 2^30), the two pairs in int64 (the total has
-        // 47 bits), and one rounding takes it to fp32.
-        {
-          constexpr int h0 = 0, h1 = 64;         // the two 64-channel halves (the same split for every lane)
-          const uint4 bfa = *reinterpret_cast<const uint4 *>(digits + g * D + h0 + 16 * t);
-          const uint4 bfb = *reinterpret_cast<const uint4 *>(digits + g * D + h1 + 16 * t);
-          int pair_lo[8], pair_hi[8];            // digit-pair sums of rows g and g+8 of each tile
-#pragma unroll
-          for (int mt = 0; mt < 8; mt++) {
-            int ca[4] = {0, 0, 0, 0}, cb[4] = {0, 0, 0, 0};
-            const int j = 16 * mt + g;
-            const uint4 alo = *reinterpret_cast<const uint4 *>(zt + j * D + h0 + 16 * t);
-            const uint4 ahi = *reinterpret_cast<const uint4 *>(zt + (j + 8) * D + h0 + 16 * t);
-            const uint4 blo = *reinterpret_cast<const uint4 *>(zt + j * D + h1 + 16 * t);
-            const uint4 bhi = *reinterpret_cast<const uint4 *>(zt + (j + 8) * D + h1 + 16 * t);
-            mma_s8(ca, alo.x, ahi.x, alo.y, ahi.y, bfa.x, bfa.y);
-            mma_s8(cb, blo.x, bhi.x, blo.y, bhi.y, bfb.x, bfb.y);
-            mma_s8(ca, alo.z, ahi.z, alo.w, ahi.w, bfa.z, bfa.w);
-            mma_s8(cb, blo.z, bhi.z, blo.w, bhi.w, bfb.z, bfb.w);
-            // c[0], c[1]: row g, planes 2t, 2t+1;  c[2], c[3]: row g+8.  Planes 4v..4v+3 are the digits of
-            // vector v: lanes t = 0, 1 carry the k sums and t = 2, 3 the q sums, even t the low digit pair.
-            pair_lo[mt] = (ca[0] + cb[0]) + ((ca[1] + cb[1]) << 8);
-            pair_hi[mt] = (ca[2] + cb[2]) + ((ca[3] + cb[3]) << 8);
-          }
-          LQ_TICK(10);
-          int oth_lo[8], oth_hi[8];
-#pragma unroll
-          for (int mt = 0; mt < 8; mt++) {
-            oth_lo[mt] = __shfl_xor_sync(FULL, pair_lo[mt], 1);
-            oth_hi[mt] = __shfl_xor_sync(FULL, pair_hi[mt], 1);
-          }
-          if (!(t & 1)) {                      // this lane has the low pairs, its neighbour sent the high pairs
-            float *dst = y + (t >> 1) * D + g;
-#pragma unroll
-            for (int mt = 0; mt < 8; mt++) {
-              dst[16 * mt] = __ll2float_rn(static_cast<long long>(oth_lo[mt]) * 65536 + pair_lo[mt]);
-              dst[16 * mt + 8] = __ll2float_rn(static_cast<long long>(oth_hi[mt]) * 65536 + pair_hi[mt]);
-            }
-          }
-        }
-        __syncwarp();
-        LQ_TICK(5);
-
-        // Per value channel (lane l: channels 4l..4l+3): scale the sums, then add the compensator and record
-        // terms with the projections of the dot warp
-        {
-          const float4 yk4 = *reinterpret_cast<const float4 *>(y + 4 * lane);
-          const float4 yq4 = *reinterpret_cast<const float4 *>(y + D + 4 * lane);
-          const float4 s4 = *reinterpret_cast<const float4 *>(bs + 4 * lane);      // code steps B_j / 127
-          float rk[4] = {s4.x * (yk4.x * back_k), s4.y * (yk4.y * back_k), s4.z * (yk4.z * back_k), s4.w * (yk4.w * back_k)};
-          float rq[4] = {s4.x * (yq4.x * back_q), s4.y * (yq4.y * back_q), s4.z * (yq4.z * back_q), s4.w * (yq4.w * back_q)};
-          const float v4[4] = {__uint_as_float(v_raw.x << 16), __uint_as_float(v_raw.x & 0xFFFF0000u),
-                               __uint_as_float(v_raw.y << 16), __uint_as_float(v_raw.y & 0xFFFF0000u)};
-          LQ_TICK(6);
-          named_arrive(B0 + 2);                     // y has been read: the dot warp may put the record terms there
-          named_sync(B0 + 3);                       // the compensator projections are complete
-          LQ_TICK(7);
-#pragma unroll 2
-          for (int h = 0; h < r; h++) {
-            const uint2 w = *reinterpret_cast<const uint2 *>(cuh + h * D + 4 * lane);
-            const float2 f01 = __half22float2(*reinterpret_cast<const __half2 *>(&w.x));
-            const float2 f23 = __half22float2(*reinterpret_cast<const __half2 *>(&w.y));
-            const float uc[4] = {f01.x, f01.y, f23.x, f23.y};
-            const float pkh = pk[h], pqh = pq[h];
-#pragma unroll
-            for (int e = 0; e < 4; e++) { rk[e] = fmaf(uc[e], pkh, rk[e]); rq[e] = fmaf(uc[e], pqh, rq[e]); }
-          }
-          __syncwarp();                        // nobody reads the head block any more (the dot warp finished with
-          if (ask && wanted(nx)) request_head(nx.bh, nx.n & 0xFFFF);    // it before barrier 3): the next head's may land
-          named_sync(B0 + 1);                       // the record terms are complete
-          {
-            const float4 tk = *reinterpret_cast<const float4 *>(y + 4 * lane);
-            const float4 tq = *reinterpret_cast<const float4 *>(y + D + 4 * lane);
-            rk[0] = rk[0] + tk.x; rk[1] = rk[1] + tk.y; rk[2] = rk[2] + tk.z; rk[3] = rk[3] + tk.w;
-            rq[0] = rq[0] + tq.x; rq[1] = rq[1] + tq.y; rq[2] = rq[2] + tq.z; rq[3] = rq[3] + tq.w;
-          }
-          const float ktq = pq[r + (trips & 1)];
-          float u[4], o[4];
-#pragma unroll
-          for (int e = 0; e < 4; e++) { u[e] = p.delta ? v4[e] - rk[e] : v4[e]; o[e] = fmaf(u[e], ktq, rq[e]); }
-          LQ_TICK(8);
-          *reinterpret_cast<float4 *>(p.o + bh * D + 4 * lane) = make_float4(o[0], o[1], o[2], o[3]);
-          store4(p.record<rec_t>(bh, n, DIAG) + REC_U + 4 * lane, u[0], u[1], u[2], u[3]);
-          if (BOUNDARY && cur.due) {           // (as above; the diagonal gate's decays reach into y, which all lanes have read)
-            rec_t *row = reinterpret_cast<rec_t *>(digits);
-            __syncwarp();
-            store4(row + REC_U + 4 * lane, u[0], u[1], u[2], u[3]);
-            if (DIAG && half == 0) {
-              float al[8];
-              widen8_bf16(nxt.a, al);          // (no other token has been loaded over a due head's)
-              store8(row + REC_A + 8 * c, al);
-            }
-          }
-        }
-        LQ_TICK(9);
       }
-      reported = reported || last;
-    }
-
-    // ---- the trip is over: on to the next head, and the one after it ----
-    const bool was_due = BOUNDARY && have_cur && cur.due;
-    PairHead after{};
-    bool have_after = false;
-    if (!turn_over) {
-      have_after = take(after);
-    } else if (draws) {
-      const unsigned tk = role == 1 ? __shfl_sync(FULL, ticket, 0) : *reinterpret_cast<volatile unsigned *>(qidx);
-      if (tk < pool) {
-        have_after = true;
-        after.bh = static_cast<unsigned>(S) * P + tk;
-        after.b = after.bh / Hv;
-        after.n = p.win_pos[after.b];        // (looked at half a trip from here)
-        after.ba = p.beta[after.bh];
-        if (!DIAG) after.ba |= static_cast<uint32_t>(p.alpha[after.bh]) << 16;
-        after.due = false;
-      } else {
-        drawing = false;
+      __syncwarp();
+      named_arrive(3);                       // the compensator projections are in pk, pq; this warp is done with the head block
+      LQ_TICK(4);
+      if (DIAG) named_wait(4);               // diagonal gate: the stream warp read the records' decays too
+      {
+        const int n_next = n_next_now();
+        if (wanted(n_next)) request_records(bh_next, n_next);
       }
-    }
-    cur = nx; have_cur = have_nx;
-    nx = after; have_nx = have_after;
-    trips++;
-    if (was_due) {
-      perform_boundaries(done);
-      done += hold;
-      if (have_cur && wanted(cur)) start();
-    }
-  }
-  if (!reported) {                           // the last trips had no head: the pair reports when both warps are here
-    if (role == 0) {
-      named_arrive(B0 + 2);
+      named_wait(2);                         // the stream warp has taken its sums out of y
+      *reinterpret_cast<float4 *>(y + 4 * lane) = make_float4(rk_rec[0], rk_rec[1], rk_rec[2], rk_rec[3]);
+      *reinterpret_cast<float4 *>(y + D + 4 * lane) = make_float4(rq_rec[0], rq_rec[1], rq_rec[2], rq_rec[3]);
+      if (draws && lane == 0) *qidx = ticket;
+      __syncwarp();
+      named_arrive(1);                       // the record terms are in shared memory (and the ticket)
+      LQ_TICK(5);
+      // append the key side of the record (and its decay)
+      {
+        rec_t *row = p.record<rec_t>(bh, n, DIAG);
+        if (half == 0) {
+          store8p(row + REC_KT + 8 * c, kt2);
+          if (DIAG) store8(row + REC_A + 8 * c, a8);
+          else if (lane == 0) p.decays[bh * (size_t)W + n] = a8[0];
+        }
+      }
+      if (lane == 0) arrive_and_set(p.win_pos, b, p.heads_v, n + 1);
+      LQ_TICK(7);
     } else {
-      named_sync(B0 + 2);
-      finish_step(lane == 0 ? report_seen(p) : 0);
+      // =========================== STREAM WARP ===========================
+      // Gamma_{1:l}: the chain of decays from the newest record back (Appendix B.2)
+      float gam[8];
+#pragma unroll
+      for (int e = 0; e < 8; e++) gam[e] = a8[e];
+      if (DIAG) {
+        for (int hi = n;;) {                        // segment after segment, in step with the dot warp
+          const int lo = seg_base(hi);
+          wait_for(barR, parR);
+#pragma unroll 2
+          for (int j = hi - 1; j >= lo; j--) {
+            float aj[8];
+            load8(rec + (j - lo) * RF + REC_A + 8 * c, aj);
+#pragma unroll
+            for (int e = 0; e < 8; e++) gam[e] = gam[e] * aj[e];
+          }
+          __syncwarp();
+          named_arrive(4);                   // this warp is done with the segment
+          if (lo == 0) break;
+          hi = lo;
+        }
+        wait_for(barA, parA);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; e++) gam[e] = gsc;
+      }
+      LQ_TICK(3);
+      // C Gamma k (lanes 0..15) and C Gamma q (lanes 16..31) on their fixed-point grids, as digit planes
+      float back_own;
+      {
+        float c8[8], x8[8];
+        load8(cs + 8 * c, c8);
+        float m = 0.0f;
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+          x8[e] = c8[e] * (gam[e] * (half ? q8[e] : k8[e]));
+          m = fmaxf(m, fabsf(x8[e]));
+        }
+#pragma unroll
+        for (int s = 1; s <= 8; s <<= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, s));
+        float scale;
+        fixed_point_scales(m, scale, back_own);
+        // X = d0 + 256 d1 + 65536 d2 + 2^24 d3 with digits in [-128, 127]: the digit is the low byte read as
+        // signed, and taking it off is (X + 128) >> 8.  The bytes of the four stages of an element are the
+        // four digits; prmt gathers the same digit of four elements into one word.
+        uint32_t st[8][4];
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+          int X = __float2int_rn(x8[e] * scale);
+#pragma unroll
+          for (int d = 0; d < 4; d++) { st[e][d] = static_cast<uint32_t>(X); X = (X + 128) >> 8; }
+        }
+#pragma unroll
+        for (int d = 0; d < 4; d++) {
+          const uint32_t lo = __byte_perm(__byte_perm(st[0][d], st[1][d], 0x0040), __byte_perm(st[2][d], st[3][d], 0x0040), 0x5410);
+          const uint32_t hi = __byte_perm(__byte_perm(st[4][d], st[5][d], 0x0040), __byte_perm(st[6][d], st[7][d], 0x0040), 0x5410);
+          *reinterpret_cast<uint2 *>(digits + (4 * half + d) * D + 8 * c) = make_uint2(lo, hi);
+        }
+      }
+      const float back_other = __shfl_xor_sync(FULL, back_own, 16);
+      const float back_k = half ? back_other : back_own, back_q = half ? back_own : back_other;
+      __syncwarp();                          // the digit planes are visible to the warp
+      LQ_TICK(4);
+
+      // The state stream on the tensor cores: eight 16-row tiles of Z^T, K = 128 as four k-blocks.  A
+      // thread's 16 bytes of a row hold key channels 64p+16t..64p+16t+15 and serve two k-blocks; the digit
+      // planes are read with the same permutation of the key index.  The two 64-channel halves of a tile
+      // accumulate separately (exact integers: any split gives the same sum), which halves the dependent
+      // chain of MMAs.  Digit pairs are recombined in int32 (|sum| < 2^30), the two pairs in int64 (the total has
+      // 47 bits), and one rounding takes it to fp32.
+      {
+        constexpr int h0 = 0, h1 = 64;         // the two 64-channel halves (the same split for every lane)
+        const uint4 bfa = *reinterpret_cast<const uint4 *>(digits + g * D + h0 + 16 * t);
+        const uint4 bfb = *reinterpret_cast<const uint4 *>(digits + g * D + h1 + 16 * t);
+        int pair_lo[8], pair_hi[8];            // digit-pair sums of rows g and g+8 of each tile
+#pragma unroll
+        for (int mt = 0; mt < 8; mt++) {
+          int ca[4] = {0, 0, 0, 0}, cb[4] = {0, 0, 0, 0};
+          const int j = 16 * mt + g;
+          const uint4 alo = *reinterpret_cast<const uint4 *>(zt + j * D + h0 + 16 * t);
+          const uint4 ahi = *reinterpret_cast<const uint4 *>(zt + (j + 8) * D + h0 + 16 * t);
+          const uint4 blo = *reinterpret_cast<const uint4 *>(zt + j * D + h1 + 16 * t);
+          const uint4 bhi = *reinterpret_cast<const uint4 *>(zt + (j + 8) * D + h1 + 16 * t);
+          mma_s8(ca, alo.x, ahi.x, alo.y, ahi.y, bfa.x, bfa.y);
+          mma_s8(cb, blo.x, bhi.x, blo.y, bhi.y, bfb.x, bfb.y);
+          mma_s8(ca, alo.z, ahi.z, alo.w, ahi.w, bfa.z, bfa.w);
+          mma_s8(cb, blo.z, bhi.z, blo.w, bhi.w, bfb.z, bfb.w);
+          // c[0], c[1]: row g, planes 2t, 2t+1;  c[2], c[3]: row g+8.  Planes 4v..4v+3 are the digits of
+          // vector v: lanes t = 0, 1 carry the k sums and t = 2, 3 the q sums, even t the low digit pair.
+          pair_lo[mt] = (ca[0] + cb[0]) + ((ca[1] + cb[1]) << 8);
+          pair_hi[mt] = (ca[2] + cb[2]) + ((ca[3] + cb[3]) << 8);
+        }
+        LQ_TICK(10);
+        int oth_lo[8], oth_hi[8];
+#pragma unroll
+        for (int mt = 0; mt < 8; mt++) {
+          oth_lo[mt] = __shfl_xor_sync(FULL, pair_lo[mt], 1);
+          oth_hi[mt] = __shfl_xor_sync(FULL, pair_hi[mt], 1);
+        }
+        if (!(t & 1)) {                      // this lane has the low pairs, its neighbour sent the high pairs
+          float *dst = y + (t >> 1) * D + g;
+#pragma unroll
+          for (int mt = 0; mt < 8; mt++) {
+            dst[16 * mt] = __ll2float_rn(static_cast<long long>(oth_lo[mt]) * 65536 + pair_lo[mt]);
+            dst[16 * mt + 8] = __ll2float_rn(static_cast<long long>(oth_hi[mt]) * 65536 + pair_hi[mt]);
+          }
+        }
+      }
+      __syncwarp();
+      LQ_TICK(5);
+
+      // Per value channel (lane l: channels 4l..4l+3): scale the sums, then add the compensator and record
+      // terms with the projections of the dot warp
+      {
+        const float4 yk4 = *reinterpret_cast<const float4 *>(y + 4 * lane);
+        const float4 yq4 = *reinterpret_cast<const float4 *>(y + D + 4 * lane);
+        const float4 s4 = *reinterpret_cast<const float4 *>(bs + 4 * lane);      // code steps B_j / 127
+        float rk[4] = {s4.x * (yk4.x * back_k), s4.y * (yk4.y * back_k), s4.z * (yk4.z * back_k), s4.w * (yk4.w * back_k)};
+        float rq[4] = {s4.x * (yq4.x * back_q), s4.y * (yq4.y * back_q), s4.z * (yq4.z * back_q), s4.w * (yq4.w * back_q)};
+        const float v4[4] = {__uint_as_float(v_raw.x << 16), __uint_as_float(v_raw.x & 0xFFFF0000u),
+                             __uint_as_float(v_raw.y << 16), __uint_as_float(v_raw.y & 0xFFFF0000u)};
+        LQ_TICK(6);
+        named_arrive(2);                     // y has been read: the dot warp may put the record terms there
+        named_wait(3);                       // the compensator projections are complete
+        LQ_TICK(7);
+#pragma unroll 2
+        for (int h = 0; h < r; h++) {
+          const uint2 w = *reinterpret_cast<const uint2 *>(cuh + h * D + 4 * lane);
+          const float2 f01 = __half22float2(*reinterpret_cast<const __half2 *>(&w.x));
+          const float2 f23 = __half22float2(*reinterpret_cast<const __half2 *>(&w.y));
+          const float uc[4] = {f01.x, f01.y, f23.x, f23.y};
+          const float pkh = pk[h], pqh = pq[h];
+#pragma unroll
+          for (int e = 0; e < 4; e++) { rk[e] = fmaf(uc[e], pkh, rk[e]); rq[e] = fmaf(uc[e], pqh, rq[e]); }
+        }
+        __syncwarp();                        // nobody reads the head block any more (the dot warp finished with
+        {
+          const int n_next = n_next_now();
+          if (wanted(n_next)) request_head(bh_next, n_next);   // it before barrier 3): the next head's may land
+        }
+        named_wait(1);                       // the record terms are complete
+        {
+          const float4 tk = *reinterpret_cast<const float4 *>(y + 4 * lane);
+          const float4 tq = *reinterpret_cast<const float4 *>(y + D + 4 * lane);
+          rk[0] = rk[0] + tk.x; rk[1] = rk[1] + tk.y; rk[2] = rk[2] + tk.z; rk[3] = rk[3] + tk.w;
+          rq[0] = rq[0] + tq.x; rq[1] = rq[1] + tq.y; rq[2] = rq[2] + tq.z; rq[3] = rq[3] + tq.w;
+        }
+        const float ktq = pq[r + (idx & 1)];
+        float u[4], o[4];
+#pragma unroll
+        for (int e = 0; e < 4; e++) { u[e] = p.delta ? v4[e] - rk[e] : v4[e]; o[e] = fmaf(u[e], ktq, rq[e]); }
+        LQ_TICK(8);
+        *reinterpret_cast<float4 *>(p.o + bh * D + 4 * lane) = make_float4(o[0], o[1], o[2], o[3]);
+        store4(p.record<rec_t>(bh, n, DIAG) + REC_U + 4 * lane, u[0], u[1], u[2], u[3]);
+      }
+      LQ_TICK(9);
     }
   }
 #ifdef LQ_TIMING
@@ -891,25 +701,26 @@ __device__ __forceinline__ void decode_pair(const Params &p, unsigned char *smem
 #endif
 }
 
-// Persistent kernel: CTAs of one pair of warps (RM < 0), or of eight warps that also perform the boundaries.
-template <int GATE, bool R16, bool LONGW, int RM>
-__global__ void __launch_bounds__(RM >= 0 ? 256 : 64, RM >= 0 ? 2 : 6) decode_kernel(const __grid_constant__ Params p, const StepPlan plan) {
-  extern __shared__ __align__(128) unsigned char lq_smem[];
+// Persistent kernel of two-warp CTAs: CTA `blockIdx.x` takes heads blockIdx.x, blockIdx.x + gridDim.x, ...
+template <int GATE, bool R16, bool LONGW>
+__global__ void __launch_bounds__(64, 6) decode_kernel(const Params p) {
+  extern __shared__ __align__(128) unsigned char lq_slot[];
   LQ_STAMP(0, 0);
-  // Resident while the kernel ahead drains: the pair asks the L2 for its first head block meanwhile (a prefetch returns
+  // Resident while the kernel ahead drains: the CTA asks the L2 for its first head block meanwhile (a prefetch returns
   // no data, so it does not matter that the kernel ahead may still be writing that block: the L2 is where its writes
-  // go).  The first head of a pair is the only one whose copy nothing hides.
-  if ((threadIdx.x & 63) == 0 && static_cast<int>(threadIdx.x >> 6) < plan.pairs) {
-    const unsigned pr = threadIdx.x >> 6, first = pr * gridDim.x + blockIdx.x;
-    if (first < static_cast<unsigned>(p.batch) * p.heads_v) bulk_prefetch_l2(p.head(first), head_bytes(p.r));
-    const uint32_t bar = smem_addr(lq_smem) + 16 * pr;
+  // go).  The first head of a CTA is the only one whose copy nothing hides.
+  if (threadIdx.x == 0 && blockIdx.x < static_cast<unsigned>(p.batch) * p.heads_v)
+    bulk_prefetch_l2(p.head(blockIdx.x), head_bytes(p.r));
+  const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {                    // the slot's two copy barriers (shared memory only)
+    const uint32_t bar = smem_addr(lq_slot + DecodeSlot(p.W, p.r, GATE == LQ_GATE_DIAG, R16).mbar);
     mbar_init(bar, 1);
     mbar_init(bar + 8, 1);
   }
   __syncthreads();
   grid_dependency_wait();                    // no data in global memory is read or written above this line
   LQ_STAMP(0, 1);
-  decode_pair<GATE, R16, LONGW, RM>(p, lq_smem, plan);
+  decode_slot<GATE, R16, LONGW>(p, lq_slot, lane, role, blockIdx.x, gridDim.x);
   LQ_STAMP(0, 3);
 #ifdef LQ_TIMING
   if (threadIdx.x == 0 && blockIdx.x < 1024) {
