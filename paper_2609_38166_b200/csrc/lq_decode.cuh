@@ -107,8 +107,10 @@ __device__ __forceinline__ void tree16x4(float (&x)[4]) {
 }
 
 // Named barriers of the CTA (64 threads each): one side arrives, the other waits.
-//   1: dot warp -> stream warp, "the projections are in shared memory"
-//   2: stream warp -> dot warp, "the slot may be overwritten"
+//   1: dot warp -> stream warp, "the record terms (and the ticket) are in shared memory"
+//   2: stream warp -> dot warp, "its sums are out of y"
+//   3: dot warp -> stream warp, "the compensator projections are in shared memory"
+//   4: stream warp -> dot warp, "the records' decays have been read" (diagonal gate)
 __device__ __forceinline__ void named_arrive(int id) {
   __threadfence_block();
   asm volatile("bar.arrive %0, 64;\n" ::"r"(id) : "memory");
@@ -333,12 +335,17 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         if (role == 0) request_head(bh_next, n_next);
         else request_records(bh_next, n_next);
       }
-      if (draws) {                           // the ticket changes hands outside the usual place
+      // The ticket changes hands outside the usual place.  As in a trip with a token, barrier 2 (the stream warp is through
+      // with the trip before) comes ahead of barrier 1: without it the dot warp could arrive at barrier 1 in two such trips
+      // before the stream warp came there once, which would complete the barrier without it and leave it waiting for good.
+      if (draws) {
         if (role == 1) {
+          named_wait(2);
           if (lane == 0) *qidx = ticket;
           __syncwarp();
           named_arrive(1);
         } else {
+          named_arrive(2);
           named_wait(1);
         }
       }

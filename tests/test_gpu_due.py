@@ -61,3 +61,43 @@ def test_dense_states_at_any_16_byte_boundary(oracle, shift):
     lq.dequantize_state(lsh, st, S)
     assert np.array_equal(gu.host(S), oracle.dequantize_state(osh, ost))
     assert not room[:shift].any() and not room[shift + S0.size:].any()
+
+
+@pytest.mark.parametrize("gate", [synth.GATE_SCALAR, synth.GATE_DIAG])
+def test_many_windows_that_come_in_full_among_drawn_heads(oracle, gate):
+    """More than three heads per resident CTA, most of them of sequences that enter with a full window and get no token: the
+    CTAs draw many such heads in a row.  Their outputs stay, the boundary takes all of them, the others step as usual."""
+    wl = synth.Workload("fullw", 90, 32, 16, W=4, r=2, gate=gate, seed=840)
+    osh, lsh = gu.shapes(wl)
+    ost = OState(osh)
+    oracle.quantize_state(osh, synth.dense_states(wl, 3), ost)
+    rng = np.random.default_rng(3)
+    pos = np.where(rng.random(wl.batch) < 0.8, wl.W, rng.integers(0, wl.W, wl.batch)).astype(np.int32)
+    pos[:4] = 1
+    ost.win_pos[:] = pos
+    ost.buf_k[...] = rng.standard_normal(ost.buf_k.shape).astype(np.float32) * 0.1
+    ost.buf_u[...] = rng.standard_normal(ost.buf_u.shape).astype(np.float32)
+    ost.buf_a[...] = rng.uniform(0.2, 1.0, ost.buf_a.shape).astype(np.float32)
+    st = gu.state_to_dev(ost, lsh)
+    o = torch.full((wl.batch, wl.heads_v, 128), 7.0, dtype=torch.float32, device="cuda")
+    tok = synth.token_inputs(wl, 0)
+    td = gu.tok_dev(tok)
+    lq.decode_step(lsh, st, td["q"], td["k"], td["v"], td["beta"], td["alpha"], o)
+    torch.cuda.synchronize()
+    assert lq.check_device() == 0 and not st.work.any()
+    full = torch.from_numpy(pos == wl.W)
+    assert torch.all(o.cpu()[full] == 7.0) and not torch.any(o.cpu()[~full] == 7.0)
+    assert st.win_pos.tolist() == [0 if p >= wl.W - 1 else int(p) + 1 for p in pos]
+    few = np.concatenate([np.flatnonzero(pos == wl.W)[:3], np.arange(3)])      # a few sequences of either kind, by the oracle
+    sub = wl.with_(batch=1)
+    osub, _ = gu.shapes(sub)
+    for b in few:
+        one = OState(osub)
+        for name in ("codes", "col_scale", "row_smooth", "comp_k", "comp_u", "buf_k", "buf_u", "buf_a", "win_pos"):
+            getattr(one, name)[...] = getattr(ost, name)[b:b + 1]
+        if pos[b] == wl.W:
+            oracle.window_flush(osub, one, force=False)
+        else:
+            want = oracle.decode_step(osub, one, **{k: np.ascontiguousarray(v[b:b + 1]) for k, v in tok.items()})
+            assert np.array_equal(gu.host(o)[b:b + 1], want)
+        assert np.array_equal(gu.gpu_codes(st)[b:b + 1], one.codes) and np.array_equal(gu.host(st.col_scale)[b:b + 1], one.col_scale)
