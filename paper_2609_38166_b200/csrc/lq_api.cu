@@ -400,6 +400,7 @@ static lq_status decode_step_impl(const lq_shape *shape, const lq_state *state, 
   p.q = q; p.k = k; p.v = v; p.beta = beta; p.alpha = alpha; p.o = o;
   const bool diag = shape->gate == LQ_GATE_DIAG;
   const long nh = (long)shape->batch * shape->heads_v;
+  p.overlap = nh >= 2L * sm_count() * shape->W;        // as many boundaries as boundary CTAs, on average
   // persistent two-warp CTAs, each with its own shared-memory slot: as many as are resident at once
   const bool r16 = shape->rec16 != 0;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);

@@ -352,6 +352,7 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
 
     for (int k = 0; k < count; k++) {
       const size_t bh = todo_bh[k];
+      if (MODE == 0 && p.overlap && count < 32 && k == count - 1) grid_dependents_may_start();
       const int n = todo_n[k];
       if (SLOT) {
         if (!DIAG && tid < n) dec[tid] = dec_next;

@@ -36,6 +36,7 @@ constexpr int REC_KT = 0, REC_U = D, REC_A = 2 * D;
 // Launch-time description of one call, passed to the kernels by value.
 struct Params {
   int batch, heads_v, heads_qk, W, r, n_iter, smooth, delta, rec16, force;
+  int overlap;       // let the next kernel of the stream start when every CTA is at its last head (else when all have ended)
   uint8_t *heads;    // [B*Hv] head blocks of head_bytes(r)
   void *records;     // [B*Hv][W] record rows of record_floats(gate) elements, fp32 or (rec16) fp16
   float *decays;     // scalar gate: [B*Hv][W]
@@ -190,11 +191,14 @@ __device__ __forceinline__ float dot128_shared(const float *a, const float *b, i
 
 // Programmatic dependent launch: a kernel launched with the stream-serialization attribute may become resident
 // before the kernel ahead of it has finished; this is where it waits for that kernel's completion and writes
-// (a no-op for an ordinary launch).  Right after it the kernel allows its own dependents to be scheduled.
-__device__ __forceinline__ void grid_dependency_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// (a no-op for an ordinary launch).
+// When the dependents may start: allowed at the very beginning, their CTAs come up one by one wherever room appears, so that
+// the few with work to do share an SM and the decode CTAs fill the gaps that boundary CTAs of another size leave.  With little
+// work (fewer boundaries than boundary CTAs, Params.overlap == 0) they start when the kernel ahead has ended, evenly over the
+// SMs: step at 32 x 32 heads 24.5 -> 19.0 us, 77 x 12 heads (W = 13) 22.0 -> 17.6 us.  With more, when every CTA has come to
+// its last head, which hides their start: 256 x 32 heads 64.7 us at the beginning or the end, 63.9 us at the last head.
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Phase timing (development aid, compiled in with -DLQ_TIMING only): clock cycles per phase of the decode
 // warps, summed over all heads by lane 0 of each warp (slots 0..15: stream warp, 16..31: dot warp; 32..: thread 0 of the boundary kernel's CTAs).

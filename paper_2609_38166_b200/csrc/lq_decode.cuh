@@ -309,6 +309,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
   };
   for (; hd.bh < nh; finish_trip()) {
     const bool draws = drawing && idx + 2 >= S;                 // a ticket is drawn in this trip
+    if (p.overlap && role == 1 && !draws && hd1.bh >= nh) grid_dependents_may_start();
     if (draws && role == 1 && lane == 0) ticket = static_cast<unsigned>(atomicAdd(p.work, 1));
     const size_t bh = hd.bh;
     const int n = __shfl_sync(FULL, sc_n, idx & 31) & 0xFFFF;
