@@ -331,6 +331,22 @@ static lq_status launch_persistent(K kernel, long items, int block, size_t smem,
   return launch_dependent(kernel, static_cast<int>(grid), block, smem, stream, p);
 }
 
+// persistent two-warp CTAs, each with its own shared-memory slot: as many as are resident at once
+template <int GATE, bool R16, bool BF16>
+static lq_status launch_decode_t(const lq_shape *s, const Params &p, cudaStream_t stream) {
+  const size_t smem = DecodeSlot(s->W, s->r, GATE == LQ_GATE_DIAG, R16, BF16).bytes;
+  const long nh = (long)s->batch * s->heads_v;
+  // (windows whose records come in more than one segment have an instance of their own)
+  return s->W - 1 > REC_SEG ? launch_persistent(decode_kernel<GATE, R16, true, BF16>, nh, 64, smem, stream, p)
+                            : launch_persistent(decode_kernel<GATE, R16, false, BF16>, nh, 64, smem, stream, p);
+}
+template <bool BF16>
+static lq_status launch_decode(const lq_shape *s, const Params &p, cudaStream_t stream) {
+  if (s->gate == LQ_GATE_DIAG)
+    return s->rec16 ? launch_decode_t<LQ_GATE_DIAG, true, BF16>(s, p, stream) : launch_decode_t<LQ_GATE_DIAG, false, BF16>(s, p, stream);
+  return s->rec16 ? launch_decode_t<LQ_GATE_SCALAR, true, BF16>(s, p, stream) : launch_decode_t<LQ_GATE_SCALAR, false, BF16>(s, p, stream);
+}
+
 // per-window BF16: persistent CTAs that stride over the heads
 template <int MODE>
 static lq_status launch_bf16w_boundary(const lq_shape *s, const Params &p, cudaStream_t stream) {
@@ -398,45 +414,10 @@ static lq_status decode_step_impl(const lq_shape *shape, const lq_state *state, 
   p.gen = generation++;
 #endif
   p.q = q; p.k = k; p.v = v; p.beta = beta; p.alpha = alpha; p.o = o;
-  const bool diag = shape->gate == LQ_GATE_DIAG;
   const long nh = (long)shape->batch * shape->heads_v;
   p.overlap = nh >= 2L * sm_count() * shape->W;        // as many boundaries as boundary CTAs, on average
-  // persistent two-warp CTAs, each with its own shared-memory slot: as many as are resident at once
-  const bool r16 = shape->rec16 != 0;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (shape->state_bf16) {                   // per-window BF16: one CTA per head
-    const int grid = static_cast<int>(nh);
-    const size_t rsm = bf16w_decode_smem(shape->W, diag, r16);
-    if (r16)
-      rc = diag ? launch_dependent(bf16w_decode_kernel<LQ_GATE_DIAG, true>, grid, 256, rsm, st, p)
-                : launch_dependent(bf16w_decode_kernel<LQ_GATE_SCALAR, true>, grid, 256, rsm, st, p);
-    else
-      rc = diag ? launch_dependent(bf16w_decode_kernel<LQ_GATE_DIAG, false>, grid, 256, rsm, st, p)
-                : launch_dependent(bf16w_decode_kernel<LQ_GATE_SCALAR, false>, grid, 256, rsm, st, p);
-    if (rc != LQ_OK) return rc;
-    if (between && cudaEventRecord(between, st) != cudaSuccess) {
-      cudaGetLastError();
-      return LQ_ERR_CUDA;
-    }
-    return launch_boundary<0>(shape, p, st);
-  }
-  const size_t smem = DecodeSlot(shape->W, shape->r, diag, r16).bytes;
-  const bool longw = shape->W - 1 > REC_SEG;               // windows whose records come in more than one segment
-  if (longw) {
-    if (r16)
-      rc = diag ? launch_persistent(decode_kernel<LQ_GATE_DIAG, true, true>, nh, 64, smem, st, p)
-                : launch_persistent(decode_kernel<LQ_GATE_SCALAR, true, true>, nh, 64, smem, st, p);
-    else
-      rc = diag ? launch_persistent(decode_kernel<LQ_GATE_DIAG, false, true>, nh, 64, smem, st, p)
-                : launch_persistent(decode_kernel<LQ_GATE_SCALAR, false, true>, nh, 64, smem, st, p);
-  } else {
-    if (r16)
-      rc = diag ? launch_persistent(decode_kernel<LQ_GATE_DIAG, true, false>, nh, 64, smem, st, p)
-                : launch_persistent(decode_kernel<LQ_GATE_SCALAR, true, false>, nh, 64, smem, st, p);
-    else
-      rc = diag ? launch_persistent(decode_kernel<LQ_GATE_DIAG, false, false>, nh, 64, smem, st, p)
-                : launch_persistent(decode_kernel<LQ_GATE_SCALAR, false, false>, nh, 64, smem, st, p);
-  }
+  rc = shape->state_bf16 ? launch_decode<true>(shape, p, st) : launch_decode<false>(shape, p, st);
   if (rc != LQ_OK) return rc;
   if (between && cudaEventRecord(between, st) != cudaSuccess) {
     cudaGetLastError();

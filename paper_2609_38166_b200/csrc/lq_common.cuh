@@ -30,6 +30,7 @@ constexpr int HB_ROW_SMOOTH = HB_COL_SCALE + 4 * D;
 constexpr int HB_COMP_K = HB_ROW_SMOOTH + 4 * D;
 __host__ __device__ constexpr int hb_comp_u(int r) { return HB_COMP_K + 2 * D * r; }
 __host__ __device__ constexpr int head_bytes(int r) { return HB_COMP_K + 4 * D * r; }
+constexpr int BF16W_HEAD_BYTES = 2 * D * D;   // per-window BF16: S0^T
 __host__ __device__ constexpr int record_floats(bool diag) { return diag ? 3 * D : 2 * D; }
 constexpr int REC_KT = 0, REC_U = D, REC_A = 2 * D;
 

@@ -44,16 +44,16 @@ constexpr int REC_SEG = 32;                // (16 was tried: no faster at W = 32
 struct DecodeSlot {
   // byte offsets inside the slot; every region starts on a 16-byte boundary
   int head, rec, bas, digits, y, pk, pq, mbar, bytes;
-  __host__ __device__ DecodeSlot(int W, int r, bool diag, bool rec16 = false) {
+  __host__ __device__ DecodeSlot(int W, int r, bool diag, bool rec16 = false, bool bf16 = false) {
     // a window holds at most W-1 records when a token arrives; they are staged REC_SEG rows at a time (newest
     // first), which keeps the slot small for long windows
     int rows = W > 1 ? W - 1 : 1;
     if (rows > REC_SEG) rows = REC_SEG;
     int o = 0;
-    head = o; o += head_bytes(r);          // the head block: codes | col_scale | row_smooth | comp_k | comp_u
+    head = o; o += bf16 ? BF16W_HEAD_BYTES : head_bytes(r);   // codes | col_scale | row_smooth | comp_k | comp_u, or S0^T
     rec = o; o += (rec16 ? 2 : 4) * record_floats(diag) * rows;   // buffered record rows (fp32 or fp16)
     bas = o; o += diag ? 0 : 2 * 4 * MAX_W;         // scalar gate: the records' decays, one copy per warp
-    digits = o; o += 8 * D;               // digit planes: plane 4v+d = digit d of vector v (0: k, 1: q)
+    digits = o; o += 8 * D;               // digit planes: plane 4v+d = digit d of vector v (0: k, 1: q); bf16: record terms
     y = o; o += 2 * 4 * D;                // [2][128]: the rounded sums of the state stream, later the record terms
     pk = o; o += (4 * (r + 2) + 15) / 16 * 16;      // compensator projections against Gamma k
     pq = o; o += (4 * (r + 2) + 15) / 16 * 16;      // ... against Gamma q; pq[r], pq[r+1] hold kt^T q of alternate heads
@@ -87,6 +87,12 @@ __device__ __forceinline__ void widen8_bf16(const uint4 w, float (&x)[8]) {
     x[2 * e + 1] = __uint_as_float(ws[e] & 0xFFFF0000u);
   }
 }
+// the same as four (even, odd) pairs
+__device__ __forceinline__ void widen8_bf16(const uint4 w, float2 (&x)[4]) {
+  const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+  for (int e = 0; e < 4; e++) x[e] = make_float2(__uint_as_float(ws[e] << 16), __uint_as_float(ws[e] & 0xFFFF0000u));
+}
 __device__ __forceinline__ void widen8_f16(const uint4 w, float (&x)[8]) {
   const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
@@ -103,6 +109,33 @@ __device__ __forceinline__ void tree16x4(float (&x)[4]) {
   for (int s = 1; s <= 8; s <<= 1) {
 #pragma unroll
     for (int v = 0; v < 4; v++) x[v] = x[v] + __shfl_xor_sync(FULL, x[v], s);
+  }
+}
+
+// Columns j0 .. j0 + 63 of the products of a bfloat16 state (S0T: [d_v][d_k] in shared memory) with two vectors, into
+// y[0][.] and y[1][.]; lane c (and its twin c + 16) holds block c of the vectors.  Eight columns at a time per half-warp: the
+// sixteen sums are taken over the sixteen lanes by halving exchanges (15 shuffles instead of 64), neighbouring blocks first.
+__device__ __forceinline__ void bf16_columns(const uint16_t *S0T, int j0, const float2 (&xk)[4], const float2 (&xq)[4], float *y, int lane) {
+  const int c = lane & 15, half = lane >> 4;
+  const bool u0 = lane & 1, u1 = lane & 2, u2 = lane & 4, u3 = lane & 8;
+#pragma unroll 1
+  for (int j = j0 + 8 * half; j < j0 + 64; j += 16) {
+    float vk[8], vq[8], x8[8], x4[4], x2[2];
+#pragma unroll
+    for (int m = 0; m < 8; m++) {
+      float2 s2[4];
+      widen8_bf16(*reinterpret_cast<const uint4 *>(S0T + (j + m) * D + 8 * c), s2);
+      vk[m] = block8(s2, xk);
+      vq[m] = block8(s2, xq);
+    }
+#pragma unroll
+    for (int e = 0; e < 8; e++) x8[e] = (u0 ? vq[e] : vk[e]) + __shfl_xor_sync(FULL, u0 ? vk[e] : vq[e], 1);
+#pragma unroll
+    for (int e = 0; e < 4; e++) x4[e] = (u1 ? x8[e + 4] : x8[e]) + __shfl_xor_sync(FULL, u1 ? x8[e] : x8[e + 4], 2);
+#pragma unroll
+    for (int e = 0; e < 2; e++) x2[e] = (u2 ? x4[e + 2] : x4[e]) + __shfl_xor_sync(FULL, u2 ? x4[e] : x4[e + 2], 4);
+    const float x = (u3 ? x2[1] : x2[0]) + __shfl_xor_sync(FULL, u3 ? x2[0] : x2[1], 8);
+    y[(u0 ? D : 0) + j + (u1 ? 4 : 0) + (u2 ? 2 : 0) + (u3 ? 1 : 0)] = x;
   }
 }
 
@@ -154,7 +187,9 @@ __device__ __forceinline__ void load_token(const Params &p, const HeadIdx h, int
 // first, first + G, first + 2G, ...
 // LONGW: the window may hold more records than the slot stages at a time (W - 1 > REC_SEG); in the instances for
 // shorter windows everything to do with a second segment drops out at compile time.
-template <int GATE, bool R16, bool LONGW>
+// BF16: the per-window BF16 state (lq_shape.state_bf16): the head block is S0^T in bfloat16, its product with Gamma x is
+// taken in binary32 by both warps, half of the columns each; there are no scales and no compensators.
+template <int GATE, bool R16, bool LONGW, bool BF16>
 __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot, const int lane, const int role,
                                             const unsigned first, const unsigned G) {
   uint32_t parA = 0, parR = 0;               // phases of the slot's two copy barriers
@@ -162,7 +197,8 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
   constexpr int RF = record_floats(DIAG);
   const int W = p.W, r = p.r;
   using rec_t = typename std::conditional<R16, __half, float>::type;   // element type of the record rows
-  const DecodeSlot L(W, r, DIAG, R16);
+  const DecodeSlot L(W, r, DIAG, R16, BF16);
+  const uint32_t block_bytes = BF16 ? BF16W_HEAD_BYTES : head_bytes(r);
   const int c = lane & 15, half = lane >> 4, g = lane >> 2, t = lane & 3;
   const int8_t *zt = reinterpret_cast<const int8_t *>(slot + L.head + HB_CODES);
   const float *bs = reinterpret_cast<const float *>(slot + L.head + HB_COL_SCALE);
@@ -197,9 +233,10 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
   const uint64_t keep = l2_keep_policy(), stream = l2_stream_policy();
   auto request_head = [&](unsigned bh, int n) {
     if (lane == 0) {
-      mbar_expect_tx(barA, head_bytes(r));
-      if (n == W - 1) bulk_g2s_hint(slot_a + L.head, p.head(bh), head_bytes(r), barA, keep);
-      else bulk_g2s_hint(slot_a + L.head, p.head(bh), head_bytes(r), barA, stream);
+      const uint8_t *block = p.heads + bh * (size_t)block_bytes;
+      mbar_expect_tx(barA, block_bytes);
+      if (n == W - 1) bulk_g2s_hint(slot_a + L.head, block, block_bytes, barA, keep);
+      else bulk_g2s_hint(slot_a + L.head, block, block_bytes, barA, stream);
     }
   };
   // first record of the segment that ends before record `hi`
@@ -505,6 +542,29 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         }
       }
       LQ_TICK(3);
+      if constexpr (BF16) {                  // this warp's half of the columns; then all goes to the stream warp
+        if (DIAG) named_wait(4);             // (the stream warp has read the records' decays too)
+        {
+          const int n_next = n_next_now();
+          if (wanted(n_next)) request_records(bh_next, n_next);
+        }
+        float2 xk[4], xq[4];
+#pragma unroll
+        for (int cc = 0; cc < 4; cc++) {
+          const float2 gm = DIAG ? g2[cc] : pair(gsc);
+          xk[cc] = __fmul2_rn(gm, k2[cc]);
+          xq[cc] = __fmul2_rn(gm, q2[cc]);
+        }
+        named_wait(2);                       // the stream warp has taken the head before out of y and the terms
+        wait_for(barA, parA);
+        bf16_columns(reinterpret_cast<const uint16_t *>(zt), 64, xk, xq, y, lane);
+        float *terms = reinterpret_cast<float *>(digits);
+        *reinterpret_cast<float4 *>(terms + 4 * lane) = make_float4(rk_rec[0], rk_rec[1], rk_rec[2], rk_rec[3]);
+        *reinterpret_cast<float4 *>(terms + D + 4 * lane) = make_float4(rq_rec[0], rq_rec[1], rq_rec[2], rq_rec[3]);
+        if (draws && lane == 0) *qidx = ticket;
+        __syncwarp();
+        named_arrive(1);                     // (this warp is done with the head block as well)
+      } else {
       // Now the head block: the compensators are projected with Gamma_{1:l}, which for the diagonal gate is where
       // the walk's chain of decays has arrived (g2), for the scalar gate the product taken before the wait.
       wait_for(barA, parA);
@@ -532,6 +592,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
       if (draws && lane == 0) *qidx = ticket;
       __syncwarp();
       named_arrive(1);                       // the record terms are in shared memory (and the ticket)
+      }
       LQ_TICK(5);
       // append the key side of the record (and its decay)
       {
@@ -572,6 +633,31 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         for (int e = 0; e < 8; e++) gam[e] = gsc;
       }
       LQ_TICK(3);
+      float rk[4], rq[4];
+      const float v4[4] = {__uint_as_float(v_raw.x << 16), __uint_as_float(v_raw.x & 0xFFFF0000u),
+                           __uint_as_float(v_raw.y << 16), __uint_as_float(v_raw.y & 0xFFFF0000u)};
+      if constexpr (BF16) {
+        float2 xk[4], xq[4];
+#pragma unroll
+        for (int cc = 0; cc < 4; cc++) {
+          const float2 gm = make_float2(gam[2 * cc], gam[2 * cc + 1]);
+          xk[cc] = __fmul2_rn(gm, make_float2(k8[2 * cc], k8[2 * cc + 1]));
+          xq[cc] = __fmul2_rn(gm, make_float2(q8[2 * cc], q8[2 * cc + 1]));
+        }
+        named_arrive(2);                     // the head before is out of y and the terms
+        bf16_columns(reinterpret_cast<const uint16_t *>(zt), 0, xk, xq, y, lane);
+        __syncwarp();
+        named_wait(1);                       // the other half of the columns and the record terms
+        {
+          const int n_next = n_next_now();
+          if (wanted(n_next)) request_head(bh_next, n_next);
+        }
+        const float *terms = reinterpret_cast<const float *>(digits);
+        const float4 yk = *reinterpret_cast<const float4 *>(y + 4 * lane), yq = *reinterpret_cast<const float4 *>(y + D + 4 * lane);
+        const float4 tk = *reinterpret_cast<const float4 *>(terms + 4 * lane), tq = *reinterpret_cast<const float4 *>(terms + D + 4 * lane);
+        rk[0] = yk.x + tk.x; rk[1] = yk.y + tk.y; rk[2] = yk.z + tk.z; rk[3] = yk.w + tk.w;
+        rq[0] = yq.x + tq.x; rq[1] = yq.y + tq.y; rq[2] = yq.z + tq.z; rq[3] = yq.w + tq.w;
+      } else {
       // C Gamma k (lanes 0..15) and C Gamma q (lanes 16..31) on their fixed-point grids, as digit planes
       float back_own;
       {
@@ -662,10 +748,8 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         const float4 yk4 = *reinterpret_cast<const float4 *>(y + 4 * lane);
         const float4 yq4 = *reinterpret_cast<const float4 *>(y + D + 4 * lane);
         const float4 s4 = *reinterpret_cast<const float4 *>(bs + 4 * lane);      // code steps B_j / 127
-        float rk[4] = {s4.x * (yk4.x * back_k), s4.y * (yk4.y * back_k), s4.z * (yk4.z * back_k), s4.w * (yk4.w * back_k)};
-        float rq[4] = {s4.x * (yq4.x * back_q), s4.y * (yq4.y * back_q), s4.z * (yq4.z * back_q), s4.w * (yq4.w * back_q)};
-        const float v4[4] = {__uint_as_float(v_raw.x << 16), __uint_as_float(v_raw.x & 0xFFFF0000u),
-                             __uint_as_float(v_raw.y << 16), __uint_as_float(v_raw.y & 0xFFFF0000u)};
+        rk[0] = s4.x * (yk4.x * back_k); rk[1] = s4.y * (yk4.y * back_k); rk[2] = s4.z * (yk4.z * back_k); rk[3] = s4.w * (yk4.w * back_k);
+        rq[0] = s4.x * (yq4.x * back_q); rq[1] = s4.y * (yq4.y * back_q); rq[2] = s4.z * (yq4.z * back_q); rq[3] = s4.w * (yq4.w * back_q);
         LQ_TICK(6);
         named_arrive(2);                     // y has been read: the dot warp may put the record terms there
         named_wait(3);                       // the compensator projections are complete
@@ -692,6 +776,9 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
           rk[0] = rk[0] + tk.x; rk[1] = rk[1] + tk.y; rk[2] = rk[2] + tk.z; rk[3] = rk[3] + tk.w;
           rq[0] = rq[0] + tq.x; rq[1] = rq[1] + tq.y; rq[2] = rq[2] + tq.z; rq[3] = rq[3] + tq.w;
         }
+      }
+      }
+      {
         const float ktq = pq[r + (idx & 1)];
         float u[4], o[4];
 #pragma unroll
@@ -710,7 +797,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
 }
 
 // Persistent kernel of two-warp CTAs: CTA `blockIdx.x` takes heads blockIdx.x, blockIdx.x + gridDim.x, ...
-template <int GATE, bool R16, bool LONGW>
+template <int GATE, bool R16, bool LONGW, bool BF16>
 __global__ void __launch_bounds__(64, 6) decode_kernel(const Params p) {
   extern __shared__ __align__(128) unsigned char lq_slot[];
   LQ_STAMP(0, 0);
@@ -718,17 +805,17 @@ __global__ void __launch_bounds__(64, 6) decode_kernel(const Params p) {
   // no data, so it does not matter that the kernel ahead may still be writing that block: the L2 is where its writes
   // go).  The first head of a CTA is the only one whose copy nothing hides.
   if (threadIdx.x == 0 && blockIdx.x < static_cast<unsigned>(p.batch) * p.heads_v)
-    bulk_prefetch_l2(p.head(blockIdx.x), head_bytes(p.r));
+    bulk_prefetch_l2(p.heads + blockIdx.x * (size_t)(BF16 ? BF16W_HEAD_BYTES : head_bytes(p.r)), BF16 ? BF16W_HEAD_BYTES : head_bytes(p.r));
   const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
   if (threadIdx.x == 0) {                    // the slot's two copy barriers (shared memory only)
-    const uint32_t bar = smem_addr(lq_slot + DecodeSlot(p.W, p.r, GATE == LQ_GATE_DIAG, R16).mbar);
+    const uint32_t bar = smem_addr(lq_slot + DecodeSlot(p.W, p.r, GATE == LQ_GATE_DIAG, R16, BF16).mbar);
     mbar_init(bar, 1);
     mbar_init(bar + 8, 1);
   }
   __syncthreads();
   grid_dependency_wait();                    // no data in global memory is read or written above this line
   LQ_STAMP(0, 1);
-  decode_slot<GATE, R16, LONGW>(p, lq_slot, lane, role, blockIdx.x, gridDim.x);
+  decode_slot<GATE, R16, LONGW, BF16>(p, lq_slot, lane, role, blockIdx.x, gridDim.x);
   LQ_STAMP(0, 3);
 #ifdef LQ_TIMING
   if (threadIdx.x == 0 && blockIdx.x < 1024) {
