@@ -36,19 +36,19 @@
 
 namespace lq {
 
-// Rows of the record buffer that a decode slot holds at a time (a multiple of four: the walk takes the records four
-// at a time from the newest back, so a group of four never straddles two segments).
-constexpr int REC_SEG = 32;                // (16 was tried: no faster at W = 32 or 64)
+// Long windows: the records come in segments of this many rows, newest first, two of which the slot holds at a time: while
+// one is walked the next is on its way (a multiple of four: the walk takes the records four at a time from the newest back).
+// Rows of 1 to 1.5 KB (fp32) and of half that (fp16); diagonal gate, fp32, W = 64: 8 rows 132 us per step at 256 x 32 heads,
+// 4: 148, 12: 149, 16: 146 (one area of 32 rows, refilled when walked: 146); fp16: 12 rows 125 us, 8: 130, 16: 123.
+__host__ __device__ constexpr int rec_seg(bool rec16) { return rec16 ? 12 : 8; }
 
 // ---- shared-memory slot of one CTA ----
 struct DecodeSlot {
   // byte offsets inside the slot; every region starts on a 16-byte boundary
   int head, rec, bas, digits, y, pk, pq, mbar, bytes;
-  __host__ __device__ DecodeSlot(int W, int r, bool diag, bool rec16 = false, bool bf16 = false) {
-    // a window holds at most W-1 records when a token arrives; they are staged REC_SEG rows at a time (newest
-    // first), which keeps the slot small for long windows
-    int rows = W > 1 ? W - 1 : 1;
-    if (rows > REC_SEG) rows = REC_SEG;
+  __host__ __device__ DecodeSlot(int W, int r, bool diag, bool rec16, bool bf16, int seg) {
+    // a window holds at most W-1 records when a token arrives; seg > 0: two segments of that many at a time
+    const int rows = seg > 0 ? 2 * seg : W > 1 ? W - 1 : 1;
     int o = 0;
     head = o; o += bf16 ? BF16W_HEAD_BYTES : head_bytes(r);   // codes | col_scale | row_smooth | comp_k | comp_u, or S0^T
     rec = o; o += (rec16 ? 2 : 4) * record_floats(diag) * rows;   // buffered record rows (fp32 or fp16)
@@ -57,7 +57,7 @@ struct DecodeSlot {
     y = o; o += 2 * 4 * D;                // [2][128]: the rounded sums of the state stream, later the record terms
     pk = o; o += (4 * (r + 2) + 15) / 16 * 16;      // compensator projections against Gamma k
     pq = o; o += (4 * (r + 2) + 15) / 16 * 16;      // ... against Gamma q; pq[r], pq[r+1] hold kt^T q of alternate heads
-    mbar = o; o += 16;
+    mbar = o; o += 32;                    // head block, records (two)
     bytes = (o + 127) / 128 * 128;
   }
 };
@@ -143,7 +143,8 @@ __device__ __forceinline__ void bf16_columns(const uint16_t *S0T, int j0, const 
 //   1: dot warp -> stream warp, "the record terms (and the ticket) are in shared memory"
 //   2: stream warp -> dot warp, "its sums are out of y"
 //   3: dot warp -> stream warp, "the compensator projections are in shared memory"
-//   4: stream warp -> dot warp, "the records' decays have been read" (diagonal gate)
+//   4, 5: stream warp -> dot warp, "the records' decays have been read" (diagonal gate; one for each half of the record area:
+//      with two segments there the stream warp may be through with both before the dot warp is with the first)
 __device__ __forceinline__ void named_arrive(int id) {
   __threadfence_block();
   asm volatile("bar.arrive %0, 64;\n" ::"r"(id) : "memory");
@@ -185,19 +186,21 @@ __device__ __forceinline__ void load_token(const Params &p, const HeadIdx h, int
 
 // The work of one pair of warps (role 0: stream warp, role 1: dot warp) on its shared-memory slot: heads
 // first, first + G, first + 2G, ...
-// LONGW: the window may hold more records than the slot stages at a time (W - 1 > REC_SEG); in the instances for
-// shorter windows everything to do with a second segment drops out at compile time.
+// LONGW: the records come in segments (launch_decode_t says when); in the other instances everything to do with a second
+// segment drops out at compile time.
 // BF16: the per-window BF16 state (lq_shape.state_bf16): the head block is S0^T in bfloat16, its product with Gamma x is
 // taken in binary32 by both warps, half of the columns each; there are no scales and no compensators.
 template <int GATE, bool R16, bool LONGW, bool BF16>
 __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot, const int lane, const int role,
                                             const unsigned first, const unsigned G) {
-  uint32_t parA = 0, parR = 0;               // phases of the slot's two copy barriers
+  uint32_t parA = 0, parR = 0;               // phase of the head block's copy barrier; bit b: of the records' barrier b
+  int buf = 0;                               // (long windows) the half of the record area that the next segment to be walked is in
   constexpr bool DIAG = GATE == LQ_GATE_DIAG;
   constexpr int RF = record_floats(DIAG);
   const int W = p.W, r = p.r;
   using rec_t = typename std::conditional<R16, __half, float>::type;   // element type of the record rows
-  const DecodeSlot L(W, r, DIAG, R16, BF16);
+  constexpr int SEG = LONGW ? rec_seg(R16) : 0;
+  const DecodeSlot L(W, r, DIAG, R16, BF16, SEG);
   const uint32_t block_bytes = BF16 ? BF16W_HEAD_BYTES : head_bytes(r);
   const int c = lane & 15, half = lane >> 4, g = lane >> 2, t = lane & 3;
   const int8_t *zt = reinterpret_cast<const int8_t *>(slot + L.head + HB_CODES);
@@ -240,26 +243,36 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
     }
   };
   // first record of the segment that ends before record `hi`
-  auto seg_base = [&](int hi) { return (LONGW && hi > REC_SEG) ? hi - REC_SEG : 0; };
-  // records [seg_base(hi), hi) of head bh, n of which are buffered in all, into the slot
-  auto request_segment = [&](unsigned bh, int n, int hi) {
+  auto seg_base = [&](int hi) { return (LONGW && hi > SEG) ? hi - SEG : 0; };
+  // records [seg_base(hi), hi) of head bh, n of which are buffered in all, into half `to` of the record area
+  auto request_segment = [&](unsigned bh, int n, int hi, int to) {
     if (lane == 0) {
       const int lo = seg_base(hi);
-      const uint32_t rb = static_cast<uint32_t>(sizeof(rec_t)) * RF * (hi - lo);
-      mbar_expect_tx(barR, rb);              // with no records the phase completes at once
+      const uint32_t rb = static_cast<uint32_t>(sizeof(rec_t)) * RF * (hi - lo), bar_to = barR + 8 * to;
+      const uint32_t dst = slot_a + L.rec + to * static_cast<uint32_t>(sizeof(rec_t)) * RF * SEG;
+      mbar_expect_tx(bar_to, rb);            // with no records the phase completes at once
       if (hi > lo) {
-        if (n == W - 1) bulk_g2s_hint(slot_a + L.rec, p.record<rec_t>(bh, lo, DIAG), rb, barR, keep);
-        else bulk_g2s_hint(slot_a + L.rec, p.record<rec_t>(bh, lo, DIAG), rb, barR, stream);
+        if (n == W - 1) bulk_g2s_hint(dst, p.record<rec_t>(bh, lo, DIAG), rb, bar_to, keep);
+        else bulk_g2s_hint(dst, p.record<rec_t>(bh, lo, DIAG), rb, bar_to, stream);
       }
     }
   };
-  auto request_records = [&](unsigned bh, int n) { request_segment(bh, n, n); };   // the newest segment
+  // the newest records of a head: with long windows the two newest segments
+  auto request_records = [&](unsigned bh, int n) {
+    request_segment(bh, n, n, buf);
+    if (LONGW && n > SEG) request_segment(bh, n, n - SEG, buf ^ 1);
+  };
   // Bounded wait for one of the two.  A copy that never lands must not hang the GPU: when the limit runs out the
   // error flag is set and the warp goes on (its results are garbage, the flag says so); the other warp, which
   // meets this one at the named barriers, is not left waiting.
   auto wait_for = [&](uint32_t bar_, uint32_t &par) {
     if (!mbar_wait(bar_, par) && lane == 0) atomicOr(&g_device_error, 1);
     par ^= 1u;
+    __syncwarp();
+  };
+  auto wait_records = [&]() {                // the segment in half `buf`
+    if (!mbar_wait(barR + 8 * buf, (parR >> buf) & 1u) && lane == 0) atomicOr(&g_device_error, 1);
+    parR ^= 1u << buf;
     __syncwarp();
   };
 
@@ -449,7 +462,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         g2[cc] = a2[cc];
         kt2[cc] = __fmul2_rn(pair(beta), k2[cc]);
       }
-      wait_for(barR, parR);                  // the newest segment of the records
+      wait_records();                        // the newest segment of the records
       // Compensator keys against Gamma_{1:l} k and Gamma_{1:l} q (the projections go to pk[h], pq[h]).
       auto project_compensators = [&](const float2 (&gam)[4]) {
         float2 gk2[4], gq2[4];
@@ -477,14 +490,17 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         }
       };
       float rk_rec[4] = {0.0f, 0.0f, 0.0f, 0.0f}, rq_rec[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-      int base = seg_base(n);                        // the slot holds records base .. (row = record - base)
+      int base = seg_base(n);                        // the segment at hand begins with record `base`
+      const rec_t *seg = rec + buf * SEG * RF;       // and lies here
       for (int jt = n - 1; jt >= 0; jt -= 4) {       // records jt, jt-1, jt-2, jt-3
-        if (LONGW && jt < base) {                    // the segment is walked: fetch the one before it
+        if (LONGW && jt < base) {                    // the segment is walked: on to the one before it
           __syncwarp();
-          if (DIAG) named_wait(4);            // (the stream warp has taken this segment's decays as well)
-          request_segment(bh, n, base);
+          if (DIAG) named_wait(4 + buf);             // (the stream warp has taken this segment's decays as well)
+          if (base > SEG) request_segment(bh, n, base - SEG, buf);      // (the one after that is on its way to the other half)
           base = seg_base(base);
-          wait_for(barR, parR);
+          buf ^= 1;
+          seg = rec + buf * SEG * RF;
+          wait_records();
         }
         float s4[4];
         int jo[2];
@@ -494,8 +510,8 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
           const int jn = jt - 2 * u, jold = jn - 1;  // newer, older
           float2 an[4], ao[4], gmine[4];
           if (DIAG) {
-            load8p(rec + ((jn > 0 ? jn : 0) - base) * RF + REC_A + 8 * c, an);
-            load8p(rec + ((jold > 0 ? jold : 0) - base) * RF + REC_A + 8 * c, ao);
+            load8p(seg + ((jn > 0 ? jn : 0) - base) * RF + REC_A + 8 * c, an);
+            load8p(seg + ((jold > 0 ? jold : 0) - base) * RF + REC_A + 8 * c, ao);
           } else {
             const float2 x = pair(bas[jn > 0 ? jn : 0]), z = pair(bas[jold > 0 ? jold : 0]);
 #pragma unroll
@@ -512,7 +528,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
           jo[u] = jn - half;
           const int j = jo[u] >= 0 ? jo[u] : 0;      // (record 0 is in the slot whenever an index runs below it)
           float2 x2[4], yk2[4], yq2[4];
-          load8p(rec + (j - base) * RF + REC_KT + 8 * c, x2);
+          load8p(seg + (j - base) * RF + REC_KT + 8 * c, x2);
 #pragma unroll
           for (int cc = 0; cc < 4; cc++) { yk2[cc] = __fmul2_rn(gmine[cc], k2[cc]); yq2[cc] = __fmul2_rn(gmine[cc], q2[cc]); }
           s4[2 * u] = block8(x2, yk2);
@@ -533,7 +549,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
             const int u = i4 >> 1;
             const bool mine = (i4 & 1) == half;
             const float pkj = mine ? s4[2 * u] : oth[2 * u], pqj = mine ? s4[2 * u + 1] : oth[2 * u + 1];
-            const float4 u4 = load4(rec + (j - base) * RF + REC_U + 4 * lane);
+            const float4 u4 = load4(seg + (j - base) * RF + REC_U + 4 * lane);
             rk_rec[0] = fmaf(u4.x, pkj, rk_rec[0]); rq_rec[0] = fmaf(u4.x, pqj, rq_rec[0]);
             rk_rec[1] = fmaf(u4.y, pkj, rk_rec[1]); rq_rec[1] = fmaf(u4.y, pqj, rq_rec[1]);
             rk_rec[2] = fmaf(u4.z, pkj, rk_rec[2]); rq_rec[2] = fmaf(u4.z, pqj, rq_rec[2]);
@@ -541,9 +557,11 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
           }
         }
       }
+      const int walked = 4 + buf;                    // the barrier of the last segment
+      if (LONGW) buf ^= 1;                           // the next head's segments follow on in turn
       LQ_TICK(3);
       if constexpr (BF16) {                  // this warp's half of the columns; then all goes to the stream warp
-        if (DIAG) named_wait(4);             // (the stream warp has read the records' decays too)
+        if (DIAG) named_wait(walked);        // (the stream warp has read the records' decays too)
         {
           const int n_next = n_next_now();
           if (wanted(n_next)) request_records(bh_next, n_next);
@@ -581,7 +599,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
       __syncwarp();
       named_arrive(3);                       // the compensator projections are in pk, pq; this warp is done with the head block
       LQ_TICK(4);
-      if (DIAG) named_wait(4);               // diagonal gate: the stream warp read the records' decays too
+      if (DIAG) named_wait(walked);          // diagonal gate: the stream warp read the records' decays too
       {
         const int n_next = n_next_now();
         if (wanted(n_next)) request_records(bh_next, n_next);
@@ -614,16 +632,18 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
       if (DIAG) {
         for (int hi = n;;) {                        // segment after segment, in step with the dot warp
           const int lo = seg_base(hi);
-          wait_for(barR, parR);
+          const rec_t *seg = rec + buf * SEG * RF;
+          wait_records();
 #pragma unroll 2
           for (int j = hi - 1; j >= lo; j--) {
             float aj[8];
-            load8(rec + (j - lo) * RF + REC_A + 8 * c, aj);
+            load8(seg + (j - lo) * RF + REC_A + 8 * c, aj);
 #pragma unroll
             for (int e = 0; e < 8; e++) gam[e] = gam[e] * aj[e];
           }
           __syncwarp();
-          named_arrive(4);                   // this warp is done with the segment
+          named_arrive(4 + buf);             // this warp is done with the segment
+          if (LONGW) buf ^= 1;
           if (lo == 0) break;
           hi = lo;
         }
@@ -808,9 +828,10 @@ __global__ void __launch_bounds__(64, 6) decode_kernel(const Params p) {
     bulk_prefetch_l2(p.heads + blockIdx.x * (size_t)(BF16 ? BF16W_HEAD_BYTES : head_bytes(p.r)), BF16 ? BF16W_HEAD_BYTES : head_bytes(p.r));
   const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
   if (threadIdx.x == 0) {                    // the slot's two copy barriers (shared memory only)
-    const uint32_t bar = smem_addr(lq_slot + DecodeSlot(p.W, p.r, GATE == LQ_GATE_DIAG, R16, BF16).mbar);
+    const uint32_t bar = smem_addr(lq_slot + DecodeSlot(p.W, p.r, GATE == LQ_GATE_DIAG, R16, BF16, LONGW ? rec_seg(R16) : 0).mbar);
     mbar_init(bar, 1);
     mbar_init(bar + 8, 1);
+    if (LONGW) mbar_init(bar + 16, 1);
   }
   __syncthreads();
   grid_dependency_wait();                    // no data in global memory is read or written above this line
