@@ -8,7 +8,6 @@
 #include <mutex>
 #include <tuple>
 
-#include "lq_bf16w.cuh"
 #include "lq_boundary.cuh"
 #include "lq_decode.cuh"
 
@@ -353,50 +352,39 @@ static lq_status launch_decode(const lq_shape *s, const Params &p, cudaStream_t 
   return s->rec16 ? launch_decode_t<LQ_GATE_SCALAR, true, BF16>(s, p, stream) : launch_decode_t<LQ_GATE_SCALAR, false, BF16>(s, p, stream);
 }
 
-// per-window BF16: persistent CTAs that stride over the heads
-template <int MODE>
-static lq_status launch_bf16w_boundary(const lq_shape *s, const Params &p, cudaStream_t stream) {
-  const bool diag = s->gate == LQ_GATE_DIAG;
-  const bool r16 = MODE != 1 && s->rec16 != 0;
-  const size_t smem = bf16w_boundary_smem(s->W, diag, r16);
-  const long nh = (long)s->batch * s->heads_v;
-  const int grid = static_cast<int>(nh < 2L * sm_count() ? nh : 2L * sm_count());      // persistent, two per SM
-  if (r16)
-    return diag ? launch_dependent(bf16w_boundary_kernel<LQ_GATE_DIAG, MODE == 1 ? 0 : MODE, true>, grid, 256, smem, stream, p)
-                : launch_dependent(bf16w_boundary_kernel<LQ_GATE_SCALAR, MODE == 1 ? 0 : MODE, true>, grid, 256, smem, stream, p);
-  return diag ? launch_dependent(bf16w_boundary_kernel<LQ_GATE_DIAG, MODE, false>, grid, 256, smem, stream, p)
-              : launch_dependent(bf16w_boundary_kernel<LQ_GATE_SCALAR, MODE, false>, grid, 256, smem, stream, p);
-}
-
 // The boundary kernels are persistent: as many CTAs as are resident at once, each striding over its heads.
-template <int GATE, int MODE, bool R16, int RM>
+template <int GATE, int MODE, bool R16, int RM, bool BF16>
 static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStream_t stream) {
-  const size_t smem = BoundarySmem<RM>(s->W, s->r, GATE == LQ_GATE_DIAG, R16, MODE != 1, s->n_iter > 1).bytes;
-  auto kernel = boundary_kernel<GATE, MODE, R16, RM>;
-  const long resident = (long)prepare_launch(reinterpret_cast<const void *>(kernel), 256, smem) * sm_count();
+  const bool diag = GATE == LQ_GATE_DIAG, iterate = RM > 0 && s->n_iter > 1;
+  auto bytes = [&](int slots) { return BoundarySmem<RM>(MODE, s->W, s->r, diag, R16, BF16, iterate, slots).bytes; };
+  // A second slot where a head is through in a few microseconds and two CTAs with two slots each still fit on an SM; a head
+  // that is requantized leaves its slot early enough for the next one (two slots: 65.3 us against 64.1 at 256 x 32 heads).
+  const int slots = (MODE == 2 || (BF16 && MODE == 0)) && bytes(2) <= (228 / 2 - 2) * 1024 ? 2 : 1;
+  auto kernel = boundary_kernel<GATE, MODE, R16, RM, BF16>;
+  const long resident = (long)prepare_launch(reinterpret_cast<const void *>(kernel), 256, bytes(slots)) * sm_count();
   if (resident < 1) return LQ_ERR_CUDA;
   const long nh = (long)s->batch * s->heads_v;
-  return launch_dependent(kernel, static_cast<int>(nh < resident ? nh : resident), 256, smem, stream, p);
+  return launch_dependent(kernel, static_cast<int>(nh < resident ? nh : resident), 256, bytes(slots), stream, p, slots);
 }
 
-template <int MODE, int RM>
+template <int MODE, int RM, bool BF16>
 static lq_status launch_boundary_gate(const lq_shape *s, const Params &p, cudaStream_t stream) {
-  if (MODE == 1) return launch_boundary_t<LQ_GATE_SCALAR, MODE, false, RM>(s, p, stream);   // (reads no records)
+  if (MODE == 1) return launch_boundary_t<LQ_GATE_SCALAR, MODE, false, RM, BF16>(s, p, stream);   // (reads no records)
   constexpr int M_ = MODE == 1 ? 0 : MODE;
   if (s->gate == LQ_GATE_DIAG)
-    return s->rec16 ? launch_boundary_t<LQ_GATE_DIAG, M_, true, RM>(s, p, stream) : launch_boundary_t<LQ_GATE_DIAG, M_, false, RM>(s, p, stream);
-  return s->rec16 ? launch_boundary_t<LQ_GATE_SCALAR, M_, true, RM>(s, p, stream) : launch_boundary_t<LQ_GATE_SCALAR, M_, false, RM>(s, p, stream);
+    return s->rec16 ? launch_boundary_t<LQ_GATE_DIAG, M_, true, RM, BF16>(s, p, stream) : launch_boundary_t<LQ_GATE_DIAG, M_, false, RM, BF16>(s, p, stream);
+  return s->rec16 ? launch_boundary_t<LQ_GATE_SCALAR, M_, true, RM, BF16>(s, p, stream) : launch_boundary_t<LQ_GATE_SCALAR, M_, false, RM, BF16>(s, p, stream);
 }
 
 // compiled for r = 0, r <= 4, r <= 8 and any r (the small matrices of the fit live in registers)
 template <int MODE>
 static lq_status launch_boundary(const lq_shape *s, const Params &p, cudaStream_t stream) {
   if (s->batch == 0) return LQ_OK;
-  if (s->state_bf16) return launch_bf16w_boundary<MODE>(s, p, stream);
-  if (s->r == 0) return launch_boundary_gate<MODE, 0>(s, p, stream);
-  if (MODE == 2 || s->r <= 4) return launch_boundary_gate<MODE, 4>(s, p, stream);
-  if (s->r <= 8) return launch_boundary_gate<MODE, MODE == 2 ? 4 : 8>(s, p, stream);
-  return launch_boundary_gate<MODE, MODE == 2 ? 4 : MAX_R>(s, p, stream);
+  if (s->state_bf16) return launch_boundary_gate<MODE, 0, true>(s, p, stream);
+  if (s->r == 0) return launch_boundary_gate<MODE, 0, false>(s, p, stream);
+  if (MODE == 2 || s->r <= 4) return launch_boundary_gate<MODE, 4, false>(s, p, stream);
+  if (s->r <= 8) return launch_boundary_gate<MODE, MODE == 2 ? 4 : 8, false>(s, p, stream);
+  return launch_boundary_gate<MODE, MODE == 2 ? 4 : MAX_R, false>(s, p, stream);
 }
 
 }  // namespace lq

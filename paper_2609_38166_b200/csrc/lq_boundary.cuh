@@ -20,12 +20,16 @@
 
 namespace lq {
 
-// Shared memory of a CTA, byte offsets: working arrays at fixed places (sized for RM vectors), then the slot (head block,
-// records), which is filled by two bulk copies.  Both parts of the slot are free again when the products with the start
-// vectors have been taken, and then receive the next head.
+// Shared memory of a CTA, byte offsets: working arrays at fixed places (sized for RM vectors), then one or two slots, which
+// are filled by bulk copies: the head block and the records, or (quantizing) a dense state.  A slot is free again when the
+// products with the start vectors have been taken; with two of them the next head is asked for when this one is begun.
+// A dense state lies in groups of eight rows, DENSE_GROUP bytes apart and shifted against one another by 16-byte units, so
+// that the four row groups that a quarter of a warp reads at a time fall on different banks.
+constexpr int DENSE_GROUP = 8 * D * 4 + 128;
+__host__ __device__ constexpr int dense_group_at(int g) { return g * DENSE_GROUP + ((g & 1) ? 16 : 0) + ((g & 2) ? 64 : 0); }
 template <int RM>
 struct BoundarySmem {
-  static constexpr int bar = 0;
+  static constexpr int bar = 0;                              // [2] copy barriers
   static constexpr int invc = 16;                            // [8][16]    1 / code step, per warp
   static constexpr int ic = invc + 4 * D;                    // [128]      1 / c
   static constexpr int gam = ic + 4 * D;                     // [128]      Gamma_{1:n}
@@ -34,13 +38,14 @@ struct BoundarySmem {
   static constexpr int ub = chol + (RM > 4 ? 4 * (RM * RM + 2 * RM) : 0);      // [8][RM][16] value sides as stored, per warp
   static constexpr int T = ub + 4 * D * RM;                  // [RM][128]  S w_h, then the keys as stored
   static constexpr int part = T + 4 * D * RM;                // [8][RM][128] per-warp row sums; later [8][128] those of |R|
-  static constexpr int head = part + 4 * D * 8 * (RM > 0 ? RM : 1);
-  int rec, dec, kd, Wv, bytes;
-  __host__ __device__ BoundarySmem(int W, int r, bool diag, bool rec16, bool slot, bool iterate) {
-    rec = head + (slot ? head_bytes(r) : 0);                 // [W] record rows
-    dec = rec + (slot ? (rec16 ? 2 : 4) * record_floats(diag) * W : 0);        // [W] scalar gate: the records' decays
-    kd = dec + (slot && !diag ? (4 * W + 15) / 16 * 16 : 0); // [W][128] fp16 records: Gamma_{j+1:n} kt_j (fp32: in place)
-    Wv = kd + (slot && rec16 ? 4 * D * W : 0);               // [r][128] several rounds: S^T q_h
+  static constexpr int head = part + 4 * D * 8 * (RM > 0 ? RM : 1);            // the slots
+  int rec, slot, dec, kd, Wv, bytes;
+  __host__ __device__ BoundarySmem(int mode, int W, int r, bool diag, bool rec16, bool bf16, bool iterate, int slots) {
+    rec = bf16 ? BF16W_HEAD_BYTES : head_bytes(r);           // within a slot: [W] record rows behind the head block
+    slot = mode == 1 ? (RM <= 8 ? 16 * DENSE_GROUP : 0) : rec + (rec16 ? 2 : 4) * record_floats(diag) * W;
+    dec = head + slots * slot;                               // [W] scalar gate: the records' decays
+    kd = dec + (mode != 1 && !diag ? (4 * W + 15) / 16 * 16 : 0);   // [W][128] fp16 records: Gamma_{j+1:n} kt_j (fp32: in place)
+    Wv = kd + (mode != 1 && rec16 ? 4 * D * W : 0);          // [r][128] several rounds: S^T q_h
     bytes = Wv + (iterate ? 4 * D * r : 0);
   }
 };
@@ -72,6 +77,14 @@ __device__ __forceinline__ void store_row8(float *dst, bool wide, const float2 (
                  : "memory");
   else
     store8p(dst, x);
+}
+
+// eight bfloat16 values
+__device__ __forceinline__ void load8_bf16(const uint16_t *src, float (&x)[8]) {
+  const uint4 w = *reinterpret_cast<const uint4 *>(src);
+  const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+  for (int e = 0; e < 4; e++) { x[2 * e] = __uint_as_float(ws[e] << 16); x[2 * e + 1] = __uint_as_float(ws[e] & 0xFFFF0000u); }
 }
 
 // Which of the lane's eight columns a column_tree leaves with it
@@ -194,63 +207,65 @@ __device__ __forceinline__ void cholesky_lower_warp(const float *G, int nv, floa
 }
 
 // Orthonormalise the r vectors X (rows of 128 floats in shared memory) in place, in order:
-// q_h = (x_h - sum_{j<h} L_hj q_j) / L_hh, one thread per element index (the upper half of the threads computes the same
-// and stores nothing).  With FINAL the results are rounded to fp16 (what is stored as compensator keys), written to keys
-// and kept in X as stored.  Up to four vectors: every thread computes the factor itself, in registers (no barriers around
-// a chain of four 1/sqrt); more: one warp does, through shared memory.
+// q_h = (x_h - sum_{j<h} L_hj q_j) / L_hh, one thread per element index (four warps).  With FINAL the results are rounded to
+// fp16 (what is stored as compensator keys), written to keys and kept in X as stored.  Up to four vectors: each of these
+// threads computes the factor itself, in registers (no barrier around a chain of four 1/sqrt; the other four warps leave the
+// issue slots to them); more: one warp does, through shared memory.
 // Returns the bit mask of the vectors that were not dropped.  Begins and ends with a barrier.
 template <bool FINAL, int RM>
 __device__ __forceinline__ uint32_t orthonormalize(float *X, int r, float *gram, float *chol, uint16_t *keys) {
-  const int tid = threadIdx.x, i = tid & (D - 1);
+  __shared__ uint32_t alive_mask;
+  const int tid = threadIdx.x, i = tid;
   __syncthreads();
   gram_lower<RM>(X, r, gram, true);
   __syncthreads();
   LQ_BTICK(7);
-  uint32_t alive = 0;
-  float x[RM];
-#pragma unroll
-  for (int h = 0; h < RM; h++) x[h] = h < r ? X[h * D + i] : 0.0f;
-  if constexpr (RM <= 4) {
-    float l[4][4], iv[4];
-#pragma unroll
-    for (int h = 0; h < 4; h++) {
-      float gr[4];
-#pragma unroll
-      for (int j = 0; j <= h; j++) gr[j] = h < r ? gram[h * RM + j] : 0.0f;
-#pragma unroll
-      for (int j = 0; j < h; j++) {
-        float s = gr[j];
-#pragma unroll
-        for (int m = 0; m < j; m++) s = fmaf(-l[h][m], l[j][m], s);
-        l[h][j] = s * iv[j];
-      }
-      float d = gr[h];
-#pragma unroll
-      for (int m = 0; m < h; m++) d = fmaf(-l[h][m], l[h][m], d);
-      const bool ok = gr[h] >= 1e-30f && d > 1e-6f * gr[h];
-      alive |= ok ? 1u << h : 0u;
-      iv[h] = ok ? 1.0f / sqrtf(d) : 0.0f;
-#pragma unroll
-      for (int j = 0; j < h; j++) x[h] = fmaf(-l[h][j], x[j], x[h]);
-      x[h] = x[h] * iv[h];
-    }
-    __syncthreads();                         // (two threads share an element of X)
-  } else {
+  if constexpr (RM > 4) {
     if (tid < 32) cholesky_lower_warp<RM>(gram, r, chol, tid);
     __syncthreads();
-    const float *iv = chol + RM * RM;
+  }
+  if (tid < D) {
+    uint32_t alive = 0;
+    float x[RM];
 #pragma unroll
-    for (int h = 0; h < RM; h++) {
-      if (h < r) {
+    for (int h = 0; h < RM; h++) x[h] = h < r ? X[h * D + i] : 0.0f;
+    if constexpr (RM <= 4) {
+      float l[4][4], iv[4];
 #pragma unroll
-        for (int j = 0; j < h; j++) x[h] = fmaf(-chol[h * RM + j], x[j], x[h]);
+      for (int h = 0; h < 4; h++) {
+        float gr[4];
+#pragma unroll
+        for (int j = 0; j <= h; j++) gr[j] = h < r ? gram[h * RM + j] : 0.0f;
+#pragma unroll
+        for (int j = 0; j < h; j++) {
+          float s = gr[j];
+#pragma unroll
+          for (int m = 0; m < j; m++) s = fmaf(-l[h][m], l[j][m], s);
+          l[h][j] = s * iv[j];
+        }
+        float d = gr[h];
+#pragma unroll
+        for (int m = 0; m < h; m++) d = fmaf(-l[h][m], l[h][m], d);
+        const bool ok = gr[h] >= 1e-30f && d > 1e-6f * gr[h];
+        alive |= ok ? 1u << h : 0u;
+        iv[h] = ok ? 1.0f / sqrtf(d) : 0.0f;
+#pragma unroll
+        for (int j = 0; j < h; j++) x[h] = fmaf(-l[h][j], x[j], x[h]);
         x[h] = x[h] * iv[h];
-        alive |= iv[RM + h] != 0.0f ? 1u << h : 0u;
+      }
+    } else {
+      const float *iv = chol + RM * RM;
+#pragma unroll
+      for (int h = 0; h < RM; h++) {
+        if (h < r) {
+#pragma unroll
+          for (int j = 0; j < h; j++) x[h] = fmaf(-chol[h * RM + j], x[j], x[h]);
+          x[h] = x[h] * iv[h];
+          alive |= iv[RM + h] != 0.0f ? 1u << h : 0u;
+        }
       }
     }
-  }
-  LQ_BTICK(8);
-  if (tid < D) {
+    LQ_BTICK(8);
 #pragma unroll
     for (int h = 0; h < RM; h++) {
       if (h < r) {
@@ -263,47 +278,41 @@ __device__ __forceinline__ uint32_t orthonormalize(float *X, int r, float *gram,
         X[h * D + i] = out;
       }
     }
+    if (FINAL && tid == 0) alive_mask = alive;
   }
   __syncthreads();
-  return alive;
+  return FINAL ? alive_mask : 0u;
 }
 
 // MODE 0 flush (window representation -> dense -> new window representation), 1 quantize dense fp32 states,
 // 2 dequantize to dense fp32 states.  RM: the largest r the instance handles; 0: no compensators at all (an instance of its
 // own: told apart inside the others, the two ways cost 400 bytes of spills).
-template <int GATE, int MODE, bool R16, int RM>
-__global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
-  constexpr bool DIAG = GATE == LQ_GATE_DIAG, SLOT = MODE != 1;
+// BF16: the per-window BF16 state (lq_shape.state_bf16, RM = 0): the dense state is rounded to bfloat16, and that is all.
+// slots: 1 or 2.
+template <int GATE, int MODE, bool R16, int RM, bool BF16>
+__global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const int slots) {
+  constexpr bool DIAG = GATE == LQ_GATE_DIAG, RECORDS = MODE != 1, STAGED = MODE != 1 || RM <= 8;
+  static_assert(!BF16 || RM == 0, "the per-window BF16 state has no compensators");
   constexpr int RF = record_floats(DIAG);
   using rec_t = typename std::conditional<R16, __half, float>::type;
   using Lay = BoundarySmem<RM>;
   extern __shared__ __align__(128) unsigned char lq_bsm[];
   __shared__ unsigned todo_bh[32];
   __shared__ int todo_n[32], todo_count, any_due;
-  const int W = p.W, r = p.r, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 1, tx = lane & 1;
+  const int W = p.W, r = RM > 0 ? p.r : 0, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 1, tx = lane & 1;
   const int v0 = 16 * warp + 8 * tx;         // the lane's first column
   if (RM > 0 && r < 1) return;               // (not launched)
   const unsigned nh = static_cast<unsigned>(p.batch) * p.heads_v;
-  const Lay L(W, r, DIAG, R16, SLOT, p.n_iter > 1);
-  rec_t *rec = reinterpret_cast<rec_t *>(lq_bsm + L.rec);
+  const Lay L(MODE, W, r, DIAG, R16, BF16, RM > 0 && p.n_iter > 1, slots);
   float *dec = reinterpret_cast<float *>(lq_bsm + L.dec), *gam = reinterpret_cast<float *>(lq_bsm + Lay::gam);
-  const uint8_t *zt = lq_bsm + Lay::head + HB_CODES;
-  const float *ss = reinterpret_cast<const float *>(lq_bsm + Lay::head + HB_COL_SCALE);
-  const float *cs = reinterpret_cast<const float *>(lq_bsm + Lay::head + HB_ROW_SMOOTH);
-  const uint16_t *ckh = reinterpret_cast<const uint16_t *>(lq_bsm + Lay::head + HB_COMP_K), *cuh = ckh + r * D;
   float *part = reinterpret_cast<float *>(lq_bsm + Lay::part), *T = reinterpret_cast<float *>(lq_bsm + Lay::T);
   float *Wv = reinterpret_cast<float *>(lq_bsm + L.Wv), *gram = reinterpret_cast<float *>(lq_bsm + Lay::gram);
   float *chol = reinterpret_cast<float *>(lq_bsm + Lay::chol), *ub = reinterpret_cast<float *>(lq_bsm + Lay::ub) + warp * 16 * RM;
   float *ic_s = reinterpret_cast<float *>(lq_bsm + Lay::ic), *invc = reinterpret_cast<float *>(lq_bsm + Lay::invc) + 16 * warp;
   const uint32_t bar = smem_addr(lq_bsm + Lay::bar);
   const bool wide = (reinterpret_cast<uintptr_t>(p.S) & 31) == 0;
-  auto kd_row = [&](int j) -> float * {      // Gamma_{j+1:n} kt_j
-    if constexpr (R16) return reinterpret_cast<float *>(lq_bsm + L.kd) + j * D;
-    else return rec + j * RF + REC_KT;
-  };
-
   LQ_STAMP(1, 0);
-  if (SLOT && tid == 0) mbar_init(bar, 1);
+  if (STAGED && tid == 0) { mbar_init(bar, 1); mbar_init(bar + 8, 1); }
   grid_dependency_wait();                    // everything the kernel before this one wrote is visible from here on
   LQ_STAMP(1, 1);
 #ifdef LQ_TIMING
@@ -312,15 +321,23 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
   // the decode kernel ahead of a flush counts the tickets of its pool of heads in the state's scratch words
   if (MODE == 0 && p.work != nullptr && blockIdx.x == 0 && tid == 0) p.work[0] = 0;
 
-  uint32_t parity = 0;
+  uint32_t parity = 0;                       // bit b: phase of copy barrier b
+  int at = 0;                                // the slot of the head at hand
   float dec_next = 0.0f;                     // this thread's decay of the head on its way (scalar gate, tid < n)
-  auto request = [&](size_t bh, int n) {     // bring head bh and its n records into the slot
-    if (!DIAG && tid < n) dec_next = p.decays[bh * (size_t)W + tid];
-    if (tid == 0) {
-      const uint32_t rb = static_cast<uint32_t>(sizeof(rec_t)) * RF * n;
-      mbar_expect_tx(bar, head_bytes(r) + rb);
-      bulk_g2s(smem_addr(lq_bsm + Lay::head), p.head(bh), head_bytes(r), bar);
-      if (n > 0) bulk_g2s(smem_addr(lq_bsm + L.rec), p.record<rec_t>(bh, 0, DIAG), rb, bar);
+  auto request = [&](size_t bh, int n, int to) {             // bring head bh and its n records, or its dense state, into slot `to`
+    const uint32_t dst = smem_addr(lq_bsm + Lay::head) + to * L.slot, bar_to = bar + 8 * to;
+    if constexpr (RECORDS) {
+      if (!DIAG && tid < n) dec_next = p.decays[bh * (size_t)W + tid];
+      if (tid == 0) {
+        const uint32_t rb = static_cast<uint32_t>(sizeof(rec_t)) * RF * n;
+        mbar_expect_tx(bar_to, L.rec + rb);
+        bulk_g2s(dst, p.heads + bh * (size_t)L.rec, L.rec, bar_to);
+        if (n > 0) bulk_g2s(dst + L.rec, p.record<rec_t>(bh, 0, DIAG), rb, bar_to);
+      }
+    } else if (warp == 0) {
+      if (lane == 0) mbar_expect_tx(bar_to, 4 * D * D);
+      __syncwarp();
+      if (lane < 16) bulk_g2s(dst + dense_group_at(lane), p.S + bh * (size_t)(D * D) + lane * 8 * D, 8 * D * 4, bar_to);
     }
   };
 
@@ -344,7 +361,7 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
     }
     __syncthreads();
     count = todo_count;
-    if (SLOT && count > 0) request(todo_bh[0], todo_n[0]);
+    if (STAGED && count > 0) request(todo_bh[0], todo_n[0], at);
     // one warp reports that this CTA has seen all of win_pos, once the first head's copies are on their way (the round
     // trip hides behind them); with nothing due there is nothing to restart
     if (MODE == 0 && count < 32 && any_due > 0 && warp == 7) restart_due_windows(p, lane);
@@ -353,11 +370,20 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
     for (int k = 0; k < count; k++) {
       const size_t bh = todo_bh[k];
       if (MODE == 0 && p.overlap && count < 32 && k == count - 1) grid_dependents_may_start();
-      const int n = todo_n[k];
-      if (SLOT) {
-        if (!DIAG && tid < n) dec[tid] = dec_next;
-        if (!mbar_wait(bar, parity) && lane == 0) atomicOr(&g_device_error, 1);
-        parity ^= 1u;
+      const int n = MODE == 0 ? max(todo_n[k], 1) : todo_n[k];          // (never 0 when due)
+      unsigned char *slot = lq_bsm + Lay::head + at * L.slot;
+      rec_t *rec = reinterpret_cast<rec_t *>(slot + L.rec);
+      auto kd_row = [&](int j) -> float * {                   // Gamma_{j+1:n} kt_j
+        if constexpr (R16) return reinterpret_cast<float *>(lq_bsm + L.kd) + j * D;
+        else return rec + j * RF + REC_KT;
+      };
+      if (RECORDS && !DIAG && tid < n) dec[tid] = dec_next;
+      if (STAGED) {
+        if (slots > 1 && k + 1 < count) request(todo_bh[k + 1], todo_n[k + 1], at ^ 1);
+        if (!mbar_wait(bar + 8 * at, (parity >> at) & 1u) && lane == 0) atomicOr(&g_device_error, 1);
+        parity ^= 1u << at;
+      }
+      if (RECORDS) {
         if (!DIAG) __syncthreads();
         if (k == 0) LQ_STAMP(1, 2);
         LQ_BTICK(1);
@@ -383,12 +409,23 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
 
       float2 M[8][4];                                         // rows 8 ty + a, columns v0 + 2 c, v0 + 2 c + 1
       // ---- the dense state (Eq. 7) ----
-      if constexpr (SLOT) {
-        {
+      if constexpr (RECORDS) {
+        const uint8_t *zt = slot + HB_CODES;
+        const uint16_t *ckh = reinterpret_cast<const uint16_t *>(slot + HB_COMP_K), *cuh = ckh + r * D;
+        if constexpr (BF16) {
+#pragma unroll
+          for (int c = 0; c < 4; c++) {
+            float lo[8], hi[8];                               // columns v0 + 2 c, v0 + 2 c + 1
+            load8_bf16(reinterpret_cast<const uint16_t *>(slot) + (v0 + 2 * c) * D + 8 * ty, lo);
+            load8_bf16(reinterpret_cast<const uint16_t *>(slot) + (v0 + 2 * c + 1) * D + 8 * ty, hi);
+#pragma unroll
+            for (int a = 0; a < 8; a++) M[a][c] = make_float2(lo[a], hi[a]);
+          }
+        } else {
           float ci[8];
           float2 sj[4];
-          load8(cs + 8 * ty, ci);
-          load8p(ss + v0, sj);
+          load8(reinterpret_cast<const float *>(slot + HB_ROW_SMOOTH) + 8 * ty, ci);
+          load8p(reinterpret_cast<const float *>(slot + HB_COL_SCALE) + v0, sj);
           uint2 zz[8];
 #pragma unroll
           for (int b = 0; b < 8; b++) {
@@ -432,6 +469,10 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
           rank1_pairs(M, kj, uj);
         }
         LQ_BTICK(3);
+      } else if constexpr (STAGED) {
+        const float *S = reinterpret_cast<const float *>(slot + dense_group_at(ty)) + v0;
+#pragma unroll
+        for (int a = 0; a < 8; a++) load8p(S + a * D, M[a]);
       } else {
         const float *S = p.S + bh * (size_t)(D * D) + 8 * ty * D + v0;
 #pragma unroll
@@ -441,12 +482,12 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
         float *S = p.S + bh * (size_t)(D * D) + 8 * ty * D + v0;
 #pragma unroll
         for (int a = 0; a < 8; a++) store_row8(S + a * D, wide, M[a]);
-      } else {
+      } else if constexpr (RM > 0) {
         // T_h = S w_h; w_h is the value side of the (h+1)-th newest record, or Walsh function h
 #pragma unroll 2
         for (int h = 0; h < r; h++) {
           float2 w[4];
-          if (SLOT && h < n) {
+          if (RECORDS && h < n) {
             load8p(rec + (n - 1 - h) * RF + REC_U + v0, w);
           } else {
 #pragma unroll
@@ -459,13 +500,28 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p) {
         }
       }
       // the slot is free when all have come here: the next head may land while this one is worked on
-      if (SLOT) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      if (STAGED) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
       __syncthreads();
-      if (SLOT && k + 1 < count) request(todo_bh[k + 1], todo_n[k + 1]);
-      if (MODE == 1 && k + 1 < count && tid < 8)              // (dense states: at least into the L2)
+      if (STAGED && slots == 1 && k + 1 < count) request(todo_bh[k + 1], todo_n[k + 1], at);
+      if (!STAGED && k + 1 < count && tid < 8)                // (dense states: at least into the L2)
         bulk_prefetch_l2(p.S + todo_bh[k + 1] * (size_t)(D * D) + tid * (D * D / 8), D * D / 2);
+      if (slots > 1) at ^= 1;
 
-      if constexpr (MODE != 2) {
+      if constexpr (BF16 && MODE != 2) {                      // round and store: that is the new boundary state
+        uint16_t *S0T = reinterpret_cast<uint16_t *>(p.heads + bh * (size_t)BF16W_HEAD_BYTES) + v0 * D + 8 * ty;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          uint32_t lo[4], hi[4];
+#pragma unroll
+          for (int e = 0; e < 4; e++) {
+            lo[e] = (uint32_t)to_bf16_bits(M[2 * e][c].x) | ((uint32_t)to_bf16_bits(M[2 * e + 1][c].x) << 16);
+            hi[e] = (uint32_t)to_bf16_bits(M[2 * e][c].y) | ((uint32_t)to_bf16_bits(M[2 * e + 1][c].y) << 16);
+          }
+          *reinterpret_cast<uint4 *>(S0T + (2 * c) * D) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+          *reinterpret_cast<uint4 *>(S0T + (2 * c + 1) * D) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        }
+        if (MODE == 1 && tid == 0) p.win_pos[bh / p.heads_v] = 0;
+      } else if constexpr (MODE != 2) {
         uint32_t alive = 0;
         if constexpr (RM > 0) {
           for (int idx = tid; idx < r * D; idx += 256) T[idx] = sum_warps(part + idx, RM * D);
