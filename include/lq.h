@@ -177,8 +177,8 @@ lq_status lq_decode_step_host(const lq_shape *shape, const lq_state *state, cons
  * starts and ends in device memory; this is a convenience of the library for callers whose tokens arrive in
  * host memory.)  The batch is cut into two sub-batches of whole sequences.  The inputs of both are brought in
  * on a copy-in stream, so the second sub-batch arrives while the first is computed; o of a sub-batch is
- * complete after its decode kernel and is copied out on a copy-out stream while the window-boundary kernel of
- * that sub-batch and the next sub-batch run.  The two side streams are created per device at the first call
+ * complete after its decode kernel and is copied out on a copy-out stream while the next sub-batch and the window
+ * boundaries (one launch for the whole batch) run.  The two side streams are created per device at the first call
  * (make that call outside any stream capture) and are tied to `stream` by events on both sides: the call
  * starts after everything already enqueued on `stream`, and anything enqueued on `stream` afterwards starts
  * after the last copy.  Same arguments, staging size, results and error codes as lq_decode_step_host; use

@@ -395,7 +395,8 @@ extern "C" {
 
 static lq_status decode_step_impl(const lq_shape *shape, const lq_state *state, const uint16_t *q, const uint16_t *k,
                                   const uint16_t *v, const uint16_t *beta, const uint16_t *alpha, float *o,
-                                  lq_stream stream, cudaEvent_t between) {
+                                  lq_stream stream, cudaEvent_t between, int part = -1) {
+  // part >= 0: the decode kernel only, of sub-batch `part` (each of them counts its tickets in a word of its own)
   lq_status rc = check_shape(shape);
   if (rc != LQ_OK) return rc;
   if ((rc = check_state(shape, state, true)) != LQ_OK) return rc;
@@ -411,13 +412,14 @@ static lq_status decode_step_impl(const lq_shape *shape, const lq_state *state, 
   const long nh = (long)shape->batch * shape->heads_v;
   p.overlap = nh >= 2L * sm_count() * shape->W;        // as many boundaries as boundary CTAs, on average
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (part > 0 && p.work) p.work += part;
   rc = shape->state_bf16 ? launch_decode<true>(shape, p, st) : launch_decode<false>(shape, p, st);
   if (rc != LQ_OK) return rc;
   if (between && cudaEventRecord(between, st) != cudaSuccess) {
     cudaGetLastError();
     return LQ_ERR_CUDA;
   }
-  return launch_boundary<0>(shape, p, st);     // sequences whose window just became full
+  return part >= 0 ? LQ_OK : launch_boundary<0>(shape, p, st);     // sequences whose window just became full
 }
 
 lq_status lq_decode_step(const lq_shape *shape, const lq_state *state, const uint16_t *q, const uint16_t *k,
@@ -569,6 +571,7 @@ lq_status lq_decode_step_host(const lq_shape *shape, const lq_state *state, cons
 // ---------------------------------------------------------------------------------------------
 namespace {
 constexpr int PIPE_CHUNKS = 2;
+static_assert(PIPE_CHUNKS <= LQ_WORK_WORDS, "a ticket counter each");
 struct HostPipe {
   bool ready = false;
   cudaStream_t s_in = nullptr, s_out = nullptr;
@@ -698,7 +701,8 @@ lq_status lq_decode_step_host_pipelined(const lq_shape *shape, const lq_state *s
     ok = ok && cudaEventRecord(hp->in[c], hp->s_in) == cudaSuccess;
   }
   // Kernels on `stream`, sub-batch after sub-batch.  o of a sub-batch is complete after its decode kernel, so
-  // its copy to the host starts there, next to the window-boundary kernel, which does not touch o.
+  // its copy to the host starts there.  The window boundaries come last, in one launch for the whole batch: between the
+  // sub-batches they would hold up the second one's decode kernel.
   for (int c = 0; ok && c < PIPE_CHUNKS; c++) {
     const uint64_t b0 = lo[c], nb = lo[c + 1] - lo[c];
     if (nb == 0) continue;
@@ -712,10 +716,14 @@ lq_status lq_decode_step_host_pipelined(const lq_shape *shape, const lq_state *s
     if (ss.decays) ss.decays += b0 * Hv * shape->W;
     ss.win_pos += b0;
     rc = decode_step_impl(&sub, &ss, q_d + b0 * eqk, k_d + b0 * eqk, v_d + b0 * ev, b_d + b0 * eb, a_d + b0 * ea,
-                          o_d + b0 * ev, stream, hp->done[c]);
+                          o_d + b0 * ev, stream, hp->done[c], c);
     if (rc != LQ_OK) break;
     ok = cudaStreamWaitEvent(hp->s_out, hp->done[c], 0) == cudaSuccess &&
          cudaMemcpyAsync(o_h + b0 * ev, o_d + b0 * ev, 4 * nb * ev, cudaMemcpyDeviceToHost, hp->s_out) == cudaSuccess;
+  }
+  if (ok && rc == LQ_OK) {                   // the windows that became full, of all sub-batches together
+    Params p = make_params(shape, state);
+    rc = launch_boundary<0>(shape, p, st);
   }
   // join: whatever was put on the side streams is waited for by `stream`, also after an error above
   // (`stream` has waited for every copy-in of this call already, sub-batch by sub-batch, unless an error cut the

@@ -318,8 +318,8 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const 
 #ifdef LQ_TIMING
   if (tid == 0) { for (int i = 0; i < 16; i++) lq_bacc[i] = 0; lq_btick = clock64(); }
 #endif
-  // the decode kernel ahead of a flush counts the tickets of its pool of heads in the state's scratch words
-  if (MODE == 0 && p.work != nullptr && blockIdx.x == 0 && tid == 0) p.work[0] = 0;
+  // the decode kernels ahead of a flush count the tickets of their pools of heads in the state's scratch words
+  if (MODE == 0 && p.work != nullptr && blockIdx.x == 0 && tid < LQ_WORK_WORDS) p.work[tid] = 0;
 
   uint32_t parity = 0;                       // bit b: phase of copy barrier b
   int at = 0;                                // the slot of the head at hand
