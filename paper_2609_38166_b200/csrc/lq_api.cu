@@ -692,7 +692,10 @@ lq_status lq_decode_step_host_pipelined(const lq_shape *shape, const lq_state *s
         g.dst[i] = reinterpret_cast<uint4 *>(dst_d[i] + b0 * per_seq[i]);
         g.units[i] = static_cast<uint32_t>((2 * nb * per_seq[i] + 15) / 16);
       }
-      ok = launch(gather_kernel, sm_count() / 2, 256, 0, hp->s_in, g) == LQ_OK;
+      // Sixteen CTAs (262 KB in flight, which the bus does not need more of): each of them keeps a decode CTA of the other
+      // sub-batch waiting for its place.  256 x 32 heads: 202 us a call by itself and 151 chained; with 74 CTAs 210 and 158
+      // (the decode kernel of half a batch took 43 us instead of 24), with 8 CTAs 222 and 172.
+      ok = launch(gather_kernel, 16, 256, 0, hp->s_in, g) == LQ_OK;
     } else {
       for (int i = 0; ok && i < 5; i++)
         ok = cudaMemcpyAsync(dst_d[i] + b0 * per_seq[i], src_h[i] + b0 * per_seq[i], 2 * nb * per_seq[i],
