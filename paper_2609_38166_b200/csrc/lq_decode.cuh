@@ -45,7 +45,7 @@ __host__ __device__ constexpr int rec_seg(bool rec16) { return rec16 ? 12 : 8; }
 // ---- shared-memory slot of one CTA ----
 struct DecodeSlot {
   // byte offsets inside the slot; every region starts on a 16-byte boundary
-  int head, rec, bas, digits, y, pk, pq, mbar, bytes;
+  int head, rec, bas, digits, y, pj, pk, pq, mbar, bytes;
   __host__ __device__ DecodeSlot(int W, int r, bool diag, bool rec16, bool bf16, int seg) {
     // a window holds at most W-1 records when a token arrives; seg > 0: two segments of that many at a time
     const int rows = seg > 0 ? 2 * seg : W > 1 ? W - 1 : 1;
@@ -55,6 +55,7 @@ struct DecodeSlot {
     bas = o; o += diag ? 0 : 2 * 4 * MAX_W;         // scalar gate: the records' decays, one copy per warp
     digits = o; o += 8 * D;               // digit planes: plane 4v+d = digit d of vector v (0: k, 1: q); bf16: record terms
     y = o; o += 2 * 4 * D;                // [2][128]: the rounded sums of the state stream, later the record terms
+    pj = o; o += 4 * 16;                  // [2][8]: projections of a group of records, on their way to all lanes of the dot warp
     pk = o; o += (4 * (r + 2) + 15) / 16 * 16;      // compensator projections against Gamma k
     pq = o; o += (4 * (r + 2) + 15) / 16 * 16;      // ... against Gamma q; pq[r], pq[r+1] hold kt^T q of alternate heads
     mbar = o; o += 32;                    // head block, records (two)
@@ -212,7 +213,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
   float *bas = reinterpret_cast<float *>(slot + L.bas) + role * MAX_W;   // this warp's copy of the decays
   int8_t *digits = reinterpret_cast<int8_t *>(slot + L.digits);
   float *y = reinterpret_cast<float *>(slot + L.y), *pk = reinterpret_cast<float *>(slot + L.pk);
-  float *pq = reinterpret_cast<float *>(slot + L.pq);
+  float *pq = reinterpret_cast<float *>(slot + L.pq), *pj = reinterpret_cast<float *>(slot + L.pj);
   const uint32_t barA = smem_addr(slot + L.mbar), barR = barA + 8, slot_a = smem_addr(slot);   // head block, records
 
   const unsigned nh = static_cast<unsigned>(p.batch) * p.heads_v, Hv = p.heads_v;
@@ -489,31 +490,27 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
             if (c == 0 && ho[u] < r) { pk[ho[u]] = s4[2 * u]; pq[ho[u]] = s4[2 * u + 1]; }
         }
       };
-      float rk_rec[4] = {0.0f, 0.0f, 0.0f, 0.0f}, rq_rec[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      // The record terms sum_j u_j (kt_j^T Gamma k) and the same for q, channels 4 lane .. 4 lane + 3, as one chain from the
+      // newest record back.
+      float2 rk_rec[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}}, rq_rec[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
       int base = seg_base(n);                        // the segment at hand begins with record `base`
       const rec_t *seg = rec + buf * SEG * RF;       // and lies here
-      for (int jt = n - 1; jt >= 0; jt -= 4) {       // records jt, jt-1, jt-2, jt-3
-        if (LONGW && jt < base) {                    // the segment is walked: on to the one before it
-          __syncwarp();
-          if (DIAG) named_wait(4 + buf);             // (the stream warp has taken this segment's decays as well)
-          if (base > SEG) request_segment(bh, n, base - SEG, buf);      // (the one after that is on its way to the other half)
-          base = seg_base(base);
-          buf ^= 1;
-          seg = rec + buf * SEG * RF;
-          wait_records();
-        }
-        float s4[4];
-        int jo[2];
+      // 2 NP records jt, jt-1, ...: half 0 projects the first, third, ... of them, half 1 the others.  The sums over the sixteen
+      // lanes are taken by halving exchanges (eight values: 4 + 2 + 1 + 1 shuffles), after which a lane holds one of them;
+      // through pj every lane gets all.  Groups of four may run past record 0.
+      auto walk_group = [&](const int jt, auto np) {
+        constexpr int NP = decltype(np)::value;
+        float v[2 * NP];
 #pragma unroll
-        for (int u = 0; u < 2; u++) {
+        for (int u = 0; u < NP; u++) {
           // the decays of the two records of this pair; the half that owns the older one steps over the newer
           const int jn = jt - 2 * u, jold = jn - 1;  // newer, older
           float2 an[4], ao[4], gmine[4];
           if (DIAG) {
-            load8p(seg + ((jn > 0 ? jn : 0) - base) * RF + REC_A + 8 * c, an);
-            load8p(seg + ((jold > 0 ? jold : 0) - base) * RF + REC_A + 8 * c, ao);
+            load8p(seg + ((NP > 2 || jn > 0 ? jn : 0) - base) * RF + REC_A + 8 * c, an);
+            load8p(seg + ((NP > 2 || jold > 0 ? jold : 0) - base) * RF + REC_A + 8 * c, ao);
           } else {
-            const float2 x = pair(bas[jn > 0 ? jn : 0]), z = pair(bas[jold > 0 ? jold : 0]);
+            const float2 x = pair(bas[NP > 2 || jn > 0 ? jn : 0]), z = pair(bas[NP > 2 || jold > 0 ? jold : 0]);
 #pragma unroll
             for (int cc = 0; cc < 4; cc++) { an[cc] = x; ao[cc] = z; }
           }
@@ -523,38 +520,73 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
             gmine[cc] = half ? go : gn;
             // past both records; the chain stops at record 0, so that it ends as Gamma_{1:l} exactly
             // (selects: a branch for the last trip of a long head was slower)
-            g2[cc] = (!DIAG || jold >= 0) ? __fmul2_rn(go, ao[cc]) : (jn >= 0 ? go : gn);
+            g2[cc] = (NP > 2 || !DIAG || jold >= 0) ? __fmul2_rn(go, ao[cc]) : (jn >= 0 ? go : gn);
           }
-          jo[u] = jn - half;
-          const int j = jo[u] >= 0 ? jo[u] : 0;      // (record 0 is in the slot whenever an index runs below it)
+          const int jm = jn - half, j = NP > 2 || jm >= 0 ? jm : 0;  // (record 0 is in the slot whenever an index runs below it)
           float2 x2[4], yk2[4], yq2[4];
           load8p(seg + (j - base) * RF + REC_KT + 8 * c, x2);
 #pragma unroll
           for (int cc = 0; cc < 4; cc++) { yk2[cc] = __fmul2_rn(gmine[cc], k2[cc]); yq2[cc] = __fmul2_rn(gmine[cc], q2[cc]); }
-          s4[2 * u] = block8(x2, yk2);
-          s4[2 * u + 1] = block8(x2, yq2);
+          v[2 * u] = block8(x2, yk2);
+          v[2 * u + 1] = block8(x2, yq2);
         }
-        tree16x4(s4);
-        // The record terms sum_j u_j (kt_j^T Gamma k) and the same for q, channels 4 lane .. 4 lane + 3, as one
-        // chain from the newest record back.  Half 0 holds the projections of records jt and jt-2, half 1
-        // those of jt-1 and jt-3: swap them, then take the four records in order.
-        {
-          float oth[4];
+        // halving exchanges over lane bits 0, 1, (2), then plain ones; lane c ends with value `mine` of its half
+        const bool u0 = lane & 1, u1 = lane & 2, u2 = lane & 4;
+        float x;
+        int mine;
+        if constexpr (NP == 4) {
+          float x4[4], x2_[2];
 #pragma unroll
-          for (int e = 0; e < 4; e++) oth[e] = __shfl_xor_sync(FULL, s4[e], 16);
+          for (int e = 0; e < 4; e++) x4[e] = (u0 ? v[e + 4] : v[e]) + __shfl_xor_sync(FULL, u0 ? v[e] : v[e + 4], 1);
 #pragma unroll
-          for (int i4 = 0; i4 < 4; i4++) {
-            const int j = jt - i4;
-            if (j < 0) break;                                  // the same for every lane
-            const int u = i4 >> 1;
-            const bool mine = (i4 & 1) == half;
-            const float pkj = mine ? s4[2 * u] : oth[2 * u], pqj = mine ? s4[2 * u + 1] : oth[2 * u + 1];
-            const float4 u4 = load4(seg + (j - base) * RF + REC_U + 4 * lane);
-            rk_rec[0] = fmaf(u4.x, pkj, rk_rec[0]); rq_rec[0] = fmaf(u4.x, pqj, rq_rec[0]);
-            rk_rec[1] = fmaf(u4.y, pkj, rk_rec[1]); rq_rec[1] = fmaf(u4.y, pqj, rq_rec[1]);
-            rk_rec[2] = fmaf(u4.z, pkj, rk_rec[2]); rq_rec[2] = fmaf(u4.z, pqj, rq_rec[2]);
-            rk_rec[3] = fmaf(u4.w, pkj, rk_rec[3]); rq_rec[3] = fmaf(u4.w, pqj, rq_rec[3]);
-          }
+          for (int e = 0; e < 2; e++) x2_[e] = (u1 ? x4[e + 2] : x4[e]) + __shfl_xor_sync(FULL, u1 ? x4[e] : x4[e + 2], 2);
+          x = (u2 ? x2_[1] : x2_[0]) + __shfl_xor_sync(FULL, u2 ? x2_[0] : x2_[1], 4);
+          mine = (u0 ? 4 : 0) + (u1 ? 2 : 0) + (u2 ? 1 : 0);
+        } else {
+          float x2_[2];
+#pragma unroll
+          for (int e = 0; e < 2; e++) x2_[e] = (u0 ? v[e + 2] : v[e]) + __shfl_xor_sync(FULL, u0 ? v[e] : v[e + 2], 1);
+          x = (u1 ? x2_[1] : x2_[0]) + __shfl_xor_sync(FULL, u1 ? x2_[0] : x2_[1], 2);
+          x = x + __shfl_xor_sync(FULL, x, 4);
+          mine = (u0 ? 2 : 0) + (u1 ? 1 : 0);
+        }
+        x = x + __shfl_xor_sync(FULL, x, 8);
+        __syncwarp();                                // (the group before has been read)
+        if (c < 2 * NP) pj[(mine & 1) * 8 + (mine & ~1) + half] = x;     // pj[vector][record]
+        __syncwarp();
+        float pk_[2 * NP], pq_[2 * NP];
+#pragma unroll
+        for (int e = 0; e < NP / 2; e++) {
+          const float4 a = *reinterpret_cast<const float4 *>(pj + 4 * e), b = *reinterpret_cast<const float4 *>(pj + 8 + 4 * e);
+          pk_[4 * e] = a.x; pk_[4 * e + 1] = a.y; pk_[4 * e + 2] = a.z; pk_[4 * e + 3] = a.w;
+          pq_[4 * e] = b.x; pq_[4 * e + 1] = b.y; pq_[4 * e + 2] = b.z; pq_[4 * e + 3] = b.w;
+        }
+#pragma unroll
+        for (int e = 0; e < 2 * NP; e++) {
+          const int j = jt - e;
+          if (NP == 2 && j < 0) break;               // the same for every lane
+          const float4 u4 = load4(seg + (j - base) * RF + REC_U + 4 * lane);
+          const float2 lo = make_float2(u4.x, u4.y), hi = make_float2(u4.z, u4.w), pk2 = pair(pk_[e]), pq2 = pair(pq_[e]);
+          rk_rec[0] = __ffma2_rn(lo, pk2, rk_rec[0]); rq_rec[0] = __ffma2_rn(lo, pq2, rq_rec[0]);
+          rk_rec[1] = __ffma2_rn(hi, pk2, rk_rec[1]); rq_rec[1] = __ffma2_rn(hi, pq2, rq_rec[1]);
+        }
+      };
+      for (int jt = n - 1; jt >= 0;) {
+        if (LONGW && jt < base) {                    // the segment is walked: on to the one before it
+          __syncwarp();
+          if (DIAG) named_wait(4 + buf);             // (the stream warp has taken this segment's decays as well)
+          if (base > SEG) request_segment(bh, n, base - SEG, buf);      // (the one after that is on its way to the other half)
+          base = seg_base(base);
+          buf ^= 1;
+          seg = rec + buf * SEG * RF;
+          wait_records();
+        }
+        if (jt - 7 >= base) {
+          walk_group(jt, std::integral_constant<int, 4>{});
+          jt -= 8;
+        } else {
+          walk_group(jt, std::integral_constant<int, 2>{});
+          jt -= 4;
         }
       }
       const int walked = 4 + buf;                    // the barrier of the last segment
@@ -577,8 +609,8 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         wait_for(barA, parA);
         bf16_columns(reinterpret_cast<const uint16_t *>(zt), 64, xk, xq, y, lane);
         float *terms = reinterpret_cast<float *>(digits);
-        *reinterpret_cast<float4 *>(terms + 4 * lane) = make_float4(rk_rec[0], rk_rec[1], rk_rec[2], rk_rec[3]);
-        *reinterpret_cast<float4 *>(terms + D + 4 * lane) = make_float4(rq_rec[0], rq_rec[1], rq_rec[2], rq_rec[3]);
+        *reinterpret_cast<float4 *>(terms + 4 * lane) = make_float4(rk_rec[0].x, rk_rec[0].y, rk_rec[1].x, rk_rec[1].y);
+        *reinterpret_cast<float4 *>(terms + D + 4 * lane) = make_float4(rq_rec[0].x, rq_rec[0].y, rq_rec[1].x, rq_rec[1].y);
         if (draws && lane == 0) *qidx = ticket;
         __syncwarp();
         named_arrive(1);                     // (this warp is done with the head block as well)
@@ -605,8 +637,8 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         if (wanted(n_next)) request_records(bh_next, n_next);
       }
       named_wait(2);                         // the stream warp has taken its sums out of y
-      *reinterpret_cast<float4 *>(y + 4 * lane) = make_float4(rk_rec[0], rk_rec[1], rk_rec[2], rk_rec[3]);
-      *reinterpret_cast<float4 *>(y + D + 4 * lane) = make_float4(rq_rec[0], rq_rec[1], rq_rec[2], rq_rec[3]);
+      *reinterpret_cast<float4 *>(y + 4 * lane) = make_float4(rk_rec[0].x, rk_rec[0].y, rk_rec[1].x, rk_rec[1].y);
+      *reinterpret_cast<float4 *>(y + D + 4 * lane) = make_float4(rq_rec[0].x, rq_rec[0].y, rq_rec[1].x, rq_rec[1].y);
       if (draws && lane == 0) *qidx = ticket;
       __syncwarp();
       named_arrive(1);                       // the record terms are in shared memory (and the ticket)
