@@ -335,12 +335,12 @@ template <int GATE, bool R16, bool BF16>
 static lq_status launch_decode_t(const lq_shape *s, const Params &p, cudaStream_t stream) {
   const bool diag = GATE == LQ_GATE_DIAG;
   const int whole = DecodeSlot(s->W, s->r, diag, R16, BF16, 0).bytes, ring = DecodeSlot(s->W, s->r, diag, R16, BF16, rec_seg(R16)).bytes;
-  // The records of a head at once, or in segments through a smaller slot: in segments where that lets an SM hold a third more
-  // CTAs (of six, which the registers allow).  At 256 x 32 heads, fp32 records, scalar gate: W = 32 (4 or 5 CTAs) 78.6 us per
-  // step at once, 79.4 in segments; W = 40 (3 or 5) 100.5 and 89.1; diagonal gate: W = 24 (4 or 4) 83.6 and 88.0, W = 32
-  // (3 or 4) 98.7 and 92.7; fp16 records, W = 64 (4 or 6) 116 and 112.
+  // The records of a head at once, or in segments through a smaller slot: in segments where an SM holds no more than three
+  // CTAs otherwise.  At 256 x 32 heads, us per step at once / in segments: scalar gate, fp32 records: W = 32 (4 or 5 CTAs)
+  // 70.3 / 73.7, W = 40 (3 or 5) 86.5 / 81.3, W = 64 (2 or 5) 129 / 104; fp16 records, W = 64 (4 or 6) 99.1 / 101.7;
+  // diagonal gate, fp32: W = 24 (4 or 4) 78.4 / 83.6, W = 32 (3 or 4) 86.8 / 85.6, W = 64 (2 or 4) 224 / 116.
   auto ctas = [](int bytes) { return std::min(6, 228 * 1024 / (bytes + 1024)); };
-  const bool longw = s->W - 1 > 2 * rec_seg(R16) && 3 * ctas(ring) >= 4 * ctas(whole);
+  const bool longw = s->W - 1 > 2 * rec_seg(R16) && ctas(whole) <= 3 && ctas(ring) > ctas(whole);
   const long nh = (long)s->batch * s->heads_v;
   return longw ? launch_persistent(decode_kernel<GATE, R16, true, BF16>, nh, 64, ring, stream, p)
                : launch_persistent(decode_kernel<GATE, R16, false, BF16>, nh, 64, whole, stream, p);
