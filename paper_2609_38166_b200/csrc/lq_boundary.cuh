@@ -289,8 +289,13 @@ __device__ __forceinline__ uint32_t orthonormalize(float *X, int r, float *gram,
 // own: told apart inside the others, the two ways cost 400 bytes of spills).
 // BF16: the per-window BF16 state (lq_shape.state_bf16, RM = 0): the dense state is rounded to bfloat16, and that is all.
 // slots: 1 or 2.
-template <int GATE, int MODE, bool R16, int RM, bool BF16>
+// EXACT: r is RM, known at compile time: without a test per vector the compiler interleaves the four or eight column sums
+// (flush at 256 x 32 heads: step 62.2 -> 61.4 us, W = 8 75.6 -> 74.4; quantizing spills with it, 57.5 -> 69.9 us).
+template <int GATE, int MODE, bool R16, int RM, bool BF16, bool EXACT>
 __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const int slots) {
+  // (exactly four vectors: registers are left for deeper unrolling, step 61.3 -> 60.8 us and 74.2 -> 73.0 at W = 8; for exactly
+  // eight it is slower, 234.3 -> 236.5 us at 512 x 32 heads, diagonal gate, W = 64)
+  constexpr bool FOUR = EXACT && RM == 4;
   constexpr bool DIAG = GATE == LQ_GATE_DIAG, RECORDS = MODE != 1, STAGED = MODE != 1 || RM <= 8;
   static_assert(!BF16 || RM == 0, "the per-window BF16 state has no compensators");
   constexpr int RF = record_floats(DIAG);
@@ -299,7 +304,7 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const 
   extern __shared__ __align__(128) unsigned char lq_bsm[];
   __shared__ unsigned todo_bh[32];
   __shared__ int todo_n[32], todo_count, any_due;
-  const int W = p.W, r = RM > 0 ? p.r : 0, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 1, tx = lane & 1;
+  const int W = p.W, r = EXACT ? RM : RM > 0 ? p.r : 0, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 1, tx = lane & 1;
   const int v0 = 16 * warp + 8 * tx;         // the lane's first column
   if (RM > 0 && r < 1) return;               // (not launched)
   const unsigned nh = static_cast<unsigned>(p.batch) * p.heads_v;
@@ -443,7 +448,7 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const 
               M[a][c] = __fmul2_rn(pair(ci[a]), __fmul2_rn(__fadd2_rn(raw, pair(-8388736.0f)), sj[c]));
             }
         }
-#pragma unroll 1
+#pragma unroll (FOUR ? 2 : 1)
         for (int h = 0; h < r; h++) {
           float kc[8];
           float2 uc[4];
@@ -459,7 +464,7 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const 
 #pragma unroll
             for (int c = 0; c < 4; c++) M[a][c] = __fmul2_rn(pair(gi[a]), M[a][c]);
         }
-        constexpr int AHEAD = MODE == 2 ? 1 : 2;              // (dequantizing spills with two records at a time)
+        constexpr int AHEAD = MODE == 2 ? 1 : FOUR ? 4 : 2;              // (dequantizing spills with two records at a time)
 #pragma unroll AHEAD
         for (int j = 0; j < n; j++) {
           float kj[8];
@@ -484,7 +489,7 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const 
         for (int a = 0; a < 8; a++) store_row8(S + a * D, wide, M[a]);
       } else if constexpr (RM > 0) {
         // T_h = S w_h; w_h is the value side of the (h+1)-th newest record, or Walsh function h
-#pragma unroll 2
+#pragma unroll (FOUR ? 4 : 2)
         for (int h = 0; h < r; h++) {
           float2 w[4];
           if (RECORDS && h < n) {
@@ -588,7 +593,7 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const 
           }
           __syncwarp();
           LQ_BTICK(14);
-#pragma unroll 1
+#pragma unroll (FOUR ? 2 : 1)
           for (int h = 0; h < r; h++) {                       // M -= k u^T with the stored values
             float kf[8];
             float2 uv[4];
