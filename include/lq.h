@@ -301,10 +301,10 @@ lq_status lq_ref_decode_step_bf16(const lq_shape *shape, uint16_t *S, const uint
 
 /*
  * Device-side error flags of the current device (0 = none), written to *flags (a host pointer).  Waits inside
- * the kernels are bounded; bit 0 is set when a decode warp gave up waiting for its asynchronous copies.  After
+ * the kernels are bounded; bit 0 is set when a warp gave up waiting for its asynchronous copies.  After
  * that, neither the outputs of that launch NOR THE STATE it worked on are valid (records may be missing or
- * half written): restore the state from a checkpoint.  Bits 1 and 2 belong to the optional fused step kernel
- * (gave up waiting for decode work / more heads than it can track), bit 3 to lq_selftest_bounded_wait.
+ * half written): restore the state from a checkpoint.  Bit 3 belongs to lq_selftest_bounded_wait; the
+ * others are not used.
  * The flags stay set until lq_clear_device_flags is called.  Both calls synchronise the device.
  */
 lq_status lq_check_device(int *flags);

@@ -8,11 +8,12 @@
 // scales, the codes - stays inside a warp, and only row sums (the products with the start vectors, the smoothing scales)
 // go through shared memory and a barrier.  Two CTAs fill the register file of an SM.
 //
-// What bounds it: a flush (W = 16, r = 4) takes 27 K cycles with two CTAs on the SM; 9 K of them are the fp32 pipes (about
-// 1150 packed FMAs per warp, two cycles each, four warps to a scheduler), the rest the waits between its dependent phases,
-// of which only the other CTA fills some.  Against tiles of 8 rows x 128 columns per half-warp, where every column sum
-// crossed the CTA (13 barriers a head, now 8), and copies by all threads into two staging buffers: 2048 dense states
-// quantized in 59.7 us (91.4 before), 2048 states dequantized in 48.4 us (54.0), 512 flushes 35.8 us (37.7).
+// What bounds it: a flush (W = 16, r = 4) takes 23 K cycles with two CTAs on the SM (27 K before two records and two start
+// vectors were in flight at a time); 9 K of them are the fp32 pipes (about 1150 packed FMAs per warp, two cycles each, four
+// warps to a scheduler), the rest the waits between its dependent phases, of which only the other CTA fills some.  Issue slots
+// are 41 % busy.  Against tiles of 8 rows x 128 columns per half-warp, where every column sum crossed the CTA (13 barriers a
+// head, now 8), and copies by all threads into two staging buffers: 2048 dense states quantized in 57.6 us (91.4 before),
+// 2048 states dequantized in 45.6 us (54.0); a step of 256 x 32 heads, 512 of them due, 73 -> 61 us.
 #pragma once
 #include <type_traits>
 

@@ -78,11 +78,6 @@ __device__ __forceinline__ uint16_t to_bf16_bits(float x) {
   return static_cast<uint16_t>(u >> 16);
 }
 
-// ---- asynchronous global -> shared copies (16 bytes each) ----
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-  unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
-}
 // L2 eviction priorities: lines that will not be read again soon / lines another kernel reads next
 __device__ __forceinline__ uint64_t l2_stream_policy() {
   uint64_t policy;
@@ -94,15 +89,6 @@ __device__ __forceinline__ uint64_t l2_keep_policy() {
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;\n" : "=l"(policy));
   return policy;
 }
-__device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
-  unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-// all but the most recently committed group have landed
-__device__ __forceinline__ void cp_async_wait_but_one() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-
 // ---- mbarrier / TMA bulk copy (1-D) ----
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 __device__ __forceinline__ void mbar_init(uint32_t bar, int count) {
@@ -308,31 +294,6 @@ __device__ __forceinline__ void store4(__half *dst, float a, float b, float c, f
   *reinterpret_cast<uint2 *>(dst) = make_uint2(pack2_f16_sat(a, b), pack2_f16_sat(c, d));
 }
 
-// Row sums.  In: p[a] = this thread's block result for row 8ty+a (block index tx).
-// Out: the full sum of row 8ty+sel, the same value in lanes tx and tx^8; sel depends on tx & 7 only.
-// Halving exchanges: after the step with mask m a lane keeps the rows whose partner-combined sums it owns.
-__device__ __forceinline__ float row_tree(const float (&p)[8], int lane, int &sel) {
-  float q4[4], q2[2], q1;
-  const bool u0 = lane & 1, u1 = lane & 2, u2 = lane & 4;
-#pragma unroll
-  for (int e = 0; e < 4; e++) {
-    const float keep = u0 ? p[e + 4] : p[e], send = u0 ? p[e] : p[e + 4];
-    q4[e] = keep + __shfl_xor_sync(FULL, send, 1);
-  }
-#pragma unroll
-  for (int e = 0; e < 2; e++) {
-    const float keep = u1 ? q4[e + 2] : q4[e], send = u1 ? q4[e] : q4[e + 2];
-    q2[e] = keep + __shfl_xor_sync(FULL, send, 2);
-  }
-  {
-    const float keep = u2 ? q2[1] : q2[0], send = u2 ? q2[0] : q2[1];
-    q1 = keep + __shfl_xor_sync(FULL, send, 4);
-  }
-  q1 = q1 + __shfl_xor_sync(FULL, q1, 8);
-  sel = (u0 ? 4 : 0) + (u1 ? 2 : 0) + (u2 ? 1 : 0);
-  return q1;
-}
-
 // Column sums.  In: p[b] = this thread's block result for column 8tx+b (block index ty).
 // part: 8*128 floats and out: 128 floats of shared memory.  Returns w[b] = full sum of column 8tx+b in
 // every thread.  Tree levels: ty^1 inside the warp (lane^16), then warps (0,1)(2,3)(4,5)(6,7), pairs of
@@ -372,20 +333,6 @@ __device__ __forceinline__ void col_blocks(const float (&M)[8][8], const float (
     p[b] = even + odd;
   }
 }
-// p[a] = block result over this thread's eight columns of  sum_b M[a][b] * x[b]
-__device__ __forceinline__ void row_blocks(const float (&M)[8][8], const float (&x)[8], float (&p)[8]) {
-#pragma unroll
-  for (int a = 0; a < 8; a++) {
-    float even = M[a][0] * x[0], odd = M[a][1] * x[1];
-#pragma unroll
-    for (int b = 2; b < 8; b += 2) {
-      even = fmaf(M[a][b], x[b], even);
-      odd = fmaf(M[a][b + 1], x[b + 1], odd);
-    }
-    p[a] = even + odd;
-  }
-}
-
 // ---- the heads that are due for a window boundary ----
 // Position of the k-th set bit of m (k < popc(m)).
 __device__ __forceinline__ int nth_set_bit(uint32_t m, unsigned k) {

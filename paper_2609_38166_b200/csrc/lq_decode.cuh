@@ -37,7 +37,7 @@
 namespace lq {
 
 // Long windows: the records come in segments of this many rows, newest first, two of which the slot holds at a time: while
-// one is walked the next is on its way (a multiple of four: the walk takes the records four at a time from the newest back).
+// one is walked the next is on its way (a multiple of four: the walk takes eight or four records at a time from the newest back).
 // Rows of 1 to 1.5 KB (fp32) and of half that (fp16); diagonal gate, W = 64, us per step at 256 x 32 heads: fp32 8 rows 132,
 // 4: 148, 12: 149, 16: 146; fp16 12 rows 125, 8: 130, 16: 123 (with records walked four at a time; eight at a time, 116 and 114).
 __host__ __device__ constexpr int rec_seg(bool rec16) { return rec16 ? 12 : 8; }

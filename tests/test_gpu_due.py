@@ -42,11 +42,12 @@ def test_boundaries_of_windows_in_any_order(oracle, batch, heads_v, heads_qk, W,
     assert st.win_pos.tolist() == [0] * batch and lq.check_device() == 0
 
 
+@pytest.mark.parametrize("r", [3, 12])
 @pytest.mark.parametrize("shift", [0, 4])
-def test_dense_states_at_any_16_byte_boundary(oracle, shift):
-    """Dense states are moved 32 bytes at a time where their base allows it; a base that is only 16-byte aligned
-    (`shift` floats into an allocation) takes the other branch.  Same bits."""
-    wl = synth.Workload("al", 3, 2, 1, W=5, r=3, seed=830)
+def test_dense_states_at_any_16_byte_boundary(oracle, shift, r):
+    """Dense states come by bulk copies (up to eight compensators) or are loaded, and stored, 32 bytes at a time where their
+    base allows it; a base that is only 16-byte aligned (`shift` floats into an allocation) takes the other branch."""
+    wl = synth.Workload("al", 3, 2, 1, W=5, r=r, seed=830)
     osh, lsh = gu.shapes(wl)
     S0 = synth.dense_states(wl, 3)
     ost = OState(osh)
