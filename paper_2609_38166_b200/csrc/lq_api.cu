@@ -369,6 +369,34 @@ static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStrea
   return launch_dependent(kernel, static_cast<int>(nh < resident ? nh : resident), 256, bytes(slots), stream, p, slots);
 }
 
+// A whole step of few heads in one launch, a CTA per head: as long as every SM has one head at most (a CTA takes most of an
+// SM's registers).  W = 16, r = 4, us per step in a graph as two launches / one: 1 head 6.7 / 5.1, 32 heads 6.7 / 5.2, 128 heads
+// 8.3 / 6.9, 148 heads of 37 sequences 13.8 / 12.7, 184 heads 14.5 / 14.5, 280 heads 14.2 / 16.1; 128 heads, diagonal gate,
+// W = 64, r = 8: 11.4 / 8.4; called one by one from the host, 1 to 128 heads: 11 / 8.4.
+static bool one_launch(const lq_shape *s) {
+  return (long)s->batch * s->heads_v <= sm_count();
+}
+template <int GATE, bool R16, int RM, bool BF16>
+static lq_status launch_step_t(const lq_shape *s, const Params &p, cudaStream_t stream) {
+  const bool diag = GATE == LQ_GATE_DIAG;
+  const int smem = std::max(BoundarySmem<RM>(0, s->W, s->r, diag, R16, BF16, RM > 0 && s->n_iter > 1, 1).bytes,
+                            TOKEN_SLOT + DecodeSlot(s->W, s->r, diag, R16, BF16, 0).bytes);
+  return launch_dependent(boundary_kernel<GATE, 0, R16, RM, BF16, false, true>, s->batch * s->heads_v, 256, smem, stream, p, 1);
+}
+template <int RM, bool BF16>
+static lq_status launch_step_gate(const lq_shape *s, const Params &p, cudaStream_t stream) {
+  if (s->gate == LQ_GATE_DIAG)
+    return s->rec16 ? launch_step_t<LQ_GATE_DIAG, true, RM, BF16>(s, p, stream) : launch_step_t<LQ_GATE_DIAG, false, RM, BF16>(s, p, stream);
+  return s->rec16 ? launch_step_t<LQ_GATE_SCALAR, true, RM, BF16>(s, p, stream) : launch_step_t<LQ_GATE_SCALAR, false, RM, BF16>(s, p, stream);
+}
+static lq_status launch_step(const lq_shape *s, const Params &p, cudaStream_t stream) {
+  if (s->state_bf16) return launch_step_gate<0, true>(s, p, stream);
+  if (s->r == 0) return launch_step_gate<0, false>(s, p, stream);
+  if (s->r <= 4) return launch_step_gate<4, false>(s, p, stream);
+  if (s->r <= 8) return launch_step_gate<8, false>(s, p, stream);
+  return launch_step_gate<MAX_R, false>(s, p, stream);
+}
+
 template <int MODE, int RM, bool BF16>
 static lq_status launch_boundary_gate(const lq_shape *s, const Params &p, cudaStream_t stream) {
   if (MODE == 1) return launch_boundary_t<LQ_GATE_SCALAR, MODE, false, RM, BF16>(s, p, stream);   // (reads no records)
@@ -414,6 +442,7 @@ static lq_status decode_step_impl(const lq_shape *shape, const lq_state *state, 
   const long nh = (long)shape->batch * shape->heads_v;
   p.overlap = nh >= 2L * sm_count() * shape->W;        // as many boundaries as boundary CTAs, on average
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (!between && part < 0 && one_launch(shape)) return launch_step(shape, p, st);
   if (part > 0 && p.work) p.work += part;
   rc = shape->state_bf16 ? launch_decode<true>(shape, p, st) : launch_decode<false>(shape, p, st);
   if (rc != LQ_OK) return rc;
@@ -952,7 +981,7 @@ int lq_debug_phase_cycles(unsigned long long *out) {
 }
 #endif
 
-int lq_decode_launches(const lq_shape *shape) { return check_shape(shape) == LQ_OK && shape->batch > 0 ? 2 : 0; }
+int lq_decode_launches(const lq_shape *shape) { return check_shape(shape) == LQ_OK && shape->batch > 0 ? one_launch(shape) ? 1 : 2 : 0; }
 
 const char *lq_status_string(lq_status status) {
   switch (status) {

@@ -18,6 +18,7 @@
 #include <type_traits>
 
 #include "lq_common.cuh"
+#include "lq_decode.cuh"
 
 namespace lq {
 
@@ -26,6 +27,7 @@ namespace lq {
 // products with the start vectors have been taken; with two of them the next head is asked for when this one is begun.
 // A dense state lies in groups of eight rows, DENSE_GROUP bytes apart and shifted against one another by 16-byte units, so
 // that the four row groups that a quarter of a warp reads at a time fall on different banks.
+constexpr int TOKEN_SLOT = 128;              // a step in one launch: where the slot of its token lies, behind the barriers
 constexpr int DENSE_GROUP = 8 * D * 4 + 128;
 __host__ __device__ constexpr int dense_group_at(int g) { return g * DENSE_GROUP + ((g & 1) ? 16 : 0) + ((g & 2) ? 64 : 0); }
 template <int RM>
@@ -292,8 +294,12 @@ __device__ __forceinline__ uint32_t orthonormalize(float *X, int r, float *gram,
 // slots: 1 or 2.
 // EXACT: r is RM, known at compile time: without a test per vector the compiler interleaves the four or eight column sums
 // (flush at 256 x 32 heads: step 62.2 -> 61.4 us, W = 8 75.6 -> 74.4; quantizing spills with it, 57.5 -> 69.9 us).
-template <int GATE, int MODE, bool R16, int RM, bool BF16, bool EXACT>
-__global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const int slots) {
+// STEP (a flush): a whole decode step of few heads in one launch.  Every CTA has one head: two of its warps take it through the
+// token (decode_slot), then, if that filled the window, the CTA through the boundary.  What bounds it: the latency of a token and
+// of a boundary, and the host time of a launch, of which it needs one instead of
+// two (figures: one_launch).
+template <int GATE, int MODE, bool R16, int RM, bool BF16, bool EXACT, bool STEP = false>
+__global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Params p, const int slots) {
   // (exactly four vectors: registers are left for deeper unrolling, step 61.3 -> 60.8 us and 74.2 -> 73.0 at W = 8; for exactly
   // eight it is slower, 234.3 -> 236.5 us at 512 x 32 heads, diagonal gate, W = 64)
   constexpr bool FOUR = EXACT && RM == 4;
@@ -319,13 +325,23 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const 
   const bool wide = (reinterpret_cast<uintptr_t>(p.S) & 31) == 0;
   LQ_STAMP(1, 0);
   if (STAGED && tid == 0) { mbar_init(bar, 1); mbar_init(bar + 8, 1); }
+  unsigned char *token_slot = lq_bsm + TOKEN_SLOT;     // (the boundary's arrays and slot take its place)
+  if constexpr (STEP) {
+    if (tid == 0) {
+      const uint32_t token_bar = smem_addr(token_slot + DecodeSlot(W, p.r, DIAG, R16, BF16, 0).mbar);
+      mbar_init(token_bar, 1);
+      mbar_init(token_bar + 8, 1);
+    }
+    __syncthreads();
+  }
   grid_dependency_wait();                    // everything the kernel before this one wrote is visible from here on
+  if (STEP) grid_dependents_may_start();     // (the next step's few CTAs find room beside these)
   LQ_STAMP(1, 1);
 #ifdef LQ_TIMING
   if (tid == 0) { for (int i = 0; i < 16; i++) lq_bacc[i] = 0; lq_btick = clock64(); }
 #endif
   // the decode kernels ahead of a flush count the tickets of their pools of heads in the state's scratch words
-  if (MODE == 0 && p.work != nullptr && blockIdx.x == 0 && tid < LQ_WORK_WORDS) p.work[tid] = 0;
+  if (MODE == 0 && !STEP && p.work != nullptr && blockIdx.x == 0 && tid < LQ_WORK_WORDS) p.work[tid] = 0;
 
   uint32_t parity = 0;                       // bit b: phase of copy barrier b
   int at = 0;                                // the slot of the head at hand
@@ -351,7 +367,26 @@ __global__ void __launch_bounds__(256, 2) boundary_kernel(const Params p, const 
   // gridDim-th head) and how many records each holds; then the CTA takes them one after the other.
   int count = 32;
   for (unsigned first = blockIdx.x; count == 32; first += 32 * gridDim.x) {
-    if (warp == 0) {
+    if constexpr (STEP) {
+      const int b = blockIdx.x / p.heads_v, n_in = p.win_pos[b] & 0xFFFF;
+      if (warp < 2) {
+        decode_slot<GATE, R16, false, BF16, true>(p, token_slot, lane, warp, blockIdx.x, gridDim.x);
+        asm volatile("fence.proxy.async;\n" ::: "memory");    // the record is written; a bulk copy may read it next
+      }
+      // (the barrier is where the whole CTA has read win_pos, ahead of its arrival)
+      const bool due = __syncthreads_or(n_in == W - 1 || n_in == W);
+      if (tid == 0) arrive_and_set(p.win_pos, b, p.heads_v, due ? 0 : n_in < W ? n_in + 1 : n_in);
+      if (!due) return;
+      if (tid == 0) {
+        const uint32_t token_bar = smem_addr(token_slot + DecodeSlot(W, p.r, DIAG, R16, BF16, 0).mbar);
+        mbar_inval(token_bar);
+        mbar_inval(token_bar + 8);
+        todo_bh[0] = blockIdx.x;
+        todo_n[0] = W;
+        todo_count = 1;
+        any_due = 0;
+      }
+    } else if (warp == 0) {
       unsigned bh_mine = first + lane * gridDim.x;
       int n_mine = 0, c, due = 0;
       if (MODE == 0) {

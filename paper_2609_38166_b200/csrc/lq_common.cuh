@@ -95,6 +95,7 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, int count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
   asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
 }
+__device__ __forceinline__ void mbar_inval(uint32_t bar) { asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(bar) : "memory"); }
 // The arrival that announces the bytes of the next copies.  Relaxed: nothing this thread wrote has to be
 // visible to anybody through this barrier (the copies' own completion is what the waiters acquire), and the
 // default release form stalls the warp for about 800 cycles here.

@@ -191,7 +191,8 @@ __device__ __forceinline__ void load_token(const Params &p, const HeadIdx h, int
 // segment drops out at compile time.
 // BF16: the per-window BF16 state (lq_shape.state_bf16): the head block is S0^T in bfloat16, its product with Gamma x is
 // taken in binary32 by both warps, half of the columns each; there are no scales and no compensators.
-template <int GATE, bool R16, bool LONGW, bool BF16>
+// ONCE: one head and no more, and the caller makes the window-position arrival.
+template <int GATE, bool R16, bool LONGW, bool BF16, bool ONCE = false>
 __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot, const int lane, const int role,
                                             const unsigned first, const unsigned G) {
   uint32_t parA = 0, parR = 0;               // phase of the head block's copy barrier; bit b: of the records' barrier b
@@ -286,9 +287,9 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
   // (barrier 1), and at the end of the trip both warps ask for that head's scalars, which they look at for the first
   // time half a trip later (ext_*) and move to the lane registers of the other heads' at the end of the next trip.
   // A pair stops when a ticket is beyond the pool.
-  const int rounds_all = static_cast<int>(nh / G);             // rounds in which every pair has a head
+  const int rounds_all = ONCE ? 1 : static_cast<int>(nh / G);  // rounds in which every pair has a head
   const int DRAWN_ROUNDS = rounds_all >= 6 ? 2 : 1;            // (with few rounds, more of them in turn)
-  const bool draw = p.work != nullptr && rounds_all >= 3;
+  const bool draw = !ONCE && p.work != nullptr && rounds_all >= 3;
   const int S = draw ? rounds_all - DRAWN_ROUNDS : 0;
   const unsigned pool = draw ? nh - static_cast<unsigned>(S) * G : 0;
   // Per-head scalars of this CTA's heads, 32 heads at a time: lane l holds those of the CTA's (32*batch+l)-th head
@@ -653,7 +654,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
           else if (lane == 0) p.decays[bh * (size_t)W + n] = a8[0];
         }
       }
-      if (lane == 0) arrive_and_set(p.win_pos, b, p.heads_v, n + 1);
+      if (!ONCE && lane == 0) arrive_and_set(p.win_pos, b, p.heads_v, n + 1);
       LQ_TICK(7);
     } else {
       // =========================== STREAM WARP ===========================

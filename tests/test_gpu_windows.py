@@ -17,7 +17,7 @@ G, K = synth.GATE_SCALAR, synth.GATE_DIAG
                                                      (K, 64, 1, 0), (G, 24, 0, 1), (G, 64, 1, 1), (K, 32, 1, 1), (K, 64, 0, 1), (G, 2, 0, 1)])
 def test_every_fill_of_a_window(oracle, gate, W, rec16, state_bf16):
     kw = dict(r=0, smooth=0, state_bf16=1) if state_bf16 else dict(r=3)
-    wl = synth.Workload("fill", W, 2, 1, W=W, gate=gate, rec16=rec16, seed=850 + W, **kw)
+    wl = synth.Workload("fill", W, 8, 4, W=W, gate=gate, rec16=rec16, seed=850 + W, **kw)
     osh, lsh = gu.shapes(wl)
     ost = OState(osh)
     oracle.quantize_state(osh, synth.dense_states(wl, 3), ost)
@@ -28,7 +28,7 @@ def test_every_fill_of_a_window(oracle, gate, W, rec16, state_bf16):
     ost.buf_u[...] = half(rng.standard_normal(ost.buf_u.shape))
     ost.buf_a[...] = half(rng.uniform(0.9, 1.0, ost.buf_a.shape))
     st = gu.state_to_dev(ost, lsh)
-    o = torch.empty((W, 2, 128), dtype=torch.float32, device="cuda")
+    o = torch.empty((W, 8, 128), dtype=torch.float32, device="cuda")
     for step in range(2):
         tok = synth.token_inputs(wl, step)
         want = oracle.decode_step(osh, ost, **tok)
