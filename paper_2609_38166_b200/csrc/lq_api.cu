@@ -372,7 +372,8 @@ static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStrea
 // A whole step of few heads in one launch, a CTA per head: as long as every SM has one head at most (a CTA takes most of an
 // SM's registers).  W = 16, r = 4, us per step in a graph as two launches / one: 1 head 6.7 / 5.1, 32 heads 6.7 / 5.2, 128 heads
 // 8.3 / 6.9, 148 heads of 37 sequences 13.8 / 12.7, 184 heads 14.5 / 14.5, 280 heads 14.2 / 16.1; 128 heads, diagonal gate,
-// W = 64, r = 8: 11.4 / 8.4; called one by one from the host, 1 to 128 heads: 11 / 8.4.
+// W = 64, r = 8: 11.4 / 8.4; called one by one from the host, 1 to 128 heads: 11 / 8.4.  (With the instances for exactly four
+// and eight compensators a step of 148 heads takes 12.0 instead of 12.7 us, of 128 heads, W = 8, 10.6 instead of 11.3.)
 static bool one_launch(const lq_shape *s) {
   return (long)s->batch * s->heads_v <= sm_count();
 }
@@ -381,7 +382,9 @@ static lq_status launch_step_t(const lq_shape *s, const Params &p, cudaStream_t 
   const bool diag = GATE == LQ_GATE_DIAG;
   const int smem = std::max(BoundarySmem<RM>(0, s->W, s->r, diag, R16, BF16, RM > 0 && s->n_iter > 1, 1).bytes,
                             TOKEN_SLOT + DecodeSlot(s->W, s->r, diag, R16, BF16, 0).bytes);
-  return launch_dependent(boundary_kernel<GATE, 0, R16, RM, BF16, false, true>, s->batch * s->heads_v, 256, smem, stream, p, 1);
+  auto kernel = boundary_kernel<GATE, 0, R16, RM, BF16, false, true>;
+  if (s->r == RM && (RM == 4 || RM == 8)) kernel = boundary_kernel<GATE, 0, R16, RM, BF16, RM == 4 || RM == 8, true>;
+  return launch_dependent(kernel, s->batch * s->heads_v, 256, smem, stream, p, 1);
 }
 template <int RM, bool BF16>
 static lq_status launch_step_gate(const lq_shape *s, const Params &p, cudaStream_t stream) {

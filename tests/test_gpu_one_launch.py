@@ -18,7 +18,7 @@ def _shape(batch, W, r, gate, rec16, bf16, n_iter):
 
 @pytest.mark.parametrize("gate,W,r,rec16,bf16,n_iter", [
     (G, 16, 4, 0, 0, 1), (G, 1, 2, 0, 0, 1), (G, 2, 0, 0, 0, 1), (G, 5, 8, 1, 0, 2), (G, 64, 3, 1, 0, 1), (G, 40, 16, 0, 0, 1),
-    (K, 16, 4, 0, 0, 1), (K, 7, 0, 1, 0, 1), (K, 33, 5, 0, 0, 1), (K, 64, 16, 0, 0, 2), (K, 13, 9, 1, 0, 1),
+    (K, 16, 4, 0, 0, 1), (K, 12, 4, 1, 0, 1), (G, 11, 4, 1, 0, 2), (K, 6, 8, 0, 0, 1), (K, 7, 0, 1, 0, 1), (K, 33, 5, 0, 0, 1), (K, 64, 16, 0, 0, 2), (K, 13, 9, 1, 0, 1),
     (G, 16, 0, 0, 1, 1), (G, 9, 0, 1, 1, 1), (K, 64, 0, 0, 1, 1), (K, 3, 0, 1, 1, 1)])
 def test_one_launch_and_two_give_the_same_bits(gate, W, r, rec16, bf16, n_iter):
     few = torch.cuda.get_device_properties(0).multi_processor_count // HEADS        # the most sequences of one launch
