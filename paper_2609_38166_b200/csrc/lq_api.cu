@@ -360,7 +360,7 @@ static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStrea
   // A second slot where a head is through in a few microseconds and two CTAs with two slots each still fit on an SM; a head
   // that is requantized leaves its slot early enough for the next one (two slots: 65.3 us against 64.1 at 256 x 32 heads).
   const int slots = (MODE == 2 || (BF16 && MODE == 0)) && bytes(2) <= (228 / 2 - 2) * 1024 ? 2 : 1;
-  constexpr bool may_be_exact = MODE == 0 && (RM == 4 || RM == 8);
+  constexpr bool may_be_exact = (MODE == 0 && (RM == 4 || RM == 8)) || (MODE == 1 && RM == 4);
   auto kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, false>;
   if (may_be_exact && s->r == RM) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, may_be_exact>;
   const long resident = (long)prepare_launch(reinterpret_cast<const void *>(kernel), 256, bytes(slots)) * sm_count();

@@ -12,7 +12,7 @@
 // vectors were in flight at a time); 9 K of them are the fp32 pipes (about 1150 packed FMAs per warp, two cycles each, four
 // warps to a scheduler), the rest the waits between its dependent phases, of which only the other CTA fills some.  Issue slots
 // are 41 % busy.  Against tiles of 8 rows x 128 columns per half-warp, where every column sum crossed the CTA (13 barriers a
-// head, now 8), and copies by all threads into two staging buffers: 2048 dense states quantized in 57.6 us (91.4 before),
+// head, now 8), and copies by all threads into two staging buffers: 2048 dense states quantized in 55.2 us (91.4 before),
 // 2048 states dequantized in 45.6 us (54.0); a step of 256 x 32 heads, 512 of them due, 73 -> 61 us.
 #pragma once
 #include <type_traits>
@@ -293,7 +293,9 @@ __device__ __forceinline__ uint32_t orthonormalize(float *X, int r, float *gram,
 // BF16: the per-window BF16 state (lq_shape.state_bf16, RM = 0): the dense state is rounded to bfloat16, and that is all.
 // slots: 1 or 2.
 // EXACT: r is RM, known at compile time: without a test per vector the compiler interleaves the four or eight column sums
-// (flush at 256 x 32 heads: step 62.2 -> 61.4 us, W = 8 75.6 -> 74.4; quantizing spills with it, 57.5 -> 69.9 us).
+// (flush at 256 x 32 heads: step 62.2 -> 61.4 us, W = 8 75.6 -> 74.4; quantizing 2048 states, r = 4: 57.5 -> 55.2 us, where only
+// the products with the start vectors must not know r: the vectors, the same for every head, would be kept in registers and
+// others spilled, 69.9 us; with eight vectors it spills all the same).
 // STEP (a flush): a whole decode step of few heads in one launch.  Every CTA has one head: two of its warps take it through the
 // token (decode_slot), then, if that filled the window, the CTA through the boundary.  What bounds it: the latency of a token and
 // of a boundary, and the host time of a launch, of which it needs one instead of
@@ -302,7 +304,7 @@ template <int GATE, int MODE, bool R16, int RM, bool BF16, bool EXACT, bool STEP
 __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Params p, const int slots) {
   // (exactly four vectors: registers are left for deeper unrolling, step 61.3 -> 60.8 us and 74.2 -> 73.0 at W = 8; for exactly
   // eight it is slower, 234.3 -> 236.5 us at 512 x 32 heads, diagonal gate, W = 64)
-  constexpr bool FOUR = EXACT && RM == 4;
+  constexpr bool FOUR = EXACT && RM == 4 && MODE == 0;
   constexpr bool DIAG = GATE == LQ_GATE_DIAG, RECORDS = MODE != 1, STAGED = MODE != 1 || RM <= 8;
   static_assert(!BF16 || RM == 0, "the per-window BF16 state has no compensators");
   constexpr int RF = record_floats(DIAG);
@@ -311,7 +313,7 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
   extern __shared__ __align__(128) unsigned char lq_bsm[];
   __shared__ unsigned todo_bh[32];
   __shared__ int todo_n[32], todo_count, any_due;
-  const int W = p.W, r = EXACT ? RM : RM > 0 ? p.r : 0, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 1, tx = lane & 1;
+  const int W = p.W, rT = MODE == 1 ? p.r : EXACT ? RM : p.r, r = EXACT ? RM : RM > 0 ? p.r : 0, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 1, tx = lane & 1;
   const int v0 = 16 * warp + 8 * tx;         // the lane's first column
   if (RM > 0 && r < 1) return;               // (not launched)
   const unsigned nh = static_cast<unsigned>(p.batch) * p.heads_v;
@@ -526,7 +528,7 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
       } else if constexpr (RM > 0) {
         // T_h = S w_h; w_h is the value side of the (h+1)-th newest record, or Walsh function h
 #pragma unroll (FOUR ? 4 : 2)
-        for (int h = 0; h < r; h++) {
+        for (int h = 0; h < rT; h++) {
           float2 w[4];
           if (RECORDS && h < n) {
             load8p(rec + (n - 1 - h) * RF + REC_U + v0, w);
