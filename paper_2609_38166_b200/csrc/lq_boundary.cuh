@@ -298,8 +298,7 @@ __device__ __forceinline__ uint32_t orthonormalize(float *X, int r, float *gram,
 // others spilled, 69.9 us; with eight vectors it spills all the same).
 // STEP (a flush): a whole decode step of few heads in one launch.  Every CTA has one head: two of its warps take it through the
 // token (decode_slot), then, if that filled the window, the CTA through the boundary.  What bounds it: the latency of a token and
-// of a boundary, and the host time of a launch, of which it needs one instead of
-// two (figures: one_launch).
+// of a boundary, and the host time of a launch, of which it needs one instead of two (figures: one_launch).
 template <int GATE, int MODE, bool R16, int RM, bool BF16, bool EXACT, bool STEP = false>
 __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Params p, const int slots) {
   // (exactly four vectors: registers are left for deeper unrolling, step 61.3 -> 60.8 us and 74.2 -> 73.0 at W = 8; for exactly
