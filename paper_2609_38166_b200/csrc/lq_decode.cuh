@@ -57,7 +57,7 @@ struct DecodeSlot {
     y = o; o += 2 * 4 * D;                // [2][128]: the rounded sums of the state stream, later the record terms
     pj = o; o += 4 * 16;                  // [2][8]: projections of a group of records, on their way to all lanes of the dot warp
     pk = o; o += (4 * (r + 2) + 15) / 16 * 16;      // compensator projections against Gamma k
-    pq = o; o += (4 * (r + 2) + 15) / 16 * 16;      // ... against Gamma q; pq[r], pq[r+1] hold kt^T q of alternate heads
+    pq = o; o += (4 * (r + 2) + 15) / 16 * 16;      // ... against Gamma q; pq[r], pq[r+1] hold kt^T q of alternate heads with a token
     mbar = o; o += 32;                    // head block, records (two)
     bytes = (o + 127) / 128 * 128;
   }
@@ -332,6 +332,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
   int ext_n = 0;                             // scalars of the head drawn a trip ago, on their way
   uint32_t ext_beta = 0, ext_alpha = 0;
   int idx = 0;                               // position of the head in this slot's list
+  int odd = 0;                               // parity of the heads with a token so far
   // end of a trip
   auto finish_trip = [&]() {
     // the next head, if it was drawn: its scalars, asked for a trip ago, go where the others' are
@@ -429,7 +430,11 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
       for (int j = n - 1; j >= 0; j--) gsc = gsc * bas[j];
     }
     // kt^T q needs only the token: the dot warp takes it before the wait as well.  It goes to one of two places
-    // in turn, because the stream warp may still be reading the previous head's.
+    // in turn, because the stream warp may still be reading the previous head's.  In turn over the heads WITH a token: the
+    // barriers of the head in between are what keeps a word from being written before the head two back has read it, and a
+    // head whose window came in full meets at none.
+    const int ktq_at = r + odd;
+    odd ^= 1;
     if (role == 1) {
       float2 k2p[4], q2p[4];
 #pragma unroll
@@ -438,7 +443,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         q2p[cc] = make_float2(q8[2 * cc], q8[2 * cc + 1]);
       }
       const float ktq_pre = tree16(block8(k2p, q2p));
-      if (lane == 0) pq[r + (idx & 1)] = ktq_pre;
+      if (lane == 0) pq[ktq_at] = ktq_pre;
     }
     LQ_TICK(1);
 
@@ -832,7 +837,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
       }
       }
       {
-        const float ktq = pq[r + (idx & 1)];
+        const float ktq = pq[ktq_at];
         float u[4], o[4];
 #pragma unroll
         for (int e = 0; e < 4; e++) { u[e] = p.delta ? v4[e] - rk[e] : v4[e]; o[e] = fmaf(u[e], ktq, rq[e]); }

@@ -102,3 +102,40 @@ def test_many_windows_that_come_in_full_among_drawn_heads(oracle, gate):
             want = oracle.decode_step(osub, one, **{k: np.ascontiguousarray(v[b:b + 1]) for k, v in tok.items()})
             assert np.array_equal(gu.host(o)[b:b + 1], want)
         assert np.array_equal(gu.gpu_codes(st)[b:b + 1], one.codes) and np.array_equal(gu.host(st.col_scale)[b:b + 1], one.col_scale)
+
+
+@pytest.mark.parametrize("state_bf16", [0, 1])
+@pytest.mark.parametrize("gate", [synth.GATE_SCALAR, synth.GATE_DIAG])
+def test_full_windows_between_heads_with_a_token(oracle, gate, state_bf16):
+    """Several heads per resident CTA, taken in turn (no scratch words), with sequences that enter with a full window in
+    between: such a head meets at no barrier, and the two warps hand kt^T q from one to the other through two words in turn.
+    Sixteen compensators make the reader of that word late."""
+    kw = dict(r=0, smooth=0, state_bf16=1) if state_bf16 else dict(r=16)
+    wl = synth.Workload("between", 60, 48, 16, W=3, gate=gate, seed=845, **kw)
+    osh, lsh = gu.shapes(wl)
+    assert lq.decode_launches(lsh) == 2
+    ost = OState(osh)
+    oracle.quantize_state(osh, synth.dense_states(wl, 3), ost)
+    rng = np.random.default_rng(5)
+    ost.buf_k[...] = rng.standard_normal(ost.buf_k.shape).astype(np.float32) * 0.1
+    ost.buf_u[...] = rng.standard_normal(ost.buf_u.shape).astype(np.float32)
+    ost.buf_a[...] = rng.uniform(0.2, 1.0, ost.buf_a.shape).astype(np.float32)
+    pieces = ["buf_k", "buf_u", "buf_a", "win_pos"] + (["S0"] if state_bf16 else ["codes", "col_scale", "row_smooth", "comp_k", "comp_u"])
+    for pattern in range(4):
+        full = np.arange(wl.batch) % 2 == pattern if pattern < 2 else rng.random(wl.batch) < 0.4
+        ost.win_pos[:] = np.where(full, wl.W, rng.integers(0, wl.W, wl.batch))
+        st = gu.state_to_dev(ost, lsh, work=False)
+        o = torch.full((wl.batch, wl.heads_v, 128), 7.0, dtype=torch.float32, device="cuda")
+        tok = synth.token_inputs(wl, pattern)
+        td = gu.tok_dev(tok)
+        lq.decode_step(lsh, st, td["q"], td["k"], td["v"], td["beta"], td["alpha"], o)
+        some = wl.with_(batch=int((~full).sum()))
+        osub, _ = gu.shapes(some)
+        sub = OState(osub)
+        for name in pieces:
+            getattr(sub, name)[...] = getattr(ost, name)[~full]
+        want = oracle.decode_step(osub, sub, **{k: np.ascontiguousarray(v[~full]) for k, v in tok.items()})
+        got = gu.host(o)
+        assert np.array_equal(got[~full], want) and (got[full] == 7.0).all(), pattern
+        assert np.array_equal(gu.host_f32(st.buf_u)[~full], sub.buf_u), pattern
+    assert lq.check_device() == 0
