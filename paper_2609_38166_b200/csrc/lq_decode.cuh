@@ -600,6 +600,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
       LQ_TICK(3);
       if constexpr (BF16) {                  // this warp's half of the columns; then all goes to the stream warp
         if (DIAG) named_wait(walked);        // (the stream warp has read the records' decays too)
+        else __syncwarp();                   // (every lane has read its last row)
         {
           const int n_next = n_next_now();
           if (wanted(n_next)) request_records(bh_next, n_next);

@@ -37,3 +37,30 @@ def test_every_fill_of_a_window(oracle, gate, W, rec16, state_bf16):
         assert np.array_equal(gu.host(o), want), f"o of step {step}"
         gu.assert_state_parity(st, ost, wl.r, f"state after step {step}")
     assert lq.check_device() == 0
+
+
+@pytest.mark.parametrize("gate,W,rec16", [(G, 3, 0), (G, 9, 1), (G, 24, 0), (K, 9, 0)])
+def test_bf16_state_several_heads_per_cta(oracle, gate, W, rec16):
+    """Per-window BF16, three and more heads per resident CTA: the records of a CTA's next head are asked for while this one's
+    state is multiplied, so every lane must be through with the rows before; every fill of a window, a boundary included."""
+    wl = synth.Workload("bfmany", 60, 48, 16, W=W, gate=gate, rec16=rec16, r=0, smooth=0, state_bf16=1, seed=880 + W)
+    osh, lsh = gu.shapes(wl)
+    assert lq.decode_launches(lsh) == 2
+    ost = OState(osh)
+    oracle.quantize_state(osh, synth.dense_states(wl, 3), ost)
+    rng = np.random.default_rng(W)
+    ost.win_pos[:] = rng.permutation(wl.batch) % W
+    half = lambda a: a.astype(np.float16).astype(np.float32)
+    ost.buf_k[...] = half(rng.standard_normal(ost.buf_k.shape, dtype=np.float32) * 0.1)
+    ost.buf_u[...] = half(rng.standard_normal(ost.buf_u.shape, dtype=np.float32))
+    ost.buf_a[...] = half(rng.uniform(0.5, 1.0, ost.buf_a.shape))
+    st = gu.state_to_dev(ost, lsh)
+    o = torch.empty((wl.batch, wl.heads_v, 128), dtype=torch.float32, device="cuda")
+    for step in range(2):
+        tok = synth.token_inputs(wl, step)
+        want = oracle.decode_step(osh, ost, **tok)
+        td = gu.tok_dev(tok)
+        lq.decode_step(lsh, st, td["q"], td["k"], td["v"], td["beta"], td["alpha"], o)
+        assert np.array_equal(gu.host(o), want), f"o of step {step}"
+        gu.assert_state_parity(st, ost, wl.r, f"state after step {step}")
+    assert lq.check_device() == 0
