@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
   using Lay = BoundarySmem<RM>;
   extern __shared__ __align__(128) unsigned char lq_bsm[];
   __shared__ unsigned todo_bh[32];
-  __shared__ int todo_n[32], todo_count, any_due;
+  __shared__ int todo_n[32], todo_count, lead_due;
   const int W = p.W, rT = MODE == 1 ? p.r : EXACT ? RM : p.r, r = EXACT ? RM : RM > 0 ? p.r : 0, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 1, tx = lane & 1;
   const int v0 = 16 * warp + 8 * tx;         // the lane's first column
   if (RM > 0 && r < 1) return;               // (not launched)
@@ -385,13 +385,13 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
         todo_bh[0] = blockIdx.x;
         todo_n[0] = W;
         todo_count = 1;
-        any_due = 0;
+        lead_due = -1;
       }
     } else if (warp == 0) {
       unsigned bh_mine = first + lane * gridDim.x;
-      int n_mine = 0, c, due = 0;
+      int n_mine = 0, c, lead = -1;
       if (MODE == 0) {
-        c = find_due_heads(p, first, gridDim.x, lane, bh_mine, n_mine, due);
+        c = find_due_heads(p, first, gridDim.x, lane, bh_mine, n_mine, lead);
       } else {
         const bool have = bh_mine < nh;
         if (MODE == 2 && have) n_mine = p.win_pos[bh_mine / p.heads_v] & 0xFFFF;
@@ -399,14 +399,14 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
       }
       todo_bh[lane] = bh_mine;
       todo_n[lane] = n_mine > W ? W : n_mine;
-      if (lane == 0) { todo_count = c; any_due = due; }
+      if (lane == 0) { todo_count = c; lead_due = lead; }
     }
     __syncthreads();
     count = todo_count;
     if (STAGED && count > 0) request(todo_bh[0], todo_n[0], at);
     // one warp reports that this CTA has seen all of win_pos, once the first head's copies are on their way (the round
     // trip hides behind them); with nothing due there is nothing to restart
-    if (MODE == 0 && count < 32 && any_due > 0 && warp == 7) restart_due_windows(p, lane);
+    if (MODE == 0 && count < 32 && lead_due >= 0 && warp == 7) restart_due_windows(p, lead_due, lane);
     LQ_BTICK(0);
 
     for (int k = 0; k < count; k++) {

@@ -350,16 +350,17 @@ __device__ __forceinline__ int nth_set_bit(uint32_t m, unsigned k) {
 // particular order, heads handed out by their own index pile up on some CTAs (256 sequences x 32 heads in random order,
 // W = 16: up to five boundaries on one CTA and none on others; a step of 100 us, 73 us with equal shares).
 // One warp finds up to 32 of a CTA's heads in one pass over win_pos: lane l looks for due head number first + l * stride.
-// Returns how many lanes found theirs (lanes 0 .. count-1); bh and n are the head and its buffered records, `total` how
-// many sequences are due in all.
+// Returns how many lanes found theirs (lanes 0 .. count-1); bh and n are the head and its buffered records, `lead` the first
+// due sequence, the same for every CTA (-1: none is due).
 __device__ __forceinline__ int find_due_heads(const Params &p, unsigned first, unsigned stride, int lane, unsigned &bh, int &n,
-                                              int &total) {
+                                              int &lead) {
   constexpr int U = 8;                       // loads in flight per lane
   const unsigned item = first + lane * stride;
   const unsigned want = item / static_cast<unsigned>(p.heads_v);       // rank of the head's sequence among the due ones
   unsigned base = 0;
+  int first_parked = -1;                     // first due sequence of any position
   bool found = false;
-  bh = 0; n = 0;
+  bh = 0; n = 0; lead = -1;
   for (int b0 = 0; b0 < p.batch; b0 += 32 * U) {
     int v[U];
 #pragma unroll
@@ -368,6 +369,11 @@ __device__ __forceinline__ int find_due_heads(const Params &p, unsigned first, u
     for (int u = 0; u < U; u++) {
       const uint32_t m = __ballot_sync(FULL, v[u] == p.W || (p.force && v[u] > 0));
       if (m == 0) continue;
+      // (a forced flush also takes sequences that a caller has parked at a position above W, upper bits and all: such a one
+      // only counts arrivals where there is no other)
+      const uint32_t counts = p.force ? __ballot_sync(FULL, v[u] > 0 && v[u] <= p.W) : m;
+      if (counts != 0 && lead < 0) lead = b0 + 32 * u + __ffs(counts) - 1;
+      if (first_parked < 0) first_parked = b0 + 32 * u + __ffs(m) - 1;
       const unsigned c = __popc(m);
       const bool mine = want - base < c;     // (unsigned: false for ranks below base)
       const int pos = mine ? nth_set_bit(m, want - base) : 0;
@@ -380,21 +386,22 @@ __device__ __forceinline__ int find_due_heads(const Params &p, unsigned first, u
       base += c;
     }
   }
-  total = base;
+  if (lead < 0 && base > 0) lead = first_parked;
   return __popc(__ballot_sync(FULL, found));
 }
 
-// A CTA that has seen all of win_pos says so on the upper bits of win_pos[0]; the last one starts the windows of the due
-// sequences afresh (nobody reads win_pos any more, and the boundaries themselves do not need it).  One warp calls this.
-__device__ __forceinline__ void restart_due_windows(const Params &p, int lane) {
+// A CTA that has seen all of win_pos says so on the upper bits of the first due sequence's entry; the last one starts the windows
+// of the due sequences afresh (nobody reads win_pos any more, and the boundaries themselves do not need it).  The other
+// entries are not touched, whatever a caller keeps there: a sequence without a request may be parked at any position from W
+// up, 2^31 - 1 or -1 included, with whose upper bits nothing could be counted.  One warp calls this.
+__device__ __forceinline__ void restart_due_windows(const Params &p, int lead, int lane) {
   int old = 0;
-  if (lane == 0) old = atomicAdd(p.win_pos, 0x10000);
+  if (lane == 0) old = atomicAdd(p.win_pos + lead, 0x10000);
   old = __shfl_sync(FULL, old, 0);
   if ((old >> 16) != static_cast<int>(gridDim.x) - 1) return;
   for (int b = lane; b < p.batch; b += 32) {
     const int v = __ldcg(p.win_pos + b) & 0xFFFF;
-    const bool due = v == p.W || (p.force && v > 0);
-    if (due || b == 0) p.win_pos[b] = due ? 0 : v;
+    if (v == p.W || (p.force && v > 0)) p.win_pos[b] = 0;
   }
 }
 

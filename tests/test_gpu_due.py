@@ -139,3 +139,40 @@ def test_full_windows_between_heads_with_a_token(oracle, gate, state_bf16):
         assert np.array_equal(got[~full], want) and (got[full] == 7.0).all(), pattern
         assert np.array_equal(gu.host_f32(st.buf_u)[~full], sub.buf_u), pattern
     assert lq.check_device() == 0
+
+
+@pytest.mark.parametrize("batch,launches", [(40, 2)])
+def test_parked_sequences_hold_up_nobody(oracle, batch, launches):
+    """Sequences at a position above W (the caller's mark for "no request here": 2^31 - 1, -1, 65535, W + 1; the first sequence
+    among them) get no token, keep their position and their rows of the output, and the windows of the others go on."""
+    wl = synth.Workload("parked", batch, 4, 2, W=3, r=2, seed=850 + batch)
+    osh, lsh = gu.shapes(wl)
+    assert lq.decode_launches(lsh) == launches
+    ost = OState(osh)
+    oracle.quantize_state(osh, synth.dense_states(wl, 3), ost)
+    marks = {0: 2 ** 31 - 1, 3: -1, 5: 65535, batch - 1: wl.W + 1}
+    parked = np.isin(np.arange(batch), list(marks))
+    st = gu.state_to_dev(ost, lsh)
+    for b, mark in marks.items():
+        st.win_pos[b] = mark
+    some = wl.with_(batch=int((~parked).sum()))
+    osub, _ = gu.shapes(some)
+    sub = OState(osub)
+    for name in ("codes", "col_scale", "row_smooth", "comp_k", "comp_u", "win_pos"):
+        getattr(sub, name)[...] = getattr(ost, name)[~parked]
+    o = torch.full((batch, 4, 128), 7.0, dtype=torch.float32, device="cuda")
+    for step in range(3 * wl.W + 1):
+        tok = synth.token_inputs(wl, step)
+        td = gu.tok_dev(tok)
+        lq.decode_step(lsh, st, td["q"], td["k"], td["v"], td["beta"], td["alpha"], o)
+        want = oracle.decode_step(osub, sub, **{k: np.ascontiguousarray(v[~parked]) for k, v in tok.items()})
+        got = gu.host(o)
+        assert np.array_equal(got[~parked], want) and (got[parked] == 7.0).all(), step
+        assert st.win_pos.cpu().numpy()[~parked].tolist() == sub.win_pos.tolist(), step
+        assert {b: int(st.win_pos[b]) for b in marks} == marks, step
+    lq.window_flush(lsh, st)                 # nothing is full
+    assert np.array_equal(gu.gpu_codes(st)[~parked], sub.codes)
+    lq.window_flush(lsh, st, force=True)     # the others' windows, whatever becomes of the parked ones
+    oracle.window_flush(osub, sub, force=True)
+    assert np.array_equal(gu.gpu_codes(st)[~parked], sub.codes) and not st.win_pos.cpu().numpy()[~parked].any()
+    assert lq.check_device() == 0
