@@ -376,7 +376,8 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
       }
       // (the barrier is where the whole CTA has read win_pos, ahead of its arrival)
       const bool due = __syncthreads_or(n_in == W - 1 || n_in == W);
-      if (tid == 0) arrive_and_set(p.win_pos, b, p.heads_v, due ? 0 : n_in < W ? n_in + 1 : n_in);
+      // (a sequence beyond W gets no token and keeps its entry, upper bits included)
+      if (tid == 0 && n_in <= W) arrive_and_set(p.win_pos, b, p.heads_v, due ? 0 : n_in + 1);
       if (!due) return;
       if (tid == 0) {
         const uint32_t token_bar = smem_addr(token_slot + DecodeSlot(W, p.r, DIAG, R16, BF16, 0).mbar);

@@ -141,7 +141,7 @@ def test_full_windows_between_heads_with_a_token(oracle, gate, state_bf16):
     assert lq.check_device() == 0
 
 
-@pytest.mark.parametrize("batch,launches", [(40, 2)])
+@pytest.mark.parametrize("batch,launches", [(40, 2), (20, 1)])
 def test_parked_sequences_hold_up_nobody(oracle, batch, launches):
     """Sequences at a position above W (the caller's mark for "no request here": 2^31 - 1, -1, 65535, W + 1; the first sequence
     among them) get no token, keep their position and their rows of the output, and the windows of the others go on."""
