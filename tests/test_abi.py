@@ -1,7 +1,10 @@
 """CPU checks of the boundary: the shared library builds, loads, exports every symbol the header declares,
 and rejects bad arguments before anything is launched (no GPU is touched)."""
+import copy
 import ctypes as C
+import dataclasses
 import os
+import pickle
 import re
 
 import pytest
@@ -93,3 +96,25 @@ def test_binding_fails_loudly_without_the_library(monkeypatch):
     monkeypatch.setattr(lq, "_LIB_PATH", "/nonexistent/liblq.so")
     with pytest.raises(lq.LqError):
         lq.lib()
+
+
+def test_shape_struct_follows_the_fields(L):
+    """The struct that a shape keeps for its calls is seen neither in the instance's dict nor in copies, and a change of a field
+    reaches the next call, whichever way it is made."""
+    sh = lq.Shape(2, 4, 2)
+    fields = dict(vars(sh))
+    assert lq.head_bytes(sh) == 19456
+    assert vars(sh) == fields and lq.Shape(**vars(sh)) == sh
+    for other in (copy.copy(sh), copy.deepcopy(sh), pickle.loads(pickle.dumps(sh)), dataclasses.replace(sh)):
+        assert other == sh and vars(other) == fields and lq.head_bytes(other) == 19456
+    sh.r = 8
+    assert lq.head_bytes(sh) == 21504
+    vars(sh)["r"] = 0
+    assert lq.head_bytes(sh) == 17408
+    sh.__dict__.update(gate=lq.GATE_DIAG)
+    assert lq.record_floats(sh) == 384
+    other = copy.copy(sh)
+    other.gate = lq.GATE_SCALAR
+    assert lq.record_floats(other) == 256 and lq.record_floats(sh) == 384
+    del sh.gate                              # (back to the default)
+    assert lq.record_floats(sh) == 256
