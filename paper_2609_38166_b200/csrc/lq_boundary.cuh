@@ -383,6 +383,8 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
         const uint32_t token_bar = smem_addr(token_slot + DecodeSlot(W, p.r, DIAG, R16, BF16, 0).mbar);
         mbar_inval(token_bar);
         mbar_inval(token_bar + 8);
+        // (the two words may lie where a bulk copy of the boundary lands: the warps' fences came before these accesses)
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         todo_bh[0] = blockIdx.x;
         todo_n[0] = W;
         todo_count = 1;
