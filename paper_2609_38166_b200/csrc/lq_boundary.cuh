@@ -310,8 +310,8 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
   using rec_t = typename std::conditional<R16, __half, float>::type;
   using Lay = BoundarySmem<RM>;
   extern __shared__ __align__(128) unsigned char lq_bsm[];
-  __shared__ unsigned todo_bh[32];
-  __shared__ int todo_n[32], todo_count, lead_due;
+  __shared__ unsigned todo_bh[32], due_counts[2][8];
+  __shared__ int todo_n[32], todo_count, lead_due[8];
   const int W = p.W, rT = MODE == 1 ? p.r : EXACT ? RM : p.r, r = EXACT ? RM : RM > 0 ? p.r : 0, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, ty = lane >> 1, tx = lane & 1;
   const int v0 = 16 * warp + 8 * tx;         // the lane's first column
   if (RM > 0 && r < 1) return;               // (not launched)
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
     }
   };
 
-  // Warp 0 puts together the next 32 heads of the CTA (a flush: of those that are due, see find_due_heads; otherwise every
+  // The CTA puts together its next 32 heads (a flush: of those that are due, see list_due_heads; otherwise warp 0, every
   // gridDim-th head) and how many records each holds; then the CTA takes them one after the other.
   int count = 32;
   for (unsigned first = blockIdx.x; count == 32; first += 32 * gridDim.x) {
@@ -388,28 +388,32 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
         todo_bh[0] = blockIdx.x;
         todo_n[0] = W;
         todo_count = 1;
-        lead_due = -1;
+      }
+    } else if constexpr (MODE == 0) {
+      if (warp < due_scan_warps(p)) {
+        int lead;
+        const int c = list_due_heads(p, first, gridDim.x, due_scan_warps(p), due_counts, todo_bh, todo_n, lead);
+        if (lane == 0) lead_due[warp] = lead;
+        if (tid == 0) todo_count = c;
       }
     } else if (warp == 0) {
-      unsigned bh_mine = first + lane * gridDim.x;
-      int n_mine = 0, c, lead = -1;
-      if (MODE == 0) {
-        c = find_due_heads(p, first, gridDim.x, lane, bh_mine, n_mine, lead);
-      } else {
-        const bool have = bh_mine < nh;
-        if (MODE == 2 && have) n_mine = p.win_pos[bh_mine / p.heads_v] & 0xFFFF;
-        c = __popc(__ballot_sync(FULL, have));
-      }
+      const unsigned bh_mine = first + lane * gridDim.x;
+      const bool have = bh_mine < nh;
+      const int n_mine = MODE == 2 && have ? p.win_pos[bh_mine / p.heads_v] & 0xFFFF : 0;
+      const int c = __popc(__ballot_sync(FULL, have));
       todo_bh[lane] = bh_mine;
       todo_n[lane] = n_mine > W ? W : n_mine;
-      if (lane == 0) { todo_count = c; lead_due = lead; }
+      if (lane == 0) todo_count = c;
     }
     __syncthreads();
     count = todo_count;
     if (STAGED && count > 0) request(todo_bh[0], todo_n[0], at);
-    // one warp reports that this CTA has seen all of win_pos, once the first head's copies are on their way (the round
-    // trip hides behind them); with nothing due there is nothing to restart
-    if (MODE == 0 && count < 32 && lead_due >= 0 && warp == 7) restart_due_windows(p, lead_due, lane);
+    // report that this CTA has seen all of win_pos, once the first head's copies are on their way (the round trip hides behind
+    // them), part by part; with nothing due in a part there is nothing to restart
+    if (MODE == 0 && !STEP && count < 32) {
+      const int warps = due_scan_warps(p), w = (warp + 1) & 7;       // (warp 7 for part 0)
+      if (w < warps && lead_due[w] >= 0) restart_due_windows(p, lead_due[w], w, warps);
+    }
     LQ_BTICK(0);
 
     for (int k = 0; k < count; k++) {

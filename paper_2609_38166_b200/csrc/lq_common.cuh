@@ -346,62 +346,109 @@ __device__ __forceinline__ int nth_set_bit(uint32_t m, unsigned k) {
   return pos;
 }
 
-// The due heads, numbered sequence by sequence, belong to CTA i mod gridDim: with the windows of a serving batch in no
-// particular order, heads handed out by their own index pile up on some CTAs (256 sequences x 32 heads in random order,
-// W = 16: up to five boundaries on one CTA and none on others; a step of 100 us, 73 us with equal shares).
-// One warp finds up to 32 of a CTA's heads in one pass over win_pos: lane l looks for due head number first + l * stride.
-// Returns how many lanes found theirs (lanes 0 .. count-1); bh and n are the head and its buffered records, `lead` the first
-// due sequence, the same for every CTA (-1: none is due).
-__device__ __forceinline__ int find_due_heads(const Params &p, unsigned first, unsigned stride, int lane, unsigned &bh, int &n,
-                                              int &lead) {
+// The due heads, in an order of their sequences that every CTA sees alike, belong to CTA i mod gridDim: with the windows of a
+// serving batch in no particular order, heads handed out by their own index pile up on some CTAs (256 sequences x 32 heads in
+// random order, W = 16: up to five boundaries on one CTA and none on others; a step of 100 us, 73 us with equal shares).
+// The CTA lists up to 32 of its heads in one pass over win_pos: due heads number first, first + stride, ..., `todo_bh` and
+// `todo_n` the head and its buffered records.  What bounds it is the round trip of the loads, of which a lane has eight in flight,
+// and where few are due, the instructions, which a CTA fetches for itself: up to 256 sequences warp 0 does it alone, in one
+// trip; more of them take all eight warps, 2048 sequences to a trip, warp w those with w in bits 5 to 7 of their index.
+// W = 16, us per step with one warp at all sizes / as it is: 512 x 2 heads 22.6 / 18.7, 1024 x 8 66.7 / 61.7, 8192 x 1 141 / 66,
+// 32768 x 1 644 / 246; with eight warps at all sizes 32 x 32 heads take 18.7 instead of 18.4.
+// Called by the `warps` first warps (due_scan_warps).  Returns how many heads are listed.  `lead`: a due sequence among those
+// this warp looks at, the same for the warp of this number in every CTA (-1: none).  `counts`: shared memory.  Ends without a
+// barrier.
+__device__ __forceinline__ bool window_due(const Params &p, int v) { return v == p.W || (p.force && v > 0); }
+__device__ __forceinline__ int due_scan_warps(const Params &p) { return p.batch <= 256 ? 1 : 8; }
+__device__ __forceinline__ int list_due_heads(const Params &p, unsigned first, unsigned stride, int warps, unsigned (*counts)[8],
+                                              unsigned *todo_bh, int *todo_n, int &lead) {
   constexpr int U = 8;                       // loads in flight per lane
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, span = 32 * warps;
   const unsigned item = first + lane * stride;
   const unsigned want = item / static_cast<unsigned>(p.heads_v);       // rank of the head's sequence among the due ones
   unsigned base = 0;
-  int first_parked = -1;                     // first due sequence of any position
-  bool found = false;
-  bh = 0; n = 0; lead = -1;
-  for (int b0 = 0; b0 < p.batch; b0 += 32 * U) {
+  int turn = 0;
+  lead = -1;
+#pragma unroll 1
+  for (int b0 = 0; b0 < p.batch; b0 += span * U, turn ^= 1) {
+    const int mine0 = b0 + 32 * warp;
     int v[U];
+    uint32_t m[U];
+    unsigned c = 0;
 #pragma unroll
-    for (int u = 0; u < U; u++) v[u] = b0 + 32 * u + lane < p.batch ? p.win_pos[b0 + 32 * u + lane] & 0xFFFF : 0;
+    for (int u = 0; u < U; u++) v[u] = mine0 + span * u + lane < p.batch ? p.win_pos[mine0 + span * u + lane] & 0xFFFF : 0;
 #pragma unroll
     for (int u = 0; u < U; u++) {
-      const uint32_t m = __ballot_sync(FULL, v[u] == p.W || (p.force && v[u] > 0));
-      if (m == 0) continue;
-      // (a forced flush also takes sequences that a caller has parked at a position above W, upper bits and all: such a one
-      // only counts arrivals where there is no other)
-      const uint32_t counts = p.force ? __ballot_sync(FULL, v[u] > 0 && v[u] <= p.W) : m;
-      if (counts != 0 && lead < 0) lead = b0 + 32 * u + __ffs(counts) - 1;
-      if (first_parked < 0) first_parked = b0 + 32 * u + __ffs(m) - 1;
-      const unsigned c = __popc(m);
-      const bool mine = want - base < c;     // (unsigned: false for ranks below base)
-      const int pos = mine ? nth_set_bit(m, want - base) : 0;
-      const int nv = __shfl_sync(FULL, v[u], pos);
-      if (mine) {
-        found = true;
-        n = nv < p.W ? nv : p.W;
-        bh = static_cast<unsigned>(b0 + 32 * u + pos) * p.heads_v + (item - want * p.heads_v);
-      }
-      base += c;
+      m[u] = __ballot_sync(FULL, window_due(p, v[u]));
+      c += __popc(m[u]);
     }
+    unsigned at = base;
+    if (warps == 1) {
+      base += c;
+    } else {
+      if (lane == 0) counts[turn][warp] = c;
+      __syncthreads();                       // (in turn: the counts of the trip before may still be read)
+#pragma unroll
+      for (int w = 0; w < 8; w++) {
+        const unsigned x = counts[turn][w];
+        if (w < warp) at += x;
+        base += x;
+      }
+    }
+    if (c == 0) continue;
+    // the sequence of rank `want`, if it is one of this trip: the word it is in, then the bit; and the first due one
+    unsigned left = want - at;               // (unsigned: beyond all words for ranks below `at`)
+    uint32_t word = 0;
+    int bit0 = 0, lead_word = 0;
+    uint32_t lead_bits = 0;
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const unsigned cu = __popc(m[u]);
+      if (word == 0) {
+        if (left < cu) { word = m[u]; bit0 = u; }
+        else left -= cu;
+      }
+      if (lead_bits == 0) { lead_bits = m[u]; lead_word = u; }
+    }
+    if (word != 0) {
+      const int b = mine0 + span * bit0 + nth_set_bit(word, left);
+      todo_bh[lane] = static_cast<unsigned>(b) * p.heads_v + (item - want * p.heads_v);
+      todo_n[lane] = p.force ? min(p.win_pos[b] & 0xFFFF, p.W) : p.W;
+    }
+    if (lead < 0) lead = mine0 + span * lead_word + __ffs(lead_bits) - 1;
   }
-  if (lead < 0 && base > 0) lead = first_parked;
-  return __popc(__ballot_sync(FULL, found));
+  return __popc(__ballot_sync(FULL, want < base));
 }
 
-// A CTA that has seen all of win_pos says so on the upper bits of the first due sequence's entry; the last one starts the windows
-// of the due sequences afresh (nobody reads win_pos any more, and the boundaries themselves do not need it).  The other
-// entries are not touched, whatever a caller keeps there: a sequence without a request may be parked at any position from W
-// up, 2^31 - 1 or -1 included, with whose upper bits nothing could be counted.  One warp calls this.
-__device__ __forceinline__ void restart_due_windows(const Params &p, int lead, int lane) {
+// A CTA whose part `w` of win_pos (of `warps` parts, as above) has been seen says so on the upper bits of the entry of a due
+// sequence of that part; the last CTA starts the windows of the due sequences of the part afresh (nobody reads these entries any
+// more, and the boundaries themselves do not need them).  The other entries are not touched, whatever a caller keeps there: a
+// sequence without a request may be parked at any position from W up, 2^31 - 1 or -1 included, with whose upper bits nothing
+// could be counted.  One warp calls this.
+__device__ __forceinline__ void restart_due_windows(const Params &p, int lead, int w, int warps) {
+  constexpr int U = 8;
+  const int lane = threadIdx.x & 31, span = 32 * warps;
+  if (p.force) {                             // (which also takes the parked ones: count on another one where there is one)
+    int ok = p.batch;
+    for (int b = 32 * w + lane; b < p.batch; b += span) {
+      const int v = p.win_pos[b] & 0xFFFF;
+      if (v > 0 && v <= p.W) { ok = b; break; }
+    }
+    ok = __reduce_min_sync(FULL, ok);
+    if (ok < p.batch) lead = ok;
+  }
   int old = 0;
   if (lane == 0) old = atomicAdd(p.win_pos + lead, 0x10000);
   old = __shfl_sync(FULL, old, 0);
   if ((old >> 16) != static_cast<int>(gridDim.x) - 1) return;
-  for (int b = lane; b < p.batch; b += 32) {
-    const int v = __ldcg(p.win_pos + b) & 0xFFFF;
-    if (v == p.W || (p.force && v > 0)) p.win_pos[b] = 0;
+#pragma unroll 1
+  for (int b0 = 32 * w + lane; b0 < p.batch; b0 += span * U) {
+    int v[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) v[u] = b0 + span * u < p.batch ? __ldcg(p.win_pos + b0 + span * u) & 0xFFFF : 0;
+#pragma unroll
+    for (int u = 0; u < U; u++)
+      if (window_due(p, v[u])) p.win_pos[b0 + span * u] = 0;
   }
 }
 

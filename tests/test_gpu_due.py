@@ -1,6 +1,6 @@
 """GPU: which heads a window boundary takes.  The kernels find the due sequences by looking over all window positions; the
-sizes here are where that can go wrong: one sequence, more sequences than one pass of loads covers (256), more due heads
-per CTA than one list holds (32), windows in random order, all due at once, none due."""
+sizes here are where that can go wrong: one sequence, more sequences than one load of every thread covers (256) and than one
+trip does (2048), more due heads per CTA than one list holds (32), in one trip and in several, windows in random order, all due at once, none due."""
 import numpy as np
 import pytest
 import torch
@@ -14,7 +14,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("state_bf16", [0, 1])
 @pytest.mark.parametrize("batch,heads_v,heads_qk,W,order", [(1, 1, 1, 4, "last"), (5, 3, 3, 5, "all"), (300, 3, 1, 4, "random"),
-                                                            (257, 2, 2, 3, "none"), (301, 32, 16, 2, "all")])
+                                                            (257, 2, 2, 3, "none"), (301, 32, 16, 2, "all"),
+                                                            (2049, 1, 1, 3, "last"), (2500, 2, 1, 4, "random"), (4750, 2, 1, 2, "all")])
 def test_boundaries_of_windows_in_any_order(oracle, batch, heads_v, heads_qk, W, order, state_bf16):
     kw = dict(r=0, smooth=0, state_bf16=1) if state_bf16 else dict(r=2)
     wl = synth.Workload("due", batch, heads_v, heads_qk, W=W, seed=800 + batch, **kw)
