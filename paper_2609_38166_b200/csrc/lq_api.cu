@@ -354,7 +354,7 @@ static lq_status launch_decode(const lq_shape *s, const Params &p, cudaStream_t 
 
 // The boundary kernels are persistent: as many CTAs as are resident at once, each striding over its heads.
 template <int GATE, int MODE, bool R16, int RM, bool BF16>
-static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStream_t stream) {
+static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStream_t stream, long due) {
   const bool diag = GATE == LQ_GATE_DIAG, iterate = RM > 0 && s->n_iter > 1;
   auto bytes = [&](int slots) { return BoundarySmem<RM>(MODE, s->W, s->r, diag, R16, BF16, iterate, slots).bytes; };
   // A second slot where a head is through in a few microseconds and two CTAs with two slots each still fit on an SM; a head
@@ -363,10 +363,17 @@ static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStrea
   constexpr bool may_be_exact = (MODE == 0 && (RM == 4 || RM == 8)) || (MODE == 1 && RM == 4);
   auto kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, false>;
   if (may_be_exact && s->r == RM) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, may_be_exact>;
-  const long resident = (long)prepare_launch(reinterpret_cast<const void *>(kernel), 256, bytes(slots)) * sm_count();
-  if (resident < 1) return LQ_ERR_CUDA;
   const long nh = (long)s->batch * s->heads_v;
-  return launch_dependent(kernel, static_cast<int>(nh < resident ? nh : resident), 256, bytes(slots), stream, p, slots);
+  // With more than eight compensators two heads on one SM take half as long again as one, and CTAs that leave room for a second
+  // one are not placed one to an SM (the first 148 of 296 come to lie on 142 SMs): where windows of every fill would have no
+  // more heads due at a time than there are SMs, though all heads at once are more than two to an SM, a CTA asks for more than
+  // half of its SM's memory.  64 x 32 heads, W = 16, us per step with one CTA / two to an SM: windows of every fill, r = 9
+  // 35.6 / 37.1, r = 12 38.5 / 42.1, r = 16 43.7 / 50.2; all windows due at once (every 16th step), r = 16, on average 37.4 / 31.5.
+  const bool alone = RM > 8 && MODE == 0 && due <= sm_count() && nh > 2L * sm_count();
+  const int smem = alone ? std::max(bytes(slots), 116 * 1024) : bytes(slots);
+  const long resident = (long)prepare_launch(reinterpret_cast<const void *>(kernel), 256, smem) * sm_count();
+  if (resident < 1) return LQ_ERR_CUDA;
+  return launch_dependent(kernel, static_cast<int>(nh < resident ? nh : resident), 256, smem, stream, p, slots);
 }
 
 // A whole step of few heads in one launch, a CTA per head: as long as every SM has one head at most (a CTA takes most of an
@@ -401,23 +408,24 @@ static lq_status launch_step(const lq_shape *s, const Params &p, cudaStream_t st
 }
 
 template <int MODE, int RM, bool BF16>
-static lq_status launch_boundary_gate(const lq_shape *s, const Params &p, cudaStream_t stream) {
-  if (MODE == 1) return launch_boundary_t<LQ_GATE_SCALAR, MODE, false, RM, BF16>(s, p, stream);   // (reads no records)
+static lq_status launch_boundary_gate(const lq_shape *s, const Params &p, cudaStream_t stream, long due) {
+  if (MODE == 1) return launch_boundary_t<LQ_GATE_SCALAR, MODE, false, RM, BF16>(s, p, stream, due);   // (reads no records)
   constexpr int M_ = MODE == 1 ? 0 : MODE;
   if (s->gate == LQ_GATE_DIAG)
-    return s->rec16 ? launch_boundary_t<LQ_GATE_DIAG, M_, true, RM, BF16>(s, p, stream) : launch_boundary_t<LQ_GATE_DIAG, M_, false, RM, BF16>(s, p, stream);
-  return s->rec16 ? launch_boundary_t<LQ_GATE_SCALAR, M_, true, RM, BF16>(s, p, stream) : launch_boundary_t<LQ_GATE_SCALAR, M_, false, RM, BF16>(s, p, stream);
+    return s->rec16 ? launch_boundary_t<LQ_GATE_DIAG, M_, true, RM, BF16>(s, p, stream, due) : launch_boundary_t<LQ_GATE_DIAG, M_, false, RM, BF16>(s, p, stream, due);
+  return s->rec16 ? launch_boundary_t<LQ_GATE_SCALAR, M_, true, RM, BF16>(s, p, stream, due) : launch_boundary_t<LQ_GATE_SCALAR, M_, false, RM, BF16>(s, p, stream, due);
 }
 
-// compiled for r = 0, r <= 4, r <= 8 and any r (the small matrices of the fit live in registers)
+// compiled for r = 0, r <= 4, r <= 8 and any r (the small matrices of the fit live in registers); due: heads that are due at a
+// time, as far as the call tells
 template <int MODE>
-static lq_status launch_boundary(const lq_shape *s, const Params &p, cudaStream_t stream) {
+static lq_status launch_boundary(const lq_shape *s, const Params &p, cudaStream_t stream, long due) {
   if (s->batch == 0) return LQ_OK;
-  if (s->state_bf16) return launch_boundary_gate<MODE, 0, true>(s, p, stream);
-  if (s->r == 0) return launch_boundary_gate<MODE, 0, false>(s, p, stream);
-  if (MODE == 2 || s->r <= 4) return launch_boundary_gate<MODE, 4, false>(s, p, stream);
-  if (s->r <= 8) return launch_boundary_gate<MODE, MODE == 2 ? 4 : 8, false>(s, p, stream);
-  return launch_boundary_gate<MODE, MODE == 2 ? 4 : MAX_R, false>(s, p, stream);
+  if (s->state_bf16) return launch_boundary_gate<MODE, 0, true>(s, p, stream, due);
+  if (s->r == 0) return launch_boundary_gate<MODE, 0, false>(s, p, stream, due);
+  if (MODE == 2 || s->r <= 4) return launch_boundary_gate<MODE, 4, false>(s, p, stream, due);
+  if (s->r <= 8) return launch_boundary_gate<MODE, MODE == 2 ? 4 : 8, false>(s, p, stream, due);
+  return launch_boundary_gate<MODE, MODE == 2 ? 4 : MAX_R, false>(s, p, stream, due);
 }
 
 }  // namespace lq
@@ -453,7 +461,7 @@ static lq_status decode_step_impl(const lq_shape *shape, const lq_state *state, 
     cudaGetLastError();
     return LQ_ERR_CUDA;
   }
-  return part >= 0 ? LQ_OK : launch_boundary<0>(shape, p, st);     // sequences whose window just became full
+  return part >= 0 ? LQ_OK : launch_boundary<0>(shape, p, st, nh / shape->W);     // sequences whose window just became full
 }
 
 lq_status lq_decode_step(const lq_shape *shape, const lq_state *state, const uint16_t *q, const uint16_t *k,
@@ -760,7 +768,7 @@ lq_status lq_decode_step_host_pipelined(const lq_shape *shape, const lq_state *s
   }
   if (ok && rc == LQ_OK) {                   // the windows that became full, of all sub-batches together
     Params p = make_params(shape, state);
-    rc = launch_boundary<0>(shape, p, st);
+    rc = launch_boundary<0>(shape, p, st, (long)shape->batch * shape->heads_v / shape->W);
   }
   // join: whatever was put on the side streams is waited for by `stream`, also after an error above
   // (`stream` has waited for every copy-in of this call already, sub-batch by sub-batch, unless an error cut the
@@ -840,7 +848,7 @@ lq_status lq_window_flush(const lq_shape *shape, const lq_state *state, int forc
   if ((rc = check_state(shape, state, true)) != LQ_OK) return rc;
   Params p = make_params(shape, state);
   p.force = force ? 1 : 0;
-  return launch_boundary<0>(shape, p, reinterpret_cast<cudaStream_t>(stream));
+  return launch_boundary<0>(shape, p, reinterpret_cast<cudaStream_t>(stream), (long)shape->batch * shape->heads_v);
 }
 
 lq_status lq_quantize_state(const lq_shape *shape, const float *S, const lq_state *state, lq_stream stream) {
@@ -850,7 +858,7 @@ lq_status lq_quantize_state(const lq_shape *shape, const float *S, const lq_stat
   if ((rc = check_ptrs({S})) != LQ_OK) return rc;
   Params p = make_params(shape, state);
   p.S = const_cast<float *>(S);
-  return launch_boundary<1>(shape, p, reinterpret_cast<cudaStream_t>(stream));
+  return launch_boundary<1>(shape, p, reinterpret_cast<cudaStream_t>(stream), (long)shape->batch * shape->heads_v);
 }
 
 lq_status lq_dequantize_state(const lq_shape *shape, const lq_state *state, float *S, lq_stream stream) {
@@ -860,7 +868,7 @@ lq_status lq_dequantize_state(const lq_shape *shape, const lq_state *state, floa
   if ((rc = check_ptrs({S})) != LQ_OK) return rc;
   Params p = make_params(shape, state);
   p.S = S;
-  return launch_boundary<2>(shape, p, reinterpret_cast<cudaStream_t>(stream));
+  return launch_boundary<2>(shape, p, reinterpret_cast<cudaStream_t>(stream), (long)shape->batch * shape->heads_v);
 }
 
 static lq_status ref_step(const lq_shape *shape, float *S, uint16_t *S16, const uint16_t *q, const uint16_t *k,

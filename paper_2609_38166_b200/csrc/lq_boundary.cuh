@@ -40,8 +40,11 @@ struct BoundarySmem {
   static constexpr int chol = gram + 4 * RM * RM;            // L [RM][RM], 1 / L_hh [RM], alive [RM] (more than four vectors)
   static constexpr int ub = chol + (RM > 4 ? 4 * (RM * RM + 2 * RM) : 0);      // [8][RM][16] value sides as stored, per warp
   static constexpr int T = ub + 4 * D * RM;                  // [RM][128]  S w_h, then the keys as stored
-  static constexpr int part = T + 4 * D * RM;                // [8][RM][128] per-warp row sums; later [8][128] those of |R|
-  static constexpr int head = part + 4 * D * 8 * (RM > 0 ? RM : 1);            // the slots
+  // Row sums go through here eight vectors at a time (r is more than eight where RM is): all sixteen at once are 64 KB, with which one CTA fits on an SM instead of
+  // two (2048 heads, W = 16, r = 16 flushed in 325 us, 239 with eight at a time).
+  static constexpr int PV = RM > 8 ? 8 : RM > 0 ? RM : 1;
+  static constexpr int part = T + 4 * D * RM;                // [8][PV][128] per-warp row sums; later [8][128] those of |R|
+  static constexpr int head = part + 4 * D * 8 * PV;         // the slots
   int rec, slot, dec, kd, Wv, bytes;
   __host__ __device__ BoundarySmem(int mode, int W, int r, bool diag, bool rec16, bool bf16, bool iterate, int slots) {
     rec = bf16 ? BF16W_HEAD_BYTES : head_bytes(r);           // within a slot: [W] record rows behind the head block
@@ -309,6 +312,7 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
   constexpr int RF = record_floats(DIAG);
   using rec_t = typename std::conditional<R16, __half, float>::type;
   using Lay = BoundarySmem<RM>;
+  constexpr int PV = Lay::PV;                // vectors whose row sums `part` holds at a time
   extern __shared__ __align__(128) unsigned char lq_bsm[];
   __shared__ unsigned todo_bh[32], due_counts[2][8];
   __shared__ int todo_n[32], todo_count, lead_due[8];
@@ -533,19 +537,39 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
         for (int a = 0; a < 8; a++) store_row8(S + a * D, wide, M[a]);
       } else if constexpr (RM > 0) {
         // T_h = S w_h; w_h is the value side of the (h+1)-th newest record, or Walsh function h
-#pragma unroll (FOUR ? 4 : 2)
-        for (int h = 0; h < rT; h++) {
-          float2 w[4];
+        auto start_vector = [&](int h, float2 (&w)[4]) {
           if (RECORDS && h < n) {
             load8p(rec + (n - 1 - h) * RF + REC_U + v0, w);
           } else {
 #pragma unroll
             for (int c = 0; c < 4; c++) w[c] = make_float2(walsh_entry(h, v0 + 2 * c), walsh_entry(h, v0 + 2 * c + 1));
           }
+        };
+        auto row_sums = [&](const float2 (&w)[4], int at) {
           float pr[8];
 #pragma unroll
           for (int a = 0; a < 8; a++) pr[a] = block8(M[a], w);
-          store_row_pairs(pr, ty, tx, part + (warp * RM + h) * D);
+          store_row_pairs(pr, ty, tx, part + (warp * PV + at) * D);
+        };
+        if constexpr (RM > PV) {
+#pragma unroll 2
+          for (int h = 0; h < rT; h++) {
+            if (h == PV) {                                    // more than eight (up to sixteen): the first eight are summed here
+              __syncthreads();
+              for (int idx = tid; idx < PV * D; idx += 256) T[idx] = sum_warps(part + idx, PV * D);
+              __syncthreads();
+            }
+            float2 w[4];
+            start_vector(h, w);
+            row_sums(w, h % PV);
+          }
+        } else {
+#pragma unroll (FOUR ? 4 : 2)
+          for (int h = 0; h < rT; h++) {
+            float2 w[4];
+            start_vector(h, w);
+            row_sums(w, h);
+          }
         }
       }
       // the slot is free when all have come here: the next head may land while this one is worked on
@@ -573,7 +597,8 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
       } else if constexpr (MODE != 2) {
         uint32_t alive = 0;
         if constexpr (RM > 0) {
-          for (int idx = tid; idx < r * D; idx += 256) T[idx] = sum_warps(part + idx, RM * D);
+          constexpr int T0 = RM > PV ? PV * D : 0;            // (those before are there)
+          for (int idx = T0 + tid; idx < r * D; idx += 256) T[idx] = sum_warps(part + idx - T0, PV * D);
           LQ_BTICK(10);
           // further rounds: W_h = S^T q_h, orthonormalise, T_h = S q_h
           for (int it = 1; it < p.n_iter; it++) {
@@ -589,15 +614,20 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
             orthonormalize<false, RM>(Wv, r, gram, chol, nullptr);
 #pragma unroll 1
             for (int h = 0; h < r; h++) {
+              if (RM > PV && h == PV) {
+                __syncthreads();
+                for (int idx = tid; idx < PV * D; idx += 256) T[idx] = sum_warps(part + idx, PV * D);
+                __syncthreads();
+              }
               float2 w[4];
               load8p(Wv + h * D + v0, w);
               float pr[8];
 #pragma unroll
               for (int a = 0; a < 8; a++) pr[a] = block8(M[a], w);
-              store_row_pairs(pr, ty, tx, part + (warp * RM + h) * D);
+              store_row_pairs(pr, ty, tx, part + (warp * PV + (RM > PV ? h % PV : h)) * D);
             }
             __syncthreads();
-            for (int idx = tid; idx < r * D; idx += 256) T[idx] = sum_warps(part + idx, RM * D);
+            for (int idx = T0 + tid; idx < r * D; idx += 256) T[idx] = sum_warps(part + idx - T0, PV * D);
           }
           alive = orthonormalize<true, RM>(T, r, gram, chol, p.comp_k(bh));       // T now holds the keys as stored
           LQ_BTICK(11);

@@ -129,6 +129,14 @@ def test_chain_with_several_rounds_of_power_iteration(oracle, gate, r, n_iter):
     _run_chain(oracle, wl, 2 * wl.W + 3, init="dense", stagger=True, check_every=4)
 
 
+@pytest.mark.parametrize("gate,r,n_iter,rec16", [(0, 9, 1, 0), (0, 16, 3, 0), (1, 16, 1, 1), (1, 10, 2, 0)])
+def test_chain_with_more_than_eight_compensators(oracle, gate, r, n_iter, rec16):
+    """Above eight the row sums go through shared memory eight vectors at a time; more heads than one launch takes."""
+    wl = synth.Workload("r16", 40, 4, 2, W=4, r=r, n_iter=n_iter, gate=gate, rec16=rec16, seed=475 + r)
+    assert lq.decode_launches(gu.shapes(wl)[1]) == 2
+    _run_chain(oracle, wl, 2 * wl.W + 1, init="dense", stagger=True, check_every=2)
+
+
 @pytest.mark.parametrize("gate", GATES)
 def test_chain_without_the_delta_rule(oracle, gate):
     """b_t = 0 (Mamba2 / GLA style instances): u = v; decode, boundaries and both baseline kernels against the oracle."""
