@@ -220,13 +220,15 @@ def _ptr(t: Optional[torch.Tensor], b0: int = 0) -> Optional[int]:
 
 def _sub(sh: Shape, b0: int, nb: Optional[int]):
     """Sequences [b0, b0+nb) of a shape, as a reference to the C struct."""
+    if nb is None and not b0:
+        return sh.ref()
     nb = sh.batch - b0 if nb is None else nb
-    return sh.ref() if nb == sh.batch else C.byref(sh.c(nb))
+    return C.byref(sh.c(nb))
 
 
 def decode_step(sh: Shape, st: State, q, k, v, beta, alpha, o, stream=None, b0: int = 0, nb: Optional[int] = None):
     """lq_decode_step on sequences [b0, b0+nb) of the tensors (all of them by default)."""
-    s = sh.ref() if nb is None and not b0 else _sub(sh, b0, nb)
+    s = _sub(sh, b0, nb)
     cs = C.byref(st.c(b0))
     rc = (_lib or lib()).lq_decode_step(s, cs, _ptr(q, b0), _ptr(k, b0), _ptr(v, b0), _ptr(beta, b0), _ptr(alpha, b0), _ptr(o, b0),
                                         _stream(stream))
