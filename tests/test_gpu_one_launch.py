@@ -12,18 +12,20 @@ G, K = synth.GATE_SCALAR, synth.GATE_DIAG
 HEADS = 4
 
 
-def _shape(batch, W, r, gate, rec16, bf16, n_iter):
-    return lq.Shape(batch, HEADS, 2, 128, 128, W, r, n_iter, gate, 0 if bf16 else 1, 1, rec16, bf16)
+def _shape(batch, W, r, gate, rec16, bf16, n_iter, plain):
+    """`plain`: without the delta rule and without residual smoothing"""
+    return lq.Shape(batch, HEADS, 2, 128, 128, W, r, n_iter, gate, 0 if bf16 or plain else 1, 0 if plain else 1, rec16, bf16)
 
 
-@pytest.mark.parametrize("gate,W,r,rec16,bf16,n_iter", [
-    (G, 16, 4, 0, 0, 1), (G, 1, 2, 0, 0, 1), (G, 2, 0, 0, 0, 1), (G, 5, 8, 1, 0, 2), (G, 64, 3, 1, 0, 1), (G, 40, 16, 0, 0, 1),
-    (K, 16, 4, 0, 0, 1), (K, 12, 4, 1, 0, 1), (G, 11, 4, 1, 0, 2), (K, 6, 8, 0, 0, 1), (K, 7, 0, 1, 0, 1), (K, 33, 5, 0, 0, 1), (K, 64, 16, 0, 0, 2), (K, 13, 9, 1, 0, 1),
-    (G, 16, 0, 0, 1, 1), (G, 9, 0, 1, 1, 1), (K, 64, 0, 0, 1, 1), (K, 3, 0, 1, 1, 1)])
-def test_one_launch_and_two_give_the_same_bits(gate, W, r, rec16, bf16, n_iter):
+@pytest.mark.parametrize("gate,W,r,rec16,bf16,n_iter,plain", [
+    (G, 16, 4, 0, 0, 1, 0), (G, 1, 2, 0, 0, 1, 0), (G, 2, 0, 0, 0, 1, 0), (G, 5, 8, 1, 0, 2, 0), (G, 64, 3, 1, 0, 1, 0), (G, 40, 16, 0, 0, 1, 0),
+    (K, 16, 4, 0, 0, 1, 0), (K, 12, 4, 1, 0, 1, 0), (G, 11, 4, 1, 0, 2, 0), (K, 6, 8, 0, 0, 1, 0), (K, 7, 0, 1, 0, 1, 0), (K, 33, 5, 0, 0, 1, 0), (K, 64, 16, 0, 0, 2, 0), (K, 13, 9, 1, 0, 1, 0),
+    (G, 16, 0, 0, 1, 1, 0), (G, 9, 0, 1, 1, 1, 0), (K, 64, 0, 0, 1, 1, 0), (K, 3, 0, 1, 1, 1, 0),
+    (G, 7, 4, 0, 0, 1, 1), (K, 5, 3, 0, 0, 1, 1), (G, 6, 8, 1, 0, 1, 1), (K, 9, 0, 1, 1, 1, 1)])
+def test_one_launch_and_two_give_the_same_bits(gate, W, r, rec16, bf16, n_iter, plain):
     few = torch.cuda.get_device_properties(0).multi_processor_count // HEADS        # the most sequences of one launch
     B = 2 * few
-    whole, part = _shape(B, W, r, gate, rec16, bf16, n_iter), _shape(few, W, r, gate, rec16, bf16, n_iter)
+    whole, part = _shape(B, W, r, gate, rec16, bf16, n_iter, plain), _shape(few, W, r, gate, rec16, bf16, n_iter, plain)
     assert lq.decode_launches(whole) == 2 and lq.decode_launches(part) == 1
     kw = dict(r=0, smooth=0, state_bf16=1) if bf16 else dict(r=r)
     wl = synth.Workload("one", B, HEADS, 2, W=W, gate=gate, rec16=rec16, seed=900 + W, **kw)

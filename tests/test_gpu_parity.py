@@ -15,6 +15,9 @@ pytestmark = pytest.mark.gpu
 
 GATES = [synth.GATE_SCALAR, synth.GATE_DIAG]
 
+# A step of no more heads than SMs is one launch, of more it is two; most chains run at either side of that line.
+either = lambda few: pytest.mark.parametrize("batch,launches", [(few, 1), (40, 2)])        # (of four heads each)
+
 
 def _close(got, want, what=""):
     assert np.allclose(got, want, rtol=1e-3, atol=1e-5), (what, float(np.abs(got - want).max()))
@@ -82,8 +85,9 @@ def test_reference_kernels(oracle, gate):
     assert np.array_equal(gu.host(S16d), S16)
 
 
-def _run_chain(oracle, wl, steps, init="zero", stagger=False, check_every=1, work=True):
+def _run_chain(oracle, wl, steps, init="zero", stagger=False, check_every=1, work=True, launches=None):
     osh, lsh = gu.shapes(wl)
+    assert launches in (None, lq.decode_launches(lsh))
     ost = OState(osh)
     S0 = np.zeros((wl.batch, wl.heads_v, 128, 128), np.float32) if init == "zero" else synth.dense_states(wl, 9)
     oracle.quantize_state(osh, S0, ost)
@@ -113,35 +117,39 @@ def test_config1_single_head_64_tokens(oracle):
 
 @pytest.mark.parametrize("gate", GATES)
 @pytest.mark.parametrize("W,r", [(8, 4), (16, 4), (32, 4), (16, 8), (1, 0), (3, 2), (64, 4)])
-def test_staggered_batch_chain(oracle, gate, W, r):
+@either(6)
+def test_staggered_batch_chain(oracle, gate, W, r, batch, launches):
     # the shape of the headline workload at a batch the oracle finishes in seconds: grouped heads,
     # window offsets spread uniformly, two full windows
-    wl = synth.Workload("c2", 6, 4, 2, W=W, r=r, gate=gate, seed=400 + W + r)
-    _run_chain(oracle, wl, 2 * W + 3 if W <= 16 else W + 5, init="dense", stagger=True, check_every=4)
+    wl = synth.Workload("c2", batch, 4, 2, W=W, r=r, gate=gate, seed=400 + W + r)
+    _run_chain(oracle, wl, 2 * W + 3 if W <= 16 else W + 5, init="dense", stagger=True, check_every=4, launches=launches)
 
 
 @pytest.mark.parametrize("gate", GATES)
 @pytest.mark.parametrize("r,n_iter", [(4, 2), (8, 3), (16, 2), (3, 4)])
-def test_chain_with_several_rounds_of_power_iteration(oracle, gate, r, n_iter):
+@either(5)
+def test_chain_with_several_rounds_of_power_iteration(oracle, gate, r, n_iter, batch, launches):
     # more than one round: the boundary kernel then also runs W = S^T T and its orthonormalisation between the passes;
     # r = 8 and 16 take the instances of the kernel whose Cholesky factor is computed by a warp
-    wl = synth.Workload("iters", 5, 4, 2, W=8, r=r, n_iter=n_iter, gate=gate, seed=470 + r + n_iter)
-    _run_chain(oracle, wl, 2 * wl.W + 3, init="dense", stagger=True, check_every=4)
+    wl = synth.Workload("iters", batch, 4, 2, W=8, r=r, n_iter=n_iter, gate=gate, seed=470 + r + n_iter)
+    _run_chain(oracle, wl, 2 * wl.W + 3, init="dense", stagger=True, check_every=4, launches=launches)
 
 
 @pytest.mark.parametrize("gate,r,n_iter,rec16", [(0, 9, 1, 0), (0, 16, 3, 0), (1, 16, 1, 1), (1, 10, 2, 0)])
 def test_chain_with_more_than_eight_compensators(oracle, gate, r, n_iter, rec16):
     """Above eight the row sums go through shared memory eight vectors at a time; more heads than one launch takes."""
     wl = synth.Workload("r16", 40, 4, 2, W=4, r=r, n_iter=n_iter, gate=gate, rec16=rec16, seed=475 + r)
-    assert lq.decode_launches(gu.shapes(wl)[1]) == 2
-    _run_chain(oracle, wl, 2 * wl.W + 1, init="dense", stagger=True, check_every=2)
+    _run_chain(oracle, wl, 2 * wl.W + 1, init="dense", stagger=True, check_every=2, launches=2)
 
 
 @pytest.mark.parametrize("gate", GATES)
-def test_chain_without_the_delta_rule(oracle, gate):
-    """b_t = 0 (Mamba2 / GLA style instances): u = v; decode, boundaries and both baseline kernels against the oracle."""
-    wl = synth.Workload("nd", 5, 4, 2, W=4, r=2, gate=gate, seed=470, delta=0)
-    _run_chain(oracle, wl, 14, init="dense", stagger=True, check_every=3)
+@pytest.mark.parametrize("smooth", [1, 0])
+@either(5)
+def test_chain_without_the_delta_rule(oracle, gate, smooth, batch, launches):
+    """b_t = 0 (Mamba2 / GLA style instances): u = v; decode, boundaries and both baseline kernels against the oracle, with and
+    without residual smoothing."""
+    wl = synth.Workload("nd", batch, 4, 2, W=4, r=2, gate=gate, seed=470, delta=0, smooth=smooth)
+    _run_chain(oracle, wl, 14, init="dense", stagger=True, check_every=3, launches=launches)
     osh, lsh = gu.shapes(wl)
     S_o = synth.dense_states(wl, 2)
     S_d = gu.dev(S_o.copy())
@@ -163,11 +171,12 @@ def test_chain_without_the_delta_rule(oracle, gate):
 
 @pytest.mark.parametrize("gate", GATES)
 @pytest.mark.parametrize("W,r", [(16, 4), (5, 2), (32, 0)])
-def test_chain_with_fp16_records(oracle, gate, W, r):
+@either(6)
+def test_chain_with_fp16_records(oracle, gate, W, r, batch, launches):
     """The record buffer in fp16 (the paper's storage): append rounds kt, u (and the diagonal gate's alpha) with
     saturation; decode, boundaries, forced flush and dequantization against the oracle, bit for bit."""
-    wl = synth.Workload("r16", 6, 4, 2, W=W, r=r, gate=gate, seed=480 + W, rec16=1)
-    ost, st = _run_chain(oracle, wl, 2 * W + 3 if W <= 16 else W + 5, init="dense", stagger=True, check_every=4)
+    wl = synth.Workload("r16", batch, 4, 2, W=W, r=r, gate=gate, seed=480 + W, rec16=1)
+    ost, st = _run_chain(oracle, wl, 2 * W + 3 if W <= 16 else W + 5, init="dense", stagger=True, check_every=4, launches=launches)
     osh, lsh = gu.shapes(wl)
     S = torch.empty((wl.batch, wl.heads_v, 128, 128), dtype=torch.float32, device="cuda")
     lq.dequantize_state(lsh, st, S)
@@ -179,12 +188,14 @@ def test_chain_with_fp16_records(oracle, gate, W, r):
 
 @pytest.mark.parametrize("gate", GATES)
 @pytest.mark.parametrize("rec16", [0, 1])
-def test_largest_supported_shape(oracle, gate, rec16):
+@pytest.mark.parametrize("batch,launches", [(2, 1), (80, 2)])
+def test_largest_supported_shape(oracle, gate, rec16, batch, launches):
     """W = 64 and r = 16 together (the largest shared-memory plans of both kernels), windows nearly full so that
     the step crosses a boundary with 64 records; without the delta rule for one of the combinations."""
-    wl = synth.Workload("max", 2, 2, 1, W=64, r=16, gate=gate, seed=490 + rec16, rec16=rec16,
+    wl = synth.Workload("max", batch, 2, 1, W=64, r=16, gate=gate, seed=490 + rec16, rec16=rec16,
                         delta=0 if (gate == synth.GATE_DIAG and rec16) else 1)
     osh, lsh = gu.shapes(wl)
+    assert lq.decode_launches(lsh) == launches
     ost = OState(osh)
     S0 = synth.dense_states(wl, 3)
     oracle.quantize_state(osh, S0, ost)
@@ -207,16 +218,6 @@ def test_largest_supported_shape(oracle, gate, rec16):
 
 
 @pytest.mark.parametrize("gate", GATES)
-def test_fused_step_kernel_gives_the_same_bits(oracle, gate, monkeypatch):
-    """The step as one cooperative kernel (decode slots and boundary CTAs side by side; off by default because it
-    is slower on this GPU): same chain, same oracle, bit for bit, with boundaries in every call."""
-    monkeypatch.setenv("LQ_FUSED_STEP", "1")
-    wl = synth.Workload("fu", 40, 4, 2, W=4, r=2, gate=gate, seed=495)
-    _run_chain(oracle, wl, 11, init="dense", stagger=True, check_every=2)
-    assert lq.check_device() == 0
-
-
-@pytest.mark.parametrize("gate", GATES)
 @pytest.mark.parametrize("work", [False, True])
 def test_heads_of_the_last_round_are_drawn(oracle, gate, work):
     """More than three heads per resident CTA: with the scratch words in the state (lq_state.work) the decode kernel
@@ -232,11 +233,13 @@ def test_heads_of_the_last_round_are_drawn(oracle, gate, work):
     assert lq.check_device() == 0
 
 
-def test_steps_captured_in_a_cuda_graph_replay_identically():
-    """W steps captured once (the two kernels of a step are programmatic dependents of each other) and replayed
-    must leave the same state and outputs as the same steps issued directly."""
-    wl = synth.Workload("cg", 24, 4, 2, W=4, r=2, seed=497)
+@either(24)
+def test_steps_captured_in_a_cuda_graph_replay_identically(batch, launches):
+    """W steps captured once (the kernels of the steps, one each or two, are programmatic dependents of each other) and
+    replayed must leave the same state and outputs as the same steps issued directly."""
+    wl = synth.Workload("cg", batch, 4, 2, W=4, r=2, seed=497)
     _, lsh = gu.shapes(wl)
+    assert lq.decode_launches(lsh) == launches
     S0 = gu.dev(synth.dense_states(wl, 4))
     toks = [gu.tok_dev(synth.token_inputs(wl, t)) for t in range(4)]
     outs = {}
@@ -443,6 +446,41 @@ def test_pipelined_host_steps_back_to_back(oracle, gate, state_bf16):
     assert lq.check_device() == 0
 
 
+@pytest.mark.parametrize("gate", GATES)
+def test_pipelined_host_steps_whose_halves_draw_their_last_heads(gate):
+    """Large enough that the decode kernel of each half of the batch hands out its last heads by tickets, each half from a
+    scratch word of its own, which the one boundary launch behind both puts back: the same tokens by plain steps give the same
+    bits, and the words are zero afterwards."""
+    wl = synth.Workload("hd", 208, 32, 16, W=3, r=2, gate=gate, seed=770)
+    _, lsh = gu.shapes(wl)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert wl.batch // 2 * wl.heads_v >= 3 * 6 * sms                # three rounds of the CTAs that fit at once
+    S = torch.randn((wl.batch, wl.heads_v, 128, 128), generator=torch.Generator("cuda").manual_seed(3), device="cuda")
+    plain, piped = lq.State(lsh), lq.State(lsh)
+    for st in (plain, piped):
+        lq.quantize_state(lsh, S, st)
+        st.win_pos.copy_(torch.arange(wl.batch, device="cuda") % wl.W)
+        st.buf_a.fill_(0.5)
+    stage = torch.empty((lq.decode_stage_bytes(lsh),), dtype=torch.uint8, device="cuda")
+    toks = [gu.tok_dev(synth.token_inputs(wl, t)) for t in range(2)]
+    pins = [{k: v.cpu().pin_memory() for k, v in tok.items()} for tok in toks]
+    steps = 2 * wl.W + 1
+    outs = [torch.full((wl.batch, wl.heads_v, 128), float("nan"), dtype=torch.float32).pin_memory() for _ in range(steps)]
+    for t in range(steps):                   # (chained: nothing waits in between)
+        d = pins[t % 2]
+        lq.decode_step_host_pipelined(lsh, piped, d["q"], d["k"], d["v"], d["beta"], d["alpha"], outs[t], stage)
+    torch.cuda.synchronize()
+    assert not piped.work.any()
+    o = torch.empty((wl.batch, wl.heads_v, 128), dtype=torch.float32, device="cuda")
+    for t in range(steps):
+        d = toks[t % 2]
+        lq.decode_step(lsh, plain, d["q"], d["k"], d["v"], d["beta"], d["alpha"], o)
+        assert torch.equal(o.cpu(), outs[t]), f"step {t}"
+    for name, a, b in zip(("heads", "records", "decays", "win_pos"), plain.tensors(), piped.tensors()):
+        assert torch.equal(a, b), name
+    assert lq.check_device() == 0
+
+
 # ---- per-window BF16 (the -w baseline): bfloat16 boundary state, no scale, smoothing or compensators ----
 
 def _bf16w(name, batch, heads_v, heads_qk, **kw):
@@ -451,10 +489,11 @@ def _bf16w(name, batch, heads_v, heads_qk, **kw):
 
 @pytest.mark.parametrize("gate", GATES)
 @pytest.mark.parametrize("W,rec16,delta", [(16, 0, 1), (1, 0, 1), (5, 1, 1), (64, 0, 1), (40, 1, 0)])
-def test_per_window_bf16_chain(oracle, gate, W, rec16, delta):
+@either(6)
+def test_per_window_bf16_chain(oracle, gate, W, rec16, delta, batch, launches):
     """Every output, the bfloat16 boundary state after every boundary and the record buffer, bit for bit."""
-    wl = _bf16w("w", 6, 4, 2, W=W, gate=gate, rec16=rec16, delta=delta, seed=600 + W)
-    _run_chain(oracle, wl, 2 * W + 3 if W <= 16 else W + 5, init="dense", stagger=True, check_every=4)
+    wl = _bf16w("w", batch, 4, 2, W=W, gate=gate, rec16=rec16, delta=delta, seed=600 + W)
+    _run_chain(oracle, wl, 2 * W + 3 if W <= 16 else W + 5, init="dense", stagger=True, check_every=4, launches=launches)
 
 
 @pytest.mark.parametrize("gate", GATES)

@@ -144,13 +144,16 @@ def test_config1_single_head_against_the_plain_definition(oracle, oracle_plain):
     _teacher_forced_chain(oracle, oracle_plain, synth.config("single_gdn"), 64, "single_gdn", init="zero", stagger=False)
 
 
-@pytest.mark.parametrize("gate,name", [(synth.GATE_SCALAR, "gdn staggered, 12 x 8 heads"),
-                                       (synth.GATE_DIAG, "kda outliers staggered, 12 x 8 heads")])
-def test_staggered_chain_against_the_plain_definition(oracle, oracle_plain, gate, name):
+@pytest.mark.parametrize("batch,launches", [(12, 1), (19, 2)])
+@pytest.mark.parametrize("gate,name", [(synth.GATE_SCALAR, "gdn staggered, %d x 8 heads"),
+                                       (synth.GATE_DIAG, "kda outliers staggered, %d x 8 heads")])
+def test_staggered_chain_against_the_plain_definition(oracle, oracle_plain, gate, name, batch, launches):
+    name = name % batch
     if gate == synth.GATE_DIAG:
-        wl = synth.config("kda_b128_outlier").with_(batch=12, heads_v=8, heads_qk=8)
+        wl = synth.config("kda_b128_outlier").with_(batch=batch, heads_v=8, heads_qk=8)
     else:
-        wl = synth.config("gdn_b256").with_(batch=12, heads_v=8, heads_qk=4)
+        wl = synth.config("gdn_b256").with_(batch=batch, heads_v=8, heads_qk=4)
+    assert lq.decode_launches(gu.shapes(wl)[1]) == launches
     _teacher_forced_chain(oracle, oracle_plain, wl, 2 * wl.W + 3, name)
 
 

@@ -40,13 +40,15 @@ def _guarded_state(sh):
 
 
 @pytest.mark.parametrize("gate", [synth.GATE_SCALAR, synth.GATE_DIAG])
-@pytest.mark.parametrize("batch,heads_v,heads_qk,W,r,rec16", [(3, 5, 5, 64, 16, 0),      # the largest window and token count
-                                                              (3, 5, 5, 64, 16, 1),
-                                                              (41, 23, 23, 4, 2, 0),     # more heads than resident CTAs, odd counts
-                                                              (2, 4, 2, 16, 4, 0)])
-def test_no_entry_point_writes_outside_its_buffers(gate, batch, heads_v, heads_qk, W, r, rec16):
+@pytest.mark.parametrize("batch,heads_v,heads_qk,W,r,rec16,launches", [
+    (3, 5, 5, 64, 16, 0, 1), (31, 5, 5, 64, 16, 0, 2),       # the largest window and token count, a step as one launch and as two
+    (3, 5, 5, 64, 16, 1, 1), (31, 5, 5, 64, 16, 1, 2),
+    (41, 23, 23, 4, 2, 0, 2),                                # more heads than resident CTAs, odd counts
+    (2, 4, 2, 16, 4, 0, 1), (38, 4, 2, 16, 4, 0, 2)])
+def test_no_entry_point_writes_outside_its_buffers(gate, batch, heads_v, heads_qk, W, r, rec16, launches):
     wl = synth.Workload("guard", batch, heads_v, heads_qk, W=W, r=r, gate=gate, rec16=rec16, seed=900 + W + r)
     _, sh = gu.shapes(wl)
+    assert lq.decode_launches(sh) == launches
     st, g = _guarded_state(sh)
     S_in = Guarded((batch, heads_v, 128, 128), torch.float32)
     S_in.t.copy_(gu.dev(synth.dense_states(wl, 2)))
@@ -76,12 +78,14 @@ def test_no_entry_point_writes_outside_its_buffers(gate, batch, heads_v, heads_q
 
 @pytest.mark.parametrize("gate", [synth.GATE_SCALAR, synth.GATE_DIAG])
 @pytest.mark.parametrize("rec16", [0, 1])
-def test_checkpoint_in_mid_window_resumes_bit_for_bit(gate, rec16):
+@pytest.mark.parametrize("batch,launches", [(6, 1), (40, 2)])
+def test_checkpoint_in_mid_window_resumes_bit_for_bit(gate, rec16, batch, launches):
     """After 5 + 2 W tokens (five records in the buffer) the four arrays of the state are copied to the host; the
     run goes on for W + 7 tokens (through a boundary).  Restored into fresh device memory and fed the same tokens,
     the copy must produce the same outputs and end in the same state, bit for bit."""
-    wl = synth.Workload("ckpt", 6, 4, 2, W=8, r=4, gate=gate, rec16=rec16, seed=950 + gate + 2 * rec16)
+    wl = synth.Workload("ckpt", batch, 4, 2, W=8, r=4, gate=gate, rec16=rec16, seed=950 + gate + 2 * rec16)
     _, sh = gu.shapes(wl)
+    assert lq.decode_launches(sh) == launches
     st = lq.State(sh)
     lq.quantize_state(sh, gu.dev(synth.dense_states(wl, 5)), st)
     # stagger the windows a little: the first three sequences take one token more than the others
