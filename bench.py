@@ -65,7 +65,7 @@ def record_bytes(diag: bool, rec16: int) -> int:
     return 4 * (256 + (128 if diag else 1))
 
 
-def algorithmic_bytes_per_head_step(W: int, r: int, diag: bool, group: int, launches_fused: bool, rec16: int = 0) -> float:
+def algorithmic_bytes_per_head_step(W: int, r: int, diag: bool, group: int, rec16: int = 0) -> float:
     """Bytes that must move per (head, token): quantized state + average record buffer + inputs + appended
     record + output + the window boundary amortised over W tokens."""
     g = 128 if diag else 1
@@ -73,7 +73,7 @@ def algorithmic_bytes_per_head_step(W: int, r: int, diag: bool, group: int, laun
     rec = record_bytes(diag, rec16)
     buf_read = (W - 1) / 2.0 * rec
     inputs = 512 / group + 256 + 2 + 2 * g
-    flush = state + (0 if launches_fused else state + W * rec)      # write back (+ re-read when a second kernel does it)
+    flush = 2 * state + W * rec                                     # re-read (also by the one launch of few heads) and written back
     return state + buf_read + inputs + rec + 512 + flush / W
 
 
@@ -460,7 +460,7 @@ def run_cuda(args, wl):
     launches = lq.decode_launches(sh)
     peak, peak_src = peaks()
     group = wl.heads_v // wl.heads_qk
-    bytes_hs = algorithmic_bytes_per_head_step(wl.W, wl.r, wl.gate == synth.GATE_DIAG, group, launches == 1, wl.rec16)
+    bytes_hs = algorithmic_bytes_per_head_step(wl.W, wl.r, wl.gate == synth.GATE_DIAG, group, wl.rec16)
     achieved = heads * bytes_hs / (ms_per_step / 1e3) / 1e9
     rec = record_bytes(wl.gate == synth.GATE_DIAG, wl.rec16)
     # what each kernel has to move per launch: the decode kernel everything but the boundary; the boundary
@@ -630,7 +630,7 @@ def run_sweep(args):
                                                                   ("q", "k", "v", "beta", "alpha")], o, stream), nrep, W)
                     flags = lq.check_device()
                     heads = B * 32
-                    bytes_hs = algorithmic_bytes_per_head_step(W, r, diag, wl.heads_v // wl.heads_qk, False, rec16)
+                    bytes_hs = algorithmic_bytes_per_head_step(W, r, diag, wl.heads_v // wl.heads_qk, rec16)
                     foot = st.heads.numel() + st.records.numel() * st.records.element_size()
                     state_b = 128 * 128 + 4 * 128 + 4 * 128 + 2 * r * 256
                     row = {"sweep": True, "gate": gate_name, "batch": B, "W": W, "r": r, "n_iter": wl.n_iter,

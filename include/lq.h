@@ -154,9 +154,10 @@ lq_status lq_decode_step(const lq_shape *shape, const lq_state *state, const uin
                          const uint16_t *v, const uint16_t *beta, const uint16_t *alpha, float *o, lq_stream stream);
 
 /*
- * lq_decode_step for a measuring harness: identical work, and in addition the CUDA event `event_between`
+ * lq_decode_step for a measuring harness: the same results, and in addition the CUDA event `event_between`
  * (a cudaEvent_t created by the caller; may be null) is recorded on `stream` between the decode kernel and
- * the window-boundary kernel, so that the two can be timed separately.
+ * the window-boundary kernel, so that the two can be timed separately.  With an event the step is always these
+ * two launches, also where lq_decode_step makes one of both (lq_decode_launches).
  */
 lq_status lq_decode_step_profiled(const lq_shape *shape, const lq_state *state, const uint16_t *q, const uint16_t *k,
                                   const uint16_t *v, const uint16_t *beta, const uint16_t *alpha, float *o,
