@@ -380,7 +380,9 @@ static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStrea
 // SM's registers).  W = 16, r = 4, us per step in a graph as two launches / one: 1 head 6.7 / 5.1, 32 heads 6.7 / 5.2, 128 heads
 // 8.3 / 6.9, 148 heads of 37 sequences 13.8 / 12.7, 184 heads 14.5 / 14.5, 280 heads 14.2 / 16.1; 128 heads, diagonal gate,
 // W = 64, r = 8: 11.4 / 8.4; called one by one from the host, 1 to 128 heads: 11 / 8.4.  (With the instances for exactly four
-// and eight compensators a step of 148 heads takes 12.0 instead of 12.7 us, of 128 heads, W = 8, 10.6 instead of 11.3.)
+// and eight compensators a step of 148 heads takes 12.0 instead of 12.7 us, of 128 heads, W = 8, 10.6 instead of 11.3.)  Two streams
+// of 40 to 148 heads each, which then share the GPU less well: 9.6 to 13.4 us for a step of both, 12.4 to 17.8 as two launches each
+// (kernels of an earlier build; r = 8 12.1 to 17.3 and 15.9 to 24.2).
 static bool one_launch(const lq_shape *s) {
   return (long)s->batch * s->heads_v <= sm_count();
 }
@@ -736,7 +738,8 @@ lq_status lq_decode_step_host_pipelined(const lq_shape *shape, const lq_state *s
       }
       // Sixteen CTAs (262 KB in flight, which the bus does not need more of): each of them keeps a decode CTA of the other
       // sub-batch waiting for its place.  256 x 32 heads: 202 us a call by itself and 151 chained; with 74 CTAs 210 and 158
-      // (the decode kernel of half a batch took 43 us instead of 24), with 8 CTAs 222 and 172.
+      // (the decode kernel of half a batch took 43 us instead of 24), with 8 CTAs 222 and 172.  From 16 to 256 sequences of 8 to 64
+      // heads and with either gate no other number did better by more than 6 %: 24, 32 and 48 are slower in most by 3 to 20 %.
       ok = launch(gather_kernel, 16, 256, 0, hp->s_in, g) == LQ_OK;
     } else {
       for (int i = 0; ok && i < 5; i++)

@@ -11,7 +11,7 @@
 // What bounds it: a flush (W = 16, r = 4) takes 23 K cycles with two CTAs on the SM (27 K before two records and two start
 // vectors were in flight at a time); 9 K of them are the fp32 pipes (about 1150 packed FMAs per warp, two cycles each, four
 // warps to a scheduler), the rest the waits between its dependent phases, of which only the other CTA fills some.  Issue slots
-// are 41 % busy.  Against tiles of 8 rows x 128 columns per half-warp, where every column sum crossed the CTA (13 barriers a
+// are 48 % busy.  Against tiles of 8 rows x 128 columns per half-warp, where every column sum crossed the CTA (13 barriers a
 // head, now 8), and copies by all threads into two staging buffers: 2048 dense states quantized in 55.2 us (91.4 before),
 // 2048 states dequantized in 45.6 us (54.0); a step of 256 x 32 heads, 512 of them due, 73 -> 61 us.
 #pragma once
@@ -292,7 +292,8 @@ __device__ __forceinline__ uint32_t orthonormalize(float *X, int r, float *gram,
 
 // MODE 0 flush (window representation -> dense -> new window representation), 1 quantize dense fp32 states,
 // 2 dequantize to dense fp32 states.  RM: the largest r the instance handles; 0: no compensators at all (an instance of its
-// own: told apart inside the others, the two ways cost 400 bytes of spills).
+// own: told apart inside the others, the two ways cost those 400 bytes of spills; in the one for r = 0 the compiler still spills
+// 280 bytes: 256 x 32 heads, W = 16, r = 0, 53.0 us a step, 71.7 with the former layout, which spilled none).
 // BF16: the per-window BF16 state (lq_shape.state_bf16, RM = 0): the dense state is rounded to bfloat16, and that is all.
 // slots: 1 or 2.
 // EXACT: r is RM, known at compile time: without a test per vector the compiler interleaves the four or eight column sums
@@ -340,7 +341,7 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
     __syncthreads();
   }
   grid_dependency_wait();                    // everything the kernel before this one wrote is visible from here on
-  if (STEP) grid_dependents_may_start();     // (the next step's few CTAs find room beside these)
+  if (STEP) grid_dependents_may_start();     // (up to half as many heads as SMs, the next step's CTAs find room beside these)
   LQ_STAMP(1, 1);
 #ifdef LQ_TIMING
   if (tid == 0) { for (int i = 0; i < 16; i++) lq_bacc[i] = 0; lq_btick = clock64(); }
