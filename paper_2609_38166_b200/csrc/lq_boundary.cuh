@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(256, STEP ? 1 : 2) boundary_kernel(const Param
     for (int k = 0; k < count; k++) {
       const size_t bh = todo_bh[k];
       if (MODE == 0 && p.overlap && count < 32 && k == count - 1) grid_dependents_may_start();
-      const int n = MODE == 0 ? max(todo_n[k], 1) : todo_n[k];          // (never 0 when due)
+      const int n = todo_n[k];                                // (never 0 when due)
       unsigned char *slot = lq_bsm + Lay::head + at * L.slot;
       rec_t *rec = reinterpret_cast<rec_t *>(slot + L.rec);
       auto kd_row = [&](int j) -> float * {                   // Gamma_{j+1:n} kt_j
