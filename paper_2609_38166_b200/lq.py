@@ -228,7 +228,7 @@ def _sub(sh: Shape, b0: int, nb: Optional[int]):
 
 def decode_step(sh: Shape, st: State, q, k, v, beta, alpha, o, stream=None, b0: int = 0, nb: Optional[int] = None):
     """lq_decode_step on sequences [b0, b0+nb) of the tensors (all of them by default)."""
-    s = _sub(sh, b0, nb)
+    s = sh.ref() if nb is None and not b0 else _sub(sh, b0, nb)
     cs = C.byref(st.c(b0))
     rc = (_lib or lib()).lq_decode_step(s, cs, _ptr(q, b0), _ptr(k, b0), _ptr(v, b0), _ptr(beta, b0), _ptr(alpha, b0), _ptr(o, b0),
                                         _stream(stream))
