@@ -122,6 +122,7 @@ __device__ __forceinline__ void bulk_prefetch_l2(const void *src, uint32_t bytes
 // Bounded wait for phase `parity`; false if the limit of LIMIT polls ran out (the caller then reports and bails out).
 template <int LIMIT = (1 << 20)>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+#pragma unroll 1                             // (unrolled, the waits were a fifth of the decode kernel's code)
   for (int spin = 0; spin < LIMIT; spin++) {
     uint32_t done;
     asm volatile(

@@ -140,6 +140,225 @@ __device__ __forceinline__ void bf16_columns(const uint16_t *S0T, int j0, const 
   }
 }
 
+// Compensator keys against Gamma_{1:l} k and Gamma_{1:l} q, by one warp: the projections go to pk[h], pq[h].  A dot product of 128
+// terms is taken by sixteen lanes (lane c owns block c of eight terms); the two halves of the warp work on different vectors, two
+// per half and trip, so that four shuffle trees overlap.  Both halves make the same number of trips (the shuffles name all 32
+// lanes); an index outside the range recomputes a valid item and is not stored.
+__device__ __forceinline__ void project_compensators(const uint16_t *ckh, int r, const float2 (&gam)[4], const float2 (&k2)[4],
+                                                     const float2 (&q2)[4], float *pk, float *pq, int lane) {
+  const int c = lane & 15, half = lane >> 4;
+  float2 gk2[4], gq2[4];
+#pragma unroll
+  for (int cc = 0; cc < 4; cc++) { gk2[cc] = __fmul2_rn(gam[cc], k2[cc]); gq2[cc] = __fmul2_rn(gam[cc], q2[cc]); }
+#pragma unroll 1
+  for (int hb = 0; hb < r; hb += 4) {
+    float s4[4];
+    int ho[2];
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      ho[u] = hb + 2 * u + half;
+      const int h = ho[u] < r ? ho[u] : r - 1;
+      float x8[8];
+      widen8_f16(*reinterpret_cast<const uint4 *>(ckh + h * D + 8 * c), x8);
+      float2 x2[4];
+#pragma unroll
+      for (int cc = 0; cc < 4; cc++) x2[cc] = make_float2(x8[2 * cc], x8[2 * cc + 1]);
+      s4[2 * u] = block8(x2, gk2);
+      s4[2 * u + 1] = block8(x2, gq2);
+    }
+    tree16x4(s4);
+#pragma unroll
+    for (int u = 0; u < 2; u++)
+      if (c == 0 && ho[u] < r) { pk[ho[u]] = s4[2 * u]; pq[ho[u]] = s4[2 * u + 1]; }
+  }
+}
+
+// 2 NP records jt, jt-1, ...: half 0 projects the first, third, ... of them, half 1 the others.  The sums over the sixteen
+// lanes are taken by halving exchanges (eight values: 4 + 2 + 1 + 1 shuffles), after which a lane holds one of them;
+// through pj every lane gets all.  A group of four may run past record `base`; what lies below is computed from that record and
+// dropped.  `seg`: the rows at hand, beginning with record `base`; bas: the records' decays (scalar gate); g2 or (scalar gate) g1:
+// Gamma_{jt+1:l}, kept up (and past record `base` exactly at the end).  With one number in place of the scalar gate's vector the walk
+// takes about 30 instructions less for a pair of records: with the waits not unrolled (mbar_wait) 1024 x 32 heads, W = 32, 259 -> 252 us a step.
+template <int GATE, int NP, typename rec_t>
+__device__ __forceinline__ void walk_group(const rec_t *seg, const int base, const float *bas, float *pj, const int jt, const int lane,
+                                           const float2 (&k2)[4], const float2 (&q2)[4], float2 (&g2)[4], float &g1,
+                                           float2 (&rk_rec)[2], float2 (&rq_rec)[2]) {
+  constexpr bool DIAG = GATE == LQ_GATE_DIAG, MASKED = NP == 2;
+  constexpr int RF = record_floats(DIAG);
+  const int c = lane & 15, half = lane >> 4;
+  float v[2 * NP];
+#pragma unroll
+  for (int u = 0; u < NP; u++) {
+    // the decays of the two records of this pair; the half that owns the older one steps over the newer
+    const int jn = jt - 2 * u, jold = jn - 1;  // newer, older
+    const int in = MASKED ? max(jn, base) : jn, iold = MASKED ? max(jold, base) : jold;
+    float2 gmine[4];
+    // past both records, as far as they are there (selects: a branch for the last trip of a long head was slower)
+    if constexpr (DIAG) {
+      float2 an[4], ao[4];
+      load8p(seg + (in - base) * RF + REC_A + 8 * c, an);
+      load8p(seg + (iold - base) * RF + REC_A + 8 * c, ao);
+#pragma unroll
+      for (int cc = 0; cc < 4; cc++) {
+        const float2 gn = g2[cc], go = __fmul2_rn(gn, an[cc]);   // Gamma_{jn+1:l}, Gamma_{jold+1:l}
+        gmine[cc] = half ? go : gn;
+        g2[cc] = !MASKED || jold >= base ? __fmul2_rn(go, ao[cc]) : jn >= base ? go : gn;
+      }
+    } else {
+      const float gn = g1, go = gn * bas[in], past = go * bas[iold];
+      g1 = !MASKED || jold >= base ? past : jn >= base ? go : gn;
+#pragma unroll
+      for (int cc = 0; cc < 4; cc++) gmine[cc] = pair(half ? go : gn);
+    }
+    const int j = half ? iold : in;
+    float2 x2[4], yk2[4], yq2[4];
+    load8p(seg + (j - base) * RF + REC_KT + 8 * c, x2);
+#pragma unroll
+    for (int cc = 0; cc < 4; cc++) { yk2[cc] = __fmul2_rn(gmine[cc], k2[cc]); yq2[cc] = __fmul2_rn(gmine[cc], q2[cc]); }
+    v[2 * u] = block8(x2, yk2);
+    v[2 * u + 1] = block8(x2, yq2);
+  }
+  // halving exchanges over lane bits 0, 1, (2), then plain ones; lane c ends with value `mine` of its half
+  const bool u0 = lane & 1, u1 = lane & 2, u2 = lane & 4;
+  float x;
+  int mine;
+  if constexpr (NP == 4) {
+    float x4[4], x2_[2];
+#pragma unroll
+    for (int e = 0; e < 4; e++) x4[e] = (u0 ? v[e + 4] : v[e]) + __shfl_xor_sync(FULL, u0 ? v[e] : v[e + 4], 1);
+#pragma unroll
+    for (int e = 0; e < 2; e++) x2_[e] = (u1 ? x4[e + 2] : x4[e]) + __shfl_xor_sync(FULL, u1 ? x4[e] : x4[e + 2], 2);
+    x = (u2 ? x2_[1] : x2_[0]) + __shfl_xor_sync(FULL, u2 ? x2_[0] : x2_[1], 4);
+    mine = (u0 ? 4 : 0) + (u1 ? 2 : 0) + (u2 ? 1 : 0);
+  } else {
+    float x2_[2];
+#pragma unroll
+    for (int e = 0; e < 2; e++) x2_[e] = (u0 ? v[e + 2] : v[e]) + __shfl_xor_sync(FULL, u0 ? v[e] : v[e + 2], 1);
+    x = (u1 ? x2_[1] : x2_[0]) + __shfl_xor_sync(FULL, u1 ? x2_[0] : x2_[1], 2);
+    x = x + __shfl_xor_sync(FULL, x, 4);
+    mine = (u0 ? 2 : 0) + (u1 ? 1 : 0);
+  }
+  x = x + __shfl_xor_sync(FULL, x, 8);
+  __syncwarp();                                // (the group before has been read)
+  if (c < 2 * NP) pj[(mine & 1) * 8 + (mine & ~1) + half] = x;     // pj[vector][record]
+  __syncwarp();
+  float pk_[2 * NP], pq_[2 * NP];
+#pragma unroll
+  for (int e = 0; e < NP / 2; e++) {
+    const float4 a = *reinterpret_cast<const float4 *>(pj + 4 * e), b = *reinterpret_cast<const float4 *>(pj + 8 + 4 * e);
+    pk_[4 * e] = a.x; pk_[4 * e + 1] = a.y; pk_[4 * e + 2] = a.z; pk_[4 * e + 3] = a.w;
+    pq_[4 * e] = b.x; pq_[4 * e + 1] = b.y; pq_[4 * e + 2] = b.z; pq_[4 * e + 3] = b.w;
+  }
+#pragma unroll
+  for (int e = 0; e < 2 * NP; e++) {
+    const int j = jt - e;
+    if (MASKED && j < base) break;             // the same for every lane
+    const float4 u4 = load4(seg + (j - base) * RF + REC_U + 4 * lane);
+    const float2 lo = make_float2(u4.x, u4.y), hi = make_float2(u4.z, u4.w), pk2 = pair(pk_[e]), pq2 = pair(pq_[e]);
+    rk_rec[0] = __ffma2_rn(lo, pk2, rk_rec[0]); rq_rec[0] = __ffma2_rn(lo, pq2, rq_rec[0]);
+    rk_rec[1] = __ffma2_rn(hi, pk2, rk_rec[1]); rq_rec[1] = __ffma2_rn(hi, pq2, rq_rec[1]);
+  }
+}
+// The records from jt back to `base`: eight at a time while they last, then four.
+template <int GATE, typename rec_t>
+__device__ __forceinline__ void walk_records(const rec_t *seg, const int base, const float *bas, float *pj, int jt, const int lane,
+                                             const float2 (&k2)[4], const float2 (&q2)[4], float2 (&g2)[4], float &g1,
+                                             float2 (&rk_rec)[2], float2 (&rq_rec)[2]) {
+#pragma unroll 1
+  for (; jt - 7 >= base; jt -= 8) walk_group<GATE, 4>(seg, base, bas, pj, jt, lane, k2, q2, g2, g1, rk_rec, rq_rec);
+#pragma unroll 1
+  for (; jt >= base; jt -= 4) walk_group<GATE, 2>(seg, base, bas, pj, jt, lane, k2, q2, g2, g1, rk_rec, rq_rec);
+}
+
+// C Gamma k (lanes 0..15) and C Gamma q (lanes 16..31) on their fixed-point grids, as digit planes; back_*: what a unit of the
+// grids is worth
+__device__ __forceinline__ void digit_planes(const float *cs, const float (&gam)[8], const float (&k8)[8], const float (&q8)[8],
+                                             int8_t *digits, int lane, float &back_k, float &back_q) {
+  const int c = lane & 15, half = lane >> 4;
+  float back_own;
+  {
+    float c8[8], x8[8];
+    load8(cs + 8 * c, c8);
+    float m = 0.0f;
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+      x8[e] = c8[e] * (gam[e] * (half ? q8[e] : k8[e]));
+      m = fmaxf(m, fabsf(x8[e]));
+    }
+#pragma unroll
+    for (int s = 1; s <= 8; s <<= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, s));
+    float scale;
+    fixed_point_scales(m, scale, back_own);
+    // X = d0 + 256 d1 + 65536 d2 + 2^24 d3 with digits in [-128, 127]: the digit is the low byte read as
+    // signed, and taking it off is (X + 128) >> 8.  The bytes of the four stages of an element are the
+    // four digits; prmt gathers the same digit of four elements into one word.
+    uint32_t st[8][4];
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+      int X = __float2int_rn(x8[e] * scale);
+#pragma unroll
+      for (int d = 0; d < 4; d++) { st[e][d] = static_cast<uint32_t>(X); X = (X + 128) >> 8; }
+    }
+#pragma unroll
+    for (int d = 0; d < 4; d++) {
+      const uint32_t lo = __byte_perm(__byte_perm(st[0][d], st[1][d], 0x0040), __byte_perm(st[2][d], st[3][d], 0x0040), 0x5410);
+      const uint32_t hi = __byte_perm(__byte_perm(st[4][d], st[5][d], 0x0040), __byte_perm(st[6][d], st[7][d], 0x0040), 0x5410);
+      *reinterpret_cast<uint2 *>(digits + (4 * half + d) * D + 8 * c) = make_uint2(lo, hi);
+    }
+  }
+  const float back_other = __shfl_xor_sync(FULL, back_own, 16);
+  back_k = half ? back_other : back_own;
+  back_q = half ? back_own : back_other;
+}
+
+// The state stream on the tensor cores: eight 16-row tiles of Z^T, K = 128 as four k-blocks.  A
+// thread's 16 bytes of a row hold key channels 64p+16t..64p+16t+15 and serve two k-blocks; the digit
+// planes are read with the same permutation of the key index.  The two 64-channel halves of a tile
+// accumulate separately (exact integers: any split gives the same sum), which halves the dependent
+// chain of MMAs.  Digit pairs are recombined in int32 (|sum| < 2^30), the two pairs in int64 (the total has
+// 47 bits), and one rounding takes it to fp32.
+__device__ __forceinline__ void code_sums(const int8_t *zt, const int8_t *digits, float *y, int lane) {
+  const int g = lane >> 2, t = lane & 3;
+  constexpr int h0 = 0, h1 = 64;         // the two 64-channel halves (the same split for every lane)
+  const uint4 bfa = *reinterpret_cast<const uint4 *>(digits + g * D + h0 + 16 * t);
+  const uint4 bfb = *reinterpret_cast<const uint4 *>(digits + g * D + h1 + 16 * t);
+  constexpr int TILES = 8, mg = 0;
+  {
+    int pair_lo[TILES], pair_hi[TILES];  // digit-pair sums of rows g and g+8 of each tile
+#pragma unroll
+    for (int mt = 0; mt < TILES; mt++) {
+      int ca[4] = {0, 0, 0, 0}, cb[4] = {0, 0, 0, 0};
+      const int j = 16 * (mg + mt) + g;
+      const uint4 alo = *reinterpret_cast<const uint4 *>(zt + j * D + h0 + 16 * t);
+      const uint4 ahi = *reinterpret_cast<const uint4 *>(zt + (j + 8) * D + h0 + 16 * t);
+      const uint4 blo = *reinterpret_cast<const uint4 *>(zt + j * D + h1 + 16 * t);
+      const uint4 bhi = *reinterpret_cast<const uint4 *>(zt + (j + 8) * D + h1 + 16 * t);
+      mma_s8(ca, alo.x, ahi.x, alo.y, ahi.y, bfa.x, bfa.y);
+      mma_s8(cb, blo.x, bhi.x, blo.y, bhi.y, bfb.x, bfb.y);
+      mma_s8(ca, alo.z, ahi.z, alo.w, ahi.w, bfa.z, bfa.w);
+      mma_s8(cb, blo.z, bhi.z, blo.w, bhi.w, bfb.z, bfb.w);
+      // c[0], c[1]: row g, planes 2t, 2t+1;  c[2], c[3]: row g+8.  Planes 4v..4v+3 are the digits of
+      // vector v: lanes t = 0, 1 carry the k sums and t = 2, 3 the q sums, even t the low digit pair.
+      pair_lo[mt] = (ca[0] + cb[0]) + ((ca[1] + cb[1]) << 8);
+      pair_hi[mt] = (ca[2] + cb[2]) + ((ca[3] + cb[3]) << 8);
+    }
+    int oth_lo[TILES], oth_hi[TILES];
+#pragma unroll
+    for (int mt = 0; mt < TILES; mt++) {
+      oth_lo[mt] = __shfl_xor_sync(FULL, pair_lo[mt], 1);
+      oth_hi[mt] = __shfl_xor_sync(FULL, pair_hi[mt], 1);
+    }
+    if (!(t & 1)) {                      // this lane has the low pairs, its neighbour sent the high pairs
+      float *dst = y + (t >> 1) * D + g + 16 * mg;
+#pragma unroll
+      for (int mt = 0; mt < TILES; mt++) {
+        dst[16 * mt] = __ll2float_rn(static_cast<long long>(oth_lo[mt]) * 65536 + pair_lo[mt]);
+        dst[16 * mt + 8] = __ll2float_rn(static_cast<long long>(oth_hi[mt]) * 65536 + pair_hi[mt]);
+      }
+    }
+  }
+}
+
 // Named barriers of the CTA (64 threads each): one side arrives, the other waits.
 //   1: dot warp -> stream warp, "the record terms (and the ticket) are in shared memory"
 //   2: stream warp -> dot warp, "its sums are out of y"
@@ -204,7 +423,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
   constexpr int SEG = LONGW ? rec_seg(R16) : 0;
   const DecodeSlot L(W, r, DIAG, R16, BF16, SEG);
   const uint32_t block_bytes = BF16 ? BF16W_HEAD_BYTES : head_bytes(r);
-  const int c = lane & 15, half = lane >> 4, g = lane >> 2, t = lane & 3;
+  const int c = lane & 15, half = lane >> 4;
   const int8_t *zt = reinterpret_cast<const int8_t *>(slot + L.head + HB_CODES);
   const float *bs = reinterpret_cast<const float *>(slot + L.head + HB_COL_SCALE);
   const float *cs = reinterpret_cast<const float *>(slot + L.head + HB_ROW_SMOOTH);
@@ -427,7 +646,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
     if (!DIAG) {
       __syncwarp();
 #pragma unroll 4
-      for (int j = n - 1; j >= 0; j--) gsc = gsc * bas[j];
+      for (int j = role == 0 ? n - 1 : -1; j >= 0; j--) gsc = gsc * bas[j];
     }
     // kt^T q needs only the token: the dot warp takes it before the wait as well.  It goes to one of two places
     // in turn, because the stream warp may still be reading the previous head's.  In turn over the heads WITH a token: the
@@ -455,10 +674,6 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
 
     if (role == 1) {
       // =========================== DOT WARP ===========================
-      // Projections.  A dot product of 128 terms is taken by sixteen lanes (lane c owns block c of eight
-      // terms); the two halves of the warp work on different vectors, two per half and trip, so that four
-      // shuffle trees overlap.  Both halves make the same number of trips (the shuffles name all 32 lanes);
-      // an index outside the range recomputes a valid item and is not stored.
       // Records are walked from the newest back, with g8 = Gamma_{j+1:l} kept up on the way (Appendix B.2).
       float2 k2[4], q2[4], a2[4], g2[4], kt2[4];
 #pragma unroll
@@ -470,131 +685,26 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         kt2[cc] = __fmul2_rn(pair(beta), k2[cc]);
       }
       wait_records();                        // the newest segment of the records
-      // Compensator keys against Gamma_{1:l} k and Gamma_{1:l} q (the projections go to pk[h], pq[h]).
-      auto project_compensators = [&](const float2 (&gam)[4]) {
-        float2 gk2[4], gq2[4];
-#pragma unroll
-        for (int cc = 0; cc < 4; cc++) { gk2[cc] = __fmul2_rn(gam[cc], k2[cc]); gq2[cc] = __fmul2_rn(gam[cc], q2[cc]); }
-        for (int hb = 0; hb < r; hb += 4) {
-          float s4[4];
-          int ho[2];
-#pragma unroll
-          for (int u = 0; u < 2; u++) {
-            ho[u] = hb + 2 * u + half;
-            const int h = ho[u] < r ? ho[u] : r - 1;
-            float x8[8];
-            widen8_f16(*reinterpret_cast<const uint4 *>(ckh + h * D + 8 * c), x8);
-            float2 x2[4];
-#pragma unroll
-            for (int cc = 0; cc < 4; cc++) x2[cc] = make_float2(x8[2 * cc], x8[2 * cc + 1]);
-            s4[2 * u] = block8(x2, gk2);
-            s4[2 * u + 1] = block8(x2, gq2);
-          }
-          tree16x4(s4);
-#pragma unroll
-          for (int u = 0; u < 2; u++)
-            if (c == 0 && ho[u] < r) { pk[ho[u]] = s4[2 * u]; pq[ho[u]] = s4[2 * u + 1]; }
-        }
-      };
       // The record terms sum_j u_j (kt_j^T Gamma k) and the same for q, channels 4 lane .. 4 lane + 3, as one chain from the
       // newest record back.
       float2 rk_rec[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}}, rq_rec[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
-      int base = seg_base(n);                        // the segment at hand begins with record `base`
+      int n_left = n, base = seg_base(n);            // the segment at hand begins with record `base`, its newest is n_left - 1
+      float g1 = alpha_s;
       const rec_t *seg = rec + buf * SEG * RF;       // and lies here
-      // 2 NP records jt, jt-1, ...: half 0 projects the first, third, ... of them, half 1 the others.  The sums over the sixteen
-      // lanes are taken by halving exchanges (eight values: 4 + 2 + 1 + 1 shuffles), after which a lane holds one of them;
-      // through pj every lane gets all.  Groups of four may run past record 0.
-      auto walk_group = [&](const int jt, auto np) {
-        constexpr int NP = decltype(np)::value;
-        float v[2 * NP];
-#pragma unroll
-        for (int u = 0; u < NP; u++) {
-          // the decays of the two records of this pair; the half that owns the older one steps over the newer
-          const int jn = jt - 2 * u, jold = jn - 1;  // newer, older
-          float2 an[4], ao[4], gmine[4];
-          if (DIAG) {
-            load8p(seg + ((NP > 2 || jn > 0 ? jn : 0) - base) * RF + REC_A + 8 * c, an);
-            load8p(seg + ((NP > 2 || jold > 0 ? jold : 0) - base) * RF + REC_A + 8 * c, ao);
-          } else {
-            const float2 x = pair(bas[NP > 2 || jn > 0 ? jn : 0]), z = pair(bas[NP > 2 || jold > 0 ? jold : 0]);
-#pragma unroll
-            for (int cc = 0; cc < 4; cc++) { an[cc] = x; ao[cc] = z; }
-          }
-#pragma unroll
-          for (int cc = 0; cc < 4; cc++) {
-            const float2 gn = g2[cc], go = __fmul2_rn(gn, an[cc]);   // Gamma_{jn+1:l}, Gamma_{jold+1:l}
-            gmine[cc] = half ? go : gn;
-            // past both records; the chain stops at record 0, so that it ends as Gamma_{1:l} exactly
-            // (selects: a branch for the last trip of a long head was slower)
-            g2[cc] = (NP > 2 || !DIAG || jold >= 0) ? __fmul2_rn(go, ao[cc]) : (jn >= 0 ? go : gn);
-          }
-          const int jm = jn - half, j = NP > 2 || jm >= 0 ? jm : 0;  // (record 0 is in the slot whenever an index runs below it)
-          float2 x2[4], yk2[4], yq2[4];
-          load8p(seg + (j - base) * RF + REC_KT + 8 * c, x2);
-#pragma unroll
-          for (int cc = 0; cc < 4; cc++) { yk2[cc] = __fmul2_rn(gmine[cc], k2[cc]); yq2[cc] = __fmul2_rn(gmine[cc], q2[cc]); }
-          v[2 * u] = block8(x2, yk2);
-          v[2 * u + 1] = block8(x2, yq2);
-        }
-        // halving exchanges over lane bits 0, 1, (2), then plain ones; lane c ends with value `mine` of its half
-        const bool u0 = lane & 1, u1 = lane & 2, u2 = lane & 4;
-        float x;
-        int mine;
-        if constexpr (NP == 4) {
-          float x4[4], x2_[2];
-#pragma unroll
-          for (int e = 0; e < 4; e++) x4[e] = (u0 ? v[e + 4] : v[e]) + __shfl_xor_sync(FULL, u0 ? v[e] : v[e + 4], 1);
-#pragma unroll
-          for (int e = 0; e < 2; e++) x2_[e] = (u1 ? x4[e + 2] : x4[e]) + __shfl_xor_sync(FULL, u1 ? x4[e] : x4[e + 2], 2);
-          x = (u2 ? x2_[1] : x2_[0]) + __shfl_xor_sync(FULL, u2 ? x2_[0] : x2_[1], 4);
-          mine = (u0 ? 4 : 0) + (u1 ? 2 : 0) + (u2 ? 1 : 0);
-        } else {
-          float x2_[2];
-#pragma unroll
-          for (int e = 0; e < 2; e++) x2_[e] = (u0 ? v[e + 2] : v[e]) + __shfl_xor_sync(FULL, u0 ? v[e] : v[e + 2], 1);
-          x = (u1 ? x2_[1] : x2_[0]) + __shfl_xor_sync(FULL, u1 ? x2_[0] : x2_[1], 2);
-          x = x + __shfl_xor_sync(FULL, x, 4);
-          mine = (u0 ? 2 : 0) + (u1 ? 1 : 0);
-        }
-        x = x + __shfl_xor_sync(FULL, x, 8);
-        __syncwarp();                                // (the group before has been read)
-        if (c < 2 * NP) pj[(mine & 1) * 8 + (mine & ~1) + half] = x;     // pj[vector][record]
+      for (;;) {
+        walk_records<GATE>(seg, base, bas, pj, n_left - 1, lane, k2, q2, g2, g1, rk_rec, rq_rec);
+        if (!LONGW || base == 0) break;
+        // the segment is walked: on to the one before it
         __syncwarp();
-        float pk_[2 * NP], pq_[2 * NP];
-#pragma unroll
-        for (int e = 0; e < NP / 2; e++) {
-          const float4 a = *reinterpret_cast<const float4 *>(pj + 4 * e), b = *reinterpret_cast<const float4 *>(pj + 8 + 4 * e);
-          pk_[4 * e] = a.x; pk_[4 * e + 1] = a.y; pk_[4 * e + 2] = a.z; pk_[4 * e + 3] = a.w;
-          pq_[4 * e] = b.x; pq_[4 * e + 1] = b.y; pq_[4 * e + 2] = b.z; pq_[4 * e + 3] = b.w;
-        }
-#pragma unroll
-        for (int e = 0; e < 2 * NP; e++) {
-          const int j = jt - e;
-          if (NP == 2 && j < 0) break;               // the same for every lane
-          const float4 u4 = load4(seg + (j - base) * RF + REC_U + 4 * lane);
-          const float2 lo = make_float2(u4.x, u4.y), hi = make_float2(u4.z, u4.w), pk2 = pair(pk_[e]), pq2 = pair(pq_[e]);
-          rk_rec[0] = __ffma2_rn(lo, pk2, rk_rec[0]); rq_rec[0] = __ffma2_rn(lo, pq2, rq_rec[0]);
-          rk_rec[1] = __ffma2_rn(hi, pk2, rk_rec[1]); rq_rec[1] = __ffma2_rn(hi, pq2, rq_rec[1]);
-        }
-      };
-      for (int jt = n - 1; jt >= 0;) {
-        if (LONGW && jt < base) {                    // the segment is walked: on to the one before it
-          __syncwarp();
-          if (DIAG) named_wait(4 + buf);             // (the stream warp has taken this segment's decays as well)
-          if (base > SEG) request_segment(bh, n, base - SEG, buf);      // (the one after that is on its way to the other half)
-          base = seg_base(base);
-          buf ^= 1;
-          seg = rec + buf * SEG * RF;
-          wait_records();
-        }
-        if (jt - 7 >= base) {
-          walk_group(jt, std::integral_constant<int, 4>{});
-          jt -= 8;
-        } else {
-          walk_group(jt, std::integral_constant<int, 2>{});
-          jt -= 4;
-        }
+        if (DIAG) named_wait(4 + buf);               // (the stream warp has taken this segment's decays as well)
+        if (base > SEG) request_segment(bh, n, base - SEG, buf);        // (the one after that is on its way to the other half)
+        n_left = base;
+        base = seg_base(base);
+        buf ^= 1;
+        seg = rec + buf * SEG * RF;
+        wait_records();
       }
+      if (!DIAG) gsc = g1;                           // (the walk has come past record 0)
       const int walked = 4 + buf;                    // the barrier of the last segment
       if (LONGW) buf ^= 1;                           // the next head's segments follow on in turn
       LQ_TICK(3);
@@ -627,12 +737,12 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
       wait_for(barA, parA);
       if (r > 0) {
         if (DIAG) {
-          project_compensators(g2);
+          project_compensators(ckh, r, g2, k2, q2, pk, pq, lane);
         } else {
           float2 gam[4];
 #pragma unroll
           for (int cc = 0; cc < 4; cc++) gam[cc] = pair(gsc);
-          project_compensators(gam);
+          project_compensators(ckh, r, gam, k2, q2, pk, pq, lane);
         }
       }
       __syncwarp();
@@ -717,87 +827,12 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
         rk[0] = yk.x + tk.x; rk[1] = yk.y + tk.y; rk[2] = yk.z + tk.z; rk[3] = yk.w + tk.w;
         rq[0] = yq.x + tq.x; rq[1] = yq.y + tq.y; rq[2] = yq.z + tq.z; rq[3] = yq.w + tq.w;
       } else {
-      // C Gamma k (lanes 0..15) and C Gamma q (lanes 16..31) on their fixed-point grids, as digit planes
-      float back_own;
-      {
-        float c8[8], x8[8];
-        load8(cs + 8 * c, c8);
-        float m = 0.0f;
-#pragma unroll
-        for (int e = 0; e < 8; e++) {
-          x8[e] = c8[e] * (gam[e] * (half ? q8[e] : k8[e]));
-          m = fmaxf(m, fabsf(x8[e]));
-        }
-#pragma unroll
-        for (int s = 1; s <= 8; s <<= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, s));
-        float scale;
-        fixed_point_scales(m, scale, back_own);
-        // X = d0 + 256 d1 + 65536 d2 + 2^24 d3 with digits in [-128, 127]: the digit is the low byte read as
-        // signed, and taking it off is (X + 128) >> 8.  The bytes of the four stages of an element are the
-        // four digits; prmt gathers the same digit of four elements into one word.
-        uint32_t st[8][4];
-#pragma unroll
-        for (int e = 0; e < 8; e++) {
-          int X = __float2int_rn(x8[e] * scale);
-#pragma unroll
-          for (int d = 0; d < 4; d++) { st[e][d] = static_cast<uint32_t>(X); X = (X + 128) >> 8; }
-        }
-#pragma unroll
-        for (int d = 0; d < 4; d++) {
-          const uint32_t lo = __byte_perm(__byte_perm(st[0][d], st[1][d], 0x0040), __byte_perm(st[2][d], st[3][d], 0x0040), 0x5410);
-          const uint32_t hi = __byte_perm(__byte_perm(st[4][d], st[5][d], 0x0040), __byte_perm(st[6][d], st[7][d], 0x0040), 0x5410);
-          *reinterpret_cast<uint2 *>(digits + (4 * half + d) * D + 8 * c) = make_uint2(lo, hi);
-        }
-      }
-      const float back_other = __shfl_xor_sync(FULL, back_own, 16);
-      const float back_k = half ? back_other : back_own, back_q = half ? back_own : back_other;
+      float back_k, back_q;
+      digit_planes(cs, gam, k8, q8, digits, lane, back_k, back_q);
       __syncwarp();                          // the digit planes are visible to the warp
       LQ_TICK(4);
 
-      // The state stream on the tensor cores: eight 16-row tiles of Z^T, K = 128 as four k-blocks.  A
-      // thread's 16 bytes of a row hold key channels 64p+16t..64p+16t+15 and serve two k-blocks; the digit
-      // planes are read with the same permutation of the key index.  The two 64-channel halves of a tile
-      // accumulate separately (exact integers: any split gives the same sum), which halves the dependent
-      // chain of MMAs.  Digit pairs are recombined in int32 (|sum| < 2^30), the two pairs in int64 (the total has
-      // 47 bits), and one rounding takes it to fp32.
-      {
-        constexpr int h0 = 0, h1 = 64;         // the two 64-channel halves (the same split for every lane)
-        const uint4 bfa = *reinterpret_cast<const uint4 *>(digits + g * D + h0 + 16 * t);
-        const uint4 bfb = *reinterpret_cast<const uint4 *>(digits + g * D + h1 + 16 * t);
-        int pair_lo[8], pair_hi[8];            // digit-pair sums of rows g and g+8 of each tile
-#pragma unroll
-        for (int mt = 0; mt < 8; mt++) {
-          int ca[4] = {0, 0, 0, 0}, cb[4] = {0, 0, 0, 0};
-          const int j = 16 * mt + g;
-          const uint4 alo = *reinterpret_cast<const uint4 *>(zt + j * D + h0 + 16 * t);
-          const uint4 ahi = *reinterpret_cast<const uint4 *>(zt + (j + 8) * D + h0 + 16 * t);
-          const uint4 blo = *reinterpret_cast<const uint4 *>(zt + j * D + h1 + 16 * t);
-          const uint4 bhi = *reinterpret_cast<const uint4 *>(zt + (j + 8) * D + h1 + 16 * t);
-          mma_s8(ca, alo.x, ahi.x, alo.y, ahi.y, bfa.x, bfa.y);
-          mma_s8(cb, blo.x, bhi.x, blo.y, bhi.y, bfb.x, bfb.y);
-          mma_s8(ca, alo.z, ahi.z, alo.w, ahi.w, bfa.z, bfa.w);
-          mma_s8(cb, blo.z, bhi.z, blo.w, bhi.w, bfb.z, bfb.w);
-          // c[0], c[1]: row g, planes 2t, 2t+1;  c[2], c[3]: row g+8.  Planes 4v..4v+3 are the digits of
-          // vector v: lanes t = 0, 1 carry the k sums and t = 2, 3 the q sums, even t the low digit pair.
-          pair_lo[mt] = (ca[0] + cb[0]) + ((ca[1] + cb[1]) << 8);
-          pair_hi[mt] = (ca[2] + cb[2]) + ((ca[3] + cb[3]) << 8);
-        }
-        LQ_TICK(10);
-        int oth_lo[8], oth_hi[8];
-#pragma unroll
-        for (int mt = 0; mt < 8; mt++) {
-          oth_lo[mt] = __shfl_xor_sync(FULL, pair_lo[mt], 1);
-          oth_hi[mt] = __shfl_xor_sync(FULL, pair_hi[mt], 1);
-        }
-        if (!(t & 1)) {                      // this lane has the low pairs, its neighbour sent the high pairs
-          float *dst = y + (t >> 1) * D + g;
-#pragma unroll
-          for (int mt = 0; mt < 8; mt++) {
-            dst[16 * mt] = __ll2float_rn(static_cast<long long>(oth_lo[mt]) * 65536 + pair_lo[mt]);
-            dst[16 * mt + 8] = __ll2float_rn(static_cast<long long>(oth_hi[mt]) * 65536 + pair_hi[mt]);
-          }
-        }
-      }
+      code_sums(zt, digits, y, lane);
       __syncwarp();
       LQ_TICK(5);
 
