@@ -356,13 +356,25 @@ static lq_status launch_decode(const lq_shape *s, const Params &p, cudaStream_t 
 template <int GATE, int MODE, bool R16, int RM, bool BF16>
 static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStream_t stream, long due) {
   const bool diag = GATE == LQ_GATE_DIAG, iterate = RM > 0 && s->n_iter > 1;
-  auto bytes = [&](int slots) { return BoundarySmem<RM>(MODE, s->W, s->r, diag, R16, BF16, iterate, slots).bytes; };
+  // Four warps to a state (8 x 16 tiles: a third fewer loads and copies of row values to an FMA) where CTAs have many states in turn and
+  // the registers suffice: quantizing with up to four vectors, 2048 states, r = 4 55.3 -> 53.0 us, r = 3 51.5 -> 49.0, r = 4 with two
+  // rounds 88.6 -> 84.6.  Eight vectors take 98 us with eight warps and 111 with four.  Flushes with four vectors: 256 x 32 heads, W = 8
+  // 74.7 / 72.9 us a step, W = 16 60.8 / 60.5, but one flush by itself is longer with four (32 x 32 heads: 18.1 / 19.1), and so is the
+  // search among many sequences: four where all CTAs have one to do and two trips cover the batch.
+  constexpr int NW = MODE == 1 && RM <= 4 ? 4 : 8;
+  const bool four = NW == 4 || (MODE == 0 && RM == 4 && s->r == RM && due >= 2L * sm_count() && s->batch <= 2048);
+  const int threads = four ? 128 : 256;
+  auto bytes = [&](int slots) {
+    return four ? BoundarySmem<RM, 4>(MODE, s->W, s->r, diag, R16, BF16, iterate, slots).bytes
+                : BoundarySmem<RM, 8>(MODE, s->W, s->r, diag, R16, BF16, iterate, slots).bytes;
+  };
   // A second slot where a head is through in a few microseconds and two CTAs with two slots each still fit on an SM; a head
   // that is requantized leaves its slot early enough for the next one (two slots: 65.3 us against 64.1 at 256 x 32 heads).
   const int slots = (MODE == 2 || (BF16 && MODE == 0)) && bytes(2) <= (228 / 2 - 2) * 1024 ? 2 : 1;
   constexpr bool may_be_exact = (MODE == 0 && (RM == 4 || RM == 8)) || (MODE == 1 && RM == 4);
-  auto kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, false>;
-  if (may_be_exact && s->r == RM) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, may_be_exact>;
+  auto kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, false, false, NW>;
+  if (may_be_exact && s->r == RM) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, may_be_exact, false, NW>;
+  if (MODE == 0 && RM == 4 && four) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, may_be_exact, false, MODE == 0 && RM == 4 ? 4 : NW>;
   const long nh = (long)s->batch * s->heads_v;
   // With more than eight compensators two heads on one SM take half as long again as one, and CTAs that leave room for a second
   // one are not placed one to an SM (the first 148 of 296 come to lie on 142 SMs): where windows of every fill would have no
@@ -371,9 +383,9 @@ static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStrea
   // 35.6 / 37.1, r = 12 38.5 / 42.1, r = 16 43.7 / 50.2; all windows due at once (every 16th step), r = 16, on average 37.4 / 31.5.
   const bool alone = RM > 8 && MODE == 0 && due <= sm_count() && nh > 2L * sm_count();
   const int smem = alone ? std::max(bytes(slots), 116 * 1024) : bytes(slots);
-  const long resident = (long)prepare_launch(reinterpret_cast<const void *>(kernel), 256, smem) * sm_count();
+  const long resident = (long)prepare_launch(reinterpret_cast<const void *>(kernel), threads, smem) * sm_count();
   if (resident < 1) return LQ_ERR_CUDA;
-  return launch_dependent(kernel, static_cast<int>(nh < resident ? nh : resident), 256, smem, stream, p, slots);
+  return launch_dependent(kernel, static_cast<int>(nh < resident ? nh : resident), threads, smem, stream, p, slots);
 }
 
 // A whole step of few heads in one launch, a CTA per head: as long as every SM has one head at most (a CTA takes most of an
@@ -389,11 +401,12 @@ static bool one_launch(const lq_shape *s) {
 template <int GATE, bool R16, int RM, bool BF16>
 static lq_status launch_step_t(const lq_shape *s, const Params &p, cudaStream_t stream) {
   const bool diag = GATE == LQ_GATE_DIAG;
-  const int smem = std::max(BoundarySmem<RM>(0, s->W, s->r, diag, R16, BF16, RM > 0 && s->n_iter > 1, 1).bytes,
+  constexpr int NW = 8;
+  const int smem = std::max(BoundarySmem<RM, NW>(0, s->W, s->r, diag, R16, BF16, RM > 0 && s->n_iter > 1, 1).bytes,
                             TOKEN_SLOT + DecodeSlot(s->W, s->r, diag, R16, BF16, 0).bytes);
-  auto kernel = boundary_kernel<GATE, 0, R16, RM, BF16, false, true>;
-  if (s->r == RM && (RM == 4 || RM == 8)) kernel = boundary_kernel<GATE, 0, R16, RM, BF16, RM == 4 || RM == 8, true>;
-  return launch_dependent(kernel, s->batch * s->heads_v, 256, smem, stream, p, 1);
+  auto kernel = boundary_kernel<GATE, 0, R16, RM, BF16, false, true, NW>;
+  if (s->r == RM && (RM == 4 || RM == 8)) kernel = boundary_kernel<GATE, 0, R16, RM, BF16, RM == 4 || RM == 8, true, NW>;
+  return launch_dependent(kernel, s->batch * s->heads_v, 32 * NW, smem, stream, p, 1);
 }
 template <int RM, bool BF16>
 static lq_status launch_step_gate(const lq_shape *s, const Params &p, cudaStream_t stream) {

@@ -102,6 +102,9 @@ __device__ __forceinline__ void mbar_inval(uint32_t bar) { asm volatile("mbarrie
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.relaxed.cta.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
 // global -> shared bulk copy; addresses and size are multiples of 16 bytes
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
@@ -360,7 +363,9 @@ __device__ __forceinline__ int nth_set_bit(uint32_t m, unsigned k) {
 // this warp looks at, the same for the warp of this number in every CTA (-1: none).  `counts`: shared memory.  Ends without a
 // barrier.
 __device__ __forceinline__ bool window_due(const Params &p, int v) { return v == p.W || (p.force && v > 0); }
-__device__ __forceinline__ int due_scan_warps(const Params &p) { return p.batch <= 256 ? 1 : 8; }
+template <int NW>
+__device__ __forceinline__ int due_scan_warps(const Params &p) { return p.batch <= 256 ? 1 : NW; }
+template <int NW>
 __device__ __forceinline__ int list_due_heads(const Params &p, unsigned first, unsigned stride, int warps, unsigned (*counts)[8],
                                               unsigned *todo_bh, int *todo_n, int &lead) {
   constexpr int U = 8;                       // loads in flight per lane
@@ -390,7 +395,7 @@ __device__ __forceinline__ int list_due_heads(const Params &p, unsigned first, u
       if (lane == 0) counts[turn][warp] = c;
       __syncthreads();                       // (in turn: the counts of the trip before may still be read)
 #pragma unroll
-      for (int w = 0; w < 8; w++) {
+      for (int w = 0; w < NW; w++) {
         const unsigned x = counts[turn][w];
         if (w < warp) at += x;
         base += x;
