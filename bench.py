@@ -457,7 +457,7 @@ def run_cuda(args, wl):
     heads = wl.batch * wl.heads_v
     ms_per_step = ms / args.steps
     hs = world * heads * args.steps / (ms / 1e3)
-    launches = lq.decode_launches(sh)
+    launches = lq.step_launches(sh, st)
     peak, peak_src = peaks()
     group = wl.heads_v // wl.heads_qk
     bytes_hs = algorithmic_bytes_per_head_step(wl.W, wl.r, wl.gate == synth.GATE_DIAG, group, wl.rec16)

@@ -115,7 +115,7 @@ typedef struct {
  * win_pos: int32 [B], records buffered per sequence, 0..W-1 between calls.  Bits 16 and up are used as a
  *     scratch counter while a call runs and are zero again when it has finished.
  * work: optional (may be null): int32 [LQ_WORK_WORDS], all zero when the state is created and zero again after
- *     every call.  With it, the decode kernel of lq_decode_step hands out the heads of its last, partial round
+ *     every call.  With it, lq_decode_step takes tokens and window boundaries of many shapes in one launch instead of two, and the decode kernel of lq_decode_step hands out the heads of its last, partial round
  *     (B*Hv heads over the CTAs that are resident at once) to the CTAs that get there first, instead of giving
  *     every CTA the same number of heads: on a GPU whose memory system does not serve all SMs alike, equal shares
  *     do not take equal time.  Results are the same bit for bit either way.  Sub-batches of one state that are
@@ -322,8 +322,10 @@ lq_status lq_selftest_bounded_wait(lq_stream stream);
 /* LQ_STATIC_STAGE_BYTES as the loaded library was built with (for bindings that cannot read the macro). */
 uint64_t lq_static_stage_bytes(void);
 
-/* Kernels one lq_decode_step call launches for `shape` (used to report launch counts). */
+/* Kernels one lq_decode_step call launches for `shape` on a state without scratch words, which is the most it launches; and for
+ * `state` as it is, which may be one where that is two (used to report launch counts; both 0 for an invalid shape). */
 int lq_decode_launches(const lq_shape *shape);
+int lq_step_launches(const lq_shape *shape, const lq_state *state);
 
 const char *lq_status_string(lq_status status);
 int lq_version(void);

@@ -10,6 +10,7 @@
 
 #include "lq_boundary.cuh"
 #include "lq_decode.cuh"
+#include "lq_step.cuh"
 
 namespace lq {
 
@@ -422,6 +423,36 @@ static lq_status launch_step(const lq_shape *s, const Params &p, cudaStream_t st
   return launch_step_gate<MAX_R, false>(s, p, stream);
 }
 
+// A step of many heads in one launch (step_kernel); false where it does not apply.  launch = false: says only whether it does.
+// It does with up to one due head to an SM, on average over windows of every fill: such a head is through its boundary while the
+// others get their tokens, and the second launch, the wait for the first kernel's last CTA and the search for due heads are saved.  r = 4, us per
+// step as two launches / one, scalar gate: 32 x 32 heads, W = 16 18.0 / 16.5, W = 8 19.6 / 15.1; 64 x 32, W = 16 25.8 / 22.3; 128 x 32,
+// W = 32 46.5 / 33.5; 2000 x 1, W = 16 26.6 / 22.9; diagonal gate: 64 x 32, W = 16 27.7 / 24.3; 128 x 32, W = 32 54.8 / 43.1.  With more
+// than one the heads of an SM go through their boundaries one after the other, which takes as long as two at a time in a kernel of
+// their own behind the tokens: 128 x 32, W = 16 34.9 / 34.7; 256 x 32 60.8 / 63; diagonal gate 38.4 / 39.6 and 67.9 / 73.  With the scalar
+// gate and long windows the tokens leave time for all of them (W = 24, 512 x 32: 128 / 122; W = 32, 1024 x 32: 243 / 236; W = 20: 117 / 118).
+// Three slots to an SM where four do not fit (W = 40, 128 x 32: 48.8 / 42.8); two are too few (W = 64, 256 x 32: 101 / 119).  fp16
+// records: no gain (diagonal gate, 64 x 32, r = 3: 26.3 / 26.5), so there are no instances for them.
+template <int GATE, int RM, bool EXACT>
+static bool launch_merged_t(const lq_shape *s, const Params &p, cudaStream_t stream, lq_status *rc, bool launch) {
+  auto bytes = [&](int pairs) { return StepSmem<RM>(pairs, s->batch, s->W, s->r, GATE == LQ_GATE_DIAG, RM > 0 && s->n_iter > 1).bytes; };
+  int pairs = STEP_PAIRS;                    // (226 of 227 KB: there are static arrays)
+  while (pairs > 0 && bytes(pairs) > 226 * 1024) pairs--;
+  if (pairs < STEP_PAIRS - 1) return false;
+  const long nh = (long)s->batch * s->heads_v, sms = sm_count();
+  if (nh > sms * s->W && !(GATE == LQ_GATE_SCALAR && s->W >= 24 && pairs == STEP_PAIRS)) return false;
+  if (launch) *rc = launch_dependent(step_kernel<GATE, RM, EXACT>, static_cast<int>(std::min(nh, sms)), STEP_THREADS, bytes(pairs), stream, p, pairs);
+  return true;
+}
+static bool launch_merged(const lq_shape *s, const Params &p, cudaStream_t stream, lq_status *rc, bool launch) {
+  if (!p.work || s->batch == 0 || s->batch > STEP_MAX_BATCH || s->r > STEP_MAX_R || s->state_bf16 || s->rec16) return false;
+  const bool diag = s->gate == LQ_GATE_DIAG;
+  if (s->r == 0) return diag ? launch_merged_t<LQ_GATE_DIAG, 0, false>(s, p, stream, rc, launch) : launch_merged_t<LQ_GATE_SCALAR, 0, false>(s, p, stream, rc, launch);
+  if (s->r == 4) return diag ? launch_merged_t<LQ_GATE_DIAG, 4, true>(s, p, stream, rc, launch) : launch_merged_t<LQ_GATE_SCALAR, 4, true>(s, p, stream, rc, launch);
+  if (s->r < 4) return diag ? launch_merged_t<LQ_GATE_DIAG, 4, false>(s, p, stream, rc, launch) : launch_merged_t<LQ_GATE_SCALAR, 4, false>(s, p, stream, rc, launch);
+  return diag ? launch_merged_t<LQ_GATE_DIAG, 8, false>(s, p, stream, rc, launch) : launch_merged_t<LQ_GATE_SCALAR, 8, false>(s, p, stream, rc, launch);
+}
+
 template <int MODE, int RM, bool BF16>
 static lq_status launch_boundary_gate(const lq_shape *s, const Params &p, cudaStream_t stream, long due) {
   if (MODE == 1) return launch_boundary_t<LQ_GATE_SCALAR, MODE, false, RM, BF16>(s, p, stream, due);   // (reads no records)
@@ -469,6 +500,7 @@ static lq_status decode_step_impl(const lq_shape *shape, const lq_state *state, 
   p.overlap = nh >= 2L * sm_count() * shape->W;        // as many boundaries as boundary CTAs, on average
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (!between && part < 0 && one_launch(shape)) return launch_step(shape, p, st);
+  if (!between && part < 0 && launch_merged(shape, p, st, &rc, true)) return rc;
   if (part > 0 && p.work) p.work += part;
   rc = shape->state_bf16 ? launch_decode<true>(shape, p, st) : launch_decode<false>(shape, p, st);
   if (rc != LQ_OK) return rc;
@@ -1007,6 +1039,12 @@ int lq_debug_phase_cycles(unsigned long long *out) {
   return cudaMemcpyToSymbol(g_phase_cycles, zero, sizeof(zero)) != cudaSuccess;
 }
 #endif
+
+int lq_step_launches(const lq_shape *shape, const lq_state *state) {
+  const int most = lq_decode_launches(shape);
+  lq_status rc = LQ_OK;
+  return most > 1 && state && launch_merged(shape, make_params(shape, state), nullptr, &rc, false) ? 1 : most;
+}
 
 int lq_decode_launches(const lq_shape *shape) { return check_shape(shape) == LQ_OK && shape->batch > 0 ? one_launch(shape) ? 1 : 2 : 0; }
 

@@ -317,13 +317,16 @@ __device__ __forceinline__ void digit_planes(const float *cs, const float (&gam)
 // accumulate separately (exact integers: any split gives the same sum), which halves the dependent
 // chain of MMAs.  Digit pairs are recombined in int32 (|sum| < 2^30), the two pairs in int64 (the total has
 // 47 bits), and one rounding takes it to fp32.
+// GROUPS: the tiles are taken in so many groups (registers); y may lie where the digits are.
+template <int GROUPS>
 __device__ __forceinline__ void code_sums(const int8_t *zt, const int8_t *digits, float *y, int lane) {
   const int g = lane >> 2, t = lane & 3;
   constexpr int h0 = 0, h1 = 64;         // the two 64-channel halves (the same split for every lane)
   const uint4 bfa = *reinterpret_cast<const uint4 *>(digits + g * D + h0 + 16 * t);
   const uint4 bfb = *reinterpret_cast<const uint4 *>(digits + g * D + h1 + 16 * t);
-  constexpr int TILES = 8, mg = 0;
-  {
+  constexpr int TILES = 8 / GROUPS;
+#pragma unroll 1
+  for (int mg = 0; mg < 8; mg += TILES) {
     int pair_lo[TILES], pair_hi[TILES];  // digit-pair sums of rows g and g+8 of each tile
 #pragma unroll
     for (int mt = 0; mt < TILES; mt++) {
@@ -377,6 +380,7 @@ struct TokenRaw {
   uint4 k, q, a;        // a: diagonal-gate alpha
   uint2 v;
   float ba_lo, ba_hi;   // scalar gate: decays of buffered records `lane` and `lane + 32` (stale beyond n)
+  uint16_t beta, alpha; // (SCALARS: the head's scalars come with its vectors)
 };
 
 // A head index with its sequence and value-head parts, stepped without divisions.
@@ -388,7 +392,7 @@ struct HeadIdx {
   }
 };
 
-template <int GATE>
+template <int GATE, bool SCALARS = false>
 __device__ __forceinline__ void load_token(const Params &p, const HeadIdx h, int group, int lane, int role, TokenRaw &tk) {
   const int c = lane & 15;
   const size_t bh = h.bh;
@@ -396,6 +400,8 @@ __device__ __forceinline__ void load_token(const Params &p, const HeadIdx h, int
   tk.k = *reinterpret_cast<const uint4 *>(p.k + qk_off + 8 * c);
   tk.q = *reinterpret_cast<const uint4 *>(p.q + qk_off + 8 * c);
   if (role == 0) tk.v = *reinterpret_cast<const uint2 *>(p.v + bh * D + 4 * lane);
+  if (SCALARS && role == 1) tk.beta = p.beta[bh];
+  if (SCALARS && GATE == LQ_GATE_SCALAR) tk.alpha = p.alpha[bh];
   if (GATE == LQ_GATE_DIAG) {
     tk.a = *reinterpret_cast<const uint4 *>(p.alpha + bh * D + 8 * c);
   } else {
@@ -832,7 +838,7 @@ __device__ __forceinline__ void decode_slot(const Params &p, unsigned char *slot
       __syncwarp();                          // the digit planes are visible to the warp
       LQ_TICK(4);
 
-      code_sums(zt, digits, y, lane);
+      code_sums<1>(zt, digits, y, lane);
       __syncwarp();
       LQ_TICK(5);
 

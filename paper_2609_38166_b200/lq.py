@@ -22,7 +22,7 @@ _lib = None
 EXPORTS = ["lq_decode_step", "lq_decode_step_profiled", "lq_decode_step_host", "lq_decode_step_host_pipelined", "lq_decode_step_host_static", "lq_decode_stage_bytes", "lq_head_bytes", "lq_record_floats",
            "lq_window_flush",
            "lq_quantize_state", "lq_dequantize_state", "lq_ref_decode_step_f32", "lq_ref_decode_step_bf16",
-           "lq_decode_launches", "lq_check_device", "lq_clear_device_flags", "lq_selftest_bounded_wait",
+           "lq_decode_launches", "lq_step_launches", "lq_check_device", "lq_clear_device_flags", "lq_selftest_bounded_wait",
            "lq_static_stage_bytes", "lq_import_state", "lq_export_state", "lq_status_string", "lq_version"]
 
 
@@ -56,6 +56,8 @@ def lib() -> C.CDLL:
             getattr(L, name).argtypes = [C.c_void_p]
         L.lq_decode_launches.restype = C.c_int
         L.lq_decode_launches.argtypes = [C.c_void_p]
+        L.lq_step_launches.restype = C.c_int
+        L.lq_step_launches.argtypes = [C.c_void_p, C.c_void_p]
         L.lq_static_stage_bytes.restype = C.c_uint64
         L.lq_static_stage_bytes.argtypes = []
         L.lq_clear_device_flags.restype = C.c_int
@@ -252,6 +254,10 @@ def decode_stage_bytes(sh: Shape) -> int:
 
 def decode_launches(sh: Shape) -> int:
     return int(lib().lq_decode_launches(sh.ref()))
+
+
+def step_launches(sh: Shape, st: State) -> int:
+    return int(lib().lq_step_launches(sh.ref(), C.byref(st.c())))
 
 
 def decode_step_host(sh: Shape, st: State, q_h, k_h, v_h, beta_h, alpha_h, o_h, stage, stream=None):
