@@ -363,30 +363,36 @@ static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStrea
   // 74.7 / 72.9 us a step, W = 16 60.8 / 60.5, but one flush by itself is longer with four (32 x 32 heads: 18.1 / 19.1), and so is the
   // search among many sequences: four where all CTAs have one to do and two trips cover the batch.
   constexpr int NW = MODE == 1 && RM <= 4 ? 4 : 8;
-  const bool four = NW == 4 || (MODE == 0 && RM == 4 && s->r == RM && due >= 2L * sm_count() && s->batch <= 2048);
+  // Dequantizing 8-bit states, more than are resident at once: four warps, and the state is put together in shared memory and leaves by
+  // bulk stores, where two CTAs still fit on an SM so (2048 states, W = 16, r = 4: diagonal gate 46.0 -> 43.8 us, scalar gate 47.1 -> 43.9;
+  // with eight warps 46.7 and 47.6; 256 states 7.35 / 7.54; the BF16 state 40.4 either way).
+  const long nh = (long)s->batch * s->heads_v;
+  const bool staged_out = MODE == 2 && RM == 4 && nh > 2L * sm_count() &&
+                          BoundarySmem<0, 4, false>(MODE, s->W, s->r, diag, R16, BF16, false, 1, true).bytes <= (228 / 2 - 1) * 1024 - 512;
+  const bool four = NW == 4 || staged_out || (MODE == 0 && RM == 4 && s->r == RM && due >= 2L * sm_count() && s->batch <= 2048);
   const int threads = four ? 128 : 256;
-  auto bytes = [&](int slots) {
-    return four ? BoundarySmem<RM, 4>(MODE, s->W, s->r, diag, R16, BF16, iterate, slots).bytes
-                : BoundarySmem<RM, 8>(MODE, s->W, s->r, diag, R16, BF16, iterate, slots).bytes;
+  constexpr int RL = MODE == 2 ? 0 : RM;
+  auto bytes = [&](int slots, bool staged_out = false) {
+    return four ? BoundarySmem<RL, 4, MODE != 2>(MODE, s->W, s->r, diag, R16, BF16, iterate && MODE != 2, slots, staged_out).bytes
+                : BoundarySmem<RL, 8, MODE != 2>(MODE, s->W, s->r, diag, R16, BF16, iterate && MODE != 2, slots, staged_out).bytes;
   };
   // A second slot where a head is through in a few microseconds and two CTAs with two slots each still fit on an SM; a head
   // that is requantized leaves its slot early enough for the next one (two slots: 65.3 us against 64.1 at 256 x 32 heads).
-  const int slots = (MODE == 2 || (BF16 && MODE == 0)) && bytes(2) <= (228 / 2 - 2) * 1024 ? 2 : 1;
+  const int slots = (MODE == 2 || (BF16 && MODE == 0)) && !staged_out && bytes(2) <= (228 / 2 - 2) * 1024 ? 2 : 1;
   constexpr bool may_be_exact = (MODE == 0 && (RM == 4 || RM == 8)) || (MODE == 1 && RM == 4);
   auto kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, false, false, NW>;
   if (may_be_exact && s->r == RM) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, may_be_exact, false, NW>;
-  if (MODE == 0 && RM == 4 && four) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, may_be_exact, false, MODE == 0 && RM == 4 ? 4 : NW>;
-  const long nh = (long)s->batch * s->heads_v;
+  if (MODE != 1 && RM == 4 && four) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, may_be_exact, false, MODE != 1 && RM == 4 ? 4 : NW>;
   // With more than eight compensators two heads on one SM take half as long again as one, and CTAs that leave room for a second
   // one are not placed one to an SM (the first 148 of 296 come to lie on 142 SMs): where windows of every fill would have no
   // more heads due at a time than there are SMs, though all heads at once are more than two to an SM, a CTA asks for more than
   // half of its SM's memory.  64 x 32 heads, W = 16, us per step with one CTA / two to an SM: windows of every fill, r = 9
   // 35.6 / 37.1, r = 12 38.5 / 42.1, r = 16 43.7 / 50.2; all windows due at once (every 16th step), r = 16, on average 37.4 / 31.5.
   const bool alone = RM > 8 && MODE == 0 && due <= sm_count() && nh > 2L * sm_count();
-  const int smem = alone ? std::max(bytes(slots), 116 * 1024) : bytes(slots);
+  const int smem = alone ? std::max(bytes(slots), 116 * 1024) : bytes(slots, staged_out);
   const long resident = (long)prepare_launch(reinterpret_cast<const void *>(kernel), threads, smem) * sm_count();
   if (resident < 1) return LQ_ERR_CUDA;
-  return launch_dependent(kernel, static_cast<int>(nh < resident ? nh : resident), threads, smem, stream, p, slots);
+  return launch_dependent(kernel, static_cast<int>(nh < resident ? nh : resident), threads, smem, stream, p, slots, staged_out ? 1 : 0);
 }
 
 // A whole step of few heads in one launch, a CTA per head: as long as every SM has one head at most (a CTA takes most of an
@@ -407,7 +413,7 @@ static lq_status launch_step_t(const lq_shape *s, const Params &p, cudaStream_t 
                             TOKEN_SLOT + DecodeSlot(s->W, s->r, diag, R16, BF16, 0).bytes);
   auto kernel = boundary_kernel<GATE, 0, R16, RM, BF16, false, true, NW>;
   if (s->r == RM && (RM == 4 || RM == 8)) kernel = boundary_kernel<GATE, 0, R16, RM, BF16, RM == 4 || RM == 8, true, NW>;
-  return launch_dependent(kernel, s->batch * s->heads_v, 32 * NW, smem, stream, p, 1);
+  return launch_dependent(kernel, s->batch * s->heads_v, 32 * NW, smem, stream, p, 1, 0);
 }
 template <int RM, bool BF16>
 static lq_status launch_step_gate(const lq_shape *s, const Params &p, cudaStream_t stream) {

@@ -15,7 +15,7 @@
 // head, now 8), and copies by all threads into two staging buffers: 2048 dense states quantized in 55.2 us (91.4 before),
 // 2048 states dequantized in 45.6 us (54.0); a step of 256 x 32 heads, 512 of them due, 73 -> 61 us.
 //
-// With NW = 4 (quantizing) four warps hold the state, 32 columns each and 16 to a lane.
+// With NW = 4 four warps hold the state, 32 columns each and 16 to a lane (launch_boundary_t says where).
 #pragma once
 #include <type_traits>
 
@@ -33,7 +33,8 @@ constexpr int TOKEN_SLOT = 128;              // a step in one launch: where the 
 constexpr int DENSE_GROUP = 8 * D * 4 + 128;
 template <int NW>
 __host__ __device__ constexpr int dense_group_at(int g) { return g * DENSE_GROUP + ((g & 1) ? 16 : 0) + ((g & 2) ? (NW == 4 ? 32 : 64) : 0); }
-template <int RM, int NW>
+// FIT = false: only what it takes to rebuild a state.
+template <int RM, int NW, bool FIT = true>
 struct BoundarySmem {
   static constexpr int bar = 0;                              // [2] copy barriers
   static constexpr int invc = 16;                            // [128]      1 / code step, per warp
@@ -47,15 +48,16 @@ struct BoundarySmem {
   // two (2048 heads, W = 16, r = 16 flushed in 325 us, 239 with eight at a time).
   static constexpr int PV = RM > 8 ? 8 : RM > 0 ? RM : 1;
   static constexpr int part = T + 4 * D * RM;                // [NW][PV][128] per-warp row sums; later [NW][128] those of |R|
-  static constexpr int head = part + 4 * D * NW * PV;         // the slots
-  int rec, slot, dec, kd, Wv, bytes;
-  __host__ __device__ BoundarySmem(int mode, int W, int r, bool diag, bool rec16, bool bf16, bool iterate, int slots) {
+  static constexpr int head = FIT ? part + 4 * D * NW * PV : gram;       // the slots
+  int rec, slot, dec, kd, Wv, out, bytes;
+  __host__ __device__ BoundarySmem(int mode, int W, int r, bool diag, bool rec16, bool bf16, bool iterate, int slots, bool staged_out = false) {
     rec = bf16 ? BF16W_HEAD_BYTES : head_bytes(r);           // within a slot: [W] record rows behind the head block
     slot = mode == 1 ? (RM <= 8 ? 16 * DENSE_GROUP : 0) : rec + (rec16 ? 2 : 4) * record_floats(diag) * W;
     dec = head + slots * slot;                               // [W] scalar gate: the records' decays
     kd = dec + (mode != 1 && !diag ? (4 * W + 15) / 16 * 16 : 0);   // [W][128] fp16 records: Gamma_{j+1:n} kt_j (fp32: in place)
     Wv = kd + (mode != 1 && rec16 ? 4 * D * W : 0);          // [r][128] several rounds: S^T q_h
-    bytes = Wv + (iterate ? 4 * D * r : 0);
+    out = (Wv + (iterate ? 4 * D * r : 0) + 127) / 128 * 128; // (dequantizing) a dense state on its way out
+    bytes = out + (staged_out ? 16 * DENSE_GROUP : 0);
   }
 };
 
@@ -371,6 +373,7 @@ struct BoundaryArrays {
   float *T, *Wv, *gram, *chol;               // see BoundarySmem
   float *ub, *ic, *invc;                     // ub, invc: this warp's
   unsigned char *rows = nullptr, *newest = nullptr;           // (GROUP) the record rows but the last one, and that
+  unsigned char *out = nullptr;              // (dequantizing) where the state is put together for bulk stores, or null
 };
 
 // One head through its boundary (MODE, RM, BF16, EXACT: see boundary_kernel): `slot` holds its head block and, behind it, its n
@@ -493,9 +496,13 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
     for (int a = 0; a < 8; a++) load_row(S + a * D, wide, M[a]);
   }
   if constexpr (MODE == 2) {
-    float *S = p.S + bh * (size_t)(D * D) + 8 * ty * D + v0;
+    if (A.out) {
+      if (warp == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");      // (the state before has left)
+    } else {
+      float *S = p.S + bh * (size_t)(D * D) + 8 * ty * D + v0;
 #pragma unroll
-    for (int a = 0; a < 8; a++) store_row(S + a * D, wide, M[a]);
+      for (int a = 0; a < 8; a++) store_row(S + a * D, wide, M[a]);
+    }
   } else if constexpr (RM > 0) {
     // T_h = S w_h; w_h is the value side of the (h+1)-th newest record, or Walsh function h
     auto start_vector = [&](int h, float2 (&w)[NP]) {
@@ -538,6 +545,23 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
   if (STAGED && !SUMS_IN_SLOT) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
   boundary_sync<GROUP, NW>();
   if (!SUMS_IN_SLOT) slot_is_free();
+  if constexpr (MODE == 2) {
+    if (A.out) {
+      float *rows = reinterpret_cast<float *>(A.out + dense_group_at<NW>(ty)) + v0;
+#pragma unroll
+      for (int a = 0; a < 8; a++) {
+#pragma unroll
+        for (int b = 0; b < NP / 2; b++)
+          *reinterpret_cast<float4 *>(rows + a * D + 4 * b) = make_float4(M[a][2 * b].x, M[a][2 * b].y, M[a][2 * b + 1].x, M[a][2 * b + 1].y);
+      }
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      boundary_sync<GROUP, NW>();
+      if (warp == 0) {
+        if (lane < 16) bulk_s2g(p.S + bh * (size_t)(D * D) + lane * 8 * D, smem_addr(A.out) + dense_group_at<NW>(lane), 8 * D * 4);
+        asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+      }
+    }
+  }
 
   if constexpr (BF16 && MODE != 2) {                      // round and store: that is the new boundary state
     uint16_t *S0T = reinterpret_cast<uint16_t *>(p.heads + bh * (size_t)BF16W_HEAD_BYTES) + v0 * D + 8 * ty;
@@ -723,7 +747,7 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
 // own: told apart inside the others, the two ways cost those 400 bytes of spills; in the one for r = 0 the compiler still spills
 // 280 bytes: 256 x 32 heads, W = 16, r = 0, 53.0 us a step, 71.7 with the former layout, which spilled none).
 // BF16: the per-window BF16 state (lq_shape.state_bf16, RM = 0): the dense state is rounded to bfloat16, and that is all.
-// slots: 1 or 2.
+// slots: 1 or 2.  staged_out (dequantizing): a state leaves by bulk stores from shared memory.
 // EXACT: r is RM, known at compile time: without a test per vector the compiler interleaves the four or eight column sums
 // (flush at 256 x 32 heads: step 62.2 -> 61.4 us, W = 8 75.6 -> 74.4; quantizing 2048 states, r = 4: 57.5 -> 55.2 us, where only
 // the products with the start vectors must not know r: the vectors, the same for every head, would be kept in registers and
@@ -732,12 +756,12 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
 // token (decode_slot), then, if that filled the window, the CTA through the boundary.  What bounds it: the latency of a token and
 // of a boundary, and the host time of a launch, of which it needs one instead of two (figures: one_launch).
 template <int GATE, int MODE, bool R16, int RM, bool BF16, bool EXACT, bool STEP, int NW>
-__global__ void __launch_bounds__(32 * NW, STEP ? 1 : 2) boundary_kernel(const Params p, const int slots) {
+__global__ void __launch_bounds__(32 * NW, STEP ? 1 : 2) boundary_kernel(const Params p, const int slots, const int staged_out) {
   constexpr bool DIAG = GATE == LQ_GATE_DIAG, RECORDS = MODE != 1, STAGED = MODE != 1 || RM <= 8;
   static_assert(!BF16 || RM == 0, "the per-window BF16 state has no compensators");
   constexpr int RF = record_floats(DIAG);
   using rec_t = typename std::conditional<R16, __half, float>::type;
-  using Lay = BoundarySmem<RM, NW>;
+  using Lay = BoundarySmem<MODE == 2 ? 0 : RM, NW, MODE != 2>;
   constexpr int PV = Lay::PV;                // vectors whose row sums `part` holds at a time
   extern __shared__ __align__(128) unsigned char lq_bsm[];
   __shared__ unsigned todo_bh[32], due_counts[2][8];
@@ -745,11 +769,12 @@ __global__ void __launch_bounds__(32 * NW, STEP ? 1 : 2) boundary_kernel(const P
   const int W = p.W, rT = MODE == 1 ? p.r : EXACT ? RM : p.r, r = EXACT ? RM : RM > 0 ? p.r : 0, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (RM > 0 && r < 1) return;               // (not launched)
   const unsigned nh = static_cast<unsigned>(p.batch) * p.heads_v;
-  const Lay L(MODE, W, r, DIAG, R16, BF16, RM > 0 && p.n_iter > 1, slots);
+  const Lay L(MODE, W, r, DIAG, R16, BF16, MODE != 2 && RM > 0 && p.n_iter > 1, slots);
   float *dec = reinterpret_cast<float *>(lq_bsm + L.dec);
   auto at_bytes = [&](int offset) { return reinterpret_cast<float *>(lq_bsm + offset); };
-  const BoundaryArrays A{dec, at_bytes(Lay::gam), at_bytes(L.kd), at_bytes(Lay::part), at_bytes(Lay::part), at_bytes(Lay::T), at_bytes(L.Wv),
+  BoundaryArrays A{dec, at_bytes(Lay::gam), at_bytes(L.kd), at_bytes(Lay::part), at_bytes(Lay::part), at_bytes(Lay::T), at_bytes(L.Wv),
                          at_bytes(Lay::gram), at_bytes(Lay::chol), at_bytes(Lay::ub) + warp * (D / NW) * RM, at_bytes(Lay::ic), at_bytes(Lay::invc) + D / NW * warp};
+  if (MODE == 2 && RM > 0 && NW == 4 && staged_out) A.out = lq_bsm + L.out;
   const uint32_t bar = smem_addr(lq_bsm + Lay::bar);
   const bool wide = (reinterpret_cast<uintptr_t>(p.S) & 31) == 0;
   LQ_STAMP(1, 0);
@@ -871,6 +896,7 @@ __global__ void __launch_bounds__(32 * NW, STEP ? 1 : 2) boundary_kernel(const P
     }
     __syncthreads();                         // the list is rewritten by the next round
   }
+  if (MODE == 2 && RM > 0 && NW == 4 && staged_out && warp == 0) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
   LQ_STAMP(1, 4);
 #ifdef LQ_TIMING
   if (tid == 0)

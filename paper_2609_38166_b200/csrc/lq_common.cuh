@@ -118,6 +118,10 @@ __device__ __forceinline__ void bulk_g2s_hint(uint32_t dst, const void *src, uin
       "l"(src), "r"(bytes), "r"(bar), "l"(policy)
       : "memory");
 }
+// shared -> global bulk copy of the issuing thread's bulk group; addresses and size are multiples of 16 bytes
+__device__ __forceinline__ void bulk_s2g(void *dst, uint32_t src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
+}
 // Ask the L2 for a piece of global memory (no data comes back, nothing waits for it).
 __device__ __forceinline__ void bulk_prefetch_l2(const void *src, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(src), "r"(bytes) : "memory");
