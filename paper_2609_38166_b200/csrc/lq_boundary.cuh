@@ -376,16 +376,20 @@ struct BoundaryArrays {
   unsigned char *out = nullptr;              // (dequantizing) where the state is put together for bulk stores, or null
 };
 
-// One head through its boundary (MODE, RM, BF16, EXACT: see boundary_kernel): `slot` holds its head block and, behind it, its n
+// One head through its boundary (MODE, RM, BF16, EXACT, ROUNDS: see boundary_kernel): `slot` holds its head block and, behind it, its n
 // records, or a dense state.  GROUP: the eight warps are the first of a larger CTA, and the row sums lie in the slot, where the codes
 // were (PV = 4 vectors at a time: each warp's sums take the place of the 2 KB of codes that only this warp reads).
 // slot_is_free() is called by every thread, behind a barrier after which nobody reads the slot.
-template <int GATE, int MODE, bool R16, int RM, bool BF16, bool EXACT, bool GROUP, int PV, int NW, typename F>
+template <int GATE, int MODE, bool R16, int RM, bool BF16, bool EXACT, bool ROUNDS, bool GROUP, int PV, int NW, typename F>
 __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArrays &A, unsigned char *slot, const size_t bh, const int n,
                                               const int r, const int rT, const bool wide, F slot_is_free) {
-  // (exactly four vectors: registers are left for deeper unrolling, step 61.3 -> 60.8 us and 74.2 -> 73.0 at W = 8; for exactly
-  // eight it is slower, 234.3 -> 236.5 us at 512 x 32 heads, diagonal gate, W = 64)
-  constexpr bool FOUR = EXACT && RM == 4 && MODE == 0;
+  // Exactly four vectors: registers are left for deeper unrolling, step 61.3 -> 60.8 us and 74.2 -> 73.0 at W = 8; for exactly
+  // eight it is slower, 234.3 -> 236.5 us at 512 x 32 heads, diagonal gate, W = 64.  Not with four warps, whose code is twice as long to
+  // begin with: behind other kernels it comes from the L2 or beyond, and that is where it runs in a model.  256 x 32 heads, scalar gate,
+  // us per step, in a loop of steps / with a projection, norms and a softmax in front of each: records 4, start vectors 4 at a time and
+  // the loops over the rounds in between 59.1 / 69.7, W = 8 72.1 / 83.9; one at a time and no such loops (ROUNDS) 59.3 / 64.4 and
+  // 71.8 / 76.9; eight warps 59.6 / 64.0 and 73.5 / 78.3.
+  constexpr bool FOUR = EXACT && RM == 4 && MODE == 0, DEEP = FOUR && NW == 8;
   constexpr bool DIAG = GATE == LQ_GATE_DIAG, RECORDS = MODE != 1, STAGED = MODE != 1 || RM <= 8;
   constexpr int RF = record_floats(DIAG);
   using rec_t = typename std::conditional<R16, __half, float>::type;
@@ -476,7 +480,7 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
 #pragma unroll
         for (int c = 0; c < NP; c++) M[a][c] = __fmul2_rn(pair(gi[a]), M[a][c]);
     }
-    constexpr int AHEAD = MODE == 2 ? 1 : FOUR ? 4 : 2;              // (dequantizing spills with two records at a time)
+    constexpr int AHEAD = MODE == 2 ? 1 : DEEP ? 4 : FOUR ? 1 : 2;   // (dequantizing spills with two records at a time)
 #pragma unroll AHEAD
     for (int j = 0; j < n; j++) {
       float kj[8];
@@ -532,7 +536,7 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
         row_sums(w, h % PV);
       }
     } else {
-#pragma unroll (FOUR ? 4 : NW == 4 && EXACT ? 1 : 2)
+#pragma unroll (DEEP ? 4 : NW == 4 && EXACT ? 1 : 2)
       for (int h = 0; h < rT; h++) {
         float2 w[NP];
         start_vector(h, w);
@@ -584,7 +588,7 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
       for (int idx = T0 + tid; idx < r * D; idx += NT) T[idx] = sum_warps<NW>(part + idx - T0, PV * D);
       LQ_BTICK(10);
       // further rounds: W_h = S^T q_h, orthonormalise, T_h = S q_h
-      for (int it = 1; it < p.n_iter; it++) {
+      for (int it = 1; ROUNDS && it < p.n_iter; it++) {
         orthonormalize<false, RM, GROUP, NW>(T, r, gram, chol, nullptr, [] {});
 #pragma unroll 1
         for (int h = 0; h < r; h++) {
@@ -752,10 +756,11 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
 // (flush at 256 x 32 heads: step 62.2 -> 61.4 us, W = 8 75.6 -> 74.4; quantizing 2048 states, r = 4: 57.5 -> 55.2 us, where only
 // the products with the start vectors must not know r: the vectors, the same for every head, would be kept in registers and
 // others spilled, 69.9 us; with eight vectors it spills all the same).
+// ROUNDS: p.n_iter may be more than one.  Without, the loops over the further rounds, a third of the code on the way, are not there.
 // STEP (a flush): a whole decode step of few heads in one launch.  Every CTA has one head: two of its warps take it through the
 // token (decode_slot), then, if that filled the window, the CTA through the boundary.  What bounds it: the latency of a token and
 // of a boundary, and the host time of a launch, of which it needs one instead of two (figures: one_launch).
-template <int GATE, int MODE, bool R16, int RM, bool BF16, bool EXACT, bool STEP, int NW>
+template <int GATE, int MODE, bool R16, int RM, bool BF16, bool EXACT, bool ROUNDS, bool STEP, int NW>
 __global__ void __launch_bounds__(32 * NW, STEP ? 1 : 2) boundary_kernel(const Params p, const int slots, const int staged_out) {
   constexpr bool DIAG = GATE == LQ_GATE_DIAG, RECORDS = MODE != 1, STAGED = MODE != 1 || RM <= 8;
   static_assert(!BF16 || RM == 0, "the per-window BF16 state has no compensators");
@@ -885,7 +890,7 @@ __global__ void __launch_bounds__(32 * NW, STEP ? 1 : 2) boundary_kernel(const P
         if (k == 0) LQ_STAMP(1, 2);
         LQ_BTICK(1);
       }
-      boundary_head<GATE, MODE, R16, RM, BF16, EXACT, false, PV, NW>(p, A, slot, bh, n, r, rT, wide, [&] {
+      boundary_head<GATE, MODE, R16, RM, BF16, EXACT, ROUNDS, false, PV, NW>(p, A, slot, bh, n, r, rT, wide, [&] {
         if (STAGED && slots == 1 && k + 1 < count) request(todo_bh[k + 1], todo_n[k + 1], at);
         if (!STAGED && k + 1 < count && tid < 8)              // (dense states: at least into the L2)
           bulk_prefetch_l2(p.S + todo_bh[k + 1] * (size_t)(D * D) + tid * (D * D / 8), D * D / 2);

@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const Params p, c
     A.part = reinterpret_cast<float *>(slot + StepSlot::head);
     A.newest = slot + SL.digits;
     A.rows = slot + SL.rec;
-    boundary_head<GATE, 0, false, RM, false, EXACT, true, 4, NW>(p, A, slot + StepSlot::head, hdr[0], W, r, r, false, [&] {
+    boundary_head<GATE, 0, false, RM, false, EXACT, true, true, 4, NW>(p, A, slot + StepSlot::head, hdr[0], W, r, r, false, [&] {
       const unsigned next = tid == 224 ? hdr[1] : NO_ITEM;
       if (next != NO_ITEM) {                 // the slot's next head
         step_request_head(p, SL, smem_addr(slot), next);
