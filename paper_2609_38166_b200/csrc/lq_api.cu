@@ -359,19 +359,24 @@ static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStrea
   const bool diag = GATE == LQ_GATE_DIAG, iterate = RM > 0 && s->n_iter > 1;
   // Four warps to a state (8 x 16 tiles: a third fewer loads and copies of row values to an FMA) where CTAs have many states in turn and
   // the registers suffice: quantizing with up to four vectors, 2048 states, r = 4 55.3 -> 53.0 us, r = 3 51.5 -> 49.0, r = 4 with two
-  // rounds 88.6 -> 84.6.  Eight vectors take 98 us with eight warps and 111 with four.  Flushes with four vectors, one round, the scalar
+  // rounds 88.6 -> 84.6.  Not with a state to an SM at most, or one in the last of two rounds: with eight / four warps 64 states 6.5 / 6.8 us,
+  // 128 6.7 / 7.1, 160 9.3 / 8.7, 288 9.7 / 9.1, 320 13.8 / 13.8, 384 13.9 / 14.2, 448 16.7 / 15.7, 768 24.2 / 22.7 (r = 4; r = 2 and two rounds alike).
+  // Without vectors the memory is the limit for many states: r = 0 416 7.1 / 5.6, 1024 12.2 / 10.9, 1536 23.4 / 23.2, 2048 28.9 / 29.5, 4096 53.0 / 54.9;
+  // the BF16 state 416 6.9 / 5.5, 1024 13.2 / 12.7, 2048 32.0 / 32.7.
+  // Eight vectors take 98 us with eight warps and 111 with four.  Flushes with four vectors, one round, the scalar
   // gate and fp32 records: figures at boundary_head.  With two rounds 137.2 / 137.7 us a step (512 x 32, W = 24, eight / four warps); 256 x 32,
   // W = 16, in a loop and behind other kernels: diagonal gate 67.3, 69.9 / 67.4, 70.9, fp16 records 58.9, 61.1 / 58.7, 62.2.  One flush by itself is longer with four (32 x 32 heads: 18.1 / 19.1), and so is the
   // search among many sequences: four where all CTAs have one to do and two trips cover the batch.
-  constexpr int NW = MODE == 1 && RM <= 4 ? 4 : 8;
+  constexpr bool QUANTIZE4 = MODE == 1 && RM <= 4, DEQUANTIZE4 = MODE == 2 && RM == 4;
   constexpr bool FLUSH4 = MODE == 0 && RM == 4 && GATE == LQ_GATE_SCALAR && !R16;
   // Dequantizing 8-bit states, more than are resident at once: four warps, and the state is put together in shared memory and leaves by
   // bulk stores, where two CTAs still fit on an SM so (2048 states, W = 16, r = 4: diagonal gate 46.0 -> 43.8 us, scalar gate 47.1 -> 43.9;
   // with eight warps 46.7 and 47.6; 256 states 7.35 / 7.54; the BF16 state 40.4 either way).
-  const long nh = (long)s->batch * s->heads_v;
-  const bool staged_out = MODE == 2 && RM == 4 && nh > 2L * sm_count() &&
+  const long nh = (long)s->batch * s->heads_v, sms = sm_count();
+  const bool staged_out = DEQUANTIZE4 && nh > 2 * sms &&
                           BoundarySmem<0, 4, false>(MODE, s->W, s->r, diag, R16, BF16, false, 1, true).bytes <= (228 / 2 - 1) * 1024 - 512;
-  const bool four = NW == 4 || staged_out || (FLUSH4 && s->r == RM && !iterate && due >= 2L * sm_count() && s->batch <= 2048);
+  const bool four = staged_out || (QUANTIZE4 && nh > sms && (RM == 0 ? nh <= 10 * sms : nh <= 2 * sms || nh > 3 * sms)) ||
+                    (FLUSH4 && s->r == RM && !iterate && due >= 2 * sms && s->batch <= 2048);
   const int threads = four ? 128 : 256;
   constexpr int RL = MODE == 2 ? 0 : RM;
   auto bytes = [&](int slots, bool staged_out = false) {
@@ -382,19 +387,23 @@ static lq_status launch_boundary_t(const lq_shape *s, const Params &p, cudaStrea
   // that is requantized leaves its slot early enough for the next one (two slots: 65.3 us against 64.1 at 256 x 32 heads).
   const int slots = (MODE == 2 || (BF16 && MODE == 0)) && !staged_out && bytes(2) <= (228 / 2 - 2) * 1024 ? 2 : 1;
   constexpr bool may_be_exact = (MODE == 0 && (RM == 4 || RM == 8)) || (MODE == 1 && RM == 4);
-  auto kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, false, true, false, NW>;
-  if (may_be_exact && s->r == RM) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, may_be_exact, true, false, NW>;
+  const bool exact = may_be_exact && s->r == RM;
   constexpr bool one_round = MODE == 0 && RM == 4;       // (instances for one round)
-  if (one_round && s->r == RM && !iterate) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, may_be_exact, !one_round, false, NW>;
-  if ((FLUSH4 || (MODE == 2 && RM == 4)) && four) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, FLUSH4, !FLUSH4, false, FLUSH4 || (MODE == 2 && RM == 4) ? 4 : NW>;
+  auto kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, false, true, false, 8>;
+  if (exact) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, may_be_exact, true, false, 8>;
+  if (one_round && exact && !iterate) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, may_be_exact, !one_round, false, 8>;
+  if constexpr (QUANTIZE4 || DEQUANTIZE4 || FLUSH4) {
+    if (four) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, FLUSH4, !FLUSH4, false, 4>;
+    if (four && exact) kernel = boundary_kernel<GATE, MODE, R16, RM, BF16, may_be_exact, !FLUSH4, false, 4>;
+  }
   // With more than eight compensators two heads on one SM take half as long again as one, and CTAs that leave room for a second
   // one are not placed one to an SM (the first 148 of 296 come to lie on 142 SMs): where windows of every fill would have no
   // more heads due at a time than there are SMs, though all heads at once are more than two to an SM, a CTA asks for more than
   // half of its SM's memory.  64 x 32 heads, W = 16, us per step with one CTA / two to an SM: windows of every fill, r = 9
   // 35.6 / 37.1, r = 12 38.5 / 42.1, r = 16 43.7 / 50.2; all windows due at once (every 16th step), r = 16, on average 37.4 / 31.5.
-  const bool alone = RM > 8 && MODE == 0 && due <= sm_count() && nh > 2L * sm_count();
+  const bool alone = RM > 8 && MODE == 0 && due <= sms && nh > 2 * sms;
   const int smem = alone ? std::max(bytes(slots), 116 * 1024) : bytes(slots, staged_out);
-  const long resident = (long)prepare_launch(reinterpret_cast<const void *>(kernel), threads, smem) * sm_count();
+  const long resident = prepare_launch(reinterpret_cast<const void *>(kernel), threads, smem) * sms;
   if (resident < 1) return LQ_ERR_CUDA;
   return launch_dependent(kernel, static_cast<int>(nh < resident ? nh : resident), threads, smem, stream, p, slots, staged_out ? 1 : 0);
 }

@@ -56,3 +56,23 @@ def test_many_due_heads_and_few_at_a_time_give_the_same_bits(gate, batch, heads,
             lq.window_flush(shape(c.stop - c.start), st, force=force)
         same(f"window_flush, force {force}")
     assert lq.check_device() == 0
+
+
+@pytest.mark.parametrize("r,bf16,n_iter", [(4, 0, 1), (4, 0, 2), (3, 0, 1), (0, 0, 1), (0, 1, 1)])
+def test_states_quantized_by_four_warps_and_by_eight_give_the_same_bits(r, bf16, n_iter):
+    """On both sides of the numbers of states where the other number of warps is taken: one, two, three and ten to an SM."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    shape = lambda n: lq.Shape(n, 1, 1, 128, 128, 8, r, n_iter, G, 0 if bf16 else 1, 1, 0, bf16)
+    most = 10 * sms + 1
+    S = torch.randn((most, 1, 128, 128), generator=torch.Generator("cuda").manual_seed(r), device="cuda")
+    want = torch.cat([_quantized(shape(min(100, most - b)), S[b:b + 100]) for b in range(0, most, 100)])
+    for n in (k * sms + e for k in (1, 2, 3, 10) for e in (0, 1)):
+        assert torch.equal(_quantized(shape(n), S[:n]), want[:n]), n
+    assert lq.check_device() == 0
+
+
+def _quantized(sh, S):
+    st = lq.State(sh)
+    lq.quantize_state(sh, S, st)
+    assert not st.win_pos.any()
+    return st.heads
