@@ -445,31 +445,48 @@ static lq_status launch_step(const lq_shape *s, const Params &p, cudaStream_t st
 // A step of many heads in one launch (step_kernel); false where it does not apply.  launch = false: says only whether it does.
 // It does with up to one due head to an SM, on average over windows of every fill: such a head is through its boundary while the
 // others get their tokens, and the second launch, the wait for the first kernel's last CTA and the search for due heads are saved.  r = 4, us per
-// step as two launches / one, scalar gate: 32 x 32 heads, W = 16 18.0 / 16.5, W = 8 19.6 / 15.1; 64 x 32, W = 16 25.8 / 22.3; 128 x 32,
-// W = 32 46.5 / 33.5; 2000 x 1, W = 16 26.6 / 22.9; diagonal gate: 64 x 32, W = 16 27.7 / 24.3; 128 x 32, W = 32 54.8 / 43.1.  With more
-// than one the heads of an SM go through their boundaries one after the other, which takes as long as two at a time in a kernel of
+// step as two launches / one, in a loop of steps and (in brackets) behind a projection, norms and a softmax, where code and state are fetched anew:
+//   scalar gate: 32 x 32 heads, W = 16 17.6 / 16.5 (18.8 / 19.1), W = 8 19.7 / 14.7 (20.9 / 17.1), W = 32 20.5 / 19.4 (20.9 / 23.1);
+//     48 x 32, W = 16 19.0 / 19.2 (20.7 / 21.5); 64 x 32, W = 16 25.8 / 22.4 (27.4 / 24.6); 128 x 32, W = 32 43.3 / 31.2 (44.5 / 33.9)
+//   diagonal gate: 32 x 32, W = 16 18.3 / 17.7 (19.3 / 21.1); 64 x 32, W = 16 27.6 / 24.5 (29.9 / 27.7); 128 x 32, W = 32 54.6 / 42.2 (56.7 / 44.7)
+// Not where every head has a CTA of the decode kernel to itself (six to an SM): 20 x 16 heads, W = 16 14.7 / 14.1 (14.9 / 18.7), diagonal gate
+// 14.2 / 14.7 (14.7 / 20.9); 24 x 32 15.7 / 15.9 (16.6 / 18.9).  A boundary of several rounds is more code and longer: from twice as many heads on.  32 x 32,
+// W = 16, r = 4, two rounds 20.9 / 20.1 (21.9 / 26.9); 48 x 32 22.2 / 22.8 (22.9 / 26.8); 64 x 32 29.8 / 26.2 (31.4 / 29.8), r = 8 41.2 / 33.8 (42.4 / 45.5);
+// 128 x 32, W = 32 47.7 / 34.8 (48.8 / 37.5).
+// With more than one due head to an SM they go through their boundaries one after the other, which takes as long as two at a time in a kernel of
 // their own behind the tokens: 128 x 32, W = 16 34.9 / 34.7; 256 x 32 60.8 / 63; diagonal gate 38.4 / 39.6 and 67.9 / 73.  With the scalar
-// gate and long windows the tokens leave time for all of them (W = 24, 512 x 32: 128 / 122; W = 32, 1024 x 32: 243 / 236; W = 20: 117 / 118).
+// gate and long windows the tokens leave time for all of them (W = 24, 512 x 32: 123.2 / 117.8 (125.4 / 119.2); W = 32, 1024 x 32: 247.7 / 232.0
+// (246.8 / 231.8); W = 20: 117 / 118).
+// The price of one boundary at a time is paid where all windows fall due in the same step, as those of sequences admitted together do: mean over the
+// window and the longest step, two launches / one: 32 x 32, W = 16 12.2 / 11.8, 66 / 75; 64 x 32 18.5 / 20.5, 105 / 133; 128 x 32, W = 32 34.8 / 35.2,
+// 255 / 311; 512 x 32, W = 24 118.7 / 124.7, 832 / 1039; 1024 x 32, W = 32 241 / 253, 1831 / 2339; 64 x 32, r = 8 21.9 / 25.4, 151 / 207.  Which it is the host does
+// not know.  And a CTA fills its SM, so two streams with a state each take turns: a step of both, two launches / one, 32 x 32, W = 16 23.2 / 24.1,
+// 64 x 32 33.3 / 40.0 (one state: 25.8 / 22.3), diagonal gate 37.4 / 43.5 (27.7 / 24.4), 128 x 32, W = 32 64.7 / 58.3.
 // Three slots to an SM where four do not fit (W = 40, 128 x 32: 48.8 / 42.8); two are too few (W = 64, 256 x 32: 101 / 119).  fp16
 // records: no gain (diagonal gate, 64 x 32, r = 3: 26.3 / 26.5), so there are no instances for them.
-template <int GATE, int RM, bool EXACT>
+template <int GATE, int RM, bool EXACT, bool ROUNDS>
 static bool launch_merged_t(const lq_shape *s, const Params &p, cudaStream_t stream, lq_status *rc, bool launch) {
   auto bytes = [&](int pairs) { return StepSmem<RM>(pairs, s->batch, s->W, s->r, GATE == LQ_GATE_DIAG, RM > 0 && s->n_iter > 1).bytes; };
   int pairs = STEP_PAIRS;                    // (226 of 227 KB: there are static arrays)
   while (pairs > 0 && bytes(pairs) > 226 * 1024) pairs--;
   if (pairs < STEP_PAIRS - 1) return false;
   const long nh = (long)s->batch * s->heads_v, sms = sm_count();
+  if (nh <= (ROUNDS ? 12 : 6) * sms) return false;
   if (nh > sms * s->W && !(GATE == LQ_GATE_SCALAR && s->W >= 24 && pairs == STEP_PAIRS)) return false;
-  if (launch) *rc = launch_dependent(step_kernel<GATE, RM, EXACT>, static_cast<int>(std::min(nh, sms)), STEP_THREADS, bytes(pairs), stream, p, pairs);
+  if (launch) *rc = launch_dependent(step_kernel<GATE, RM, EXACT, ROUNDS>, static_cast<int>(sms), STEP_THREADS, bytes(pairs), stream, p, pairs);
   return true;
 }
 static bool launch_merged(const lq_shape *s, const Params &p, cudaStream_t stream, lq_status *rc, bool launch) {
   if (!p.work || s->batch == 0 || s->batch > STEP_MAX_BATCH || s->r > STEP_MAX_R || s->state_bf16 || s->rec16) return false;
   const bool diag = s->gate == LQ_GATE_DIAG;
-  if (s->r == 0) return diag ? launch_merged_t<LQ_GATE_DIAG, 0, false>(s, p, stream, rc, launch) : launch_merged_t<LQ_GATE_SCALAR, 0, false>(s, p, stream, rc, launch);
-  if (s->r == 4) return diag ? launch_merged_t<LQ_GATE_DIAG, 4, true>(s, p, stream, rc, launch) : launch_merged_t<LQ_GATE_SCALAR, 4, true>(s, p, stream, rc, launch);
-  if (s->r < 4) return diag ? launch_merged_t<LQ_GATE_DIAG, 4, false>(s, p, stream, rc, launch) : launch_merged_t<LQ_GATE_SCALAR, 4, false>(s, p, stream, rc, launch);
-  return diag ? launch_merged_t<LQ_GATE_DIAG, 8, false>(s, p, stream, rc, launch) : launch_merged_t<LQ_GATE_SCALAR, 8, false>(s, p, stream, rc, launch);
+  auto by_gate = [&](auto rm, auto exact, auto rounds) {
+    return diag ? launch_merged_t<LQ_GATE_DIAG, rm, exact, rounds>(s, p, stream, rc, launch) : launch_merged_t<LQ_GATE_SCALAR, rm, exact, rounds>(s, p, stream, rc, launch);
+  };
+  constexpr std::integral_constant<int, 0> r0; constexpr std::integral_constant<int, 4> r4; constexpr std::integral_constant<int, 8> r8;
+  constexpr std::true_type yes; constexpr std::false_type no;
+  if (s->r == 0) return by_gate(r0, no, no);
+  if (s->n_iter > 1) return s->r <= 4 ? by_gate(r4, no, yes) : by_gate(r8, no, yes);
+  return s->r == 4 ? by_gate(r4, yes, no) : s->r < 4 ? by_gate(r4, no, no) : by_gate(r8, no, no);
 }
 
 template <int MODE, int RM, bool BF16>

@@ -389,7 +389,7 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
   // us per step, in a loop of steps / with a projection, norms and a softmax in front of each: records 4, start vectors 4 at a time and
   // the loops over the rounds in between 59.1 / 69.7, W = 8 72.1 / 83.9; one at a time and no such loops (ROUNDS) 59.3 / 64.4 and
   // 71.8 / 76.9; eight warps 59.6 / 64.0 and 73.5 / 78.3.
-  constexpr bool FOUR = EXACT && RM == 4 && MODE == 0, DEEP = FOUR && NW == 8;
+  constexpr bool FOUR = EXACT && RM == 4 && MODE == 0, DEEP = FOUR && NW == 8 && !GROUP;
   constexpr bool DIAG = GATE == LQ_GATE_DIAG, RECORDS = MODE != 1, STAGED = MODE != 1 || RM <= 8;
   constexpr int RF = record_floats(DIAG);
   using rec_t = typename std::conditional<R16, __half, float>::type;
@@ -464,7 +464,7 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
           M[a][c] = __fmul2_rn(pair(ci[a]), __fmul2_rn(__fadd2_rn(raw, pair(-8388736.0f)), sj[c]));
         }
     }
-#pragma unroll (FOUR ? 2 : 1)
+#pragma unroll (FOUR && !GROUP ? 2 : 1)
     for (int h = 0; h < r; h++) {
       float kc[8];
       float2 uc[NP];
@@ -480,7 +480,7 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
 #pragma unroll
         for (int c = 0; c < NP; c++) M[a][c] = __fmul2_rn(pair(gi[a]), M[a][c]);
     }
-    constexpr int AHEAD = MODE == 2 ? 1 : DEEP ? 4 : FOUR ? 1 : 2;   // (dequantizing spills with two records at a time)
+    constexpr int AHEAD = MODE == 2 ? 1 : DEEP ? 4 : FOUR || GROUP ? 1 : 2;   // (dequantizing spills with two records at a time)
 #pragma unroll AHEAD
     for (int j = 0; j < n; j++) {
       float kj[8];
@@ -536,7 +536,7 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
         row_sums(w, h % PV);
       }
     } else {
-#pragma unroll (DEEP ? 4 : NW == 4 && EXACT ? 1 : 2)
+#pragma unroll (DEEP ? 4 : GROUP || (NW == 4 && EXACT) ? 1 : 2)
       for (int h = 0; h < rT; h++) {
         float2 w[NP];
         start_vector(h, w);
@@ -625,21 +625,31 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
 
       // ---- value sides and removal of the stored tokens ----
       float x[RM];                                        // S^T k_h for the lane's column
-#pragma unroll
-      for (int h = 0; h < RM; h++) {
-        x[h] = 0.0f;
-        if (h < r) {
-          float kf[8], pc[NC];
-          load8(T + h * D + 8 * ty, kf);
-          column_blocks(M, kf, pc);
-          x[h] = column_tree(pc, lane, [](float a, float b) { return a + b; });
+      const int col = column_of<NC>(lane);
+      auto column_sum = [&](int h) {
+        float kf[8], pc[NC];
+        load8(T + h * D + 8 * ty, kf);
+        column_blocks(M, kf, pc);
+        return column_tree(pc, lane, [](float a, float b) { return a + b; });
+      };
+      if constexpr (GROUP) {                              // (one after the other through ub: one copy of the code, see step_kernel)
+#pragma unroll 1
+        for (int h = 0; h < r; h++) {
+          const float sum = column_sum(h);
+          if (NC == 16 || lane < 16) ub[CW * h + NC * tx + col] = sum;
         }
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < RM; h++) x[h] = h < r ? ub[CW * h + NC * tx + col] : 0.0f;
+        __syncwarp();
+      } else {
+#pragma unroll
+        for (int h = 0; h < RM; h++) x[h] = h < r ? column_sum(h) : 0.0f;
       }
       boundary_sync<GROUP, NW>();                                    // K^T K is complete
       LQ_BTICK(13);
       // u_h = S^T k_h - sum_{a<h} u_a (k_a^T k_h) with the stored values: what tokens 0..h-1 leave
       float uf[RM];
-      const int col = column_of<NC>(lane);
       uint16_t *cu_out = p.comp_u(bh) + v0 + col;
 #pragma unroll
       for (int h = 0; h < RM; h++) {
@@ -657,7 +667,7 @@ __device__ __forceinline__ void boundary_head(const Params &p, const BoundaryArr
       }
       __syncwarp();
       LQ_BTICK(14);
-#pragma unroll (FOUR || NW == 4 ? 2 : 1)
+#pragma unroll ((FOUR && !GROUP) || NW == 4 ? 2 : 1)
       for (int h = 0; h < r; h++) {                       // M -= k u^T with the stored values
         float kf[8];
         float2 uv[NP];

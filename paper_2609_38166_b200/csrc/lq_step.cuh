@@ -17,7 +17,11 @@
 // themselves: together they take about as long as one after the other.  Two things decide how well they go together.  Instructions:
 // an SM keeps some 32 KB of them, and a straight line beyond that is fetched at 6 cycles an instruction instead of 3.4, so loops
 // stay rolled where the unrolled ones gain little (256 x 32 heads 74 -> 62 us with the waits, the products of the codes and the
-// projections rolled).  Registers: a spilled value comes back from the L2, because the slots leave little of the L1; 128 of them
+// projections rolled).  And a launch brings only the first of a kernel's code along; behind other kernels what lies beyond comes from the L2
+// or the memory when it is reached: of a boundary (15.2 K cycles) the phases behind the products with the start vectors then took 14.6 K
+// cycles instead of 7.8.  So the boundary's loops over records, start vectors and columns are rolled as well, and one round has an instance
+// without the loops over further ones: 32 x 32 heads, W = 16, behind a projection, norms and a softmax 21.0 -> 19.1 us (two launches 18.8),
+// in a loop of steps 16.6 -> 16.4.  Registers: a spilled value comes back from the L2, because the slots leave little of the L1; 128 of them
 // (four pairs) spill nothing, 96 (six pairs) up to 180 bytes: diagonal gate, 64 x 32 heads, W = 16 24.7 / 29.2 us.
 #pragma once
 #include "lq_boundary.cuh"
@@ -431,7 +435,7 @@ struct StepSmem {
   }
 };
 
-template <int GATE, int RM, bool EXACT>
+template <int GATE, int RM, bool EXACT, bool ROUNDS>
 __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const Params p, const int pairs) {
   constexpr int NW = STEP_WARPS, NT = 32 * NW, U = STEP_MAX_BATCH / NT;
   constexpr bool DIAG = GATE == LQ_GATE_DIAG;
@@ -565,7 +569,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const Params p, c
     A.part = reinterpret_cast<float *>(slot + StepSlot::head);
     A.newest = slot + SL.digits;
     A.rows = slot + SL.rec;
-    boundary_head<GATE, 0, false, RM, false, EXACT, true, true, 4, NW>(p, A, slot + StepSlot::head, hdr[0], W, r, r, false, [&] {
+    boundary_head<GATE, 0, false, RM, false, EXACT, ROUNDS, true, 4, NW>(p, A, slot + StepSlot::head, hdr[0], W, r, r, false, [&] {
       const unsigned next = tid == 224 ? hdr[1] : NO_ITEM;
       if (next != NO_ITEM) {                 // the slot's next head
         step_request_head(p, SL, smem_addr(slot), next);

@@ -1,7 +1,7 @@
 """GPU: a step of more heads than SMs in one launch (tokens and boundaries side by side) against the same step in two.  A state
 without the scratch words takes two launches always, so each case steps two copies of a state, one with and one without the words, and
-every array has to end with the same bits.  The sizes are where the one launch can go wrong: one head more than there are SMs, several
-due heads for a CTA, all heads due, none, windows that come in full, parked sequences, three and four slots to an SM, the longest
+every array has to end with the same bits.  The sizes are where the one launch can go wrong: one head more than the decode kernel has
+CTAs (six to an SM; up to there both copies take two launches), several due heads for a CTA, all heads due, none, windows that come in full, parked sequences, three and four slots to an SM, the longest
 list of sequences, few sequences of many heads and the reverse, and the largest numbers of heads that are taken this way."""
 import pytest
 import torch
@@ -29,11 +29,19 @@ def _tokens(sh, gen):
     (G, 200, 1, 1, 2, 2, 1, 0), (K, 33, 9, 3, 3, 4, 1, 0),           # short windows
     (G, 20, 32, 16, 40, 4, 1, 0), (K, 40, 16, 16, 28, 5, 1, 0),      # three slots to an SM
     (G, 96, 64, 16, 32, 4, 1, 0), (G, 256, 32, 16, 24, 2, 1, 0),     # long windows, more due heads than SMs
-    (G, 2048, 1, 1, 14, 4, 1, 0), (K, 1025, 2, 2, 16, 4, 1, 0), (G, 3, 64, 1, 16, 4, 1, 0)])
+    (G, 2048, 1, 1, 14, 4, 1, 0), (K, 1025, 2, 2, 16, 4, 1, 0), (G, 3, 64, 1, 16, 4, 1, 0),
+    (G, 888, 1, 1, 16, 4, 1, 0), (G, 889, 1, 1, 16, 4, 1, 0), (K, 889, 1, 1, 9, 4, 1, 0),        # the last of two launches and the first of one (148 SMs)
+    (G, 64, 16, 4, 8, 4, 1, 0), (K, 100, 10, 5, 7, 3, 1, 0), (G, 14, 64, 1, 16, 2, 1, 0), (G, 90, 11, 11, 8, 1, 1, 1), (K, 64, 32, 32, 16, 8, 1, 0),
+    (G, 128, 7, 7, 8, 0, 1, 0), (K, 150, 7, 1, 8, 0, 1, 1), (G, 128, 32, 16, 32, 0, 1, 0),
+    (G, 222, 8, 8, 12, 4, 2, 0), (G, 170, 11, 11, 14, 1, 3, 1), (G, 128, 32, 16, 32, 4, 2, 0), (K, 64, 32, 32, 16, 8, 2, 0),       # several rounds: from twelve to an SM on
+    (G, 40, 32, 16, 40, 4, 1, 0), (K, 60, 16, 16, 28, 5, 1, 0), (K, 128, 32, 32, 32, 4, 1, 0),   # three slots, the last with drawn heads
+    (G, 120, 32, 16, 24, 8, 1, 0), (K, 80, 32, 32, 20, 2, 1, 0)])                                # drawn heads with r > 4; diagonal gate, four slots
 def test_one_launch_of_many_heads_and_two_give_the_same_bits(gate, batch, heads_v, heads_qk, W, r, n_iter, plain):
     sh = lq.Shape(batch, heads_v, heads_qk, 128, 128, W, r, n_iter, gate, 0 if plain else 1, 0 if plain else 1, 0, 0)
     gen = torch.Generator("cuda").manual_seed(batch * W + r)
     one, two = lq.State(sh), lq.State(sh, work=False)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert lq.step_launches(sh, one) == (1 if batch * heads_v > (12 if n_iter > 1 else 6) * sms else 2) and lq.step_launches(sh, two) == 2
     lq.quantize_state(sh, torch.randn((batch, heads_v, 128, 128), generator=gen, device="cuda"), one)
     one.records.copy_(0.2 * torch.randn(one.records.shape, generator=gen, device="cuda"))
     one.decays.copy_(torch.rand(one.decays.shape, generator=gen, device="cuda") * 0.8 + 0.2)
