@@ -458,8 +458,8 @@ static lq_status launch_step(const lq_shape *s, const Params &p, cudaStream_t st
 // gate and long windows the tokens leave time for all of them (W = 24, 512 x 32: 123.2 / 117.8 (125.4 / 119.2); W = 32, 1024 x 32: 247.7 / 232.0
 // (246.8 / 231.8); W = 20: 117 / 118).
 // The price of one boundary at a time is paid where all windows fall due in the same step, as those of sequences admitted together do: mean over the
-// window and the longest step, two launches / one: 32 x 32, W = 16 12.2 / 11.8, 66 / 75; 64 x 32 18.5 / 20.5, 105 / 133; 128 x 32, W = 32 34.8 / 35.2,
-// 255 / 311; 512 x 32, W = 24 118.7 / 124.7, 832 / 1039; 1024 x 32, W = 32 241 / 253, 1831 / 2339; 64 x 32, r = 8 21.9 / 25.4, 151 / 207.  Which it is the host does
+// window and the longest step, two launches / one: 32 x 32, W = 16 12.3 / 11.6, 65 / 72; 64 x 32 18.6 / 20.4, 105 / 131; 128 x 32, W = 32 35.0 / 35.2,
+// 256 / 305; 512 x 32, W = 24 119.9 / 124.8, 834 / 1037; 1024 x 32, W = 32 247 / 254, 1911 / 2378; 64 x 32, r = 0 16.1 / 16.5, r = 8 21.8 / 25.2.  Which it is the host does
 // not know.  And a CTA fills its SM, so two streams with a state each take turns: a step of both, two launches / one, 32 x 32, W = 16 23.2 / 24.1,
 // 64 x 32 33.3 / 40.0 (one state: 25.8 / 22.3), diagonal gate 37.4 / 43.5 (27.7 / 24.4), 128 x 32, W = 32 64.7 / 58.3.
 // Three slots to an SM where four do not fit (W = 40, 128 x 32: 48.8 / 42.8); two are too few (W = 64, 256 x 32: 101 / 119).  fp16

@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const Params p, c
     }
     // Items: a pair takes those of sequences without a boundary in turn, the last two rounds by tickets (word 0 of the scratch words
     // counts them), as in the decode kernel; a CTA's due heads go to whichever of its pairs looks for one.  The first pair's first
-    // head is a due one.
+    // head is a due one, and so are those of pairs that find nothing in turn (all windows due: every slot has one to hand over).
     if (warp == 0 && lane < pairs) {
       const unsigned items = normal * Hv, due = (all >> 16) * Hv, G = gridDim.x * pairs, mine = gridDim.x - 1 - blockIdx.x;
       const unsigned rounds = items / G, in_turn = rounds >= 4 ? (rounds - 2) * G : items;
@@ -504,11 +504,13 @@ __global__ void __launch_bounds__(STEP_THREADS, 1) step_kernel(const Params p, c
       unsigned turn = lane * gridDim.x + blockIdx.x, taken = 0;
 #pragma unroll
       for (int e = 0; e < 2; e++) {
+        const bool wants_due = (e == 0 && lane == 0) || turn >= in_turn;
+        const unsigned want = __ballot_sync((1u << pairs) - 1u, wants_due), idx = taken + __popc(want & below);
         unsigned it = NO_ITEM;
-        if (e == 0 && lane == 0 && taken < m) it = items + mine + taken++ * gridDim.x;
+        if (wants_due && idx < m) it = items + mine + idx * gridDim.x;
         else if (turn < in_turn) { it = turn; turn += G; }
-        else if (lane == 0 && taken < m) it = items + mine + taken++ * gridDim.x;
         sh.first[lane][e] = it;
+        taken = min(m, taken + __popc(want));
       }
       reinterpret_cast<unsigned *>(lq_stp + L.slots + lane * L.slot_bytes + StepSlot::words)[3] = turn;
       if (lane == 0) {
