@@ -114,7 +114,6 @@ def test_full_windows_between_heads_with_a_token(oracle, gate, state_bf16):
     kw = dict(r=0, smooth=0, state_bf16=1) if state_bf16 else dict(r=16)
     wl = synth.Workload("between", 60, 48, 16, W=3, gate=gate, seed=845, **kw)
     osh, lsh = gu.shapes(wl)
-    assert lq.decode_launches(lsh) == 2
     ost = OState(osh)
     oracle.quantize_state(osh, synth.dense_states(wl, 3), ost)
     rng = np.random.default_rng(5)
@@ -126,6 +125,7 @@ def test_full_windows_between_heads_with_a_token(oracle, gate, state_bf16):
         full = np.arange(wl.batch) % 2 == pattern if pattern < 2 else rng.random(wl.batch) < 0.4
         ost.win_pos[:] = np.where(full, wl.W, rng.integers(0, wl.W, wl.batch))
         st = gu.state_to_dev(ost, lsh, work=False)
+        assert lq.step_launches(lsh, st) == 2
         o = torch.full((wl.batch, wl.heads_v, 128), 7.0, dtype=torch.float32, device="cuda")
         tok = synth.token_inputs(wl, pattern)
         td = gu.tok_dev(tok)
@@ -148,12 +148,12 @@ def test_parked_sequences_hold_up_nobody(oracle, batch, launches):
     among them) get no token, keep their position and their rows of the output, and the windows of the others go on."""
     wl = synth.Workload("parked", batch, 4, 2, W=3, r=2, seed=850 + batch)
     osh, lsh = gu.shapes(wl)
-    assert lq.decode_launches(lsh) == launches
     ost = OState(osh)
     oracle.quantize_state(osh, synth.dense_states(wl, 3), ost)
     marks = {0: 2 ** 31 - 1, 3: -1, 5: 65535, batch - 1: wl.W + 1}
     parked = np.isin(np.arange(batch), list(marks))
     st = gu.state_to_dev(ost, lsh)
+    assert lq.step_launches(lsh, st) == launches
     for b, mark in marks.items():
         st.win_pos[b] = mark
     some = wl.with_(batch=int((~parked).sum()))

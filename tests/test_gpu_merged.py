@@ -3,10 +3,13 @@ without the scratch words takes two launches always, so each case steps two copi
 every array has to end with the same bits.  The sizes are where the one launch can go wrong: one head more than the decode kernel has
 CTAs (six to an SM; up to there both copies take two launches), several due heads for a CTA, all heads due, none, windows that come in full, parked sequences, three and four slots to an SM, the longest
 list of sequences, few sequences of many heads and the reverse, and the largest numbers of heads that are taken this way."""
+import numpy as np
 import pytest
 import torch
 
+from oracle.lq_oracle import State as OState
 from paper_2609_38166_b200 import lq, synth
+from tests import gpu_util as gu
 
 pytestmark = pytest.mark.gpu
 
@@ -66,3 +69,33 @@ def test_one_launch_of_many_heads_and_two_give_the_same_bits(gate, batch, heads_
             assert torch.equal(getattr(one, name), getattr(two, name)), f"{name}, pattern {i}"
         assert not one.work.any(), f"scratch words, pattern {i}"
     assert lq.check_device() == 0
+
+
+@pytest.mark.parametrize("gate,batch,heads", [(G, 128, 8), (K, 112, 9)])
+def test_one_launch_of_many_heads_against_the_oracle_and_in_a_graph(oracle, gate, batch, heads):
+    """A window and a half of steps, windows of every fill: called one by one against the oracle, and captured once and replayed."""
+    wl = synth.Workload("merged", batch, heads, heads, W=8, r=4, gate=gate, seed=1300 + gate)
+    osh, sh = gu.shapes(wl)
+    ost = OState(osh)
+    oracle.quantize_state(osh, synth.dense_states(wl, 2), ost)
+    ost.win_pos[:] = np.random.default_rng(4).permutation(batch) % wl.W
+    ost.buf_a[...] = 1.0
+    states = [gu.state_to_dev(ost, sh) for _ in range(2)]
+    assert lq.step_launches(sh, states[0]) == 1
+    toks = [synth.token_inputs(wl, t) for t in range(12)]
+    tds = [[gu.tok_dev(t)[x] for x in ("q", "k", "v", "beta", "alpha")] for t in toks]
+    outs = [torch.zeros((12, batch, heads, 128), dtype=torch.float32, device="cuda") for _ in range(2)]
+    for t, tok in enumerate(toks):
+        lq.decode_step(sh, states[0], *tds[t], outs[0][t])
+        assert np.array_equal(gu.host(outs[0][t]), oracle.decode_step(osh, ost, **tok)), t
+    gu.assert_state_parity(states[0], ost, wl.r, "after the steps")
+    g, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=stream):
+        for t in range(12):
+            lq.decode_step(sh, states[1], *tds[t], outs[1][t], stream)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(outs[0], outs[1])
+    for a, b in zip(states[0].tensors(), states[1].tensors()):
+        assert torch.equal(a, b)
+    assert not states[1].work.any() and lq.check_device() == 0

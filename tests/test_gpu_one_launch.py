@@ -26,11 +26,11 @@ def test_one_launch_and_two_give_the_same_bits(gate, W, r, rec16, bf16, n_iter, 
     few = torch.cuda.get_device_properties(0).multi_processor_count // HEADS        # the most sequences of one launch
     B = 2 * few
     whole, part = _shape(B, W, r, gate, rec16, bf16, n_iter, plain), _shape(few, W, r, gate, rec16, bf16, n_iter, plain)
-    assert lq.decode_launches(whole) == 2 and lq.decode_launches(part) == 1
     kw = dict(r=0, smooth=0, state_bf16=1) if bf16 else dict(r=r)
     wl = synth.Workload("one", B, HEADS, 2, W=W, gate=gate, rec16=rec16, seed=900 + W, **kw)
     S = torch.randn((B, HEADS, 128, 128), generator=torch.Generator("cuda").manual_seed(W), device="cuda")
     st = lq.State(whole)
+    assert lq.step_launches(whole, st) == 2 and lq.step_launches(part, lq.State(part)) == 1
     lq.quantize_state(whole, S, st)
     cuts = [slice(0, few), slice(few, B)]
     parts = []

@@ -15,7 +15,8 @@ pytestmark = pytest.mark.gpu
 
 GATES = [synth.GATE_SCALAR, synth.GATE_DIAG]
 
-# A step of no more heads than SMs is one launch, of more it is two; most chains run at either side of that line.
+# A step of no more heads than SMs is one launch, of more it is two (up to six to an SM; what comes behind: test_gpu_merged.py);
+# most chains run at either side of that line.
 either = lambda few: pytest.mark.parametrize("batch,launches", [(few, 1), (40, 2)])        # (of four heads each)
 
 
@@ -87,7 +88,6 @@ def test_reference_kernels(oracle, gate):
 
 def _run_chain(oracle, wl, steps, init="zero", stagger=False, check_every=1, work=True, launches=None):
     osh, lsh = gu.shapes(wl)
-    assert launches in (None, lq.decode_launches(lsh))
     ost = OState(osh)
     S0 = np.zeros((wl.batch, wl.heads_v, 128, 128), np.float32) if init == "zero" else synth.dense_states(wl, 9)
     oracle.quantize_state(osh, S0, ost)
@@ -98,6 +98,7 @@ def _run_chain(oracle, wl, steps, init="zero", stagger=False, check_every=1, wor
         ost.win_pos[:] = pos
         ost.buf_a[...] = 1.0
         st = gu.state_to_dev(ost, lsh, work=work)
+    assert launches in (None, lq.step_launches(lsh, st))
     o = torch.empty((wl.batch, wl.heads_v, 128), dtype=torch.float32, device="cuda")
     for step in range(steps):
         tok = synth.token_inputs(wl, step)
@@ -195,7 +196,6 @@ def test_largest_supported_shape(oracle, gate, rec16, batch, launches):
     wl = synth.Workload("max", batch, 2, 1, W=64, r=16, gate=gate, seed=490 + rec16, rec16=rec16,
                         delta=0 if (gate == synth.GATE_DIAG and rec16) else 1)
     osh, lsh = gu.shapes(wl)
-    assert lq.decode_launches(lsh) == launches
     ost = OState(osh)
     S0 = synth.dense_states(wl, 3)
     oracle.quantize_state(osh, S0, ost)
@@ -206,6 +206,7 @@ def test_largest_supported_shape(oracle, gate, rec16, batch, launches):
     ost.buf_a[:, :, :n0] = rng.uniform(0.9, 1.0, ost.buf_a[:, :, :n0].shape).astype(np.float16).astype(np.float32)
     ost.win_pos[:] = n0
     st = gu.state_to_dev(ost, lsh)
+    assert lq.step_launches(lsh, st) == launches
     o = torch.empty((wl.batch, wl.heads_v, 128), dtype=torch.float32, device="cuda")
     for step in range(4):
         tok = synth.token_inputs(wl, step)
@@ -239,12 +240,12 @@ def test_steps_captured_in_a_cuda_graph_replay_identically(batch, launches):
     replayed must leave the same state and outputs as the same steps issued directly."""
     wl = synth.Workload("cg", batch, 4, 2, W=4, r=2, seed=497)
     _, lsh = gu.shapes(wl)
-    assert lq.decode_launches(lsh) == launches
     S0 = gu.dev(synth.dense_states(wl, 4))
     toks = [gu.tok_dev(synth.token_inputs(wl, t)) for t in range(4)]
     outs = {}
     for mode in ("direct", "graph"):
         st = lq.State(lsh)
+        assert lq.step_launches(lsh, st) == launches
         lq.quantize_state(lsh, S0, st)
         o = torch.zeros((4, wl.batch, wl.heads_v, 128), dtype=torch.float32, device="cuda")
         stream = torch.cuda.Stream()

@@ -153,7 +153,8 @@ def test_staggered_chain_against_the_plain_definition(oracle, oracle_plain, gate
         wl = synth.config("kda_b128_outlier").with_(batch=batch, heads_v=8, heads_qk=8)
     else:
         wl = synth.config("gdn_b256").with_(batch=batch, heads_v=8, heads_qk=4)
-    assert lq.decode_launches(gu.shapes(wl)[1]) == launches
+    sh = gu.shapes(wl)[1]
+    assert lq.step_launches(sh, lq.State(sh)) == launches
     _teacher_forced_chain(oracle, oracle_plain, wl, 2 * wl.W + 3, name)
 
 

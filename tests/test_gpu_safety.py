@@ -48,8 +48,8 @@ def _guarded_state(sh):
 def test_no_entry_point_writes_outside_its_buffers(gate, batch, heads_v, heads_qk, W, r, rec16, launches):
     wl = synth.Workload("guard", batch, heads_v, heads_qk, W=W, r=r, gate=gate, rec16=rec16, seed=900 + W + r)
     _, sh = gu.shapes(wl)
-    assert lq.decode_launches(sh) == launches
     st, g = _guarded_state(sh)
+    assert lq.step_launches(sh, st) == launches
     S_in = Guarded((batch, heads_v, 128, 128), torch.float32)
     S_in.t.copy_(gu.dev(synth.dense_states(wl, 2)))
     S_out = Guarded((batch, heads_v, 128, 128), torch.float32)
@@ -85,8 +85,8 @@ def test_checkpoint_in_mid_window_resumes_bit_for_bit(gate, rec16, batch, launch
     the copy must produce the same outputs and end in the same state, bit for bit."""
     wl = synth.Workload("ckpt", batch, 4, 2, W=8, r=4, gate=gate, rec16=rec16, seed=950 + gate + 2 * rec16)
     _, sh = gu.shapes(wl)
-    assert lq.decode_launches(sh) == launches
     st = lq.State(sh)
+    assert lq.step_launches(sh, st) == launches
     lq.quantize_state(sh, gu.dev(synth.dense_states(wl, 5)), st)
     # stagger the windows a little: the first three sequences take one token more than the others
     o = torch.empty((wl.batch, wl.heads_v, 128), dtype=torch.float32, device="cuda")

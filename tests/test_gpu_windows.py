@@ -28,6 +28,7 @@ def test_every_fill_of_a_window(oracle, gate, W, rec16, state_bf16):
     ost.buf_u[...] = half(rng.standard_normal(ost.buf_u.shape))
     ost.buf_a[...] = half(rng.uniform(0.9, 1.0, ost.buf_a.shape))
     st = gu.state_to_dev(ost, lsh)
+    assert lq.step_launches(lsh, st) == (1 if W == 2 else 2)
     o = torch.empty((W, 8, 128), dtype=torch.float32, device="cuda")
     for step in range(2):
         tok = synth.token_inputs(wl, step)
@@ -45,7 +46,6 @@ def test_bf16_state_several_heads_per_cta(oracle, gate, W, rec16):
     state is multiplied, so every lane must be through with the rows before; every fill of a window, a boundary included."""
     wl = synth.Workload("bfmany", 60, 48, 16, W=W, gate=gate, rec16=rec16, r=0, smooth=0, state_bf16=1, seed=880 + W)
     osh, lsh = gu.shapes(wl)
-    assert lq.decode_launches(lsh) == 2
     ost = OState(osh)
     oracle.quantize_state(osh, synth.dense_states(wl, 3), ost)
     rng = np.random.default_rng(W)
@@ -55,6 +55,7 @@ def test_bf16_state_several_heads_per_cta(oracle, gate, W, rec16):
     ost.buf_u[...] = half(rng.standard_normal(ost.buf_u.shape, dtype=np.float32))
     ost.buf_a[...] = half(rng.uniform(0.5, 1.0, ost.buf_a.shape))
     st = gu.state_to_dev(ost, lsh)
+    assert lq.step_launches(lsh, st) == 2
     o = torch.empty((wl.batch, wl.heads_v, 128), dtype=torch.float32, device="cuda")
     for step in range(2):
         tok = synth.token_inputs(wl, step)
