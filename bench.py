@@ -458,6 +458,7 @@ def run_cuda(args, wl):
     ms_per_step = ms / args.steps
     hs = world * heads * args.steps / (ms / 1e3)
     launches = lq.step_launches(sh, st)
+    two = launches == 2                      # else one kernel takes tokens and boundaries, and the profiled entry point is another path
     peak, peak_src = peaks()
     group = wl.heads_v // wl.heads_qk
     bytes_hs = algorithmic_bytes_per_head_step(wl.W, wl.r, wl.gate == synth.GATE_DIAG, group, wl.rec16)
@@ -470,11 +471,13 @@ def run_cuda(args, wl):
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": None, "peak_source": peak_src,
                 "kernel": "one step = decode_kernel + boundary_kernel (algorithmic bytes of both over the step time "
-                          "of the timed region; the decode kernel carries 93 % of the bytes)",
+                          "of the timed region; the decode kernel carries 93 % of the bytes)" if two else
+                          "one step = one launch that takes tokens and window boundaries (algorithmic bytes of both over the "
+                          "step time of the timed region)",
                 "algorithmic_bytes_per_head_step": bytes_hs, "algorithmic_bytes_per_step": heads * bytes_hs,
                 "frac_of_nominal_8TBps": achieved / 8000.0}
     cold, warm = captured_traffic(wl, NCU_TRAFFIC_BYTES_PER_LAUNCH), captured_traffic(wl, NCU_TRAFFIC_WARM_BYTES_PER_LAUNCH)
-    if kern:
+    if kern and two:
         dk, bk = kern["decode_ms"], kern["boundary_ms"]
         roofline["kernels"] = {
             "decode_kernel": {"ms": dk, "algorithmic_bytes": decode_bytes, "achieved": decode_bytes / dk / 1e6,
@@ -488,8 +491,8 @@ def run_cuda(args, wl):
                    kern["steps"]}
     # ncu's DRAM bytes of one step: only for the workload the capture was taken on (profiles/), else null
     t_d, t_b = cold["decode_kernel"], cold["boundary_kernel"]
-    roofline["traffic"] = (t_d + t_b) if (t_d and t_b) else None
-    roofline["traffic_warm_caches"] = sum(warm.values()) if all(warm.values()) else None
+    roofline["traffic"] = (t_d + t_b) if (two and t_d and t_b) else None
+    roofline["traffic_warm_caches"] = sum(warm.values()) if two and all(warm.values()) else None
 
     # speed baselines in the same run: dense fp32 / bf16 state, read and written every token
     base = {}
