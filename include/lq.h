@@ -115,10 +115,11 @@ typedef struct {
  * win_pos: int32 [B], records buffered per sequence, 0..W-1 between calls.  Bits 16 and up are used as a
  *     scratch counter while a call runs and are zero again when it has finished.
  * work: optional (may be null): int32 [LQ_WORK_WORDS], all zero when the state is created and zero again after
- *     every call.  With it, lq_decode_step takes tokens and window boundaries of many shapes in one launch instead of two, and the decode kernel of lq_decode_step hands out the heads of its last, partial round
- *     (B*Hv heads over the CTAs that are resident at once) to the CTAs that get there first, instead of giving
- *     every CTA the same number of heads: on a GPU whose memory system does not serve all SMs alike, equal shares
- *     do not take equal time.  Results are the same bit for bit either way.  Sub-batches of one state that are
+ *     every call.  With it, lq_decode_step takes tokens and window boundaries of many shapes in one launch instead
+ *     of two, and the decode kernel of the others hands out the heads of its last, partial round (B*Hv heads over
+ *     the CTAs that are resident at once) to the CTAs that get there first, instead of giving every CTA the same
+ *     number of heads: on a GPU whose memory system does not serve all SMs alike, equal shares do not take equal
+ *     time.  Results are the same bit for bit either way.  Sub-batches of one state that are
  *     addressed by pointer offset may share one `work` as long as their calls do not run at the same time (calls
  *     in one stream never do).  After a call that returned LQ_ERR_CUDA the words are to be zeroed again (and the
  *     state restored from a checkpoint: a step that was enqueued in part leaves neither valid).
@@ -157,7 +158,7 @@ lq_status lq_decode_step(const lq_shape *shape, const lq_state *state, const uin
  * lq_decode_step for a measuring harness: the same results, and in addition the CUDA event `event_between`
  * (a cudaEvent_t created by the caller; may be null) is recorded on `stream` between the decode kernel and
  * the window-boundary kernel, so that the two can be timed separately.  With an event the step is always these
- * two launches, also where lq_decode_step makes one of both (lq_decode_launches).
+ * two launches, also where lq_decode_step makes one of both (lq_step_launches).
  */
 lq_status lq_decode_step_profiled(const lq_shape *shape, const lq_state *state, const uint16_t *q, const uint16_t *k,
                                   const uint16_t *v, const uint16_t *beta, const uint16_t *alpha, float *o,
@@ -322,8 +323,9 @@ lq_status lq_selftest_bounded_wait(lq_stream stream);
 /* LQ_STATIC_STAGE_BYTES as the loaded library was built with (for bindings that cannot read the macro). */
 uint64_t lq_static_stage_bytes(void);
 
-/* Kernels one lq_decode_step call launches for `shape` on a state without scratch words, which is the most it launches; and for
- * `state` as it is, which may be one where that is two (used to report launch counts; both 0 for an invalid shape). */
+/* Kernels one lq_decode_step call launches (used to report launch counts; both 0 for an invalid shape):
+ * lq_decode_launches: for `shape` on a state without scratch words, which is the most it launches;
+ * lq_step_launches: on `state` as it is, which may be one where that is two. */
 int lq_decode_launches(const lq_shape *shape);
 int lq_step_launches(const lq_shape *shape, const lq_state *state);
 

@@ -360,8 +360,8 @@ __device__ __forceinline__ int nth_set_bit(uint32_t m, unsigned k) {
 // The CTA lists up to 32 of its heads in one pass over win_pos: due heads number first, first + stride, ..., `todo_bh` and
 // `todo_n` the head and its buffered records.  What bounds it is the round trip of the loads, of which a lane has eight in flight,
 // and where few are due, the instructions, which a CTA fetches for itself: up to 256 sequences warp 0 does it alone, in one
-// trip; more of them take all eight warps, 2048 sequences to a trip, warp w those with w in bits 5 to 7 of their index.
-// W = 16, us per step with one warp at all sizes / as it is: 512 x 2 heads 22.6 / 18.7, 1024 x 8 66.7 / 61.7, 8192 x 1 141 / 66,
+// trip; more of them take all NW warps of the CTA, 256 NW sequences to a trip, warp w those whose index / 32 is w modulo NW.
+// W = 16, eight warps, us per step with one warp at all sizes / as it is: 512 x 2 heads 22.6 / 18.7, 1024 x 8 66.7 / 61.7, 8192 x 1 141 / 66,
 // 32768 x 1 644 / 246; with eight warps at all sizes 32 x 32 heads take 18.7 instead of 18.4.
 // Called by the `warps` first warps (due_scan_warps).  Returns how many heads are listed.  `lead`: a due sequence among those
 // this warp looks at, the same for the warp of this number in every CTA (-1: none).  `counts`: shared memory.  Ends without a

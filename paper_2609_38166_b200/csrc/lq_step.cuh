@@ -57,7 +57,6 @@ struct StepSlot {
 };
 // what the warps of a CTA share
 struct StepShared {
-  unsigned seqs_normal, seqs_due;
   unsigned turn_items, pool;                 // items handed out in turn, and those drawn
   unsigned due_first, due_mine;              // this CTA's first due item, and how many it has (gridDim apart)
   unsigned due_taken, flushed;               // how many of them a pair has taken, and how many are through their boundary

@@ -147,8 +147,9 @@ class State:
     def __init__(self, sh: Shape, device="cuda", storage=None, work=True):
         """``storage``: optionally the four tensors (heads, records, decays, win_pos) to use instead of fresh
         ones - contiguous, of the shapes and dtypes below (callers that place the state in memory of their own).
-        ``work``: give the state the ``work`` words (LQ_WORK_WORDS) with which the decode kernel hands out the heads
-        of its last round to the CTAs that get there first; without them every CTA takes the same number."""
+        ``work``: give the state the ``work`` words (LQ_WORK_WORDS).  With them a step of many shapes is one launch instead
+        of two (``step_launches``), and the decode kernel of the others hands out the heads of its last rounds to the CTAs that
+        get there first; without them every CTA takes the same number."""
         B, H, K, V, W, r = sh.batch, sh.heads_v, sh.d_k, sh.d_v, sh.W, sh.r
         self.shape = sh
         self.work = torch.zeros((8,), dtype=torch.int32, device=device) if work else None
