@@ -602,6 +602,13 @@ __global__ void __launch_bounds__(256) gather_kernel(const GatherSegs g) {
   }
 }
 
+// About five microseconds ahead of a decode kernel, in which the next sub-batch's gather gets its places (see below).  With an empty kernel
+// in its place the decode kernel is launched early behind it, and the order is as before.
+__global__ void head_start_kernel() {
+  const long long t0 = clock64();
+  for (int i = 0; i < 4096 && clock64() - t0 < 10000; i++) __nanosleep(100);
+}
+
 // The device alias of a pinned, mapped host pointer; null if the memory is not mapped into the device.
 template <typename T>
 T *device_alias(T *host) {
@@ -836,6 +843,19 @@ lq_status lq_decode_step_host_pipelined(const lq_shape *shape, const lq_state *s
     const uint64_t b0 = lo[c], nb = lo[c + 1] - lo[c];
     if (nb == 0) continue;
     ok = cudaStreamWaitEvent(st, hp->in[c], 0) == cudaSuccess;
+    // The end of a gather lets both go, this sub-batch's decode kernel and the next one's gather, and which of them is first decides how the
+    // call goes, and changed with every build of the library: decode CTAs fill every SM, so a gather behind them waits until the first of them
+    // leave (20 us), and then shares SMs with the others, whose loads queue up behind its reads over the bus (that decode kernel takes 43 us
+    // instead of 28).  So a long gather gets a head start.  us of a call by itself and back to back with those of other states, without (two builds) and
+    // with: 256 x 32 heads 216 - 224, 183 - 204 / 201, 183; 180 x 32 179, 144 - 167 / 161, 143; 512 x 32 408, 342 - 396 / 357, 338; diagonal gate 128 x 32
+    // 168, 153 / 160, 144, 96 x 32 147, 130 / 136, 118; chained 256 x 32 150 - 165 / 160, 96 x 32 105 - 110 / 99.  Not below 1.25 MB a sub-batch (128 x 32 124, 106 - 113 / 129,
+    // 115), not for the BF16 state, whose decode kernel needs the SMs more (199, 184 / 216, 199), and not in long chained calls (512 x 32 302 / 321).
+    uint64_t next_bytes = 0;
+    for (int i = 0; c + 1 < PIPE_CHUNKS && i < 5; i++) next_bytes += 2 * (lo[c + 2] - lo[c + 1]) * per_seq[i];
+    if (ok && mapped && !shape->state_bf16 && next_bytes >= 1250000 && (!chained || next_bytes < 4000000)) {
+      head_start_kernel<<<1, 32, 0, st>>>();
+      ok = cudaGetLastError() == cudaSuccess;
+    }
     if (!ok) break;
     lq_shape sub = *shape;
     sub.batch = static_cast<int>(nb);
