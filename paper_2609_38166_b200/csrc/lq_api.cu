@@ -450,7 +450,11 @@ static lq_status launch_step(const lq_shape *s, const Params &p, cudaStream_t st
 //     48 x 32, W = 16 19.0 / 19.2 (20.7 / 21.5); 64 x 32, W = 16 25.8 / 22.4 (27.4 / 24.6); 128 x 32, W = 32 43.3 / 31.2 (44.5 / 33.9)
 //   diagonal gate: 32 x 32, W = 16 18.3 / 17.7 (19.3 / 21.1); 64 x 32, W = 16 27.6 / 24.5 (29.9 / 27.7); 128 x 32, W = 32 54.6 / 42.2 (56.7 / 44.7)
 // Not where every head has a CTA of the decode kernel to itself (six to an SM): 20 x 16 heads, W = 16 14.7 / 14.1 (14.9 / 18.7), diagonal gate
-// 14.2 / 14.7 (14.7 / 20.9); 24 x 32 15.7 / 15.9 (16.6 / 18.9).  A boundary of several rounds is more code and longer: from twice as many heads on.  32 x 32,
+// 14.2 / 14.7 (14.7 / 20.9); 24 x 32 15.7 / 15.9 (16.6 / 18.9).  A boundary of several rounds is more code and longer: from twice as many heads on, or
+// where two SMs of three have a due head: a loop of steps gains up to a quarter then, steps behind other kernels lose up to a fifth.
+// Two rounds, r = 4, two / one: 32 x 32, W = 8 24.3 / 18.6 (25.8 / 27.3), W = 10 21.1 / 19.0 (24.8 / 27.3), W = 7 24.3 / 23.9 (26.7 / 32.6), r = 8,
+// W = 8 35.7 / 27.6 (37.7 / 43.5); 48 x 32, W = 12 26.3 / 21.9 (30.3 / 28.4), W = 15 23.3 / 22.5 (27.0 / 30.4); diagonal gate, 32 x 32, W = 8
+// 24.2 / 19.2 (27.5 / 29.1), 48 x 32, W = 12 28.2 / 23.1 (32.0 / 31.6).  With fewer due, 32 x 32,
 // W = 16, r = 4, two rounds 20.9 / 20.1 (21.9 / 26.9); 48 x 32 22.2 / 22.8 (22.9 / 26.8); 64 x 32 29.8 / 26.2 (31.4 / 29.8), r = 8 41.2 / 33.8 (42.4 / 45.5);
 // 128 x 32, W = 32 47.7 / 34.8 (48.8 / 37.5).
 // With more than one due head to an SM they go through their boundaries one after the other, which takes as long as two at a time in a kernel of
@@ -471,7 +475,7 @@ static bool launch_merged_t(const lq_shape *s, const Params &p, cudaStream_t str
   while (pairs > 0 && bytes(pairs) > 226 * 1024) pairs--;
   if (pairs < STEP_PAIRS - 1) return false;
   const long nh = (long)s->batch * s->heads_v, sms = sm_count();
-  if (nh <= (ROUNDS ? 12 : 6) * sms) return false;
+  if (nh <= 6 * sms || (ROUNDS && nh <= 12 * sms && 3 * nh <= 2 * sms * s->W)) return false;
   if (nh > sms * s->W && !(GATE == LQ_GATE_SCALAR && s->W >= 24 && pairs == STEP_PAIRS)) return false;
   if (launch) *rc = launch_dependent(step_kernel<GATE, RM, EXACT, ROUNDS>, static_cast<int>(sms), STEP_THREADS, bytes(pairs), stream, p, pairs);
   return true;
